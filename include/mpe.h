@@ -90,9 +90,10 @@ int mpe_reserve(mpe_handle* h, int32_t max_batch, int64_t max_total_indices);
  *   d_offsets[T*batch+1]      non-decreasing, first 0, last total_indices.
  *   d_out[batch][T*dim]       FP32, row-major; bag (t,b) lands in d_out[b][t*dim .. (t+1)*dim);
  *                             an empty bag gives zeros; rows are added in index order starting from +0.
- * The call sorts and de-duplicates the indices (Section 5.1), probes the cache tags, gathers FP32
+ * The call looks up where each row lives, gathers FP32
  * rows on hits and dequantizes (q*scale+bias, Algorithm 1) on misses.  It reads but never changes
- * table, cache or policy state.  Work is enqueued on `cuda_stream` (a cudaStream_t; NULL = the
+ * table, cache or policy state.  It records the batch for the backward that may follow, which sorts and
+ * de-duplicates it (Section 5.1); a forward alone does not.  Work is enqueued on `cuda_stream` (a cudaStream_t; NULL = the
  * default stream) and the call returns without waiting.  Row ids outside [0, num_rows) contribute
  * nothing and raise the sticky MPE_ERR_INDEX.
  */
@@ -100,12 +101,12 @@ int mpe_forward(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offset
                 int64_t total_indices, float* d_out, void* cuda_stream);
 
 /*
- * Optional: start on the NEXT batch while the current step still runs.  The first part of a forward pass -- sorting the
+ * Optional: start on the NEXT batch while the current step still runs.  The first part of a step's backward -- sorting the
  * indices and merging duplicates (Section 5.1) -- needs the indices only, not the tables, the cache or the policy state,
  * and its kernels leave most of the GPU idle.  mpe_prepare enqueues that part for the given batch on `cuda_stream`
  * (any stream on which the indices and offsets are ready; typically not the stream of the training step) into a second
  * workspace of the handle.  A later mpe_forward / mpe_forward_routed with the same d_indices, d_offsets, batch and
- * total_indices takes the result over (it waits for it on its own stream) and only looks up the tags and pools;
+ * total_indices takes the result over (its backward waits for the sort on its own stream) and only pools;
  * results are bit-identical with and without the call.  Layouts as in mpe_forward; the two buffers must stay
  * unchanged until that forward.  One batch can be prepared at a time; a forward with other arguments discards it.
  * The call does nothing (and returns MPE_OK) when the batch does not fit the workspace reserved with mpe_reserve, or
@@ -204,21 +205,17 @@ int mpe_step_host_wait(mpe_handle* h);
  * does.)
  *
  * Same inputs, outputs, layouts and result as mpe_forward -- the pooled FP32 sums of the bags, bit for bit
- * -- but every intermediate array of the step (sort keys and payloads, digit counts, per-tile words, the
- * distinct-row list and its maps) lives in ONE fixed array compiled into the library
- * (`static __device__`, about 2.5 MB; every GPU that loads the library holds it until the process exits).
+ * -- but the little device memory it needs lives in ONE fixed array compiled into the library
+ * (`static __device__`; every GPU that loads the library holds it until the process exits).
  * Limits: total_indices <= MPE_STATIC_MAX_INDICES, num_tables * batch <= MPE_STATIC_MAX_BAGS,
  * num_tables <= MPE_STATIC_MAX_TABLES; a larger call returns MPE_ERR_TOO_LARGE and does nothing.
  * It calls no cudaMalloc / cudaFree and no allocating library routine.
  *
- * It is an evaluation forward: it never changes the tables, the cached rows, the tags or the priority values
- * (the only handle memory it writes are the per-slot marks "hit in forward call number e", which every forward
- * rewrites under a fresh call number before anything reads them) and cannot be followed by mpe_backward; calling it between the mpe_forward and mpe_backward of a training step returns
+ * It is an evaluation forward: it writes no memory of the handle and cannot be followed by mpe_backward; calling it between the mpe_forward and mpe_backward of a training step returns
  * MPE_ERR_SEQUENCE.  Out-of-range row ids contribute nothing and inconsistent offsets give all-zero
  * output, as in mpe_forward, but this entry point does not record them for mpe_last_error.
  *
- * All calls, from every handle on that GPU, share the one array, and it keeps the previous call's
- * contents (the call clears the counters it needs at zero): two calls whose GPU work overlaps -- different
+ * All calls, from every handle on that GPU, share the one array: two calls whose GPU work overlaps -- different
  * streams, or different handles -- race on it.  Issue them on one stream, or wait between them.
  * The first call on each device looks up the array's device address (cudaGetSymbolAddress); make that
  * first call outside any stream capture.  The look-up is guarded by a lock, so first calls may come from
@@ -286,11 +283,10 @@ int mpe_export_cache(mpe_handle* h, int32_t table, int32_t* h_tags, float* h_row
 int mpe_export_aux(mpe_handle* h, int32_t table, const int64_t* h_rows, int64_t n, uint32_t* h_cnt,
                    float* h_adagrad);
 
-/* Steps of up to about four million indices are bound by kernel-launch latency, so by default each half of
- * the step is captured once into a CUDA graph (sized for the reserved workspace) and replayed; the per-call
+/* Steps of up to about four million indices are bound by kernel-launch latency, so by default the
+ * backward is captured once into a CUDA graph (sized for the reserved workspace) and replayed (a forward is one kernel); the per-call
  * arguments reach the kernels through device memory.  enable = 0 switches to plain launches (larger steps and
- * steps issued while profiling or while the caller captures the stream always use plain launches).  A backward
- * is replayed only if its forward was.  Not allowed between a forward and its backward (MPE_ERR_SEQUENCE).
+ * steps issued while profiling or while the caller captures the stream always use plain launches).  Not allowed between a forward and its backward (MPE_ERR_SEQUENCE).
  * A graph the CALLER captured around steps of this library may be replayed about 10^8 times in a row: the pass
  * numbers in the sort's per-tile words (30 bits) are started over by mpe_forward's host code, which counts the calls
  * it sees, not by the captured kernels.  For more replays, every 10^8 of them call

@@ -45,6 +45,7 @@ struct mpe_handle {
     uint64_t sort_passes_bound = 0;                        // no more than this many sort passes have run on either workspace
     std::vector<void*> ws_allocs;
     cudaEvent_t ev_free = nullptr;          // recorded behind the last kernel that uses this workspace
+    cudaEvent_t ev_keys = nullptr, ev_prep = nullptr;      // of a batch sorted ahead in it: its indices have been read; it is sorted
     // A second workspace, allocated on the first mpe_prepare: the next batch is sorted and de-duplicated there while the
     // kernels of the current step still run.  `alt` holds exactly the members above that belong to a workspace.
     struct WsSet {
@@ -52,14 +53,14 @@ struct mpe_handle {
         uint32_t *sortA = nullptr, *sortB = nullptr, *ghist = nullptr, *block_sums = nullptr;
         unsigned long long* sort_status = nullptr; SortCtl* sort_ctl = nullptr;
         int64_t sort_n = 0;
-        const uint32_t *skey = nullptr, *spos = nullptr;
+        const uint32_t *skey = nullptr;
         std::vector<void*> allocs;
-        cudaEvent_t ev_free = nullptr;
+        cudaEvent_t ev_free = nullptr, ev_keys = nullptr, ev_prep = nullptr;
         uint64_t bytes = 0;
     } alt;
     bool prepared = false;                  // `alt` holds a sorted batch that the next forward may take over
     StepArgs prep_args{};                   // ... of these inputs
-    cudaEvent_t ev_prep = nullptr;
+    bool prep_running = false;              // the current workspace's batch was sorted ahead and ev_prep has not been waited for yet
     cudaStream_t prep = nullptr;            // mpe_step_host_submit prepares on this stream
     // staging for mpe_step_host / mpe_step_host_submit: two slots, so that the copies of one step run next to the kernels of another
     struct HostSlot {
@@ -75,21 +76,21 @@ struct mpe_handle {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStream_t copy_in = nullptr, copy_out = nullptr;   // mpe_step_host: host<->device copies next to the kernels
     bool have_forward = false;
-    bool fwd_replayed = false;              // the pending forward ran as a graph replay, so the device copy of its arguments is current
     int64_t last_step = 0;
     uint64_t steps = 0;
     uint32_t epoch = 0;
     int32_t B = 0; int64_t L = 0;
-    const uint32_t *skey = nullptr, *spos = nullptr;
+    const uint32_t* skey = nullptr;         // the sorted keys of the current batch
+    bool chain_done = false;                // the current batch has been sorted and its distinct rows are known
     StepArgs args{};                        // the current call's arguments (passed by value when launching directly)
     Route* d_route = nullptr;               // destinations of the pooled vectors when the tables are spread over several GPUs
-    // CUDA graphs of the two halves of a step (small batches are launch-latency bound)
+    // CUDA graph of a backward (small batches are launch-latency bound; a forward is one kernel)
     bool graphs_enabled = true;
     cudaStream_t cap = nullptr;             // stream the step is captured on
-    cudaGraph_t g_fwd = nullptr, g_bwd = nullptr;
-    cudaGraphExec_t x_fwd = nullptr, x_bwd = nullptr;
-    cudaGraphNode_t n_fwd = nullptr, n_bwd = nullptr;      // the nodes that write the per-call arguments
-    uint64_t k_fwd = 0, k_bwd = 0;                         // kernel nodes per graph
+    cudaGraph_t g_bwd = nullptr;
+    cudaGraphExec_t x_bwd = nullptr;
+    cudaGraphNode_t n_bwd = nullptr;        // the node that writes the per-call arguments
+    uint64_t k_bwd = 0;                     // kernel nodes of the graph
     // instrumentation
     uint64_t launches = 0;
     bool profiling = false;
@@ -165,11 +166,9 @@ int dmalloc(mpe_handle* h, T** p, int64_t n, std::vector<void*>* track) {
 }
 
 void drop_graphs(mpe_handle* h) {
-    if (h->x_fwd) cudaGraphExecDestroy(h->x_fwd);
     if (h->x_bwd) cudaGraphExecDestroy(h->x_bwd);
-    if (h->g_fwd) cudaGraphDestroy(h->g_fwd);
     if (h->g_bwd) cudaGraphDestroy(h->g_bwd);
-    h->x_fwd = h->x_bwd = nullptr; h->g_fwd = h->g_bwd = nullptr; h->n_fwd = h->n_bwd = nullptr;
+    h->x_bwd = nullptr; h->g_bwd = nullptr; h->n_bwd = nullptr;
 }
 
 // the current workspace and the other one change places
@@ -179,9 +178,9 @@ void swap_sets(mpe_handle* h) {
     std::swap(h->ghist, h->alt.ghist); std::swap(h->block_sums, h->alt.block_sums);
     std::swap(h->sort_status, h->alt.sort_status); std::swap(h->sort_ctl, h->alt.sort_ctl);
     std::swap(h->sort_n, h->alt.sort_n);
-    std::swap(h->skey, h->alt.skey); std::swap(h->spos, h->alt.spos);
+    std::swap(h->skey, h->alt.skey);
     std::swap(h->ws_allocs, h->alt.allocs);
-    std::swap(h->ev_free, h->alt.ev_free);
+    std::swap(h->ev_free, h->alt.ev_free); std::swap(h->ev_keys, h->alt.ev_keys); std::swap(h->ev_prep, h->alt.ev_prep);
     std::swap(h->ws_bytes, h->alt.bytes);
 }
 
@@ -263,13 +262,11 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags) {
     A(h->block_sums, n / std::min<int64_t>(SCAN_TILE, PRI_CHUNK) + 2);
     A(w.ctr, 1); A(w.args, 1);
     A(w.table_start, T + 1); A(w.tile_base, T + 1); A(w.ustart, T + 1); A(w.ctile_base, T + 1);
-    A(w.bag_of, n); A(w.kidx, n); A(w.occ_loc, n); A(w.occ_b, n);
+    A(w.occ_b, n);
     A(w.uniq_row, nu); A(w.uniq_t, nu); A(w.seg, nu + 1); A(w.loc, nu); A(w.final_loc, nu);
-    A(w.hot_base, nu); A(w.uset, nu); A(w.cand_key, nu); A(w.cand_cnt, T); A(w.cstart, T + 1);
+    A(w.victim, nu); A(w.defer_k, nu); A(w.heads, nu);
+    A(w.hot_base, nu); A(w.cand_key, nu); A(w.cand_cnt, T); A(w.cstart, T + 1);
     CK(h, cudaMemset(w.cand_cnt, 0, sizeof(int32_t) * T));
-    // written and read by backward only, at most one entry per distinct row: they take the place of per-index arrays
-    // that only forward uses
-    w.victim = w.bag_of; w.defer_k = reinterpret_cast<int32_t*>(w.kidx); w.heads = w.occ_loc;
     const int64_t max_tasks = hot_capacity(L);
     A(w.task_k, max_tasks); A(w.partial, max_tasks * h->dim); A(w.hot_k, max_tasks);
 #undef A
@@ -277,47 +274,44 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags) {
     return MPE_OK;
 }
 
-// The sort's memory: two buffers of 2 * n words each.  The keys to sort are expected in the first n words of B
-// (sort_input()); between passes the elements are (key, payload) records that alternate between A and B; the last
-// pass leaves the sorted keys in the first n words and the sorted payloads in the second n words of its buffer.
+// The sort's memory: two buffers of 2 * n words each.  The (key, payload) records to sort are expected in B (sort_input());
+// between passes they alternate between A and B; the last pass leaves the sorted keys in the first n words of its buffer and
+// the sorted payloads wherever the caller wants them.
 struct SortBufs { uint32_t *A, *B; int64_t n; uint32_t* ghist; unsigned long long* status; SortCtl* ctl; uint32_t* abort_flag; int tile; };
-uint32_t* sort_input(const SortBufs& b) { return b.B; }
+uint2* sort_input(const SortBufs& b) { return reinterpret_cast<uint2*>(b.B); }
+SortBufs sort_bufs(const mpe_handle* h) {
+    return SortBufs{h->sortA, h->sortB, h->sort_n, h->ghist, h->sort_status, h->sort_ctl, &h->wk.ctr->abort, h->wk.sort_tile};
+}
 
-// stable sort of every segment [seg_start[t], seg_start[t+1]) by the low `key_bits` bits of the key, the payload being
-// the element's position before the sort; *skey / *sval receive where the sorted keys / payloads are
+// stable sort of every segment [seg_start[t], seg_start[t+1]) by the low `key_bits` bits of the key; *skey receives where the
+// sorted keys are.  The sorted payloads go to `vals`, or (vals == nullptr) behind the keys, and *sval receives where.
 // tile_base: the segments' tile bookkeeping (warp_tile_bases), filled by the kernel that produced seg_start
 void seg_sort(mpe_handle* h, const SortBufs& b, const int32_t* seg_start, const int32_t* tile_base,
-              int key_bits, int64_t n_upper, const uint32_t** skey, const uint32_t** sval, bool input_pairs = false) {
+              int key_bits, int64_t n_upper, uint32_t* vals, const uint32_t** skey, const uint32_t** sval) {
     const int T = h->T;
     const int64_t max_tiles = (n_upper + b.tile - 1) / b.tile + T;
     const int passes = (key_bits + 7) / 8;
     const int split = b.tile == sort_tile(true) ? 4 : 1;         // pieces of a tile the digit count hands to its warps
     const int gh = grid_for(h, max_tiles * split, SORT_THREADS / 32, 4);
-    if (input_pairs) LAUNCH(h, "sort_digits", k_sort_digits<true>, gh, SORT_THREADS, 0, (const uint32_t*)b.B, seg_start, tile_base, T, passes, b.ghist, b.tile, split);
-    else LAUNCH(h, "sort_digits", k_sort_digits<false>, gh, SORT_THREADS, 0, (const uint32_t*)b.B, seg_start, tile_base, T, passes, b.ghist, b.tile, split);
+    LAUNCH(h, "sort_digits", k_sort_digits, gh, SORT_THREADS, 0, (const uint2*)sort_input(b), seg_start, tile_base, T, passes, b.ghist, b.tile, split);
     for (int p = 0; p < passes; ++p) {
-        const bool first = p == 0 && !input_pairs, last = p == passes - 1;    // input_pairs: B holds (key, payload) records already
+        const bool last = p == passes - 1;
         uint32_t* src = (p & 1) ? b.A : b.B;                      // pass p reads B and writes A when p is even, the other way round when odd
         uint32_t* dst = (p & 1) ? b.B : b.A;
-        const uint32_t* kin = src; const uint2* pin = reinterpret_cast<const uint2*>(src);
-        uint2* pout = reinterpret_cast<uint2*>(dst); uint32_t* ok = dst; uint32_t* ov = dst + b.n;
+        const uint2* pin = reinterpret_cast<const uint2*>(src);
+        uint2* pout = reinterpret_cast<uint2*>(dst); uint32_t* ok = dst; uint32_t* ov = vals ? vals : dst + b.n;
         // tiles are handed out by ticket, so the grid only has to be large enough to fill the GPU
-#define SCATTER(F, L) do { \
-        if (b.tile == sort_tile(true)) { \
-            auto kern = k_sort_scatter<F, L, SORT_ITEMS_SMALL>; \
-            LAUNCH(h, "sort_scatter", kern, grid_for(h, max_tiles, 1, resident_blocks(h, kern, SORT_THREADS, 0)), SORT_THREADS, 0, kin, pin, pout, ok, ov, \
-                   seg_start, tile_base, T, p, b.ghist, b.status, b.ctl, b.abort_flag); \
-        } else { \
-            auto kern = k_sort_scatter<F, L, SORT_ITEMS_LARGE>; \
-            LAUNCH(h, "sort_scatter", kern, grid_for(h, max_tiles, 1, resident_blocks(h, kern, SORT_THREADS, 0)), SORT_THREADS, 0, kin, pin, pout, ok, ov, \
-                   seg_start, tile_base, T, p, b.ghist, b.status, b.ctl, b.abort_flag); \
-        } } while (0)
-        if (first && last) SCATTER(true, true);
-        else if (first) SCATTER(true, false);
-        else if (last) SCATTER(false, true);
-        else SCATTER(false, false);
+#define SCATTER(L, ITEMS) do { \
+        auto kern = k_sort_scatter<L, ITEMS>; \
+        LAUNCH(h, "sort_scatter", kern, grid_for(h, max_tiles, 1, resident_blocks(h, kern, SORT_THREADS, 0)), SORT_THREADS, 0, pin, pout, ok, ov, \
+               seg_start, tile_base, T, p, b.ghist, b.status, b.ctl, b.abort_flag); } while (0)
+        const bool small = b.tile == sort_tile(true);
+        if (last && small) SCATTER(true, SORT_ITEMS_SMALL);
+        else if (last) SCATTER(true, SORT_ITEMS_LARGE);
+        else if (small) SCATTER(false, SORT_ITEMS_SMALL);
+        else SCATTER(false, SORT_ITEMS_LARGE);
 #undef SCATTER
-        if (last) { *skey = dst; *sval = dst + b.n; }
+        if (last) { *skey = dst; if (sval) *sval = ov; }
     }
 }
 
@@ -327,8 +321,7 @@ void dispatch(int bits, int lanes, F&& f) {
 #ifdef MPE_ONLY_BITS        // development builds: one code width and one row width only (much shorter compile)
     (void)bits; (void)lanes;
     f(std::integral_constant<int, MPE_ONLY_BITS>{}, std::integral_constant<int, MPE_ONLY_LANES>{});
-    return;
-#endif
+#else
     auto by_lanes = [&](auto bc) {
         switch (lanes) {
             case 1: f(bc, std::integral_constant<int, 1>{}); break;
@@ -343,6 +336,7 @@ void dispatch(int bits, int lanes, F&& f) {
     else if (bits == 4) by_lanes(std::integral_constant<int, 4>{});
     else if (bits == 2) by_lanes(std::integral_constant<int, 2>{});
     else by_lanes(std::integral_constant<int, 16>{});
+#endif
 }
 
 int check_launch(mpe_handle* h) {
@@ -411,9 +405,9 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
         cudaStreamCreateWithFlags(&h->copy_in, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&h->copy_out, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&h->prep, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->ev_free, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->ev_prep, cudaEventDisableTiming) != cudaSuccess ||
         false) { delete h; return MPE_ERR_CUDA; }
+    for (cudaEvent_t* e : {&h->ev_free, &h->ev_keys, &h->ev_prep, &h->alt.ev_free, &h->alt.ev_keys, &h->alt.ev_prep})
+        if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) { delete h; return MPE_ERR_CUDA; }
     for (auto& sl : h->slot)
         for (cudaEvent_t* e : {&sl.ev_idx, &sl.ev_grad, &sl.ev_fwd, &sl.ev_done, &sl.ev_down})
             if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) { delete h; return MPE_ERR_CUDA; }
@@ -457,10 +451,11 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
         if ((rc = dmalloc(h, &s.codes, h->total_rows * h->code_bytes, nullptr)) != MPE_OK) return fail(rc);
         if (bits != 16 && (rc = dmalloc(h, &s.sb, h->total_rows, nullptr)) != MPE_OK) return fail(rc);   // an FP16 table has no scale/bias
     }
-    if (policy == MPE_LFU && (rc = dmalloc(h, &s.cnt, h->total_rows, nullptr)) != MPE_OK) return fail(rc);
     if (optimizer == MPE_ROWWISE_ADAGRAD && (rc = dmalloc(h, &s.G, h->total_rows, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.slab, h->total_slots * dim, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.tags, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
+    s.home_shift = policy == MPE_LFU ? 1 : 0;
+    if ((rc = dmalloc(h, &s.home, h->total_rows << s.home_shift, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.ts, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.hit_epoch, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.hit_k, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
@@ -468,13 +463,13 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
     if ((rc = dmalloc(h, &s.stats, (int64_t)num_tables * 8, nullptr)) != MPE_OK) return fail(rc);
 #define CKC(expr) do { cudaError_t e_ = (expr); if (e_ != cudaSuccess) { h->last_cuda_error = (int)e_; return fail(MPE_ERR_CUDA); } } while (0)
     CKC(cudaMemcpy(h->d_tables, h->tables.data(), sizeof(TableDev) * num_tables, cudaMemcpyHostToDevice));
-    if (s.cnt) CKC(cudaMemset(s.cnt, 0, sizeof(uint32_t) * h->total_rows));
     if (s.G) CKC(cudaMemset(s.G, 0, sizeof(float) * h->total_rows));
     CKC(cudaMemset(s.slab, 0, sizeof(float) * std::max<int64_t>(1, h->total_slots * dim)));
     if (s.ts) CKC(cudaMemset(s.ts, 0, sizeof(uint32_t) * std::max<int64_t>(1, h->total_slots)));
     CKC(cudaMemset(s.hit_epoch, 0, sizeof(uint32_t) * std::max<int64_t>(1, h->total_slots)));
     CKC(cudaMemset(s.floor, 0, sizeof(uint32_t) * std::max<int64_t>(1, h->total_sets)));
     CKC(cudaMemset(s.stats, 0, sizeof(unsigned long long) * 8 * num_tables));
+    LAUNCH(h, "init_home", k_init_home, grid_for(h, h->total_rows, 256, 8), 256, 0, s, h->total_rows);
     LAUNCH(h, "fill_tags", k_fill_i32, grid_for(h, h->total_slots, 256, 8), 256, 0, s.tags, h->total_slots, -1);
     for (int t = 0; t < num_tables; ++t) {
         const int g = grid_for(h, h->tables[t].N, 256 / s.lanes, 8);
@@ -497,7 +492,7 @@ int mpe_reserve(mpe_handle* h, int32_t max_batch, int64_t max_total_indices) {
     if (max_total_indices <= h->cap_L && bags <= h->cap_bags && h->wk.ctr) return MPE_OK;
     if (h->have_forward) return MPE_ERR_SEQUENCE;     // a pending backward still needs the old workspace
     CK(h, cudaStreamSynchronize(h->stream));
-    if (h->ev_prep) CK(h, cudaEventSynchronize(h->ev_prep));       // so does a batch that is being prepared
+    CK(h, cudaEventSynchronize(h->ev_prep)); CK(h, cudaEventSynchronize(h->alt.ev_prep));       // so does a batch that is being prepared
     return alloc_workspace(h, std::max(max_total_indices, h->cap_L), std::max(bags, h->cap_bags));
 }
 
@@ -505,55 +500,42 @@ int mpe_reserve(mpe_handle* h, int32_t max_batch, int64_t max_total_indices) {
 
 namespace {
 
-// Launch sizes follow L_grid / bags_grid (upper bounds: every kernel walks its range with a grid stride and reads the
+// Launch sizes follow L_grid (an upper bound: every kernel walks its range with a grid stride and reads the
 // true sizes from device memory), so one captured graph serves every batch that fits the workspace.
-// First half of forward, which needs the indices only (no table, cache or policy state): keys, sort, distinct rows.
-void enqueue_index_chain(mpe_handle* h, int64_t L_grid, int64_t bags_grid, bool ind, const StepArgs& av) {
-    const State& s = h->st;
+// What backward needs of the batch and the indices alone decide (no table, cache or policy state): the sorted batch and its
+// distinct rows.  The records to sort are in sort_input().
+void enqueue_index_chain(mpe_handle* h, int64_t L_grid, bool ind) {
     Work& w = h->wk;
-    const int T = h->T;
-    LAUNCH(h, "prelude", (ind ? k_prelude<true> : k_prelude<false>), 1, 32, 0, w, T, av);
-    const SortBufs sb{h->sortA, h->sortB, h->sort_n, h->ghist, h->sort_status, h->sort_ctl, &h->wk.ctr->abort, h->wk.sort_tile};
-    LAUNCH(h, "make_keys", (ind ? k_make_keys<true> : k_make_keys<false>), grid_for(h, bags_grid, 32, 8), 256, 0, s, w, sort_input(sb), av);
     // sort the row indices of the mini-batch (Section 5.1), table by table
-    seg_sort(h, sb, w.table_start, w.tile_base, bits_for((uint32_t)h->max_rows), L_grid, &h->skey, &h->spos);
+    seg_sort(h, sort_bufs(h), w.table_start, w.tile_base, bits_for((uint32_t)h->max_rows), L_grid,
+             reinterpret_cast<uint32_t*>(w.occ_b), &h->skey, nullptr);
     // distinct rows
     const int gs = grid_for(h, L_grid, SCAN_TILE, 8);
     if (ind) {
-        LAUNCH(h, "unique", k_unique, gs, SCAN_THREADS, 0, w, T, h->skey, h->sort_status, h->sort_ctl);
+        LAUNCH(h, "unique", k_unique, gs, SCAN_THREADS, 0, h->st, w, h->skey, h->sort_status, h->sort_ctl);
     } else {
-        LAUNCH(h, "unique_count", k_unique_pass<false>, gs, SCAN_THREADS, 0, w, T, h->skey, h->block_sums);
+        LAUNCH(h, "unique_count", k_unique_pass<false>, gs, SCAN_THREADS, 0, h->st, w, h->skey, h->block_sums);
         LAUNCH(h, "scan_block_sums", k_scan_block_sums, 1, BSUM_THREADS, 0, h->block_sums, (const uint32_t*)&w.ctr->L, (uint32_t)SCAN_TILE, &w.ctr->U);
-        LAUNCH(h, "unique_write", k_unique_pass<true>, gs, SCAN_THREADS, 0, w, T, h->skey, h->block_sums);
-        LAUNCH(h, "ustart", k_ustart, 1, 256, 0, w, T);
+        LAUNCH(h, "unique_write", k_unique_pass<true>, gs, SCAN_THREADS, 0, h->st, w, h->skey, h->block_sums);
     }
 }
 
-// Second half: tag lookup, then fetch + pool.
-void enqueue_lookup(mpe_handle* h, int64_t L_grid, int64_t bags_grid, bool ind, const StepArgs& av) {
+// fetch + pool, and (MODE) the record of the batch
+template <int MODE>
+void enqueue_pool(mpe_handle* h, const Work& w, uint2* records, int64_t bags, const StepArgs& av) {
     const State& s = h->st;
-    Work& w = h->wk;
-    LAUNCH(h, "probe", (ind ? k_probe<true> : k_probe<false>), grid_for(h, L_grid, 256, 8), 256, 0, s, w, av);
-    LAUNCH(h, "broadcast", (ind ? k_broadcast<true> : k_broadcast<false>), grid_for(h, L_grid, 256, 8), 256, 0, s, w, h->spos, av);
-    const int gp = grid_for(h, bags_grid, 256 / s.lanes, 8);
+    const int gp = grid_for(h, bags, 256 / s.lanes, 8);
     dispatch(h->bits, s.lanes, [&](auto bc, auto lc) {
-        constexpr int BITS = decltype(bc)::value, LANES = decltype(lc)::value;
-        auto kern = ind ? k_pool<BITS, LANES, true> : k_pool<BITS, LANES, false>;
-        LAUNCH(h, "pool", kern, gp, 256, 0, s, w, av);
+        auto kern = k_pool<decltype(bc)::value, decltype(lc)::value, MODE>;
+        LAUNCH(h, "pool", kern, gp, 256, 0, s, w, records, av);
     });
 }
 
-int enqueue_forward(mpe_handle* h, int64_t L_grid, int64_t bags_grid, bool ind) {
-    const StepArgs av = h->args;
-    enqueue_index_chain(h, L_grid, bags_grid, ind, av);
-    enqueue_lookup(h, L_grid, bags_grid, ind, av);
-    return check_launch(h);
-}
-
-int enqueue_backward(mpe_handle* h, int64_t L, bool ind) {
+int enqueue_backward(mpe_handle* h, int64_t L, bool ind, bool chain) {
     const State& s = h->st;
     Work& w = h->wk;
     const StepArgs av = h->args;
+    if (chain) enqueue_index_chain(h, L, ind);
     // the hot rows' partial gradient sums only need the sorted batch: they run on a second stream next to the
     // priority / candidate-sort / policy kernels, which leave most of the machine idle
     CK(h, cudaEventRecord(h->ev_fork, h->stream));
@@ -564,19 +546,19 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool ind) {
         LAUNCH_ON(h, h->side, "hot_partial", hot, grid_for(h, hot_capacity(L), 1, 2), 8 * LANES, 32 * s.dim * sizeof(float), s, w, av);
     });
     CK(h, cudaEventRecord(h->ev_join, h->side));
-    const SortBufs sb{h->sortA, h->sortB, h->sort_n, h->ghist, h->sort_status, h->sort_ctl, &h->wk.ctr->abort, h->wk.sort_tile};
-    // new priority values; the rows that may be admitted (few, once the caches are warm) are gathered in row order ...
+    const SortBufs sb = sort_bufs(h);
+    // where the rows live, new priority values; the rows that may be admitted (few, once the caches are warm) are gathered in row order ...
     LAUNCH(h, "priority", (ind ? k_priority<true> : k_priority<false>), grid_for(h, L, PRI_CHUNK, 8), 256, 0, s, w,
-           h->max_sets > 0 ? reinterpret_cast<uint2*>(sb.B) : (uint2*)nullptr, h->sort_status, h->sort_ctl, h->block_sums, av);
+           h->max_sets > 0 ? sort_input(sb) : (uint2*)nullptr, h->sort_status, h->sort_ctl, h->block_sums, av);
     if (h->max_sets > 0) {
         if (!ind) {        // large steps: the list is made by three small kernels
             LAUNCH(h, "scan_block_sums", k_scan_block_sums, 1, BSUM_THREADS, 0, h->block_sums, (const uint32_t*)&w.ctr->U, (uint32_t)PRI_CHUNK, &w.ctr->n_cand);
-            LAUNCH(h, "cand_write", k_cand_write, grid_for(h, L, PRI_CHUNK, 8), 256, 0, s, w, (const uint32_t*)h->block_sums, reinterpret_cast<uint2*>(sb.B));
+            LAUNCH(h, "cand_write", k_cand_write, grid_for(h, L, PRI_CHUNK, 8), 256, 0, s, w, (const uint32_t*)h->block_sums, sort_input(sb));
             LAUNCH(h, "cand_starts", k_cand_starts, 1, 32, 0, w, h->T);
         }
         // ... and grouped by cache set, keeping ascending row id inside a set
         const uint32_t *ck = nullptr, *cv = nullptr;
-        seg_sort(h, sb, w.cstart, w.ctile_base, bits_for((uint32_t)h->max_sets), L, &ck, &cv, true);
+        seg_sort(h, sb, w.cstart, w.ctile_base, bits_for((uint32_t)h->max_sets), L, nullptr, &ck, &cv);
         LAUNCH(h, "policy_heads", k_policy_heads, grid_for(h, L, 256, 8), 256, 0, s, w, ck);
         auto pol = ind ? k_policy<true> : k_policy<false>;
         LAUNCH(h, "policy", pol, grid_for(h, std::min<int64_t>(L, h->total_sets), 256 / s.ways, resident_blocks(h, pol, 256, 0)), 256, 0, s, w, ck, cv, av);
@@ -595,7 +577,6 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool ind) {
     });
     return check_launch(h);
 }
-
 
 bool may_use_graph(mpe_handle* h) {
     if (!h->graphs_enabled || h->profiling || h->cap_L > GRAPH_MAX_INDICES) return false;
@@ -638,6 +619,14 @@ int capture(mpe_handle* h, cudaGraph_t* graph, cudaGraphExec_t* exec, cudaGraphN
     return *args_node ? MPE_OK : MPE_ERR_CUDA;
 }
 
+// the handle's stream waits for the sort of the current batch, if that was done ahead
+int await_prepared(mpe_handle* h) {
+    if (!h->prep_running) return MPE_OK;
+    h->prep_running = false;
+    CK(h, cudaStreamWaitEvent(h->stream, h->ev_prep, 0));
+    return MPE_OK;
+}
+
 // forward with the pooled vectors going either to d_out (route == nullptr) or to the buffers the route names
 int forward_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offsets, int32_t batch,
                  int64_t total_indices, float* d_out, const Route* route) {
@@ -649,47 +638,30 @@ int forward_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
     }
     h->sort_passes_bound += 4 * SORT_MAX_PASSES;       // this step's two sorts, and those of a batch prepared meanwhile
     if (h->sort_passes_bound > SORT_TAG_MASK - 1024) { int rc = renew_sort_tags(h); if (rc != MPE_OK) return rc; }
-    Work& w = h->wk;
     uint32_t L = (uint32_t)total_indices;
     h->B = batch; h->L = total_indices; ++h->epoch;
     h->args.indices = d_indices; h->args.offsets = d_offsets; h->args.out = d_out; h->args.B = batch; h->args.L = L; h->args.epoch = h->epoch;
     h->args.route = route;
-    int rc = MPE_OK;
-    if (may_use_graph(h)) {
-        if (!h->x_fwd) {
-            // the graph's first kernel, k_prelude, is the one whose parameters change from call to call
-            rc = capture(h, &h->g_fwd, &h->x_fwd, &h->n_fwd, &h->k_fwd, (const void*)k_prelude<true>, [&]() {
-                return enqueue_forward(h, h->cap_L, h->cap_bags, true);
-            });
-            if (rc != MPE_OK) { drop_graphs(h); h->graphs_enabled = false; }      // fall back to plain launches for good
-        }
-        if (rc == MPE_OK) {
-            Work wv = w; int T = h->T; StepArgs av = h->args;
-            void* params[] = {&wv, &T, &av};
-            cudaKernelNodeParams kp{};
-            kp.func = (void*)k_prelude<true>; kp.gridDim = dim3(1); kp.blockDim = dim3(32); kp.kernelParams = params;
-            CK(h, cudaGraphExecKernelNodeSetParams(h->x_fwd, h->n_fwd, &kp));
-            CK(h, cudaGraphLaunch(h->x_fwd, h->stream));
-            h->launches += h->k_fwd;
-            h->have_forward = true; h->fwd_replayed = true;
-            return MPE_OK;
-        }
-    }
+    { int rc = await_prepared(h); if (rc != MPE_OK) return rc; }       // a forward whose backward never came
     if (h->prepared && h->prep_args.indices == d_indices && h->prep_args.offsets == d_offsets && h->prep_args.B == batch &&
         h->prep_args.L == L) {
         // the batch was sorted and de-duplicated ahead of time in the other workspace: it becomes the current one
         h->prepared = false;
         swap_sets(h);
-        CK(h, cudaStreamWaitEvent(h->stream, h->ev_prep, 0));
-        enqueue_lookup(h, total_indices, bags, false, h->args);
-        rc = check_launch(h);
+        // pooling needs nothing of it, only the caller's indices must have been read; backward waits for the rest
+        CK(h, cudaStreamWaitEvent(h->stream, h->ev_keys, 0));
+        h->prep_running = true;
+        enqueue_pool<FWD_PREPARED>(h, h->wk, nullptr, bags, h->args);
+        h->chain_done = true;
     } else {
         h->prepared = false;                 // whatever was prepared was for another batch
-        rc = enqueue_forward(h, total_indices, bags, false);
+        enqueue_pool<FWD_RECORD>(h, h->wk, sort_input(sort_bufs(h)), bags, h->args);
+        h->chain_done = false;
     }
+    int rc = check_launch(h);
     if (rc != MPE_OK) return rc;
-    if (h->ev_free) CK(h, cudaEventRecord(h->ev_free, h->stream));
-    h->have_forward = true; h->fwd_replayed = false;
+    CK(h, cudaEventRecord(h->ev_free, h->stream));
+    h->have_forward = true;
     return MPE_OK;
 }
 
@@ -704,7 +676,6 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
     if (!h->alt.wk.ctr) {                    // first use: the second workspace
         swap_sets(h);
         int rc = alloc_set(h, h->cap_L, h->cap_bags);
-        if (rc == MPE_OK && !h->ev_free && cudaEventCreateWithFlags(&h->ev_free, cudaEventDisableTiming) != cudaSuccess) rc = MPE_ERR_CUDA;
         if (rc != MPE_OK) free_set(h);
         swap_sets(h);
         if (rc != MPE_OK) return rc;
@@ -714,10 +685,14 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
     cudaStream_t user = h->stream;
     swap_sets(h);
     h->stream = stream;
-    cudaError_t e = h->ev_free ? cudaStreamWaitEvent(stream, h->ev_free, 0) : cudaSuccess;   // the step that used this workspace last has finished
+    cudaError_t e = cudaStreamWaitEvent(stream, h->ev_free, 0);       // the step that used this workspace last has finished,
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, h->ev_prep, 0);   // and so has a batch that was prepared in it and discarded
     if (e == cudaSuccess) {
-        enqueue_index_chain(h, total_indices, bags, false, av);
-        e = cudaEventRecord(h->ev_prep, stream);
+        LAUNCH(h, "prelude", k_prelude, 1, 32, 0, h->wk, h->T, av);
+        LAUNCH(h, "make_keys", k_make_keys, grid_for(h, bags, 32, 8), 256, 0, h->st, h->wk, sort_input(sort_bufs(h)), av);
+        e = cudaEventRecord(h->ev_keys, stream);
+        enqueue_index_chain(h, total_indices, false);
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_prep, stream);
     }
     int rc = check_launch(h);
     h->stream = user;
@@ -846,23 +821,22 @@ int mpe_backward(mpe_handle* h, const float* d_grad_out, float lr, int64_t step)
     if (step <= h->last_step) return MPE_ERR_SEQUENCE;
     DeviceGuard guard(h->device);
     Work& w = h->wk;
-    unsigned long long ustep = (unsigned long long)step;
-    h->args.grad = d_grad_out; h->args.lr = lr; h->args.step = ustep;
-    int rc = MPE_OK;
+    h->args.grad = d_grad_out; h->args.lr = lr; h->args.step = (unsigned long long)step;
+    int rc = await_prepared(h);
+    if (rc != MPE_OK) return rc;
     bool done = false;
-    // the replayed kernels read the forward's arguments (indices, offsets, batch, epoch) from the device copy, which only
-    // a replayed forward writes; after a plainly launched forward the backward is launched plainly too
-    if (h->fwd_replayed && may_use_graph(h)) {
+    if (!h->chain_done && may_use_graph(h)) {
         if (!h->x_bwd) {
             rc = capture(h, &h->g_bwd, &h->x_bwd, &h->n_bwd, &h->k_bwd, (const void*)k_set_args_backward, [&]() {
-                LAUNCH(h, "set_args", k_set_args_backward, 1, 1, 0, w.args, d_grad_out, lr, ustep);
-                return enqueue_backward(h, h->cap_L, true);
+                LAUNCH(h, "set_args", k_set_args_backward, 1, 1, 0, w.args, h->args);
+                return enqueue_backward(h, h->cap_L, true, true);
             });
-            if (rc != MPE_OK) { drop_graphs(h); h->graphs_enabled = false; }
+            if (rc != MPE_OK) { drop_graphs(h); h->graphs_enabled = false; }      // fall back to plain launches for good
         }
         if (rc == MPE_OK) {
             StepArgs* a = w.args;
-            void* params[] = {&a, &d_grad_out, &lr, &ustep};
+            StepArgs av = h->args;
+            void* params[] = {&a, &av};
             cudaKernelNodeParams kp{};
             kp.func = (void*)k_set_args_backward; kp.gridDim = dim3(1); kp.blockDim = dim3(1); kp.kernelParams = params;
             CK(h, cudaGraphExecKernelNodeSetParams(h->x_bwd, h->n_bwd, &kp));
@@ -872,10 +846,10 @@ int mpe_backward(mpe_handle* h, const float* d_grad_out, float lr, int64_t step)
         }
     }
     if (!done) {
-        rc = enqueue_backward(h, h->L, false);
+        rc = enqueue_backward(h, h->L, false, !h->chain_done);
         if (rc != MPE_OK) return rc;
     }
-    if (h->ev_free) CK(h, cudaEventRecord(h->ev_free, h->stream));
+    CK(h, cudaEventRecord(h->ev_free, h->stream));
     h->have_forward = false;
     h->last_step = step;
     ++h->steps;
@@ -1001,7 +975,7 @@ int mpe_destroy(mpe_handle* h) {
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->prep) { cudaStreamSynchronize(h->prep); cudaStreamDestroy(h->prep); }
-    for (cudaEvent_t e : {h->ev_free, h->alt.ev_free, h->ev_prep}) if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : {h->ev_free, h->alt.ev_free, h->ev_keys, h->ev_prep, h->alt.ev_keys, h->alt.ev_prep}) if (e) cudaEventDestroy(e);
     if (h->copy_in) { cudaStreamSynchronize(h->copy_in); cudaStreamDestroy(h->copy_in); }
     if (h->copy_out) { cudaStreamSynchronize(h->copy_out); cudaStreamDestroy(h->copy_out); }
     for (auto& sl : h->slot) {
@@ -1012,8 +986,8 @@ int mpe_destroy(mpe_handle* h) {
     State& s = h->st;
     if (h->table_on_host) { cudaFreeHost(s.codes); cudaFreeHost(s.sb); } else { cudaFree(s.codes); cudaFree(s.sb); }
     cudaFree(h->d_route);
-    cudaFree(h->d_tables); cudaFree(s.cnt); cudaFree(s.G); cudaFree(s.slab);
-    cudaFree(s.tags); cudaFree(s.ts); cudaFree(s.hit_epoch); cudaFree(s.hit_k); cudaFree(s.floor); cudaFree(s.stats);
+    cudaFree(h->d_tables); cudaFree(s.G); cudaFree(s.slab);
+    cudaFree(s.tags); cudaFree(s.home); cudaFree(s.ts); cudaFree(s.hit_epoch); cudaFree(s.hit_k); cudaFree(s.floor); cudaFree(s.stats);
     for (auto& r : h->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (auto e : h->event_pool) cudaEventDestroy(e);
     delete h;
@@ -1026,6 +1000,7 @@ int mpe_last_error(mpe_handle* h, int32_t* code, int64_t* detail) {
     if (!h->wk.ctr) return MPE_OK;
     DeviceGuard guard(h->device);
     CK(h, cudaStreamSynchronize(h->stream));
+    if (h->prep_running) CK(h, cudaEventSynchronize(h->ev_prep));
     Counters c;
     CK(h, cudaMemcpy(&c, h->wk.ctr, sizeof(c), cudaMemcpyDeviceToHost));
     CK(h, cudaMemset(&h->wk.ctr->err[0], 0, sizeof(c.err)));
@@ -1109,7 +1084,12 @@ int mpe_step_info(mpe_handle* h, int64_t* out6) {
     for (int i = 0; i < 6; ++i) out6[i] = 0;
     if (!h->wk.ctr) return MPE_OK;
     DeviceGuard guard(h->device);
+    if (h->have_forward && !h->chain_done) {           // a forward alone does not sort its batch: the distinct rows are counted on demand
+        enqueue_index_chain(h, h->L, false);
+        h->chain_done = true;
+    }
     CK(h, cudaStreamSynchronize(h->stream));
+    if (h->prep_running) CK(h, cudaEventSynchronize(h->ev_prep));
     Counters c;
     CK(h, cudaMemcpy(&c, h->wk.ctr, sizeof(c), cudaMemcpyDeviceToHost));
     if (c.abort) return MPE_OK;
@@ -1244,27 +1224,15 @@ namespace {
 constexpr int64_t STATIC_MAX_INDICES = MPE_STATIC_MAX_INDICES;
 constexpr int64_t STATIC_MAX_BAGS = MPE_STATIC_MAX_BAGS;
 constexpr int STATIC_MAX_TABLES = MPE_STATIC_MAX_TABLES;
-constexpr size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
-constexpr size_t STATIC_SCRATCH_BYTES =
-    2 * align256(2 * (STATIC_MAX_INDICES + 4) * 4) + 12 * align256((STATIC_MAX_INDICES + 4) * 4) +                                 // keys, payloads, per-index and per-row maps
-    align256(256 * ((STATIC_MAX_INDICES + sort_tile(true) - 1) / sort_tile(true) + STATIC_MAX_TABLES + 1) * 8) +   // the sort's per-tile words
-    align256(STATIC_MAX_TABLES * SORT_MAX_PASSES * 256 * 4) + align256(sizeof(SortCtl)) +              // its per-table digit counts and its counters
-    4 * align256((STATIC_MAX_TABLES + 1) * 4) +                                                        // per-table starts
-    2 * align256(hot_capacity(STATIC_MAX_INDICES) * 4) +                                             // hot-row lists
-    align256(sizeof(Counters)) + align256(sizeof(StepArgs));
+constexpr size_t STATIC_SCRATCH_BYTES = (sizeof(Counters) + 255) & ~size_t(255);
 
-// The scratch itself.  In host code this name is only a handle for cudaGetSymbolAddress; it is not a device address.
+// What a forward needs of device memory besides the caller's buffers: the counters by which its blocks agree that they have
+// finished.  In host code this name is only a handle for cudaGetSymbolAddress; it is not a device address.
 static __device__ __align__(256) unsigned char g_static_scratch[STATIC_SCRATCH_BYTES];
 
 constexpr int MAX_DEVICES = 64;
 unsigned char* g_scratch_addr[MAX_DEVICES] = {};     // device address of g_static_scratch, per device, filled on first use
-uint64_t g_scratch_passes[MAX_DEVICES] = {};         // sort passes run in the array so far, per device (an upper bound)
 std::mutex g_scratch_lock;                           // first calls from several host threads fill the table one at a time
-
-struct Carver {
-    unsigned char* p; size_t used = 0;
-    template <class T> T* take(size_t count) { T* r = reinterpret_cast<T*>(p + used); used += align256(count * sizeof(T)); return r; }
-};
 
 }  // namespace
 
@@ -1274,11 +1242,10 @@ extern "C" int mpe_forward_static(mpe_handle* h, const int32_t* d_indices, const
     if ((total_indices > 0 && !d_indices) || (batch > 0 && !d_out)) return MPE_ERR_ARG;
     const int64_t bags = (int64_t)h->T * batch;
     if (total_indices > STATIC_MAX_INDICES || bags > STATIC_MAX_BAGS || h->T > STATIC_MAX_TABLES) return MPE_ERR_TOO_LARGE;
-    if (h->have_forward) return MPE_ERR_SEQUENCE;      // a training step is half done: its backward still needs the probe marks
+    if (h->have_forward) return MPE_ERR_SEQUENCE;      // a training step is half done
     if (h->device < 0 || h->device >= MAX_DEVICES) return MPE_ERR_ARG;
     DeviceGuard guard(h->device);
-    unsigned char* scratch = nullptr;
-    bool renew_tags = false;          // the pass numbers in the sort's per-tile words are about to come round: start them over
+    Work w{};
     {
         std::lock_guard<std::mutex> lock(g_scratch_lock);
         if (!g_scratch_addr[h->device]) {
@@ -1287,60 +1254,13 @@ extern "C" int mpe_forward_static(mpe_handle* h, const int32_t* d_indices, const
             CK(h, cudaGetSymbolAddress(&addr, g_static_scratch));
             g_scratch_addr[h->device] = static_cast<unsigned char*>(addr);
         }
-        scratch = g_scratch_addr[h->device];
-        g_scratch_passes[h->device] += SORT_MAX_PASSES;
-        renew_tags = g_scratch_passes[h->device] > SORT_TAG_MASK - 1024;
-        if (renew_tags) g_scratch_passes[h->device] = 0;
+        // a static array starts zeroed, and every forward leaves the counters it uses at zero
+        w.ctr = reinterpret_cast<Counters*>(g_scratch_addr[h->device]);
     }
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     if (stream != h->stream) { CK(h, cudaStreamSynchronize(h->stream)); h->stream = stream; }
-
-    // carve the step's arrays out of the scratch (same roles as the handle's own workspace)
-    Carver c{scratch};
-    const size_t n = (size_t)STATIC_MAX_INDICES + 4;
-    uint32_t *sortA = c.take<uint32_t>(2 * n), *sortB = c.take<uint32_t>(2 * n);
-    Work w{};
-    w.bag_of = c.take<int32_t>(n); w.kidx = c.take<uint32_t>(n); w.occ_loc = c.take<int32_t>(n); w.occ_b = c.take<int32_t>(n);
-    w.uniq_row = c.take<int32_t>(n); w.uniq_t = c.take<int32_t>(n); w.seg = c.take<int32_t>(n); w.loc = c.take<int32_t>(n);
-    w.final_loc = c.take<int32_t>(n); w.uset = c.take<int32_t>(n); w.hot_base = c.take<int32_t>(n); w.victim = c.take<int32_t>(n);
-    const size_t max_tiles = (STATIC_MAX_INDICES + sort_tile(true) - 1) / sort_tile(true) + STATIC_MAX_TABLES + 1;
-    unsigned long long* sort_status = c.take<unsigned long long>(256 * max_tiles);
-    uint32_t* ghist = c.take<uint32_t>((size_t)STATIC_MAX_TABLES * SORT_MAX_PASSES * 256);
-    SortCtl* sort_ctl = c.take<SortCtl>(1);
-    w.table_start = c.take<int32_t>(STATIC_MAX_TABLES + 1); w.tile_base = c.take<int32_t>(STATIC_MAX_TABLES + 1);
-    w.ustart = c.take<int32_t>(STATIC_MAX_TABLES + 1); w.ctile_base = c.take<int32_t>(STATIC_MAX_TABLES + 1);
-    w.hot_k = c.take<int32_t>(hot_capacity(STATIC_MAX_INDICES)); w.task_k = c.take<int32_t>(hot_capacity(STATIC_MAX_INDICES));
-    w.ctr = c.take<Counters>(1);
-    w.args = c.take<StepArgs>(1);
-    if (c.used > STATIC_SCRATCH_BYTES) return MPE_ERR_ARG;      // cannot happen: the size formula above mirrors this list
-
-    const State& s = h->st;
-    const int T = h->T;
-    const uint32_t L = (uint32_t)total_indices;
-    ++h->epoch;
-    // the array keeps whatever the previous call left: the counters are the only part that must start from zero
-    CK(h, cudaMemsetAsync(w.ctr, 0, sizeof(Counters), stream));
-    if (renew_tags) {
-        CK(h, cudaMemsetAsync(sort_status, 0, sizeof(unsigned long long) * 256 * max_tiles, stream));
-        CK(h, cudaMemsetAsync(sort_ctl, 0, sizeof(SortCtl), stream));
-    }
     StepArgs av{};
-    av.indices = d_indices; av.offsets = d_offsets; av.out = d_out; av.B = batch; av.L = L; av.epoch = h->epoch;
-    w.sort_tile = sort_tile(true);
-    const SortBufs sb{sortA, sortB, (int64_t)n, ghist, sort_status, sort_ctl, &w.ctr->abort, w.sort_tile};
-    LAUNCH(h, "prelude", k_prelude<false>, 1, 32, 0, w, T, av);
-    LAUNCH(h, "make_keys", k_make_keys<false>, grid_for(h, bags, 32, 8), 256, 0, s, w, sort_input(sb), av);
-    // segmented radix sort, as in mpe_forward, on the carved buffers
-    const uint32_t *skey = nullptr, *spos = nullptr;
-    seg_sort(h, sb, w.table_start, w.tile_base, bits_for((uint32_t)h->max_rows), total_indices, &skey, &spos);
-    const int gs = grid_for(h, total_indices, SCAN_TILE, 8);
-    LAUNCH(h, "unique", k_unique, gs, SCAN_THREADS, 0, w, T, skey, sort_status, sort_ctl);
-    LAUNCH(h, "probe", k_probe<false>, grid_for(h, total_indices, 256, 8), 256, 0, s, w, av);
-    LAUNCH(h, "broadcast", k_broadcast<false>, grid_for(h, total_indices, 256, 8), 256, 0, s, w, spos, av);
-    const int gp = grid_for(h, bags, 256 / s.lanes, 8);
-    dispatch(h->bits, s.lanes, [&](auto bc, auto lc) {
-        auto kern = k_pool<decltype(bc)::value, decltype(lc)::value, false>;
-        LAUNCH(h, "pool", kern, gp, 256, 0, s, w, av);
-    });
+    av.indices = d_indices; av.offsets = d_offsets; av.out = d_out; av.B = batch; av.L = (uint32_t)total_indices;
+    enqueue_pool<FWD_EVAL>(h, w, nullptr, bags, av);
     return check_launch(h);
 }

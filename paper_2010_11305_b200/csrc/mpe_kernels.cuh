@@ -9,14 +9,16 @@ namespace mpe {
 
 constexpr int HOT_SPAN = 1024;        // occurrences covered by one multi-block gradient task (two tree levels)
 constexpr int HOT_MIN = 256;          // rows with more occurrences than this take the multi-block path
-// A step with few distinct rows has few warps' worth of work in k_update, and its duration is that of the warp with the
+// A small step has few warps' worth of work in k_update, and its duration is that of the warp with the
 // longest rows: there the multi-block path starts earlier.
 constexpr int HOT_MIN_SMALL = 64;
-constexpr int HOT_SMALL_U = 131072;   // "few": at most this many distinct rows
+constexpr int HOT_SMALL_L = 1 << 20;  // "small": at most this many indices
 // upper bound of the number of hot rows, and of their tasks, in a step of L indices (either threshold)
 __host__ __device__ constexpr int64_t hot_capacity(int64_t L) {
-    return (L / HOT_MIN_SMALL < HOT_SMALL_U ? L / HOT_MIN_SMALL : HOT_SMALL_U) + L / HOT_MIN + L / HOT_SPAN + 4;
+    return (L < HOT_SMALL_L ? L : HOT_SMALL_L) / HOT_MIN_SMALL + L / HOT_MIN + L / HOT_SPAN + 4;
 }
+// more occurrences than this: the multi-block path
+__host__ __device__ constexpr uint32_t hot_threshold(int64_t L) { return L <= HOT_SMALL_L ? (uint32_t)HOT_MIN_SMALL : (uint32_t)HOT_MIN; }
 constexpr int ERR_INDEX = 0, ERR_OFFSETS = 1;
 
 struct TableDev {
@@ -31,7 +33,7 @@ struct TableDev {
 struct Counters {
     uint32_t L;            // indices in this batch
     uint32_t U;            // distinct (table,row) pairs incl. one pseudo row per table that had bad indices
-    uint32_t unused0, unused1;
+    uint32_t fwd_bad, fwd_done;      // of the running forward: offsets were inconsistent; blocks that have finished
     uint32_t hot_rows;
     uint32_t hot_tasks;
     uint32_t abort;        // offsets were inconsistent: every later kernel of the step returns at once
@@ -39,6 +41,7 @@ struct Counters {
     uint32_t n_heads;      // cache sets that have miss candidates in this step
     uint32_t upd_next;     // next block of 32 distinct rows to hand to a warp of k_update
     uint32_t n_cand;       // candidates for admission in this step
+    unsigned long long fwd_dropped;  // out-of-range indices met by the running forward
     unsigned long long dropped;      // out-of-range indices in this batch
     unsigned long long hot_occ;      // indices that belong to hot rows
     unsigned long long err[2];       // sticky: ERR_INDEX, ERR_OFFSETS
@@ -52,16 +55,21 @@ struct State {
     const TableDev* tables;
     uint8_t* codes;        // [sum N][dim*bits/8]
     float2* sb;            // [sum N] (scale, bias)
-    uint32_t* cnt;         // LFU: [sum N]
     float* G;              // Adagrad: [sum N]
     float* slab;           // [slots][dim]
     int32_t* tags;         // [slots], -1 empty
+    int32_t* home;         // per row: its cache slot, or LOC_MISS (the inverse of tags); LFU: {slot, access count} in one 8-byte
+                           // record, so that a row's slot and count are one memory access
+    int home_shift;        // 0, or 1 where a record holds the count too
     uint32_t* ts;          // [slots] priority value of the resident row: LRU time stamp, or a copy of its LFU count
     uint32_t* hit_epoch;   // [slots] forward call in which the slot was last hit
     int32_t* hit_k;        // [slots] unique-row index of that hit
     uint32_t* floor;       // [sets] a lower bound of the lowest priority value among the set's residents (0: none known)
     unsigned long long* stats;   // [T][8]
 };
+
+__device__ __forceinline__ int32_t* slot_of(const State& s, int64_t row) { return s.home + (row << s.home_shift); }
+__device__ __forceinline__ uint32_t* count_of(const State& s, int64_t row) { return reinterpret_cast<uint32_t*>(s.home + 2 * row + 1); }   // LFU
 
 // What changes from call to call.  It lives in device memory so that a captured CUDA graph of the step stays valid:
 // the kernels read it, one tiny kernel at the head of the graph writes it.
@@ -84,11 +92,8 @@ struct Work {
     Counters* ctr;
     StepArgs* args;
     int32_t *table_start, *tile_base, *ustart, *ctile_base;   // [T+1]
-    int32_t* bag_of;       // [L] bag of every index position
-    uint32_t* kidx;        // [L] unique-row index of the i-th sorted element
-    int32_t* occ_loc;      // [L] by position: cache slot, LOC_MISS or LOC_INVALID
     int32_t* occ_b;        // [L] by sorted order: sample of the element; sign bit: last occurrence of its row
-    int32_t *uniq_row, *uniq_t, *seg, *loc, *final_loc, *victim, *hot_base, *uset;   // per unique row
+    int32_t *uniq_row, *uniq_t, *seg, *loc, *final_loc, *victim, *hot_base;   // per unique row
     int32_t* task_k;       // [hot tasks]
     int32_t* hot_k;        // [hot rows]
     uint32_t* cand_key;    // [distinct rows] large steps: the row's set if it is a candidate for admission, else the table's number of sets
@@ -100,6 +105,12 @@ struct Work {
     int32_t sort_tile;     // keys per tile of the sorts of this workspace
 };
 
+// the counters of a step, as its first kernel leaves them
+__device__ __forceinline__ void reset_step(Counters* c, uint32_t L, uint32_t abort, unsigned long long dropped) {
+    c->L = L; c->U = 0; c->hot_rows = 0; c->hot_tasks = 0; c->abort = abort; c->dropped = dropped; c->hot_occ = 0; c->deferred = 0;
+    c->n_heads = 0; c->upd_next = 0;
+}
+
 // ---------------------------------------------------------------------------------------------
 // step prologue
 // ---------------------------------------------------------------------------------------------
@@ -107,30 +118,20 @@ __global__ void k_set_route(Route* dst, Route r) {
     for (int g = threadIdx.x; g < MAX_RANKS; g += blockDim.x) dst->out[g] = r.out[g];
     if (threadIdx.x == 0) { dst->B_local = r.B_local; dst->T_global = r.T_global; dst->t_base = r.t_base; dst->n_ranks = r.n_ranks; }
 }
-__global__ void k_set_args_backward(StepArgs* a, const float* grad, float lr, unsigned long long step) {
-    a->grad = grad; a->lr = lr; a->step = step;
-}
+// a replayed backward starts with this node, the one whose parameters change from call to call
+__global__ void k_set_args_backward(StepArgs* a, StepArgs v) { *a = v; }
 
-// one warp: resets the step's counters and reads where each table's bags begin (the offsets of bags 0, B, 2B, ...), 32
+// First kernel of a batch that is sorted ahead of its forward (mpe_prepare); for the others the forward's pooling kernel does this.
+// One warp: resets the step's counters and reads where each table's bags begin (the offsets of bags 0, B, 2B, ...), 32
 // tables at a time so that the loads overlap; offsets that do not start at 0, end at L or grow abandon the step
-// In a replayed step this is the graph's first kernel and the one whose parameters change from call to call: it passes the
-// forward's arguments on to the kernels behind it through the block in device memory.
-template <bool IND>
-__global__ void k_prelude(Work w, int T, StepArgs av) {
-    const StepArgs a = av;
+__global__ void k_prelude(Work w, int T, StepArgs a) {
     if (blockIdx.x != 0 || threadIdx.x >= 32) return;
     const int lane = threadIdx.x;
-    if (IND && lane == 0) {
-        StepArgs* d = w.args;
-        d->indices = a.indices; d->offsets = a.offsets; d->out = a.out; d->B = a.B; d->L = a.L; d->epoch = a.epoch; d->route = a.route;
-    }
     const int32_t* __restrict__ offsets = a.offsets;
     const int B = a.B;
     const uint32_t L = a.L;
     Counters* c = w.ctr;
-    if (lane == 0) {
-        c->L = L; c->U = 0; c->hot_rows = 0; c->hot_tasks = 0; c->abort = 0; c->dropped = 0; c->hot_occ = 0; c->deferred = 0; c->n_heads = 0; c->upd_next = 0;
-    }
+    if (lane == 0) reset_step(c, L, 0, 0);
     bool bad = false;
     for (int t0 = 0; t0 <= T; t0 += 32) {
         const int t = t0 + lane;
@@ -150,11 +151,10 @@ __global__ void k_prelude(Work w, int T, StepArgs av) {
     warp_tile_bases(w.table_start, T, w.tile_base, bad, w.sort_tile);     // the sort's tiles, table by table
 }
 
-// keys for the sort: the row id, or N_t for an id outside [0, N_t); eight lanes per bag, four bags per warp
-template <bool IND>
+// Records for the sort of a batch that is sorted ahead: the row id, or N_t for an id outside [0, N_t), and the sample;
+// eight lanes per bag, four bags per warp
 __global__ void __launch_bounds__(256)
-k_make_keys(State s, Work w, uint32_t* __restrict__ keys, StepArgs av) {
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
+k_make_keys(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
     const int32_t* __restrict__ indices = a.indices;
     const int32_t* __restrict__ offsets = a.offsets;
     const int B = a.B;
@@ -175,8 +175,7 @@ k_make_keys(State s, Work w, uint32_t* __restrict__ keys, StepArgs av) {
             for (int32_t p = lo + sub; p < hi; p += 8) {
                 const int32_t r = indices[p];
                 const bool ok = r >= 0 && r < N;
-                keys[p] = ok ? (uint32_t)r : (uint32_t)N;
-                w.bag_of[p] = (int32_t)bag;
+                pairs[p] = make_uint2(ok ? (uint32_t)r : (uint32_t)N, (uint32_t)b);
                 bad += !ok;
             }
         }
@@ -187,59 +186,116 @@ k_make_keys(State s, Work w, uint32_t* __restrict__ keys, StepArgs av) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// distinct rows of the sorted batch (I_U), multiplicities, element -> distinct-row map
+// distinct rows of the sorted batch (I_U) and their multiplicities
 // ---------------------------------------------------------------------------------------------
+// One thread's SCAN_ITEMS consecutive sorted elements, starting at `base`: their keys, which of them begin a run of equal
+// (table, row) (bit i of *heads) and which end one (bit i of *lasts), and the table of the first.
+__device__ __forceinline__ void unique_items(const int32_t* __restrict__ table_start, int T, const uint32_t* __restrict__ skey, uint32_t n,
+                                             uint32_t base, uint32_t (&key)[SCAN_ITEMS], uint32_t* heads, uint32_t* lasts, int* t_first) {
+    static_assert(SCAN_ITEMS == 16, "four 16-byte loads, 16-bit masks");
+    *heads = 0; *lasts = 0; *t_first = 0;
+    if (base >= n) return;
+    int t = find_segment(table_start, T, (int32_t)base);
+    while (table_start[t + 1] <= (int32_t)base) ++t;               // skip empty tables that start here
+    *t_first = t;
+    uint32_t prev = base > 0 ? skey[base - 1] : 0;
+    uint32_t next = base + SCAN_ITEMS < n ? skey[base + SCAN_ITEMS] : 0;
+    if (base + SCAN_ITEMS <= n) {
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; i += 4) {
+            const uint4 v = *reinterpret_cast<const uint4*>(skey + base + i);
+            key[i] = v.x; key[i + 1] = v.y; key[i + 2] = v.z; key[i + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; ++i) key[i] = base + i < n ? skey[base + i] : 0;
+    }
+    int32_t tend = table_start[t + 1];
+    uint32_t h = base == (uint32_t)table_start[t] || key[0] != prev ? 1u : 0u;      // bit i: element i begins a run (bit 16: the one behind)
+#pragma unroll
+    for (int i = 1; i <= SCAN_ITEMS; ++i) {
+        const uint32_t e = base + i;
+        const uint32_t k = i < SCAN_ITEMS ? key[i < SCAN_ITEMS ? i : 0] : next;
+        bool head = e >= n || k != key[i - 1];
+        if (e < n && (int32_t)e >= tend) { head = true; do { ++t; tend = table_start[t + 1]; } while (tend <= (int32_t)e); }
+        if (head) h |= 1u << i;
+    }
+    const uint32_t live = n - base >= SCAN_ITEMS ? 0xffffu : (1u << (n - base)) - 1u;
+    *heads = h & live;
+    *lasts = (h >> 1) & live;
+}
+// ... and writes them out: the thread's first run has the index k.  The last occurrence of a row is marked in the sign bit of its
+// sample id (samples are below 2^31); ustart receives where each table's distinct rows begin.  A row with more occurrences than
+// the threshold (the element that many places behind its first one is still the same row) is listed for the multi-block
+// gradient path, HOT_SPAN occurrences per task; only for such a row the end of its run is searched for.
+__device__ __forceinline__ void unique_write(const State& s, const Work& w, const uint32_t* __restrict__ skey, uint32_t n, uint32_t base, const uint32_t (&key)[SCAN_ITEMS], uint32_t heads,
+                                             uint32_t lasts, int t, uint32_t k) {
+    if (base >= n) return;
+    const int32_t hot_min = (int32_t)hot_threshold(n);
+    int32_t tend = w.table_start[t + 1];
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+        const int32_t e = (int32_t)base + i;
+        if ((heads >> i) & 1u) {
+            while (tend <= e) { ++t; tend = w.table_start[t + 1]; }
+            w.uniq_row[k] = (int32_t)key[i]; w.uniq_t[k] = t; w.seg[k] = e;
+            if (e == w.table_start[t])                             // and of the empty tables before it
+                for (int u = t; u >= 0 && w.table_start[u] == e; --u) w.ustart[u] = (int32_t)k;
+            if (e + hot_min < tend && skey[e + hot_min] == key[i] && (int32_t)key[i] < s.tables[t].N) {
+                int32_t lo = e + hot_min, hi = tend;               // same row at lo, another one (or the table's end) at hi
+                while (hi - lo > 1) {
+                    const int32_t mid = lo + ((hi - lo) >> 1);
+                    if (skey[mid] == key[i]) lo = mid; else hi = mid;
+                }
+                const uint32_t m = (uint32_t)(hi - e), nt = (m + HOT_SPAN - 1) / HOT_SPAN;
+                const uint32_t hb = atomicAdd(&w.ctr->hot_tasks, nt);
+                w.hot_base[k] = (int32_t)hb;
+                w.hot_k[atomicAdd(&w.ctr->hot_rows, 1u)] = (int32_t)k;
+                atomicAdd(&w.ctr->hot_occ, (unsigned long long)m);
+                for (uint32_t j = 0; j < nt; ++j) w.task_k[hb + j] = (int32_t)k;
+            }
+            ++k;
+        }
+    }
+    if (lasts == 0) return;
+    if (base + SCAN_ITEMS <= n) {
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; i += 4) {
+            if (((lasts >> i) & 15u) == 0) continue;
+            uint4* q = reinterpret_cast<uint4*>(w.occ_b + base + i);
+            uint4 v = *q;
+            v.x |= ((lasts >> i) & 1u) << 31; v.y |= ((lasts >> (i + 1)) & 1u) << 31;
+            v.z |= ((lasts >> (i + 2)) & 1u) << 31; v.w |= ((lasts >> (i + 3)) & 1u) << 31;
+            *q = v;
+        }
+    } else {
+        for (int i = 0; i < SCAN_ITEMS; ++i) if ((lasts >> i) & 1u) w.occ_b[base + i] |= (int32_t)0x80000000;
+    }
+}
+// what lies behind the last distinct row: its end mark, and the start of the tables without indices at the end of the batch
+__device__ __forceinline__ void unique_close(const Work& w, int T, uint32_t n, uint32_t U) {
+    for (int t = threadIdx.x; t <= T; t += blockDim.x) if ((uint32_t)w.table_start[t] >= n) w.ustart[t] = (int32_t)U;
+    if (threadIdx.x == 0) w.seg[U] = (int32_t)n;
+}
+
 // Small steps (the ones replayed from a graph, where every launch counts), one pass: a tile of the sorted batch flags the first element of every run of equal (table, row), learns how many
-// distinct rows the tiles before it hold (look-back over one word per tile), and writes its part of the lists.  The block
-// that ends the pass fills in where each table's distinct rows begin.
+// distinct rows the tiles before it hold (look-back over one word per tile), and writes its part of the lists.
 __global__ void __launch_bounds__(SCAN_THREADS)
-k_unique(Work w, int T, const uint32_t* __restrict__ skey, unsigned long long* __restrict__ words, SortCtl* __restrict__ ctl) {
+k_unique(State s, Work w, const uint32_t* __restrict__ skey, unsigned long long* __restrict__ words, SortCtl* __restrict__ ctl) {
     __shared__ uint32_t tmp[SCAN_THREADS / 32 + 1];
     __shared__ uint32_t s_turn[2];
     __shared__ uint32_t s_prefix[2];
     const bool off = w.ctr->abort != 0;                 // an abandoned step has no tiles
     const uint32_t n = off ? 0u : w.ctr->L;
     const uint32_t nblk = (n + SCAN_TILE - 1) / SCAN_TILE;
+    const int T = s.T;
     uint32_t b, tag;
     while (draw_tile(ctl, nblk, s_turn, &b, &tag)) {
         const uint32_t base = b * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
-        uint32_t flag[SCAN_ITEMS];
-        int tcur[SCAN_ITEMS];
-        uint32_t sum = 0;
-        uint32_t keyv[SCAN_ITEMS];
-        if (base < n) {
-            int t = find_segment(w.table_start, T, (int32_t)base);
-            while (w.table_start[t + 1] <= (int32_t)base) ++t;     // skip empty tables that start here
-            uint32_t prev = base > 0 ? skey[base - 1] : 0;
-            if (base + SCAN_ITEMS <= n) {                           // 16 keys as four 16-byte loads
-#pragma unroll
-                for (int i = 0; i < SCAN_ITEMS; i += 4) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(skey + base + i);
-                    keyv[i] = v.x; keyv[i + 1] = v.y; keyv[i + 2] = v.z; keyv[i + 3] = v.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < SCAN_ITEMS; ++i) keyv[i] = base + i < n ? skey[base + i] : 0;
-            }
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; ++i) {
-                const uint32_t e = base + i;
-                flag[i] = 0; tcur[i] = t;
-                if (e < n) {
-                    while (w.table_start[t + 1] <= (int32_t)e) ++t;
-                    tcur[i] = t;
-                    const uint32_t k = keyv[i];
-                    flag[i] = (e == (uint32_t)w.table_start[t] || k != prev) ? 1u : 0u;
-                    prev = k;
-                    sum += flag[i];
-                }
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; ++i) { flag[i] = 0; tcur[i] = 0; keyv[i] = 0; }
-        }
+        uint32_t key[SCAN_ITEMS], heads, lasts; int t;
+        unique_items(w.table_start, T, skey, n, base, key, &heads, &lasts, &t);
         uint32_t total;
-        uint32_t ex = block_exclusive_scan<SCAN_THREADS>(sum, &total, tmp);
+        const uint32_t ex = block_exclusive_scan<SCAN_THREADS>(__popc(heads), &total, tmp);
         if (threadIdx.x < 32) {
             if (threadIdx.x == 0) tile_publish(words, b, total, tag);
             bool poison;
@@ -251,206 +307,39 @@ k_unique(Work w, int T, const uint32_t* __restrict__ skey, unsigned long long* _
             if (threadIdx.x == 0) { atomicAdd(&ctl->timeout, 1u); w.ctr->abort = 1; }
             continue;
         }
-        ex += s_prefix[0];
-        if (b == nblk - 1 && threadIdx.x == 0) w.ctr->U = s_prefix[0] + total;
-        uint32_t kout[SCAN_ITEMS];
-#pragma unroll
-        for (int i = 0; i < SCAN_ITEMS; ++i) {
-            const uint32_t e = base + i;
-            ex += flag[i];
-            kout[i] = ex - 1;
-            if (e < n && flag[i]) { w.uniq_row[kout[i]] = (int32_t)keyv[i]; w.uniq_t[kout[i]] = tcur[i]; w.seg[kout[i]] = (int32_t)e; }
-        }
-        if (base + SCAN_ITEMS <= n) {
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; i += 4)
-                *reinterpret_cast<uint4*>(w.kidx + base + i) = make_uint4(kout[i], kout[i + 1], kout[i + 2], kout[i + 3]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; ++i) if (base + i < n) w.kidx[base + i] = kout[i];
+        unique_write(s, w, skey, n, base, key, heads, lasts, t, ex + s_prefix[0]);
+        if (b == nblk - 1) {
+            if (threadIdx.x == 0) w.ctr->U = s_prefix[0] + total;
+            unique_close(w, T, n, s_prefix[0] + total);
         }
     }
-    if (last_block_of_pass(ctl, s_turn)) {
-        // every tile is done and its results are visible: where each table's distinct rows begin, and the end mark
-        if (!off && !__ldcg(&w.ctr->abort)) {
-            const uint32_t U = __ldcg(&w.ctr->U);
-            for (int t = threadIdx.x; t <= T; t += blockDim.x) {
-                const int32_t s0 = w.table_start[t];
-                w.ustart[t] = (uint32_t)s0 < n ? (int32_t)__ldcg(w.kidx + s0) : (int32_t)U;
-            }
-            if (threadIdx.x == 0) w.seg[U] = (int32_t)n;
-        }
-        close_pass(ctl, tag);
-    }
+    if (n == 0 && b == 0) unique_close(w, T, 0, 0);                // an empty batch
+    if (last_block_of_pass(ctl, s_turn)) close_pass(ctl, tag);
 }
 
 // Large steps: the same in two passes over the sorted batch with a prefix sum over the tiles' counts between them
-// (count, k_scan_block_sums, write), and one small kernel for the tables' starts; nothing waits for anything there.
+// (count, k_scan_block_sums, write); nothing waits for anything there.
 template <bool WRITE>
 __global__ void __launch_bounds__(SCAN_THREADS)
-k_unique_pass(Work w, int T, const uint32_t* __restrict__ skey, uint32_t* __restrict__ block_sums) {
+k_unique_pass(State s, Work w, const uint32_t* __restrict__ skey, uint32_t* __restrict__ block_sums) {
     __shared__ uint32_t tmp[SCAN_THREADS / 32 + 1];
     if (w.ctr->abort) return;
     const uint32_t n = w.ctr->L;
     const uint32_t nblk = (n + SCAN_TILE - 1) / SCAN_TILE;
+    const int T = s.T;
     for (uint32_t b = blockIdx.x; b < nblk; b += gridDim.x) {
         const uint32_t base = b * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
-        uint32_t flag[SCAN_ITEMS];
-        int tcur[SCAN_ITEMS];
-        uint32_t sum = 0;
-        uint32_t keyv[SCAN_ITEMS];
-        if (base < n) {
-            int t = find_segment(w.table_start, T, (int32_t)base);
-            while (w.table_start[t + 1] <= (int32_t)base) ++t;     // skip empty tables that start here
-            uint32_t prev = base > 0 ? skey[base - 1] : 0;
-            if (base + SCAN_ITEMS <= n) {                           // 16 keys as four 16-byte loads
-#pragma unroll
-                for (int i = 0; i < SCAN_ITEMS; i += 4) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(skey + base + i);
-                    keyv[i] = v.x; keyv[i + 1] = v.y; keyv[i + 2] = v.z; keyv[i + 3] = v.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < SCAN_ITEMS; ++i) keyv[i] = base + i < n ? skey[base + i] : 0;
-            }
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; ++i) {
-                const uint32_t e = base + i;
-                flag[i] = 0; tcur[i] = t;
-                if (e < n) {
-                    while (w.table_start[t + 1] <= (int32_t)e) ++t;
-                    tcur[i] = t;
-                    const uint32_t k = keyv[i];
-                    flag[i] = (e == (uint32_t)w.table_start[t] || k != prev) ? 1u : 0u;
-                    prev = k;
-                    sum += flag[i];
-                }
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; ++i) { flag[i] = 0; tcur[i] = 0; keyv[i] = 0; }
-        }
+        uint32_t key[SCAN_ITEMS], heads, lasts; int t;
+        unique_items(w.table_start, T, skey, n, base, key, &heads, &lasts, &t);
         uint32_t total;
-        uint32_t ex = block_exclusive_scan<SCAN_THREADS>(sum, &total, tmp);
+        const uint32_t ex = block_exclusive_scan<SCAN_THREADS>(__popc(heads), &total, tmp);
         if (!WRITE) {
             if (threadIdx.x == 0) block_sums[b] = total;
         } else {
-            ex += block_sums[b];
-            uint32_t kout[SCAN_ITEMS];
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; ++i) {
-                const uint32_t e = base + i;
-                ex += flag[i];
-                kout[i] = ex - 1;
-                if (e < n && flag[i]) { w.uniq_row[kout[i]] = (int32_t)keyv[i]; w.uniq_t[kout[i]] = tcur[i]; w.seg[kout[i]] = (int32_t)e; }
-            }
-            if (base + SCAN_ITEMS <= n) {
-#pragma unroll
-                for (int i = 0; i < SCAN_ITEMS; i += 4)
-                    *reinterpret_cast<uint4*>(w.kidx + base + i) = make_uint4(kout[i], kout[i + 1], kout[i + 2], kout[i + 3]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < SCAN_ITEMS; ++i) if (base + i < n) w.kidx[base + i] = kout[i];
-            }
+            unique_write(s, w, skey, n, base, key, heads, lasts, t, ex + block_sums[b]);
         }
     }
-}
-
-__global__ void k_ustart(Work w, int T) {
-    if (w.ctr->abort) return;
-    const uint32_t L = w.ctr->L, U = w.ctr->U;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t <= T; t += gridDim.x * blockDim.x) {
-        const int32_t s = w.table_start[t];
-        w.ustart[t] = (uint32_t)s < L ? (int32_t)w.kidx[s] : (int32_t)U;
-        if (t == 0) w.seg[U] = (int32_t)L;
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
-// cache tag lookup: one lane per distinct row, which reads the `ways` tags of the row's set (Section 3 "Cache Structure")
-// ---------------------------------------------------------------------------------------------
-template <bool IND>
-__global__ void __launch_bounds__(256)
-k_probe(State s, Work w, StepArgs av) {
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
-    const uint32_t epoch = a.epoch;
-    if (w.ctr->abort) return;
-    const int ways = s.ways;
-    const int lane = threadIdx.x & 31;
-    const int64_t U = w.ctr->U;
-    const uint32_t hot_min = U <= HOT_SMALL_U ? (uint32_t)HOT_MIN_SMALL : (uint32_t)HOT_MIN;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t k0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; k0 < U; k0 += nwarps * 32) {
-        const int64_t k = k0 + lane;
-        int32_t row = 0, set = 0, gset = -1;         // gset: index of the row's set in the concatenated cache, -1 = no probe
-        int myloc = LOC_MISS;
-        if (k < U) {
-            const TableDev tb = s.tables[w.uniq_t[k]];
-            row = w.uniq_row[k];
-            if (row >= tb.N) myloc = LOC_INVALID;
-            else if (tb.n_sets > 0) { set = set_of((uint32_t)row, tb.salt, tb.n_sets); gset = (int32_t)(tb.set_base + set); }
-        }
-        // every lane compares its own row with the tags of the row's set (contiguous: `ways` INT32, read 16 bytes at a
-        // time with all loads in flight before any comparison); a set holds a row at most once
-        if (gset >= 0) {
-            const int32_t* __restrict__ tg = s.tags + (int64_t)gset * ways;
-            int mw = -1;
-            if (ways >= 4) {
-                for (int w0 = 0; w0 < ways; w0 += 32) {
-                    int4 t4[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        t4[j] = w0 + 4 * j < ways ? *reinterpret_cast<const int4*>(tg + w0 + 4 * j) : make_int4(-1, -1, -1, -1);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (t4[j].x == row) mw = w0 + 4 * j;
-                        if (t4[j].y == row) mw = w0 + 4 * j + 1;
-                        if (t4[j].z == row) mw = w0 + 4 * j + 2;
-                        if (t4[j].w == row) mw = w0 + 4 * j + 3;
-                    }
-                }
-            } else {
-                for (int w0 = 0; w0 < ways; ++w0) if (tg[w0] == row) mw = w0;
-            }
-            if (mw >= 0) {
-                const int64_t slot = (int64_t)gset * ways + mw;
-                myloc = (int)slot;
-                s.hit_epoch[slot] = epoch; s.hit_k[slot] = (int32_t)k;
-            }
-        }
-        if (k < U) {
-            w.loc[k] = myloc; w.final_loc[k] = myloc; w.uset[k] = set;
-            // rows with very many occurrences get their gradient summed by whole blocks, HOT_SPAN occurrences per task
-            int hb = -1;
-            const uint32_t mult = (uint32_t)(w.seg[k + 1] - w.seg[k]);
-            if (myloc != LOC_INVALID && mult > hot_min) {
-                const uint32_t nt = (mult + HOT_SPAN - 1) / HOT_SPAN;
-                hb = (int)atomicAdd(&w.ctr->hot_tasks, nt);
-                w.hot_k[atomicAdd(&w.ctr->hot_rows, 1u)] = (int32_t)k;
-                atomicAdd(&w.ctr->hot_occ, (unsigned long long)mult);
-                for (uint32_t j = 0; j < nt; ++j) w.task_k[hb + j] = (int32_t)k;
-            }
-            w.hot_base[k] = hb;
-        }
-    }
-}
-
-// per sorted element: where its row lives (by index position) and which sample it belongs to
-template <bool IND>
-__global__ void __launch_bounds__(256)
-k_broadcast(State s, Work w, const uint32_t* __restrict__ spos, StepArgs av) {
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
-    if (w.ctr->abort) return;
-    const int B = a.B;
-    const int64_t L = w.ctr->L;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < L; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t k = w.kidx[i];
-        const uint32_t p = spos[i];
-        w.occ_loc[p] = w.loc[k];
-        // the sign bit marks the last occurrence of a distinct row (sample ids are below 2^31)
-        const bool last = i + 1 >= L || w.kidx[i + 1] != k;
-        w.occ_b[i] = (w.bag_of[p] - w.uniq_t[k] * B) | (last ? (int32_t)0x80000000 : 0);
-    }
+    if (WRITE && blockIdx.x == 0) unique_close(w, T, n, w.ctr->U);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -467,14 +356,69 @@ __device__ __forceinline__ float4 fetch4(const State& s, const TableDev& tb, int
     return dequant4<BITS, RO>(s.codes, s.sb, tb.row_base + row, s.dim, sub);
 }
 
-template <int BITS, int LANES, bool IND>
-__global__ void __launch_bounds__(256)
-k_pool(State s, Work w, StepArgs av) {
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
+// What a forward leaves behind besides the pooled vectors.
+//   FWD_EVAL      nothing (the allocation-free evaluation forward)
+//   FWD_RECORD    the batch as sort records, where its tables begin, and its counters: what a backward needs, since the caller
+//                 may overwrite the indices once the forward has run
+//   FWD_PREPARED  nothing: the batch was recorded (and sorted) ahead by mpe_prepare
+constexpr int FWD_EVAL = 0, FWD_RECORD = 1, FWD_PREPARED = 2;
+
+// The end of a forward: conditions met by its blocks, and (by the block that finishes last) the step's counters and the tiles
+// of its sort.  Inconsistent offsets make the whole output zero and abandon the step.
+template <int MODE>
+__device__ __forceinline__ void forward_close(const State& s, const Work& w, const StepArgs& a, bool bad_offsets, uint32_t bad_rows) {
+    __shared__ uint32_t s_last;
+    Counters* c = w.ctr;
+    if (MODE == FWD_RECORD && bad_rows) atomicAdd(&c->fwd_dropped, (unsigned long long)bad_rows);
+    const int bad = __syncthreads_or(bad_offsets);                 // also: every store of the block has been issued
+    if (threadIdx.x == 0) {
+        if (bad) atomicAdd(&c->fwd_bad, 1u);
+        __threadfence();
+        s_last = atomicAdd(&c->fwd_done, 1u) == gridDim.x - 1u;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const uint32_t nbad = __ldcg(&c->fwd_bad);
+    if (MODE == FWD_RECORD && threadIdx.x < 32) {
+        if (threadIdx.x == 0) {
+            const unsigned long long dropped = __ldcg(&c->fwd_dropped);
+            reset_step(c, a.L, nbad != 0, dropped);
+            if (nbad) c->err[ERR_OFFSETS] += nbad;
+            if (dropped) c->err[ERR_INDEX] += dropped;
+            w.table_start[s.T] = (int32_t)a.L;
+            if (a.B == 0) for (int t = 0; t < s.T; ++t) w.table_start[t] = 0;
+        }
+        __syncwarp();
+        warp_tile_bases<true>(w.table_start, s.T, w.tile_base, nbad != 0, w.sort_tile);
+    }
+    if (nbad) {
+        const int64_t row4 = (int64_t)s.T * s.dim / 4, total = (int64_t)a.B * row4;
+        for (int64_t i = threadIdx.x; i < total; i += blockDim.x) {
+            float* dst = a.out + 4 * i;
+            if (a.route) {
+                const int64_t b = i / row4, x = i - b * row4;
+                const int g = (int)(b / a.route->B_local);
+                dst = a.route->out[g] + ((b - (int64_t)g * a.route->B_local) * a.route->T_global + a.route->t_base) * s.dim + 4 * x;
+            }
+            *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    if (threadIdx.x == 0) { c->fwd_bad = 0; c->fwd_done = 0; c->fwd_dropped = 0; }
+}
+
+
+// Fetch + pool straight from the row ids: the row's home record says where it lives, so the forward needs no sort and no tag look-up per
+// distinct row, and a replayed or launched forward is this one kernel.  A bag's offsets, its row ids and their slots are three
+// dependent loads; they are fetched three, two and one bags ahead.
+template <int BITS, int LANES, int MODE>
+__global__ void __launch_bounds__(256, 4)
+k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
     const int32_t* __restrict__ indices = a.indices;
     const int32_t* __restrict__ offsets = a.offsets;
     float* __restrict__ out = a.out;
     const int B = a.B;
+    const int32_t L = (int32_t)a.L;
     constexpr int NB = LANES < 4 ? LANES : 4;        // rows per batch; two batches are in flight
     constexpr int dim = 4 * LANES;
     const int sub = threadIdx.x & (LANES - 1);
@@ -482,26 +426,46 @@ k_pool(State s, Work w, StepArgs av) {
     const uint32_t gmask = group_mask(LANES);
     const int64_t nbags = (int64_t)s.T * B;
     const int64_t gpb = blockDim.x / LANES, ng = gpb * gridDim.x;
-    const bool abort = w.ctr->abort != 0;
     const char* slab_col = reinterpret_cast<const char*>(s.slab) + 16 * sub;
-    int64_t bag = blockIdx.x * gpb + threadIdx.x / LANES;
-    int t = (int)(bag / B);
-    int64_t b = bag - (int64_t)t * B;
-    // (slot, row id) of the first LANES indices of a bag, one per lane; fetched one bag ahead
-    int32_t lo = 0, hi = 0; int wloc = LOC_INVALID; int32_t wrow = 0;
-    auto open_bag = [&](int64_t bg) {
-        wloc = LOC_INVALID;
-        if (bg < nbags && !abort) {
-            lo = offsets[bg]; hi = offsets[bg + 1];
-            if (lo + sub < hi) { wloc = w.occ_loc[lo + sub]; wrow = indices[lo + sub]; }
-        } else { lo = hi = 0; }
+    const int64_t bag0 = blockIdx.x * gpb + threadIdx.x / LANES;
+    int t = (int)(bag0 / B), b = (int)(bag0 - (int64_t)t * B);
+    const int32_t* off = offsets + bag0;             // of the bag whose offsets are fetched next
+    int32_t to_fetch = bag0 < nbags ? (int32_t)((nbags - bag0 + ng - 1) / ng) : 0, to_pool = to_fetch;
+    bool bad_offsets = false;
+    uint32_t bad_rows = 0;
+    int32_t lo0, hi0, lo1, hi1;                      // this bag's range and the next one's
+    auto next_range = [&](int32_t* lo, int32_t* hi) {
+        *lo = *hi = 0;
+        if (to_fetch > 0) { *lo = off[0]; *hi = off[1]; off += ng; --to_fetch; }
     };
-    open_bag(bag);
-    for (; bag < nbags; bag += ng) {
-        const int64_t row_base = s.tables[t].row_base;
-        const int32_t clo = lo, chi = hi;
-        int myloc = wloc; int32_t myrow = wrow;
-        open_bag(bag + ng);                           // the next bag's first window is on its way while this one is pooled
+    auto check_range = [&](int32_t* lo, int32_t* hi) {       // a bag whose offsets make no sense is not read
+        if (*lo < 0 || *hi < *lo || *hi > L) { bad_offsets = true; *lo = *hi = 0; }
+    };
+    next_range(&lo0, &hi0);
+    check_range(&lo0, &hi0);
+    int32_t row0 = lo0 + sub < hi0 ? indices[lo0 + sub] : 0;
+    next_range(&lo1, &hi1);
+    auto slot_at = [&](const TableDev& tb, int32_t row, bool live) {
+        if (!live) return LOC_INVALID;
+        if (row < 0 || row >= tb.N) { ++bad_rows; return LOC_INVALID; }
+        return __ldg(slot_of(s, tb.row_base + row));
+    };
+    auto record = [&](const TableDev& tb, int32_t p, int32_t row) {
+        if (MODE == FWD_RECORD) __stcs(pairs + p, make_uint2(row < 0 || row >= tb.N ? (uint32_t)tb.N : (uint32_t)row, (uint32_t)b));
+    };
+    for (; to_pool > 0; --to_pool) {
+        const TableDev tb = s.tables[t];
+        const int64_t row_base = tb.row_base;
+        const int32_t clo = lo0, chi = hi0;
+        int32_t myrow = row0;
+        int myloc = slot_at(tb, myrow, clo + sub < chi);
+        if (clo + sub < chi) record(tb, clo + sub, myrow);
+        if (MODE == FWD_RECORD && b == 0 && sub == 0) w.table_start[t] = clo;
+        // the next bag's first row ids are on their way while this bag is pooled, and the offsets of the one after it
+        check_range(&lo1, &hi1);
+        lo0 = lo1; hi0 = hi1;
+        row0 = lo0 + sub < hi0 ? indices[lo0 + sub] : 0;
+        next_range(&lo1, &hi1);
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         // one row: cache resident -> the FP32 row; uncached -> up-convert the codes; out of range -> +0 (never changes the sum)
         auto fetch = [&](int src_lane) {
@@ -521,8 +485,10 @@ k_pool(State s, Work w, StepArgs av) {
         };
         for (int32_t p0 = clo; p0 < chi; p0 += LANES) {
             if (p0 > clo) {                           // later windows of a long bag
-                myloc = LOC_INVALID;
-                if (p0 + sub < chi) { myloc = w.occ_loc[p0 + sub]; myrow = indices[p0 + sub]; }
+                const bool live = p0 + sub < chi;
+                myrow = live ? indices[p0 + sub] : 0;
+                myloc = slot_at(tb, myrow, live);
+                if (live) record(tb, p0 + sub, myrow);
             }
             const int n = min(LANES, chi - p0);
             const uint32_t hits = (__ballot_sync(gmask, myloc >= 0) & gmask) >> gbase;    // bit u: row u of the window is cached
@@ -562,20 +528,23 @@ k_pool(State s, Work w, StepArgs av) {
                 }
             }
         }
-        float* dst = out + (b * s.T + t) * dim;
+        float* dst = out + ((int64_t)b * s.T + t) * dim;
         if (a.route) {                                // the owner of sample b gets the vector, straight into its buffer
             const Route* __restrict__ r = a.route;
-            const int g = (int)(b / r->B_local);
-            dst = r->out[g] + ((b - (int64_t)g * r->B_local) * r->T_global + r->t_base + t) * dim;
+            const int g = b / r->B_local;
+            dst = r->out[g] + ((int64_t)(b - g * r->B_local) * r->T_global + r->t_base + t) * dim;
         }
         __stcs(reinterpret_cast<float4*>(dst) + sub, acc);      // written once, read by somebody else: not worth a place in L2
-        b += ng;
-        while (b >= B) { b -= B; ++t; }
+        int64_t nb = b + ng;
+        while (nb >= B) { nb -= B; ++t; }
+        b = (int)nb;
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && (offsets[0] != 0 || offsets[nbags] != L)) bad_offsets = true;
+    forward_close<MODE>(s, w, a, bad_offsets, bad_rows);
 }
 
 // ---------------------------------------------------------------------------------------------
-// backward 1: new priority value of every row of I_U (Section 3 "Cache Replacement Policy"), candidate keys, counters
+// backward 1: where every row of I_U lives, its new priority value (Section 3 "Cache Replacement Policy"), candidate keys, counters
 // ---------------------------------------------------------------------------------------------
 constexpr int PRI_Q = 4;                 // independent rows per thread: the counter updates are random accesses
 constexpr int PRI_CHUNK = PRI_Q * 256;   // rows per block and round
@@ -627,21 +596,27 @@ k_priority(State s, Work w, uint2* __restrict__ pairs, unsigned long long* __res
         if (FUSED) { if (!draw_tile(ctl, nchunk, s_turn, &chunk, &tag)) break; }
         else if (chunk >= nchunk) break;
         const int64_t c0 = (int64_t)chunk * PRI_CHUNK;
-        int t[Q], loc[Q]; int32_t row[Q]; uint32_t mult[Q], old[Q]; int64_t rb[Q], sbase[Q]; int32_t nsets[Q];
+        int t[Q], loc[Q]; int32_t row[Q], set[Q]; uint32_t mult[Q], old[Q]; int64_t rb[Q], sbase[Q]; int32_t nsets[Q];
         uint32_t ckey[Q]; uint32_t cmask = 0;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int64_t k = c0 + q * 256 + threadIdx.x;
             t[q] = -1;
-            if (k < U) { t[q] = w.uniq_t[k]; row[q] = w.uniq_row[k]; loc[q] = w.loc[k]; mult[q] = (uint32_t)(w.seg[k + 1] - w.seg[k]); }
+            if (k < U) { t[q] = w.uniq_t[k]; row[q] = w.uniq_row[k]; mult[q] = (uint32_t)(w.seg[k + 1] - w.seg[k]); }
         }
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-            old[q] = 0;
+            old[q] = 0; loc[q] = LOC_INVALID; set[q] = 0;
             if (t[q] >= 0) {
                 const TableDev tb = s.tables[t[q]];
                 rb[q] = tb.row_base; nsets[q] = tb.n_sets; sbase[q] = tb.set_base;
-                if (s.policy == 1 && loc[q] != LOC_INVALID) old[q] = s.cnt[rb[q] + row[q]];
+                if (row[q] < tb.N) {
+                    if (s.policy == 1) {
+                        const int2 rec = *reinterpret_cast<const int2*>(slot_of(s, rb[q] + row[q]));
+                        loc[q] = rec.x; old[q] = (uint32_t)rec.y;
+                    } else loc[q] = *slot_of(s, rb[q] + row[q]);
+                    if (tb.n_sets > 0) set[q] = set_of((uint32_t)row[q], tb.salt, tb.n_sets);
+                }
             }
         }
 #pragma unroll
@@ -649,25 +624,27 @@ k_priority(State s, Work w, uint2* __restrict__ pairs, unsigned long long* __res
             const int64_t k = c0 + q * 256 + threadIdx.x;
             unsigned long long m = 0, hitm = 0, uh = 0, un = 0, byp = 0, cand = 0;
             ckey[q] = t[q] >= 0 ? (uint32_t)nsets[q] : 0u;           // large steps: "not a candidate"
+            if (t[q] >= 0) { w.loc[k] = loc[q]; w.final_loc[k] = loc[q]; }
             if (t[q] >= 0 && loc[q] != LOC_INVALID) {
                 m = mult[q]; un = 1;
                 uint32_t pv = step;                      // the priority value the row has from now on
                 if (s.policy == 1) {                     // LFU: access count of the row, saturating
                     pv = old[q] + mult[q] < old[q] ? 0xffffffffU : old[q] + mult[q];
-                    s.cnt[rb[q] + row[q]] = pv;
+                    *count_of(s, rb[q] + row[q]) = pv;
                 }
                 // the cached row's priority value, kept per slot: the LRU time stamp, or a copy of the LFU count (so
                 // that the policy kernel reads one line per set instead of one counter per resident row)
-                if (loc[q] >= 0) s.ts[loc[q]] = pv;
-                if (loc[q] >= 0) { hitm = mult[q]; uh = 1; }
-                else if (nsets[q] > 0) {
+                if (loc[q] >= 0) {
+                    s.ts[loc[q]] = pv;
+                    s.hit_epoch[loc[q]] = a.epoch; s.hit_k[loc[q]] = (int32_t)k;
+                    hitm = mult[q]; uh = 1;
+                } else if (nsets[q] > 0) {
                     // The lowest priority value in a set never falls (counts and time stamps only grow, a replacement
                     // puts a larger value in the place of the lowest, no way is ever emptied), so a row that does not
                     // beat a bound recorded earlier is bypassed whatever happens in this step (Algorithm 2's test).
-                    const int32_t set = w.uset[k];
                     const bool always = s.ways == 1 && s.policy == 0;
-                    if (!always && pv <= s.floor[sbase[q] + set]) byp = 1;
-                    else { ckey[q] = (uint32_t)set; cand = 1; cmask |= 1u << q; }
+                    if (!always && pv <= s.floor[sbase[q] + set[q]]) byp = 1;
+                    else { ckey[q] = (uint32_t)set[q]; cand = 1; cmask |= 1u << q; }
                 }
             }
             // counters: one atomic per warp when the warp sits inside one table
@@ -848,6 +825,7 @@ k_policy(State s, Work w, const uint32_t* __restrict__ ckey, const uint32_t* __r
         const TableDev tb = s.tables[t];
         const int64_t slot = (tb.set_base + key) * ways + way;
         int32_t tag = s.tags[slot];
+        const int32_t resident = tag;
         uint32_t pri = 0;
         if (tag >= 0) pri = s.ts[slot];
         int32_t cand = -1, vict = VICTIM_NONE;
@@ -860,7 +838,7 @@ k_policy(State s, Work w, const uint32_t* __restrict__ ckey, const uint32_t* __r
             if (valid) {
                 ckk = (int32_t)cval[jj];
                 crow = w.uniq_row[ckk];
-                if (s.policy == 1) cpv = s.cnt[tb.row_base + crow];
+                if (s.policy == 1) cpv = *count_of(s, tb.row_base + crow);
             }
             const int n = __popc(__ballot_sync(gmask, valid) & gmask);   // the valid lanes are a prefix of the group
             // Between two replacements the set does not change, so every candidate that cannot beat the current
@@ -908,6 +886,8 @@ k_policy(State s, Work w, const uint32_t* __restrict__ ckey, const uint32_t* __r
         if (cand >= 0) {
             s.tags[slot] = tag;
             s.ts[slot] = pri;                            // the newcomer's priority value (LRU: this step)
+            if (resident >= 0) *slot_of(s, tb.row_base + resident) = LOC_MISS;
+            *slot_of(s, tb.row_base + tag) = (int32_t)slot;
             w.final_loc[cand] = (int32_t)slot;
             w.victim[cand] = vict;
             if (vict == VICTIM_DEFER) w.defer_k[atomicAdd(&w.ctr->deferred, 1u)] = cand;
@@ -1100,6 +1080,7 @@ k_update(State s, Work w, StepArgs av) {
     // C = {victim's key, victim's global row lo, hi, gradient column}
     int4* recs = reinterpret_cast<int4*>(upd_smem + UPD_WARPS * UPD_DEPTH * UPD_NB * 32 * 16) + warp * 96;
     const int64_t U = w.ctr->U;
+    const uint32_t hot_min = hot_threshold(w.ctr->L);
     // rows per hand-out and per group: 32 per warp when there is plenty of work; a step with few distinct rows is cut
     // finer, because there the kernel lasts as long as its longest chain of rows (each row ends in dependent loads)
     const int rpt = U > UPD_SMALL_U ? 32 : (G > 8 ? G : 8);
@@ -1117,12 +1098,13 @@ k_update(State s, Work w, StepArgs av) {
         bool skip = true; int myt = -1;
         if (lane < rpt && k < U) {
             const int32_t first = w.seg[k], row = w.uniq_row[k];
-            const int loc = w.loc[k], floc = w.final_loc[k], hb = w.hot_base[k], victim = w.victim[k], t = w.uniq_t[k];
+            const int loc = w.loc[k], floc = w.final_loc[k], victim = w.victim[k], t = w.uniq_t[k];
+            const int32_t m = w.seg[k + 1] - first;
             myt = t;
             // pseudo rows, hot rows (own kernel) and newcomers that wait for a write-back are not ours
             const bool newcomer = loc < 0 && floc >= 0;
-            skip = loc == LOC_INVALID || hb >= 0 || (newcomer && victim == VICTIM_DEFER);
-            int4 A = make_int4(loc, floc, 0, 0), Bq = make_int4(0, w.seg[k + 1] - first, first, victim), C = make_int4(0, 0, 0, t * dim);
+            skip = loc == LOC_INVALID || (uint32_t)m > hot_min || (newcomer && victim == VICTIM_DEFER);
+            int4 A = make_int4(loc, floc, 0, 0), Bq = make_int4(0, m, first, victim), C = make_int4(0, 0, 0, t * dim);
             if (!skip) {
                 const int64_t rb = s.tables[t].row_base;
                 const int64_t grow = rb + row;
@@ -1287,6 +1269,7 @@ k_update_list(State s, Work w, const int32_t* __restrict__ list, const uint32_t*
     const int sub = lane & (LANES - 1), gbase = lane & ~(LANES - 1);
     const uint32_t gmask = group_mask(LANES);
     const int64_t n = *count;
+    const uint32_t hot_min = hot_threshold(w.ctr->L);
     const int64_t gpb = blockDim.x / LANES, ng = gpb * gridDim.x;
     const uint32_t stride_bytes = (uint32_t)s.T * (uint32_t)dim * 4u;
     for (int64_t i = blockIdx.x * gpb + threadIdx.x / LANES; i < n; i += ng) {
@@ -1302,13 +1285,12 @@ k_update_list(State s, Work w, const int32_t* __restrict__ list, const uint32_t*
         const char* gcol = reinterpret_cast<const char*>(grad + (int64_t)t * dim + 4 * sub);
         const float4 x = fetch4<BITS, false>(s, tb, row, loc, sub);
         float4 g;
-        const int hb = w.hot_base[k];
-        if (hb < 0) {
+        if ((uint32_t)m <= hot_min) {
             g = sum_chunk<LANES>(w.occ_b, gcol, stride_bytes, first, min(32, m), gmask, gbase, sub);
             for (int32_t c = 32; c < m; c += 32)
                 g = add4(g, sum_chunk<LANES>(w.occ_b, gcol, stride_bytes, first + c, min(32, m - c), gmask, gbase, sub));
         } else {
-            const float* part = w.partial + (int64_t)hb * dim + 4 * sub;
+            const float* part = w.partial + (int64_t)w.hot_base[k] * dim + 4 * sub;
             auto term = [&](int64_t j) { return *reinterpret_cast<const float4*>(part + j * dim); };
             g = tree_reduce<4>(term, 0, (m + HOT_SPAN - 1) / HOT_SPAN);
         }
@@ -1384,7 +1366,7 @@ __global__ void k_gather_rows(State s, int t, const int64_t* __restrict__ rows, 
             for (int c = 0; c < code_bytes; ++c) codes[i * code_bytes + c] = s.codes[g * code_bytes + c];
             scale[i] = s.sb ? s.sb[g].x : 1.0f; bias[i] = s.sb ? s.sb[g].y : 0.0f;
         }
-        if (cnt) cnt[i] = s.cnt ? s.cnt[g] : 0u;
+        if (cnt) cnt[i] = s.policy == 1 ? *count_of(s, g) : 0u;
         if (G) G[i] = s.G ? s.G[g] : 0.0f;
     }
 }
@@ -1400,6 +1382,14 @@ k_gather_grad(const Route* __restrict__ r, float* __restrict__ dst, int64_t B, i
         const int g = (int)(b / r->B_local);
         const float4* src = reinterpret_cast<const float4*>(r->out[g] + ((b - (int64_t)g * r->B_local) * r->T_global + r->t_base) * dim);
         reinterpret_cast<float4*>(dst)[i] = src[c];
+    }
+}
+
+// no row is resident, no row has been accessed
+__global__ void k_init_home(State s, int64_t rows) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x) {
+        *slot_of(s, i) = LOC_MISS;
+        if (s.policy == 1) *count_of(s, i) = 0u;
     }
 }
 

@@ -63,12 +63,15 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* t
 // ---- segment -> tile bookkeeping ----------------------------------------------
 // tile_base[t] = number of tiles (of `tile` keys) of segments 0..t-1; tile_base[T] = total.  Called by one warp whose
 // lanes all take part; `off` (the step was abandoned) yields zero tiles, which turns the whole sort into a no-op.
+// FRESH: the starts were written by other blocks of the running kernel (read them from L2).
+template <bool FRESH = false>
 __device__ __forceinline__ void warp_tile_bases(const int32_t* seg_start, int T, int32_t* tile_base, bool off, int tile) {
     const int lane = threadIdx.x & 31;
     int32_t run = 0;
     for (int t0 = 0; t0 < T; t0 += 32) {
         const int t = t0 + lane;
-        const int32_t len = (t < T && !off) ? seg_start[t + 1] - seg_start[t] : 0;
+        int32_t len = 0;
+        if (t < T && !off) len = FRESH ? __ldcg(seg_start + t + 1) - __ldcg(seg_start + t) : seg_start[t + 1] - seg_start[t];
         const int32_t c = (len + tile - 1) / tile;
         int32_t inc = c;
 #pragma unroll
@@ -208,16 +211,13 @@ __device__ __forceinline__ uint32_t sort_look_back(const unsigned long long* wor
 // The counts do not depend on the order of the keys, so one read of the unsorted keys serves all passes.
 // ghist[t][pass][digit] must be zero on entry; the pass that uses a row of it clears it again, and a pass that finds the
 // step abandoned clears all of its rows.
-// PAIRS: the keys are the .x members of (key, payload) records
-template <bool PAIRS>
 __global__ void __launch_bounds__(SORT_THREADS)
-k_sort_digits(const uint32_t* __restrict__ keys, const int32_t* __restrict__ seg_start, const int32_t* __restrict__ tile_base,
+k_sort_digits(const uint2* __restrict__ pairs, const int32_t* __restrict__ seg_start, const int32_t* __restrict__ tile_base,
               int T, int passes, uint32_t* __restrict__ ghist, int tile_keys, int split) {
     // one warp per piece of a tile (`split` pieces per tile: whole tiles in large steps, where the cost of emptying the
     // counters wants many keys to spread over; quarters in small steps, where whole tiles would leave most SMs idle):
     // its own counters, eight key loads in flight per lane, no block-wide barrier
     constexpr int WARPS = SORT_THREADS / 32;
-    constexpr int STRIDE = PAIRS ? 2 : 1;
     __shared__ uint32_t cnt[WARPS][SORT_MAX_PASSES * 256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int npieces = tile_base[T] * split;
@@ -234,7 +234,7 @@ k_sort_digits(const uint32_t* __restrict__ keys, const int32_t* __restrict__ seg
         for (int32_t i0 = start + lane; i0 < end; i0 += 32 * 8) {
             uint32_t k[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) k[q] = i0 + 32 * q < end ? keys[(size_t)(i0 + 32 * q) * STRIDE] : 0u;
+            for (int q = 0; q < 8; ++q) k[q] = i0 + 32 * q < end ? pairs[i0 + 32 * q].x : 0u;
 #pragma unroll
             for (int q = 0; q < 8; ++q)
                 if (i0 + 32 * q < end)
@@ -251,14 +251,13 @@ k_sort_digits(const uint32_t* __restrict__ keys, const int32_t* __restrict__ seg
 }
 
 // ---- one pass: stable scatter ---------------------------------------------------
-// Between passes an element travels as one 8-byte (key, payload) record, so a pass reads and writes it with one
+// An element travels as one 8-byte (key, payload) record, so a pass reads and writes it with one
 // instruction each and a digit's run of a tile is one contiguous piece of memory.
-// FIRST: the input is the bare key array and the payload is the element's position.
 // LAST: the output is split into the sorted keys and the sorted payloads (out_keys / out_vals), which is what the
 // kernels after the sort read.
-template <bool FIRST, bool LAST, int SORT_ITEMS>
+template <bool LAST, int SORT_ITEMS>
 __global__ void __launch_bounds__(SORT_THREADS, MPE_SORT_MINB)
-k_sort_scatter(const uint32_t* __restrict__ keys_in, const uint2* __restrict__ pairs_in, uint2* __restrict__ pairs_out,
+k_sort_scatter(const uint2* __restrict__ pairs_in, uint2* __restrict__ pairs_out,
                uint32_t* __restrict__ out_keys, uint32_t* __restrict__ out_vals,
                const int32_t* __restrict__ seg_start, const int32_t* __restrict__ tile_base, int T, int pass,
                uint32_t* __restrict__ ghist, unsigned long long* __restrict__ status, SortCtl* __restrict__ ctl,
@@ -300,18 +299,14 @@ k_sort_scatter(const uint32_t* __restrict__ keys_in, const uint2* __restrict__ p
 #pragma unroll
             for (int i = 0; i < SORT_ITEMS; ++i) {
                 const int e = e0 + i * 32;
-                if (FIRST) { key[i] = keys_in[start + e]; val[i] = (uint32_t)(start + e); }
-                else { const uint2 kv = pairs_in[start + e]; key[i] = kv.x; val[i] = kv.y; }
+                const uint2 kv = pairs_in[start + e]; key[i] = kv.x; val[i] = kv.y;
             }
         } else {
 #pragma unroll
             for (int i = 0; i < SORT_ITEMS; ++i) {
                 const int e = e0 + i * 32;
                 key[i] = 0xffffffffU; val[i] = 0u;                     // padding: digit 255 in every pass, behind every real key
-                if (e < count) {
-                    if (FIRST) { key[i] = keys_in[start + e]; val[i] = (uint32_t)(start + e); }
-                    else { const uint2 kv = pairs_in[start + e]; key[i] = kv.x; val[i] = kv.y; }
-                }
+                if (e < count) { const uint2 kv = pairs_in[start + e]; key[i] = kv.x; val[i] = kv.y; }
             }
         }
 #pragma unroll
