@@ -283,11 +283,9 @@ def run_ours(args, cfg, rank, world, local_rank):
             h.prepare(batches[i + 1][0], batches[i + 1][1], cfg.batch, side.cuda_stream)
         h.backward(grad, cfg.lr, counter[0])
 
-    # Small steps are replayed from CUDA graphs (which per-kernel event records would break up) and large steps run
-    # beside the next batch's preparation (which makes a kernel's bracketing events include its neighbours): the timed
-    # region runs without the records, and the per-kernel times come from a second pass over the same batches, launched
-    # plainly and without the preparation.
-    graph_sized = maxL <= (4 << 20)
+    # Steps run beside the next batch's preparation, which makes a kernel's bracketing events include its neighbours: the timed
+    # region runs without the records, and the per-kernel times come from a second pass over the same batches, without the
+    # preparation.
 
     def barrier():
         if world > 1:
@@ -386,8 +384,8 @@ def run_ours(args, cfg, rank, world, local_rank):
         "warmup": args.warmup, "ms_per_step": ms_step, "ms_per_step_median": ms_median, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": describe(cfg), "l2": "inputs larger than L2; a new batch every step",
-                   "launch": ("CUDA graph replay" if graph_sized else "plain launches") + "; per-kernel times from a second, plainly launched pass without the preparation",
-                   "next_batch": "sorted ahead on a second stream of lower priority (mpe_prepare) while the current step runs" if ahead and not graph_sized else "not prepared ahead",
+                   "launch": "plain launches; per-kernel times from a second pass without the preparation",
+                   "next_batch": "sorted ahead on a second stream of lower priority (mpe_prepare) while the current step runs" if ahead else "not prepared ahead",
                    "sharding": "each rank trains its own tables (no data-path collective)" if world > 1 else "one GPU"},
         "clocks": clocks,
         "e2e": {"value": e2e_rows / e2e_s if e2e_s > 0 else None, "unit": "rows/s", "h2d_bytes_per_step": h2d,

@@ -109,8 +109,7 @@ int mpe_forward(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offset
  * total_indices takes the result over (its backward waits for the sort on its own stream) and only pools;
  * results are bit-identical with and without the call.  Layouts as in mpe_forward; the two buffers must stay
  * unchanged until that forward.  One batch can be prepared at a time; a forward with other arguments discards it.
- * The call does nothing (and returns MPE_OK) when the batch does not fit the workspace reserved with mpe_reserve, or
- * when steps of this size are replayed from a CUDA graph.  Do not prepare a batch whose forward will be issued while
+ * The call does nothing (and returns MPE_OK) when the batch does not fit the workspace reserved with mpe_reserve.  Do not prepare a batch whose forward will be issued while
  * the caller captures its stream into a graph (the hand-over is an event recorded outside that capture).
  * The first call allocates the second workspace
  * (cudaMalloc; as large as the first, see mpe_workspace_bytes).
@@ -283,10 +282,9 @@ int mpe_export_cache(mpe_handle* h, int32_t table, int32_t* h_tags, float* h_row
 int mpe_export_aux(mpe_handle* h, int32_t table, const int64_t* h_rows, int64_t n, uint32_t* h_cnt,
                    float* h_adagrad);
 
-/* Steps of up to about four million indices are bound by kernel-launch latency, so by default the
- * backward is captured once into a CUDA graph (sized for the reserved workspace) and replayed (a forward is one kernel); the per-call
- * arguments reach the kernels through device memory.  enable = 0 switches to plain launches (larger steps and
- * steps issued while profiling or while the caller captures the stream always use plain launches).  Not allowed between a forward and its backward (MPE_ERR_SEQUENCE).
+/* Kept for its callers: small steps used to be replayed from CUDA graphs because they were chains of some twenty kernels; a
+ * step is a few launches now, made directly whatever is asked for here.  Not allowed between a forward and its
+ * backward (MPE_ERR_SEQUENCE).
  * A graph the CALLER captured around steps of this library may be replayed about 10^8 times in a row: the pass
  * numbers in the sort's per-tile words (30 bits) are started over by mpe_forward's host code, which counts the calls
  * it sees, not by the captured kernels.  For more replays, every 10^8 of them call

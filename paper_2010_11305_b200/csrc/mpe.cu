@@ -2,7 +2,7 @@
 // kernel sequence of one training step.  Nothing here computes on the host;
 // every step of the path runs in the kernels of mpe_kernels.cuh.
 #include "../../include/mpe.h"
-#include "mpe_kernels.cuh"
+#include "mpe_table.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -10,6 +10,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <set>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -39,7 +40,7 @@ struct mpe_handle {
     uint64_t ws_bytes = 0;                  // bytes of the per-step workspace
     uint32_t *sortA = nullptr, *sortB = nullptr;   // two buffers of 2 * sort_n words: (key, payload) records, or keys | payloads
     int64_t sort_n = 0;
-    uint32_t *ghist = nullptr, *block_sums = nullptr;      // the sort's per-table digit counts; candidates per chunk of distinct rows (large steps)
+    uint32_t *ghist = nullptr, *block_sums = nullptr;      // the sort's per-table digit counts; distinct rows per tile
     unsigned long long* sort_status = nullptr;             // the sort's per-tile words
     SortCtl* sort_ctl = nullptr;
     uint64_t sort_passes_bound = 0;                        // no more than this many sort passes have run on either workspace
@@ -84,13 +85,7 @@ struct mpe_handle {
     bool chain_done = false;                // the current batch has been sorted and its distinct rows are known
     StepArgs args{};                        // the current call's arguments (passed by value when launching directly)
     Route* d_route = nullptr;               // destinations of the pooled vectors when the tables are spread over several GPUs
-    // CUDA graph of a backward (small batches are launch-latency bound; a forward is one kernel)
-    bool graphs_enabled = true;
-    cudaStream_t cap = nullptr;             // stream the step is captured on
-    cudaGraph_t g_bwd = nullptr;
-    cudaGraphExec_t x_bwd = nullptr;
-    cudaGraphNode_t n_bwd = nullptr;        // the node that writes the per-call arguments
-    uint64_t k_bwd = 0;                     // kernel nodes of the graph
+    bool graphs_enabled = true;             // accepted and remembered; see mpe_use_graphs
     // instrumentation
     uint64_t launches = 0;
     bool profiling = false;
@@ -99,6 +94,7 @@ struct mpe_handle {
     std::vector<cudaEvent_t> event_pool;
     int last_cuda_error = 0;
     std::map<const void*, int> resident;    // blocks per SM, per kernel
+    std::set<const void*> table_ready;      // cluster kernels whose launch attributes have been set
 };
 
 namespace {
@@ -165,12 +161,6 @@ int dmalloc(mpe_handle* h, T** p, int64_t n, std::vector<void*>* track) {
     return MPE_OK;
 }
 
-void drop_graphs(mpe_handle* h) {
-    if (h->x_bwd) cudaGraphExecDestroy(h->x_bwd);
-    if (h->g_bwd) cudaGraphDestroy(h->g_bwd);
-    h->x_bwd = nullptr; h->g_bwd = nullptr; h->n_bwd = nullptr;
-}
-
 // the current workspace and the other one change places
 void swap_sets(mpe_handle* h) {
     std::swap(h->wk, h->alt.wk);
@@ -192,20 +182,19 @@ void free_set(mpe_handle* h) {
 }
 
 void free_workspace(mpe_handle* h) {
-    drop_graphs(h);                       // they hold the workspace's addresses
     free_set(h);
     swap_sets(h); free_set(h); swap_sets(h);
     h->prepared = false;
     h->cap_L = 0; h->cap_bags = 0;
 }
 
-// Steps this small are bound by launch latency (they are replayed from CUDA graphs); above it the launches hide behind the kernels.
-constexpr int64_t GRAPH_MAX_INDICES = 4 << 20;
+// Batches up to this size are sorted in small tiles: large ones would leave SMs without a tile.
+constexpr int64_t SMALL_TILE_MAX_INDICES = 4 << 20;
 
 int alloc_set(mpe_handle* h, int64_t L, int64_t bags);
 
 int64_t sort_max_tiles(const mpe_handle* h, int64_t L) {
-    const int tile = sort_tile(L <= GRAPH_MAX_INDICES);
+    const int tile = sort_tile(L <= SMALL_TILE_MAX_INDICES);
     return (L + tile - 1) / tile + h->T + 1;
 }
 
@@ -251,22 +240,21 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags) {
     // results have been consumed, and uses the same two
     h->sort_n = (n + 3) & ~int64_t(3);
     A(h->sortA, 2 * h->sort_n); A(h->sortB, 2 * h->sort_n);
-    // small batches (the ones that are replayed from a graph) get small tiles, so that every SM has one
-    w.sort_tile = sort_tile(L <= GRAPH_MAX_INDICES);
+    // small batches get small tiles, so that every SM has one
+    w.sort_tile = sort_tile(L <= SMALL_TILE_MAX_INDICES);
     const int64_t max_tiles = sort_max_tiles(h, L);
     A(h->sort_status, 256 * max_tiles); A(h->ghist, (int64_t)T * SORT_MAX_PASSES * 256); A(h->sort_ctl, 1);
     // the sort keeps these consistent by itself from one pass to the next; they start from zero
     CK(h, cudaMemset(h->sort_status, 0, sizeof(unsigned long long) * 256 * max_tiles));
     CK(h, cudaMemset(h->ghist, 0, sizeof(uint32_t) * T * SORT_MAX_PASSES * 256));
     CK(h, cudaMemset(h->sort_ctl, 0, sizeof(SortCtl)));
-    A(h->block_sums, n / std::min<int64_t>(SCAN_TILE, PRI_CHUNK) + 2);
-    A(w.ctr, 1); A(w.args, 1);
-    A(w.table_start, T + 1); A(w.tile_base, T + 1); A(w.ustart, T + 1); A(w.ctile_base, T + 1);
+    A(h->block_sums, n / SCAN_TILE + 2);
+    A(w.ctr, 1);
+    A(w.table_start, T + 1); A(w.tile_base, T + 1); A(w.ustart, T + 1);
     A(w.occ_b, n);
     A(w.uniq_row, nu); A(w.uniq_t, nu); A(w.seg, nu + 1); A(w.loc, nu); A(w.final_loc, nu);
     A(w.victim, nu); A(w.defer_k, nu); A(w.heads, nu);
-    A(w.hot_base, nu); A(w.cand_key, nu); A(w.cand_cnt, T); A(w.cstart, T + 1);
-    CK(h, cudaMemset(w.cand_cnt, 0, sizeof(int32_t) * T));
+    A(w.hot_base, nu); A(w.cand_key, nu);
     const int64_t max_tasks = hot_capacity(L);
     A(w.task_k, max_tasks); A(w.partial, max_tasks * h->dim); A(w.hot_k, max_tasks);
 #undef A
@@ -283,11 +271,11 @@ SortBufs sort_bufs(const mpe_handle* h) {
     return SortBufs{h->sortA, h->sortB, h->sort_n, h->ghist, h->sort_status, h->sort_ctl, &h->wk.ctr->abort, h->wk.sort_tile};
 }
 
-// stable sort of every segment [seg_start[t], seg_start[t+1]) by the low `key_bits` bits of the key; *skey receives where the
-// sorted keys are.  The sorted payloads go to `vals`, or (vals == nullptr) behind the keys, and *sval receives where.
+// stable sort of every segment [seg_start[t], seg_start[t+1]) by the low `key_bits` bits of the key; the sorted payloads go to
+// `vals`, *skey receives where the sorted keys are
 // tile_base: the segments' tile bookkeeping (warp_tile_bases), filled by the kernel that produced seg_start
 void seg_sort(mpe_handle* h, const SortBufs& b, const int32_t* seg_start, const int32_t* tile_base,
-              int key_bits, int64_t n_upper, uint32_t* vals, const uint32_t** skey, const uint32_t** sval) {
+              int key_bits, int64_t n_upper, uint32_t* vals, const uint32_t** skey) {
     const int T = h->T;
     const int64_t max_tiles = (n_upper + b.tile - 1) / b.tile + T;
     const int passes = (key_bits + 7) / 8;
@@ -299,7 +287,7 @@ void seg_sort(mpe_handle* h, const SortBufs& b, const int32_t* seg_start, const 
         uint32_t* src = (p & 1) ? b.A : b.B;                      // pass p reads B and writes A when p is even, the other way round when odd
         uint32_t* dst = (p & 1) ? b.B : b.A;
         const uint2* pin = reinterpret_cast<const uint2*>(src);
-        uint2* pout = reinterpret_cast<uint2*>(dst); uint32_t* ok = dst; uint32_t* ov = vals ? vals : dst + b.n;
+        uint2* pout = reinterpret_cast<uint2*>(dst); uint32_t* ok = dst; uint32_t* ov = vals;
         // tiles are handed out by ticket, so the grid only has to be large enough to fill the GPU
 #define SCATTER(L, ITEMS) do { \
         auto kern = k_sort_scatter<L, ITEMS>; \
@@ -311,7 +299,7 @@ void seg_sort(mpe_handle* h, const SortBufs& b, const int32_t* seg_start, const 
         else if (small) SCATTER(false, SORT_ITEMS_SMALL);
         else SCATTER(false, SORT_ITEMS_LARGE);
 #undef SCATTER
-        if (last) { *skey = dst; if (sval) *sval = ov; }
+        if (last) *skey = dst;
     }
 }
 
@@ -399,7 +387,6 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
     DeviceGuard guard(device);
     cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess ||
         cudaStreamCreateWithFlags(&h->copy_in, cudaStreamNonBlocking) != cudaSuccess ||
@@ -459,6 +446,8 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
     if ((rc = dmalloc(h, &s.ts, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.hit_epoch, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.hit_k, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
+    if ((rc = dmalloc(h, &s.set_cnt, std::max<int64_t>(1, h->total_sets), nullptr)) != MPE_OK) return fail(rc);
+    if ((rc = dmalloc(h, &s.bucket, h->total_sets * bucket_cap(ways), nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.floor, std::max<int64_t>(1, h->total_sets), nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.stats, (int64_t)num_tables * 8, nullptr)) != MPE_OK) return fail(rc);
 #define CKC(expr) do { cudaError_t e_ = (expr); if (e_ != cudaSuccess) { h->last_cuda_error = (int)e_; return fail(MPE_ERR_CUDA); } } while (0)
@@ -467,6 +456,7 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
     CKC(cudaMemset(s.slab, 0, sizeof(float) * std::max<int64_t>(1, h->total_slots * dim)));
     if (s.ts) CKC(cudaMemset(s.ts, 0, sizeof(uint32_t) * std::max<int64_t>(1, h->total_slots)));
     CKC(cudaMemset(s.hit_epoch, 0, sizeof(uint32_t) * std::max<int64_t>(1, h->total_slots)));
+    CKC(cudaMemset(s.set_cnt, 0, sizeof(uint32_t) * std::max<int64_t>(1, h->total_sets)));
     CKC(cudaMemset(s.floor, 0, sizeof(uint32_t) * std::max<int64_t>(1, h->total_sets)));
     CKC(cudaMemset(s.stats, 0, sizeof(unsigned long long) * 8 * num_tables));
     LAUNCH(h, "init_home", k_init_home, grid_for(h, h->total_rows, 256, 8), 256, 0, s, h->total_rows);
@@ -500,24 +490,65 @@ int mpe_reserve(mpe_handle* h, int32_t max_batch, int64_t max_total_indices) {
 
 namespace {
 
-// Launch sizes follow L_grid (an upper bound: every kernel walks its range with a grid stride and reads the
-// true sizes from device memory), so one captured graph serves every batch that fits the workspace.
-// What backward needs of the batch and the indices alone decide (no table, cache or policy state): the sorted batch and its
-// distinct rows.  The records to sort are in sort_input().
-void enqueue_index_chain(mpe_handle* h, int64_t L_grid, bool ind) {
-    Work& w = h->wk;
-    // sort the row indices of the mini-batch (Section 5.1), table by table
-    seg_sort(h, sort_bufs(h), w.table_start, w.tile_base, bits_for((uint32_t)h->max_rows), L_grid,
-             reinterpret_cast<uint32_t*>(w.occ_b), &h->skey, nullptr);
-    // distinct rows
-    const int gs = grid_for(h, L_grid, SCAN_TILE, 8);
-    if (ind) {
-        LAUNCH(h, "unique", k_unique, gs, SCAN_THREADS, 0, h->st, w, h->skey, h->sort_status, h->sort_ctl);
-    } else {
-        LAUNCH(h, "unique_count", k_unique_pass<false>, gs, SCAN_THREADS, 0, h->st, w, h->skey, h->block_sums);
-        LAUNCH(h, "scan_block_sums", k_scan_block_sums, 1, BSUM_THREADS, 0, h->block_sums, (const uint32_t*)&w.ctr->L, (uint32_t)SCAN_TILE, &w.ctr->U);
-        LAUNCH(h, "unique_write", k_unique_pass<true>, gs, SCAN_THREADS, 0, h->st, w, h->skey, h->block_sums);
+// How a step's index work is done.  Table by table, a cluster of `blocks` thread blocks each (mpe_table.cuh), if the tables'
+// segments are of a size for that; else (blocks == 0) by grid-wide kernels.
+// Only the average segment is known here.  A table with a larger one than its cluster's shared memory holds is sorted through
+// global memory by the same kernel: slower, not wrong.
+struct TablePlan { int blocks; int items; };
+constexpr int TBL_ITEMS_SMALL = 4, TBL_ITEMS_LARGE = 12;            // elements per thread: 4096 and 12288 per block
+constexpr int64_t TBL_MAX_SEGMENT = 150000;                         // average; sixteen blocks hold 196608
+TablePlan table_plan(const mpe_handle* h, int64_t L) {
+    const int64_t avg = (L + h->T - 1) / h->T;
+    if (avg > TBL_MAX_SEGMENT) return {0, 0};
+    // about four elements per thread keep a block's phases short; more where the clusters would not fit the GPU side by side
+    int blocks = 1;
+    while (blocks < TBL_MAX_CLUSTER && (int64_t)blocks * TBL_ITEMS_SMALL * TBL_THREADS < avg + avg / 8) blocks *= 2;
+    while (blocks > 1 && (int64_t)h->T * blocks > h->num_sms && (int64_t)(blocks / 2) * TBL_ITEMS_LARGE * TBL_THREADS >= avg + avg / 8) blocks /= 2;
+    const int items = (int64_t)blocks * TBL_ITEMS_SMALL * TBL_THREADS >= avg + avg / 8 ? TBL_ITEMS_SMALL : TBL_ITEMS_LARGE;
+    return {blocks, items};
+}
+
+template <int ITEMS, bool STATE>
+int launch_table(mpe_handle* h, int blocks, const StepArgs& av) {
+    auto kern = k_table<ITEMS, STATE>;
+    const size_t smem = (size_t)ITEMS * TBL_THREADS * sizeof(uint2) + sizeof(TableShared);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)blocks; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(h->T * blocks)); cfg.blockDim = dim3(TBL_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = h->stream;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    if (!h->table_ready.count(reinterpret_cast<const void*>(kern))) {
+        CK(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CK(h, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        h->table_ready.insert(reinterpret_cast<const void*>(kern));
     }
+    LaunchScope ls(h, STATE ? "table" : "table_sort", h->stream);
+    CK(h, cudaLaunchKernelEx(&cfg, kern, h->st, h->wk, sort_input(sort_bufs(h)), reinterpret_cast<uint2*>(h->sortA), h->sort_status, h->sort_ctl,
+                             (uint32_t)av.step, av.epoch));
+    return MPE_OK;
+}
+// the sort and the distinct rows; `state`: the priorities and the admission too (a cluster of one block)
+int enqueue_table(mpe_handle* h, const TablePlan& plan, const StepArgs& av, bool state) {
+    if (plan.items == TBL_ITEMS_LARGE) return launch_table<TBL_ITEMS_LARGE, false>(h, plan.blocks, av);
+    return state ? launch_table<TBL_ITEMS_SMALL, true>(h, plan.blocks, av) : launch_table<TBL_ITEMS_SMALL, false>(h, plan.blocks, av);
+}
+
+// What backward needs of the batch and the indices alone decide (no table, cache or policy state): the sorted batch and its
+// distinct rows.  The records to sort are in sort_input().  Launch sizes follow L, an upper bound of what the kernels read from
+// device memory.
+int enqueue_index_chain(mpe_handle* h, int64_t L) {
+    Work& w = h->wk;
+    const TablePlan plan = table_plan(h, L);
+    if (plan.blocks) return enqueue_table(h, plan, StepArgs{}, false);
+    // sort the row indices of the mini-batch (Section 5.1), table by table
+    seg_sort(h, sort_bufs(h), w.table_start, w.tile_base, bits_for((uint32_t)h->max_rows), L, reinterpret_cast<uint32_t*>(w.occ_b), &h->skey);
+    // distinct rows
+    const int gs = grid_for(h, L, SCAN_TILE, 8);
+    LAUNCH(h, "unique_count", k_unique_pass<false>, gs, SCAN_THREADS, 0, h->st, w, h->skey, h->block_sums);
+    LAUNCH(h, "scan_block_sums", k_scan_block_sums, 1, BSUM_THREADS, 0, h->block_sums, (const uint32_t*)&w.ctr->L, (uint32_t)SCAN_TILE, &w.ctr->U);
+    LAUNCH(h, "unique_write", k_unique_pass<true>, gs, SCAN_THREADS, 0, h->st, w, h->skey, h->block_sums);
+    return MPE_OK;
 }
 
 // fetch + pool, and (MODE) the record of the batch
@@ -531,44 +562,44 @@ void enqueue_pool(mpe_handle* h, const Work& w, uint2* records, int64_t bags, co
     });
 }
 
-int enqueue_backward(mpe_handle* h, int64_t L, bool ind, bool chain) {
+int enqueue_backward(mpe_handle* h, int64_t L, bool chain) {
     const State& s = h->st;
     Work& w = h->wk;
     const StepArgs av = h->args;
-    if (chain) enqueue_index_chain(h, L, ind);
-    // the hot rows' partial gradient sums only need the sorted batch: they run on a second stream next to the
-    // priority / candidate-sort / policy kernels, which leave most of the machine idle
-    CK(h, cudaEventRecord(h->ev_fork, h->stream));
-    CK(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
-    dispatch(h->bits, s.lanes, [&](auto bc, auto lc) {
-        constexpr int LANES = decltype(lc)::value;
-        auto hot = ind ? k_hot_partial<LANES, true> : k_hot_partial<LANES, false>;
-        LAUNCH_ON(h, h->side, "hot_partial", hot, grid_for(h, hot_capacity(L), 1, 2), 8 * LANES, 32 * s.dim * sizeof(float), s, w, av);
-    });
-    CK(h, cudaEventRecord(h->ev_join, h->side));
-    const SortBufs sb = sort_bufs(h);
-    // where the rows live, new priority values; the rows that may be admitted (few, once the caches are warm) are gathered in row order ...
-    LAUNCH(h, "priority", (ind ? k_priority<true> : k_priority<false>), grid_for(h, L, PRI_CHUNK, 8), 256, 0, s, w,
-           h->max_sets > 0 ? sort_input(sb) : (uint2*)nullptr, h->sort_status, h->sort_ctl, h->block_sums, av);
-    if (h->max_sets > 0) {
-        if (!ind) {        // large steps: the list is made by three small kernels
-            LAUNCH(h, "scan_block_sums", k_scan_block_sums, 1, BSUM_THREADS, 0, h->block_sums, (const uint32_t*)&w.ctr->U, (uint32_t)PRI_CHUNK, &w.ctr->n_cand);
-            LAUNCH(h, "cand_write", k_cand_write, grid_for(h, L, PRI_CHUNK, 8), 256, 0, s, w, (const uint32_t*)h->block_sums, sort_input(sb));
-            LAUNCH(h, "cand_starts", k_cand_starts, 1, 32, 0, w, h->T);
-        }
-        // ... and grouped by cache set, keeping ascending row id inside a set
-        const uint32_t *ck = nullptr, *cv = nullptr;
-        seg_sort(h, sb, w.cstart, w.ctile_base, bits_for((uint32_t)h->max_sets), L, nullptr, &ck, &cv);
-        LAUNCH(h, "policy_heads", k_policy_heads, grid_for(h, L, 256, 8), 256, 0, s, w, ck);
-        auto pol = ind ? k_policy<true> : k_policy<false>;
-        LAUNCH(h, "policy", pol, grid_for(h, std::min<int64_t>(L, h->total_sets), 256 / s.ways, resident_blocks(h, pol, 256, 0)), 256, 0, s, w, ck, cv, av);
+    const TablePlan plan = table_plan(h, L);
+    int rc = MPE_OK;
+    // the hot rows' partial gradient sums: on a second stream, next to the kernels that leave most of the machine idle
+    auto hot_partial = [&]() -> int {
+        CK(h, cudaEventRecord(h->ev_fork, h->stream));
+        CK(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+        dispatch(h->bits, s.lanes, [&](auto bc, auto lc) {
+            constexpr int LANES = decltype(lc)::value;
+            LAUNCH_ON(h, h->side, "hot_partial", k_hot_partial<LANES>, grid_for(h, hot_capacity(L), 1, 2), 8 * LANES, 32 * s.dim * sizeof(float), s, w, av);
+        });
+        CK(h, cudaEventRecord(h->ev_join, h->side));
+        return MPE_OK;
+    };
+    if (plan.blocks == 1 && plan.items == TBL_ITEMS_SMALL && chain) {
+        rc = enqueue_table(h, plan, av, true);
+        if (rc == MPE_OK) rc = hot_partial();
+    } else {
+        // (the cluster kernel leaves the hot rows to k_priority; the grid-wide kernels list them with the distinct rows, so that
+        // their partial sums can start before it)
+        const bool by_table = plan.blocks != 0;
+        if (chain) rc = enqueue_index_chain(h, L);
+        if (rc == MPE_OK && !by_table) rc = hot_partial();
+        LAUNCH(h, "priority", k_priority, grid_for(h, L, PRI_CHUNK, 8), 256, 0, s, w, av, by_table ? 1 : 0);
+        if (rc == MPE_OK && by_table) rc = hot_partial();
+        if (h->max_sets > 0)
+            LAUNCH(h, "policy", k_policy, grid_for(h, std::min<int64_t>(L, h->total_sets), 256 / s.ways, resident_blocks(h, k_policy, 256, 0)), 256, 0, s, w, av);
     }
+    if (rc != MPE_OK) return rc;
     const int gu = grid_for(h, (L + 7) / 8, UPD_WARPS, 8);
     const int gh = grid_for(h, hot_capacity(L), 256 / s.lanes, 4);
     dispatch(h->bits, s.lanes, [&](auto bc, auto lc) {
         constexpr int BITS = decltype(bc)::value, LANES = decltype(lc)::value;
-        auto upd = ind ? k_update<BITS, LANES, true> : k_update<BITS, LANES, false>;
-        auto lst = ind ? k_update_list<BITS, LANES, true> : k_update_list<BITS, LANES, false>;
+        auto lst = k_update_list<BITS, LANES>;
+        auto upd = k_update<BITS, LANES>;
         LAUNCH(h, "update", upd, gu, UPD_WARPS * 32, UPD_SMEM, s, w, av);
         cudaStreamWaitEvent(h->stream, h->ev_join, 0);
         LAUNCH(h, "update_hot", lst, gh, 256, 0, s, w, (const int32_t*)w.hot_k, (const uint32_t*)&w.ctr->hot_rows, 0, av);
@@ -576,47 +607,6 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool ind, bool chain) {
             LAUNCH(h, "update_deferred", lst, gh, 256, 0, s, w, (const int32_t*)w.defer_k, (const uint32_t*)&w.ctr->deferred, 1, av);
     });
     return check_launch(h);
-}
-
-bool may_use_graph(mpe_handle* h) {
-    if (!h->graphs_enabled || h->profiling || h->cap_L > GRAPH_MAX_INDICES) return false;
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;   // the caller captures: plain launches join his graph
-    return true;
-}
-
-// Capture one half of the step (sized for the whole workspace) into a graph; `head` is the kernel that writes the arguments.
-template <class Body>
-int capture(mpe_handle* h, cudaGraph_t* graph, cudaGraphExec_t* exec, cudaGraphNode_t* args_node, uint64_t* kernels, const void* head,
-            Body&& body) {
-    cudaStream_t user = h->stream;
-    const uint64_t launches_before = h->launches;
-    h->stream = h->cap;
-    cudaError_t e = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal);
-    int rc = MPE_OK;
-    if (e == cudaSuccess) {
-        rc = body();
-        e = cudaStreamEndCapture(h->cap, graph);
-    }
-    h->stream = user;
-    h->launches = launches_before;
-    if (e != cudaSuccess || rc != MPE_OK || !*graph) { h->last_cuda_error = (int)e; cudaGetLastError(); return rc != MPE_OK ? rc : MPE_ERR_CUDA; }
-    CK(h, cudaGraphInstantiate(exec, *graph, 0));
-    size_t n = 0;
-    CK(h, cudaGraphGetNodes(*graph, nullptr, &n));
-    std::vector<cudaGraphNode_t> nodes(n);
-    CK(h, cudaGraphGetNodes(*graph, nodes.data(), &n));
-    *args_node = nullptr; *kernels = 0;
-    for (cudaGraphNode_t nd : nodes) {
-        cudaGraphNodeType ty;
-        CK(h, cudaGraphNodeGetType(nd, &ty));
-        if (ty != cudaGraphNodeTypeKernel) continue;
-        ++*kernels;
-        cudaKernelNodeParams kp{};
-        CK(h, cudaGraphKernelNodeGetParams(nd, &kp));
-        if (kp.func == head) *args_node = nd;
-    }
-    return *args_node ? MPE_OK : MPE_ERR_CUDA;
 }
 
 // the handle's stream waits for the sort of the current batch, if that was done ahead
@@ -670,9 +660,8 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
                  cudaStream_t stream) {
     const int64_t bags = (int64_t)h->T * batch;
     h->prepared = false;
-    // only what fits the reserved workspace, and only steps that are launched plainly (replayed steps are bound by launch
-    // latency, not by their kernels): otherwise the forward simply does all of its work itself
-    if (total_indices > h->cap_L || bags > h->cap_bags || !h->wk.ctr || may_use_graph(h)) return MPE_OK;
+    // only what fits the reserved workspace: otherwise the step simply does all of its work itself
+    if (total_indices > h->cap_L || bags > h->cap_bags || !h->wk.ctr) return MPE_OK;
     if (!h->alt.wk.ctr) {                    // first use: the second workspace
         swap_sets(h);
         int rc = alloc_set(h, h->cap_L, h->cap_bags);
@@ -680,6 +669,7 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
         swap_sets(h);
         if (rc != MPE_OK) return rc;
     }
+    int rc = MPE_OK;
     StepArgs av{};
     av.indices = d_indices; av.offsets = d_offsets; av.B = batch; av.L = (uint32_t)total_indices;
     cudaStream_t user = h->stream;
@@ -691,10 +681,10 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
         LAUNCH(h, "prelude", k_prelude, 1, 32, 0, h->wk, h->T, av);
         LAUNCH(h, "make_keys", k_make_keys, grid_for(h, bags, 32, 8), 256, 0, h->st, h->wk, sort_input(sort_bufs(h)), av);
         e = cudaEventRecord(h->ev_keys, stream);
-        enqueue_index_chain(h, total_indices, false);
+        rc = enqueue_index_chain(h, total_indices);
         if (e == cudaSuccess) e = cudaEventRecord(h->ev_prep, stream);
     }
-    int rc = check_launch(h);
+    if (rc == MPE_OK) rc = check_launch(h);
     h->stream = user;
     swap_sets(h);
     if (e != cudaSuccess) { h->last_cuda_error = (int)e; return MPE_ERR_CUDA; }
@@ -820,35 +810,11 @@ int mpe_backward(mpe_handle* h, const float* d_grad_out, float lr, int64_t step)
     if (reinterpret_cast<uintptr_t>(d_grad_out) & 15) return MPE_ERR_ARG;   // rows are moved 16 bytes at a time
     if (step <= h->last_step) return MPE_ERR_SEQUENCE;
     DeviceGuard guard(h->device);
-    Work& w = h->wk;
     h->args.grad = d_grad_out; h->args.lr = lr; h->args.step = (unsigned long long)step;
     int rc = await_prepared(h);
     if (rc != MPE_OK) return rc;
-    bool done = false;
-    if (!h->chain_done && may_use_graph(h)) {
-        if (!h->x_bwd) {
-            rc = capture(h, &h->g_bwd, &h->x_bwd, &h->n_bwd, &h->k_bwd, (const void*)k_set_args_backward, [&]() {
-                LAUNCH(h, "set_args", k_set_args_backward, 1, 1, 0, w.args, h->args);
-                return enqueue_backward(h, h->cap_L, true, true);
-            });
-            if (rc != MPE_OK) { drop_graphs(h); h->graphs_enabled = false; }      // fall back to plain launches for good
-        }
-        if (rc == MPE_OK) {
-            StepArgs* a = w.args;
-            StepArgs av = h->args;
-            void* params[] = {&a, &av};
-            cudaKernelNodeParams kp{};
-            kp.func = (void*)k_set_args_backward; kp.gridDim = dim3(1); kp.blockDim = dim3(1); kp.kernelParams = params;
-            CK(h, cudaGraphExecKernelNodeSetParams(h->x_bwd, h->n_bwd, &kp));
-            CK(h, cudaGraphLaunch(h->x_bwd, h->stream));
-            h->launches += h->k_bwd;
-            done = true;
-        }
-    }
-    if (!done) {
-        rc = enqueue_backward(h, h->L, false, !h->chain_done);
-        if (rc != MPE_OK) return rc;
-    }
+    rc = enqueue_backward(h, h->L, !h->chain_done);
+    if (rc != MPE_OK) return rc;
     CK(h, cudaEventRecord(h->ev_free, h->stream));
     h->have_forward = false;
     h->last_step = step;
@@ -862,7 +828,6 @@ int mpe_set_rounding(mpe_handle* h, int32_t mode) {
     DeviceGuard guard(h->device);
     CK(h, cudaStreamSynchronize(h->stream));
     h->st.rounding = mode;
-    drop_graphs(h);           // the captured kernels carry the old setting
     return MPE_OK;
 }
 
@@ -971,7 +936,6 @@ int mpe_destroy(mpe_handle* h) {
     DeviceGuard guard(h->device);
     cudaStreamSynchronize(h->stream);
     if (h->side) { cudaStreamSynchronize(h->side); cudaStreamDestroy(h->side); }
-    if (h->cap) cudaStreamDestroy(h->cap);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->prep) { cudaStreamSynchronize(h->prep); cudaStreamDestroy(h->prep); }
@@ -987,7 +951,7 @@ int mpe_destroy(mpe_handle* h) {
     if (h->table_on_host) { cudaFreeHost(s.codes); cudaFreeHost(s.sb); } else { cudaFree(s.codes); cudaFree(s.sb); }
     cudaFree(h->d_route);
     cudaFree(h->d_tables); cudaFree(s.G); cudaFree(s.slab);
-    cudaFree(s.tags); cudaFree(s.home); cudaFree(s.ts); cudaFree(s.hit_epoch); cudaFree(s.hit_k); cudaFree(s.floor); cudaFree(s.stats);
+    cudaFree(s.tags); cudaFree(s.home); cudaFree(s.ts); cudaFree(s.hit_epoch); cudaFree(s.hit_k); cudaFree(s.floor); cudaFree(s.set_cnt); cudaFree(s.bucket); cudaFree(s.stats);
     for (auto& r : h->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (auto e : h->event_pool) cudaEventDestroy(e);
     delete h;
@@ -1085,7 +1049,8 @@ int mpe_step_info(mpe_handle* h, int64_t* out6) {
     if (!h->wk.ctr) return MPE_OK;
     DeviceGuard guard(h->device);
     if (h->have_forward && !h->chain_done) {           // a forward alone does not sort its batch: the distinct rows are counted on demand
-        enqueue_index_chain(h, h->L, false);
+        int rc = enqueue_index_chain(h, h->L);
+        if (rc != MPE_OK) return rc;
         h->chain_done = true;
     }
     CK(h, cudaStreamSynchronize(h->stream));

@@ -40,7 +40,6 @@ struct Counters {
     uint32_t deferred;     // newcomers that wait for the write-back of an updated row
     uint32_t n_heads;      // cache sets that have miss candidates in this step
     uint32_t upd_next;     // next block of 32 distinct rows to hand to a warp of k_update
-    uint32_t n_cand;       // candidates for admission in this step
     unsigned long long fwd_dropped;  // out-of-range indices met by the running forward
     unsigned long long dropped;      // out-of-range indices in this batch
     unsigned long long hot_occ;      // indices that belong to hot rows
@@ -64,6 +63,8 @@ struct State {
     uint32_t* ts;          // [slots] priority value of the resident row: LRU time stamp, or a copy of its LFU count
     uint32_t* hit_epoch;   // [slots] forward call in which the slot was last hit
     int32_t* hit_k;        // [slots] unique-row index of that hit
+    uint32_t* set_cnt;     // [sets] candidates for admission dropped into the set's bucket in this step; zero between steps
+    int32_t* bucket;       // [sets][bucket_cap(ways)] their distinct-row indices
     uint32_t* floor;       // [sets] a lower bound of the lowest priority value among the set's residents (0: none known)
     unsigned long long* stats;   // [T][8]
 };
@@ -71,8 +72,6 @@ struct State {
 __device__ __forceinline__ int32_t* slot_of(const State& s, int64_t row) { return s.home + (row << s.home_shift); }
 __device__ __forceinline__ uint32_t* count_of(const State& s, int64_t row) { return reinterpret_cast<uint32_t*>(s.home + 2 * row + 1); }   // LFU
 
-// What changes from call to call.  It lives in device memory so that a captured CUDA graph of the step stays valid:
-// the kernels read it, one tiny kernel at the head of the graph writes it.
 // Destination of the pooled vectors when the tables are partitioned over several GPUs (Section 1: model parallelism
 // with no replication): sample b belongs to rank b / B_local, whose buffer is [B_local][T_global * dim].
 constexpr int MAX_RANKS = 72;
@@ -81,6 +80,7 @@ struct Route {
     int32_t B_local, T_global, t_base, n_ranks;
 };
 
+// what changes from call to call
 struct StepArgs {
     const int32_t* indices; const int32_t* offsets; float* out; const float* grad;
     int32_t B; uint32_t L; uint32_t epoch; float lr;
@@ -90,17 +90,14 @@ struct StepArgs {
 
 struct Work {
     Counters* ctr;
-    StepArgs* args;
-    int32_t *table_start, *tile_base, *ustart, *ctile_base;   // [T+1]
+    int32_t *table_start, *tile_base, *ustart;   // [T+1]
     int32_t* occ_b;        // [L] by sorted order: sample of the element; sign bit: last occurrence of its row
     int32_t *uniq_row, *uniq_t, *seg, *loc, *final_loc, *victim, *hot_base;   // per unique row
     int32_t* task_k;       // [hot tasks]
     int32_t* hot_k;        // [hot rows]
-    uint32_t* cand_key;    // [distinct rows] large steps: the row's set if it is a candidate for admission, else the table's number of sets
-    int32_t* cand_cnt;     // [T] candidates of each table (counted by k_priority, cleared once the candidates' segments are known)
-    int32_t* cstart;       // [T+1] where each table's candidates begin in the compacted candidate list
+    int32_t* cand_key;     // [distinct rows] the row's set if it is a candidate for admission, else CAND_NONE
     int32_t* defer_k;      // [deferred newcomers]
-    int32_t* heads;        // [sets with candidates] position of the set's first candidate in the set-sorted list
+    int32_t* heads;        // [sets with candidates] one candidate of each (small steps: the set itself, table by table)
     float* partial;        // [hot tasks][dim]
     int32_t sort_tile;     // keys per tile of the sorts of this workspace
 };
@@ -118,9 +115,6 @@ __global__ void k_set_route(Route* dst, Route r) {
     for (int g = threadIdx.x; g < MAX_RANKS; g += blockDim.x) dst->out[g] = r.out[g];
     if (threadIdx.x == 0) { dst->B_local = r.B_local; dst->T_global = r.T_global; dst->t_base = r.t_base; dst->n_ranks = r.n_ranks; }
 }
-// a replayed backward starts with this node, the one whose parameters change from call to call
-__global__ void k_set_args_backward(StepArgs* a, StepArgs v) { *a = v; }
-
 // First kernel of a batch that is sorted ahead of its forward (mpe_prepare); for the others the forward's pooling kernel does this.
 // One warp: resets the step's counters and reads where each table's bags begin (the offsets of bags 0, B, 2B, ...), 32
 // tables at a time so that the loads overlap; offsets that do not start at 0, end at L or grow abandon the step
@@ -188,6 +182,15 @@ k_make_keys(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
 // ---------------------------------------------------------------------------------------------
 // distinct rows of the sorted batch (I_U) and their multiplicities
 // ---------------------------------------------------------------------------------------------
+// a row on the multi-block gradient path: HOT_SPAN occurrences per task
+__device__ __forceinline__ void list_hot_row(const Work& w, int32_t k, uint32_t m) {
+    const uint32_t nt = (m + HOT_SPAN - 1) / HOT_SPAN;
+    const uint32_t hb = atomicAdd(&w.ctr->hot_tasks, nt);
+    w.hot_base[k] = (int32_t)hb;
+    w.hot_k[atomicAdd(&w.ctr->hot_rows, 1u)] = k;
+    atomicAdd(&w.ctr->hot_occ, (unsigned long long)m);
+    for (uint32_t j = 0; j < nt; ++j) w.task_k[hb + j] = k;
+}
 // One thread's SCAN_ITEMS consecutive sorted elements, starting at `base`: their keys, which of them begin a run of equal
 // (table, row) (bit i of *heads) and which end one (bit i of *lasts), and the table of the first.
 __device__ __forceinline__ void unique_items(const int32_t* __restrict__ table_start, int T, const uint32_t* __restrict__ skey, uint32_t n,
@@ -247,12 +250,7 @@ __device__ __forceinline__ void unique_write(const State& s, const Work& w, cons
                     const int32_t mid = lo + ((hi - lo) >> 1);
                     if (skey[mid] == key[i]) lo = mid; else hi = mid;
                 }
-                const uint32_t m = (uint32_t)(hi - e), nt = (m + HOT_SPAN - 1) / HOT_SPAN;
-                const uint32_t hb = atomicAdd(&w.ctr->hot_tasks, nt);
-                w.hot_base[k] = (int32_t)hb;
-                w.hot_k[atomicAdd(&w.ctr->hot_rows, 1u)] = (int32_t)k;
-                atomicAdd(&w.ctr->hot_occ, (unsigned long long)m);
-                for (uint32_t j = 0; j < nt; ++j) w.task_k[hb + j] = (int32_t)k;
+                list_hot_row(w, (int32_t)k, (uint32_t)(hi - e));
             }
             ++k;
         }
@@ -278,47 +276,7 @@ __device__ __forceinline__ void unique_close(const Work& w, int T, uint32_t n, u
     if (threadIdx.x == 0) w.seg[U] = (int32_t)n;
 }
 
-// Small steps (the ones replayed from a graph, where every launch counts), one pass: a tile of the sorted batch flags the first element of every run of equal (table, row), learns how many
-// distinct rows the tiles before it hold (look-back over one word per tile), and writes its part of the lists.
-__global__ void __launch_bounds__(SCAN_THREADS)
-k_unique(State s, Work w, const uint32_t* __restrict__ skey, unsigned long long* __restrict__ words, SortCtl* __restrict__ ctl) {
-    __shared__ uint32_t tmp[SCAN_THREADS / 32 + 1];
-    __shared__ uint32_t s_turn[2];
-    __shared__ uint32_t s_prefix[2];
-    const bool off = w.ctr->abort != 0;                 // an abandoned step has no tiles
-    const uint32_t n = off ? 0u : w.ctr->L;
-    const uint32_t nblk = (n + SCAN_TILE - 1) / SCAN_TILE;
-    const int T = s.T;
-    uint32_t b, tag;
-    while (draw_tile(ctl, nblk, s_turn, &b, &tag)) {
-        const uint32_t base = b * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
-        uint32_t key[SCAN_ITEMS], heads, lasts; int t;
-        unique_items(w.table_start, T, skey, n, base, key, &heads, &lasts, &t);
-        uint32_t total;
-        const uint32_t ex = block_exclusive_scan<SCAN_THREADS>(__popc(heads), &total, tmp);
-        if (threadIdx.x < 32) {
-            if (threadIdx.x == 0) tile_publish(words, b, total, tag);
-            bool poison;
-            const uint32_t before = tile_look_back(words, b, total, tag, &poison);
-            if (threadIdx.x == 0) { s_prefix[0] = before; s_prefix[1] = poison; }
-        }
-        __syncthreads();
-        if (s_prefix[1]) {                                         // a look-back gave up: write nothing, abandon the step
-            if (threadIdx.x == 0) { atomicAdd(&ctl->timeout, 1u); w.ctr->abort = 1; }
-            continue;
-        }
-        unique_write(s, w, skey, n, base, key, heads, lasts, t, ex + s_prefix[0]);
-        if (b == nblk - 1) {
-            if (threadIdx.x == 0) w.ctr->U = s_prefix[0] + total;
-            unique_close(w, T, n, s_prefix[0] + total);
-        }
-    }
-    if (n == 0 && b == 0) unique_close(w, T, 0, 0);                // an empty batch
-    if (last_block_of_pass(ctl, s_turn)) close_pass(ctl, tag);
-}
-
-// Large steps: the same in two passes over the sorted batch with a prefix sum over the tiles' counts between them
-// (count, k_scan_block_sums, write); nothing waits for anything there.
+// Two passes over the sorted batch with a prefix sum over the tiles' counts between them (count, k_scan_block_sums, write).
 template <bool WRITE>
 __global__ void __launch_bounds__(SCAN_THREADS)
 k_unique_pass(State s, Work w, const uint32_t* __restrict__ skey, uint32_t* __restrict__ block_sums) {
@@ -544,60 +502,205 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// backward 1: where every row of I_U lives, its new priority value (Section 3 "Cache Replacement Policy"), candidate keys, counters
+// backward 2: admission / eviction, integer only.  The rows that may be admitted are dropped into their cache set's bucket as
+// their priority values are formed, in whatever order they come; a group of `ways` lanes then takes a set, puts its candidates
+// in ascending row order and applies Algorithm 2's admission test (a candidate whose priority value does
+// not exceed the lowest one among the residents bypasses, otherwise it takes that resident's place).  No row value is read or
+// written here.
+// A bucket holds twice as many candidates as the set has ways (a few more for narrow sets).  A set with more candidates than that
+// finds them by walking its table's distinct rows, which are in row order, and picking those whose candidate key is the set.
 // ---------------------------------------------------------------------------------------------
-constexpr int PRI_Q = 4;                 // independent rows per thread: the counter updates are random accesses
+constexpr int VICTIM_NONE = -1;       // the way was empty, or the displaced row writes itself back
+constexpr int VICTIM_DEFER = -2;      // the displaced row was hit in this step: the newcomer waits for its write-back
+constexpr int CAND_NONE = -1;         // candidate key of a row that is not to be admitted
+__host__ __device__ constexpr int bucket_cap(int ways) { return ways >= 8 ? 2 * ways : (4 * ways < 16 ? 4 * ways : 16); }
+constexpr int BUCKET_CAP_MAX = 64;
+constexpr int BUCKET_PER_LANE = 4;    // bucket_cap(ways) / ways is at most this
+
+// the candidate k joins the bucket of set `gset`; true if it is the set's first one in this step
+__device__ __forceinline__ bool bucket_put(const State& s, int64_t gset, int cap, int32_t k) {
+    const uint32_t pos = atomicAdd(s.set_cnt + gset, 1u);
+    if (pos < (uint32_t)cap) s.bucket[gset * cap + pos] = k;
+    return pos == 0;
+}
+
+struct PolicyCounts { uint32_t admit, evict, bypass; };
+
+// One set.  All lanes of the group (`gmask`, first lane `gbase`) take part; `sorted` is the group's own piece of shared memory,
+// bucket_cap(ways) words.  The table's distinct rows are [ub, ub + n_rows).
+__device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w, const TableDev& tb, int64_t gset, int32_t ub, int32_t n_rows,
+                                                   uint32_t step, uint32_t epoch, uint32_t gmask, int gbase, int way, volatile int32_t* sorted) {
+    const int ways = s.ways, cap = bucket_cap(ways);
+    const int64_t slot = gset * ways + way;
+    const int32_t set = (int32_t)(gset - tb.set_base);
+    const int n = (int)__ldcg(s.set_cnt + gset);                   // candidates
+    int32_t tag = s.tags[slot];
+    uint32_t pri = s.ts[slot];
+    const bool in_bucket = n <= cap;
+    int32_t c[BUCKET_PER_LANE];
+#pragma unroll
+    for (int j = 0; j < BUCKET_PER_LANE; ++j) {
+        c[j] = 0x7fffffff;
+        if (in_bucket && way + j * ways < n) c[j] = __ldcg(s.bucket + gset * cap + way + j * ways);
+    }
+    const int32_t resident = tag;
+    if (tag < 0) pri = 0;
+    if (in_bucket) {                                               // distinct rows are numbered in row order: a candidate's place is the number of smaller ones
+        int place[BUCKET_PER_LANE] = {};
+#pragma unroll
+        for (int j = 0; j < BUCKET_PER_LANE; ++j) {
+            const int live = min(ways, n - j * ways);
+            for (int u = 0; u < live; ++u) {
+                const int32_t v = __shfl_sync(gmask, c[j], gbase + u);
+#pragma unroll
+                for (int i = 0; i < BUCKET_PER_LANE; ++i) place[i] += v < c[i];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < BUCKET_PER_LANE; ++j) if (way + j * ways < n) sorted[place[j]] = c[j];
+    }
+    __syncwarp(gmask);
+    if (way == 0) s.set_cnt[gset] = 0;                             // every lane has read it; empty again for the next step
+    // next `ways` candidates in row order, one per lane: from the sorted bucket, or by walking the table's distinct rows
+    int taken = 0, cursor = 0;                                     // candidates handed out; distinct rows walked
+    auto next_batch = [&](int32_t* k) {
+        if (in_bucket) {
+            *k = taken + way < n ? sorted[taken + way] : -1;
+            const int m = min(ways, n - taken);
+            taken += m;
+            return m;
+        }
+        int m = 0;                                                 // found so far; the first `ways` of them wait in `sorted`
+        *k = -1;
+        while (m < ways && cursor < n_rows) {
+            const int i = cursor + way;
+            const bool mine = i < n_rows && __ldcg(w.cand_key + ub + i) == set;
+            const uint32_t found = (__ballot_sync(gmask, mine) & gmask) >> gbase;
+            const int at = m + __popc(found & ((1u << way) - 1u));
+            const bool take = mine && at < ways;
+            if (take) sorted[at] = ub + i;
+            const uint32_t taken_m = (__ballot_sync(gmask, take) & gmask) >> gbase;
+            m += __popc(taken_m);
+            // a batch that is full ends the walk behind its last candidate
+            cursor = m == ways ? cursor + (32 - __clz(taken_m)) : cursor + ways;
+        }
+        __syncwarp(gmask);
+        if (way < m) *k = sorted[way];
+        __syncwarp(gmask);
+        return m;
+    };
+    int32_t cand = -1, vict = VICTIM_NONE;
+    PolicyCounts pc{0, 0, 0};
+    auto displace = [&]() {                                        // a row that was resident when the step began leaves the cache
+        if (s.hit_epoch[slot] == epoch) { w.final_loc[s.hit_k[slot]] = LOC_MISS; vict = VICTIM_DEFER; }
+        else vict = tag;
+    };
+    if (s.policy == 0 && ways > 1) {
+        // LRU: every candidate has the time stamp of this step, the highest there is.  So the candidates, in row order, take the
+        // empty ways and then the ways with the oldest stamps (ties: lowest way), and bypass once every way was touched in this step.
+        const bool open = tag < 0 || pri < step;
+        const uint32_t age = tag < 0 ? 0u : pri + 1u;
+        const uint32_t opens = (__ballot_sync(gmask, open) & gmask) >> gbase;
+        const int m = min(n, __popc(opens));
+        int order = 0;
+        if (m > 0) {
+            for (int u = 0; u < ways; ++u) {
+                const uint32_t v = __shfl_sync(gmask, age, gbase + u);
+                order += ((opens >> u) & 1u) && (v < age || (v == age && u < way));
+            }
+            int32_t k;
+            next_batch(&k);
+            const int32_t mine = __shfl_sync(gmask, k, gbase + min(order, ways - 1));
+            if (open && order < m) {
+                if (tag >= 0) displace();
+                cand = mine; tag = w.uniq_row[mine]; pri = step;
+            }
+        }
+        const int empties = __popc((__ballot_sync(gmask, resident < 0) & gmask) >> gbase);
+        pc.admit = (uint32_t)m; pc.evict = (uint32_t)max(0, m - empties); pc.bypass = (uint32_t)(n - m);
+    } else {
+        for (int left = n; left > 0;) {
+            int32_t ckk; int32_t crow = 0; uint32_t cpv = step;
+            const int nb = next_batch(&ckk);
+            if (nb == 0) break;
+            left -= nb;
+            const bool valid = way < nb;
+            if (valid) {
+                crow = w.uniq_row[ckk];
+                if (s.policy == 1) cpv = *count_of(s, tb.row_base + crow);
+            }
+            // Between two replacements the set does not change, so every candidate that cannot beat the current
+            // minimum bypasses at once; only the candidates that replace are walked one by one.
+            int u = 0;
+            while (u < nb) {
+                // empty ways rank below every priority; ties go to the lowest way
+                const uint32_t empties = __ballot_sync(gmask, tag < 0) & gmask;
+                int jw; bool jempty; uint32_t jpri = 0;
+                if (empties) { jw = __ffs(empties) - 1 - gbase; jempty = true; }
+                else {
+                    jpri = __reduce_min_sync(gmask, pri);
+                    jw = __ffs(__ballot_sync(gmask, pri == jpri) & gmask) - 1 - gbase;
+                    jempty = false;
+                }
+                // lane `way` holds candidate number `way` of this batch
+                const bool always = ways == 1 && s.policy == 0;                 // direct-mapped LRU never compares
+                const bool would = valid && way >= u && (jempty || always || cpv > jpri);
+                const uint32_t wm = (__ballot_sync(gmask, would) & gmask) >> gbase;
+                if (wm == 0) { pc.bypass += (uint32_t)(nb - u); break; }
+                const int f = __ffs(wm) - 1;                                    // the first candidate that replaces
+                pc.bypass += (uint32_t)(f - u);
+                const int32_t kk = __shfl_sync(gmask, ckk, gbase + f);
+                const int32_t row = __shfl_sync(gmask, crow, gbase + f);
+                const uint32_t pv = __shfl_sync(gmask, cpv, gbase + f);
+                ++pc.admit;
+                if (!jempty) ++pc.evict;
+                if (way == jw) {
+                    if (tag >= 0 && cand < 0) displace();
+                    tag = row; pri = pv; cand = kk;
+                }
+                u = f + 1;
+            }
+        }
+    }
+    {   // what the set's lowest priority value is now bounds it from below for good
+        const bool any_empty = (__ballot_sync(gmask, tag < 0) & gmask) != 0;
+        const uint32_t low = __reduce_min_sync(gmask, tag < 0 ? 0u : pri);
+        if (way == 0) s.floor[gset] = any_empty ? 0u : low;
+    }
+    if (cand >= 0) {
+        s.tags[slot] = tag;
+        s.ts[slot] = pri;                                // the newcomer's priority value (LRU: this step)
+        if (resident >= 0) *slot_of(s, tb.row_base + resident) = LOC_MISS;
+        *slot_of(s, tb.row_base + tag) = (int32_t)slot;
+        w.final_loc[cand] = (int32_t)slot;
+        w.victim[cand] = vict;
+        if (vict == VICTIM_DEFER) w.defer_k[atomicAdd(&w.ctr->deferred, 1u)] = cand;
+    }
+    return pc;
+}
+
+// ---------------------------------------------------------------------------------------------
+// backward 1: where every row of I_U lives, its new priority value (Section 3 "Cache Replacement Policy"), the candidates for
+// admission in their sets' buckets, counters.  (Large steps; small ones do this table by table, mpe_table.cuh.)
+// ---------------------------------------------------------------------------------------------
+constexpr int PRI_Q = 4;                 // independent rows per thread: the home records are random accesses
 constexpr int PRI_CHUNK = PRI_Q * 256;   // rows per block and round
 
-// The rows that may be admitted (few, once the caches are warm) are to become a list of (set, distinct-row index)
-// records in the order of the distinct rows (table, then row id).
-// Small steps (the ones replayed from a graph, where every launch counts): the list leaves this kernel.  A chunk learns
-// how many candidates the chunks before it hold by look-back over one word per chunk, and the block that ends the pass
-// turns the per-table candidate counts into the segments and tiles of the sort by set that follows.
-// Large steps: this kernel leaves each row's candidate key and each chunk's number of candidates, and three small kernels
-// (prefix sum, k_cand_write, k_cand_starts) make the list -- waiting for the chunks before costs more there than
-// reading the keys again.
-// pairs == nullptr: no table has a cache, no list.
-template <bool IND>
-__global__ void __launch_bounds__(256, IND ? 2 : 3)
-k_priority(State s, Work w, uint2* __restrict__ pairs, unsigned long long* __restrict__ words, SortCtl* __restrict__ ctl,
-           uint32_t* __restrict__ block_sums, StepArgs av) {
-    constexpr bool FUSED = IND;
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
-    __shared__ uint32_t wcand[8][PRI_Q];        // candidates per warp and round
-    __shared__ uint32_t s_turn[2];
-    __shared__ uint32_t s_prefix[2];
-    __shared__ uint2 stash[2][PRI_CHUNK];       // the candidates of this chunk and of the one before, in row order
-    const bool off = w.ctr->abort != 0;         // an abandoned step has no chunks
+__global__ void __launch_bounds__(256, 3)
+k_priority(State s, Work w, StepArgs a, int list_hot) {
+    __shared__ uint32_t sums[8][5];
+    if (w.ctr->abort) return;
     const uint32_t step = (uint32_t)a.step;
     constexpr int Q = PRI_Q;
-    const int64_t U = off ? 0 : w.ctr->U;
-    const uint32_t nchunk = (uint32_t)((U + PRI_CHUNK - 1) / PRI_CHUNK);
+    const int64_t U = w.ctr->U;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // A chunk's candidates wait in shared memory while the block works on its next chunk, and go out once that is done:
-    // by then the chunks before it have said how many candidates they hold, so the look-back finds its answer at once.
-    bool have_prev = false; uint32_t prev_chunk = 0, prev_total = 0; int buf = 0;
-    auto write_out = [&](uint32_t chunk_id, uint32_t total, int b) {
-        if (warp == 0) {
-            bool poison;
-            const uint32_t before = tile_look_back(words, chunk_id, total, s_turn[1], &poison);
-            if (lane == 0) { s_prefix[0] = before; s_prefix[1] = poison; }
-        }
-        __syncthreads();
-        if (s_prefix[1]) {                                         // a look-back gave up: write nothing, abandon the step
-            if (threadIdx.x == 0) { atomicAdd(&ctl->timeout, 1u); w.ctr->abort = 1; }
-        } else {
-            for (uint32_t j = threadIdx.x; j < total; j += 256) pairs[s_prefix[0] + j] = stash[b][j];
-        }
-    };
-    uint32_t chunk = blockIdx.x, tag = 0;
+    const int cap = bucket_cap(s.ways);
+    const bool always = s.ways == 1 && s.policy == 0;
+    const uint32_t hot_min = list_hot ? hot_threshold(w.ctr->L) : 0xffffffffU;      // 0: the kernel that listed the distinct rows did it
     // a block takes PRI_CHUNK consecutive rows at a time, thread i the rows i, i + 256, i + 512, i + 768 of them
-    for (;; chunk += gridDim.x) {
-        if (FUSED) { if (!draw_tile(ctl, nchunk, s_turn, &chunk, &tag)) break; }
-        else if (chunk >= nchunk) break;
-        const int64_t c0 = (int64_t)chunk * PRI_CHUNK;
+    for (int64_t c0 = (int64_t)blockIdx.x * PRI_CHUNK; c0 < U; c0 += (int64_t)gridDim.x * PRI_CHUNK) {
         int t[Q], loc[Q]; int32_t row[Q], set[Q]; uint32_t mult[Q], old[Q]; int64_t rb[Q], sbase[Q]; int32_t nsets[Q];
-        uint32_t ckey[Q]; uint32_t cmask = 0;
+        uint32_t low[Q];
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int64_t k = c0 + q * 256 + threadIdx.x;
@@ -620,284 +723,94 @@ k_priority(State s, Work w, uint2* __restrict__ pairs, unsigned long long* __res
             }
         }
 #pragma unroll
+        for (int q = 0; q < Q; ++q)
+            low[q] = t[q] >= 0 && loc[q] == LOC_MISS && nsets[q] > 0 && !always ? s.floor[sbase[q] + set[q]] : 0u;
+        uint32_t m = 0, hitm = 0, un = 0, uh = 0, byp = 0;          // this thread's share of the chunk, if one table fills it
+        const int t_first = w.uniq_t[c0], t_last = w.uniq_t[min(c0 + PRI_CHUNK, U) - 1];
+        const bool one_table = t_first == t_last;
+#pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int64_t k = c0 + q * 256 + threadIdx.x;
-            unsigned long long m = 0, hitm = 0, uh = 0, un = 0, byp = 0, cand = 0;
-            ckey[q] = t[q] >= 0 ? (uint32_t)nsets[q] : 0u;           // large steps: "not a candidate"
-            if (t[q] >= 0) { w.loc[k] = loc[q]; w.final_loc[k] = loc[q]; }
+            int32_t ckey = CAND_NONE;
+            bool lists = false;                          // this candidate is the first of its set
             if (t[q] >= 0 && loc[q] != LOC_INVALID) {
-                m = mult[q]; un = 1;
                 uint32_t pv = step;                      // the priority value the row has from now on
                 if (s.policy == 1) {                     // LFU: access count of the row, saturating
                     pv = old[q] + mult[q] < old[q] ? 0xffffffffU : old[q] + mult[q];
                     *count_of(s, rb[q] + row[q]) = pv;
                 }
+                bool hit = false, bypass = false;
+                if (mult[q] > hot_min) list_hot_row(w, (int32_t)k, mult[q]);
                 // the cached row's priority value, kept per slot: the LRU time stamp, or a copy of the LFU count (so
                 // that the policy kernel reads one line per set instead of one counter per resident row)
                 if (loc[q] >= 0) {
                     s.ts[loc[q]] = pv;
                     s.hit_epoch[loc[q]] = a.epoch; s.hit_k[loc[q]] = (int32_t)k;
-                    hitm = mult[q]; uh = 1;
+                    hit = true;
                 } else if (nsets[q] > 0) {
                     // The lowest priority value in a set never falls (counts and time stamps only grow, a replacement
                     // puts a larger value in the place of the lowest, no way is ever emptied), so a row that does not
                     // beat a bound recorded earlier is bypassed whatever happens in this step (Algorithm 2's test).
-                    const bool always = s.ways == 1 && s.policy == 0;
-                    if (!always && pv <= s.floor[sbase[q] + set[q]]) byp = 1;
-                    else { ckey[q] = (uint32_t)set[q]; cand = 1; cmask |= 1u << q; }
+                    if (!always && pv <= low[q]) bypass = true;
+                    else { ckey = set[q]; lists = bucket_put(s, sbase[q] + set[q], cap, (int32_t)k); }
+                }
+                if (one_table) { m += mult[q]; ++un; if (hit) { hitm += mult[q]; ++uh; } byp += bypass; }
+                else {
+                    unsigned long long* st = s.stats + (int64_t)t[q] * 8;
+                    atomicAdd(st + 0, (unsigned long long)mult[q]); atomicAdd(st + 2, 1ULL);
+                    if (hit) { atomicAdd(st + 1, (unsigned long long)mult[q]); atomicAdd(st + 3, 1ULL); }
+                    if (bypass) atomicAdd(st + 6, 1ULL);
                 }
             }
-            // counters: one atomic per warp when the warp sits inside one table
-            if (c0 + q * 256 + (threadIdx.x & ~31) >= U) continue;           // warp-uniform: nothing left for this q
-            const int t0 = __shfl_sync(0xffffffffU, t[q], 0);
-            const bool same = __all_sync(0xffffffffU, t[q] == t0 || t[q] < 0);
-            if (same && t0 >= 0) {
-                for (int o = 16; o > 0; o >>= 1) {
-                    m += __shfl_xor_sync(0xffffffffU, m, o); hitm += __shfl_xor_sync(0xffffffffU, hitm, o);
-                    uh += __shfl_xor_sync(0xffffffffU, uh, o); un += __shfl_xor_sync(0xffffffffU, un, o);
-                    byp += __shfl_xor_sync(0xffffffffU, byp, o); cand += __shfl_xor_sync(0xffffffffU, cand, o);
-                }
-                if (lane == 0) {
-                    unsigned long long* st = s.stats + (int64_t)t0 * 8;
-                    atomicAdd(st + 0, m); atomicAdd(st + 1, hitm); atomicAdd(st + 2, un); atomicAdd(st + 3, uh);
-                    if (byp) atomicAdd(st + 6, byp);
-                    if (cand) atomicAdd(&w.cand_cnt[t0], (int32_t)cand);
-                }
-            } else if (t[q] >= 0) {
-                unsigned long long* st = s.stats + (int64_t)t[q] * 8;
-                atomicAdd(st + 0, m); atomicAdd(st + 1, hitm); atomicAdd(st + 2, un); atomicAdd(st + 3, uh);
-                if (byp) atomicAdd(st + 6, byp);
-                if (cand) atomicAdd(&w.cand_cnt[t[q]], 1);
+            if (t[q] >= 0) { w.loc[k] = loc[q]; w.final_loc[k] = loc[q]; w.cand_key[k] = ckey; }
+            const uint32_t lm = __ballot_sync(0xffffffffU, lists);
+            if (lm) {
+                uint32_t at = 0;
+                if (lane == 0) at = atomicAdd(&w.ctr->n_heads, (uint32_t)__popc(lm));
+                at = __shfl_sync(0xffffffffU, at, 0) + (uint32_t)__popc(lm & ((1u << lane) - 1u));
+                if (lists) w.heads[at] = (int32_t)k;
             }
         }
-        if (!pairs) continue;
-        if constexpr (!FUSED) {
-            // large steps: the keys and the chunk's number of candidates, for the kernels that make the list
-#pragma unroll
-            for (int q = 0; q < Q; ++q) if (t[q] >= 0) w.cand_key[c0 + q * 256 + threadIdx.x] = ckey[q];
-            const uint32_t nc = (uint32_t)__syncthreads_count(cmask & 1u) + (uint32_t)__syncthreads_count(cmask & 2u) +
-                                (uint32_t)__syncthreads_count(cmask & 4u) + (uint32_t)__syncthreads_count(cmask & 8u);
-            if (threadIdx.x == 0) block_sums[chunk] = nc;
-        } else {
-        // the chunk's candidates in row order: round q's rows come before round q + 1's, a warp's before the next warp's
-        uint32_t below[Q];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const uint32_t bq = __ballot_sync(0xffffffffU, (cmask >> q) & 1u);
-            below[q] = (uint32_t)__popc(bq & ((1u << lane) - 1u));
-            if (lane == 0) wcand[warp][q] = (uint32_t)__popc(bq);
-        }
-        __syncthreads();
-        uint32_t total = 0, mine[Q];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            mine[q] = total + below[q];
-#pragma unroll
-            for (int v = 0; v < 8; ++v) { const uint32_t c = wcand[v][q]; total += c; if (v < warp) mine[q] += c; }
-        }
-        if (threadIdx.x == 0) tile_publish(words, chunk, total, tag);
-#pragma unroll
-        for (int q = 0; q < Q; ++q)
-            if ((cmask >> q) & 1u) stash[buf][mine[q]] = make_uint2(ckey[q], (uint32_t)(c0 + q * 256 + threadIdx.x));
-        if (have_prev) write_out(prev_chunk, prev_total, buf ^ 1);
-        have_prev = true; prev_chunk = chunk; prev_total = total; buf ^= 1;
-        }
-    }
-    if constexpr (FUSED) {
-    if (have_prev) { __syncthreads(); write_out(prev_chunk, prev_total, buf ^ 1); }
-    if (last_block_of_pass(ctl, s_turn)) {
-        // every chunk is done and the per-table candidate counts are complete: where each table's candidates begin in
-        // the list, and the tiles of the sort by set (one warp; the counts are cleared for the next step)
-        if (pairs && warp == 0) {
-            const bool dead = off || __ldcg(&w.ctr->abort) != 0;
-            const int T = s.T;
-            int32_t run = 0;
-            for (int t0 = 0; t0 < T; t0 += 32) {
-                const int tt = t0 + lane;
-                const int32_t c = tt < T ? __ldcg(w.cand_cnt + tt) : 0;
-                int32_t inc = c;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) { const int32_t v = __shfl_up_sync(0xffffffffU, inc, o); if (lane >= o) inc += v; }
-                if (tt < T) { w.cstart[tt] = run + inc - c; w.cand_cnt[tt] = 0; }
-                run += __shfl_sync(0xffffffffU, inc, 31);
+        if (one_table) {
+            m = __reduce_add_sync(0xffffffffU, m); hitm = __reduce_add_sync(0xffffffffU, hitm); un = __reduce_add_sync(0xffffffffU, un);
+            uh = __reduce_add_sync(0xffffffffU, uh); byp = __reduce_add_sync(0xffffffffU, byp);
+            if (lane == 0) { sums[warp][0] = m; sums[warp][1] = hitm; sums[warp][2] = un; sums[warp][3] = uh; sums[warp][4] = byp; }
+            __syncthreads();
+            if (threadIdx.x < 5) {
+                uint32_t v = 0;
+                for (int x = 0; x < 8; ++x) v += sums[x][threadIdx.x];
+                if (v) atomicAdd(s.stats + (int64_t)t_first * 8 + (threadIdx.x < 4 ? threadIdx.x : 6), (unsigned long long)v);
             }
-            if (lane == 0) { w.cstart[T] = dead ? 0 : run; w.ctr->n_cand = dead ? 0u : (uint32_t)run; }
-            __syncwarp();
-            warp_tile_bases(w.cstart, T, w.ctile_base, dead, w.sort_tile);
+            __syncthreads();
         }
-        close_pass(ctl, tag);
-    }
     }
 }
 
-// The candidates for admission, in the order of the distinct rows (table, then row id), as (set, distinct-row index)
-// records: block_sums holds the exclusive prefix of the per-chunk counts.
+// every set that has candidates (w.heads: the first candidate each of them got)
 __global__ void __launch_bounds__(256)
-k_cand_write(State s, Work w, const uint32_t* __restrict__ block_sums, uint2* __restrict__ pairs) {
-    __shared__ uint32_t tmp[256 / 32 + 1];
+k_policy(State s, Work w, StepArgs a) {
+    __shared__ int32_t scratch[256 * BUCKET_PER_LANE];             // a group of `ways` lanes has bucket_cap(ways) <= BUCKET_PER_LANE * ways words
     if (w.ctr->abort) return;
-    const int64_t U = w.ctr->U;
-    const uint32_t* __restrict__ ckey = w.cand_key;
-    for (int64_t c0 = (int64_t)blockIdx.x * PRI_CHUNK; c0 < U; c0 += (int64_t)gridDim.x * PRI_CHUNK) {
-        const int64_t k0 = c0 + 4 * threadIdx.x;             // four consecutive rows per thread
-        uint32_t key[4]; bool is[4]; uint32_t n = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            is[i] = false; key[i] = 0;
-            if (k0 + i < U) {
-                key[i] = ckey[k0 + i];
-                is[i] = key[i] < (uint32_t)s.tables[w.uniq_t[k0 + i]].n_sets;
-            }
-            n += is[i];
-        }
-        uint32_t total;
-        uint32_t pos = block_exclusive_scan<256>(n, &total, tmp) + block_sums[c0 / PRI_CHUNK];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (is[i]) pairs[pos++] = make_uint2(key[i], (uint32_t)(k0 + i));
-    }
-}
-
-// where each table's candidates begin (one warp; the per-table counts are cleared for the next step)
-__global__ void k_cand_starts(Work w, int T) {
-    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
-    const int lane = threadIdx.x;
-    int32_t run = 0;
-    for (int t0 = 0; t0 < T; t0 += 32) {
-        const int t = t0 + lane;
-        const int32_t c = t < T ? w.cand_cnt[t] : 0;
-        int32_t inc = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int32_t v = __shfl_up_sync(0xffffffffU, inc, o); if (lane >= o) inc += v; }
-        if (t < T) { w.cstart[t] = run + inc - c; w.cand_cnt[t] = 0; }
-        run += __shfl_sync(0xffffffffU, inc, 31);
-    }
-    if (lane == 0) w.cstart[T] = w.ctr->abort ? 0 : run;
-    __syncwarp();
-    warp_tile_bases(w.cstart, T, w.ctile_base, w.ctr->abort != 0, w.sort_tile);     // the tiles of the sort by set
-}
-
-// ---------------------------------------------------------------------------------------------
-// backward 2: admission / eviction, integer only.  One group of `ways` lanes walks the miss
-// candidates of one set in ascending row id (Algorithm 2's admission test: a candidate whose priority value does
-// not exceed the lowest one among the residents bypasses, otherwise it takes that resident's place).  Lane w holds way w of the set; the candidates are fetched `ways`
-// at a time (one per lane) and handed round with shuffles.  No row value is read or written here.
-// ---------------------------------------------------------------------------------------------
-constexpr int VICTIM_NONE = -1;       // the way was empty, or the displaced row writes itself back
-constexpr int VICTIM_DEFER = -2;      // the displaced row was hit in this step: the newcomer waits for its write-back
-
-// the first candidate of every set that has any (the set-sorted list is grouped by table, then set)
-__global__ void k_policy_heads(State s, Work w, const uint32_t* __restrict__ ckey) {
-    if (w.ctr->abort) return;
-    const int64_t U = w.cstart[s.T];                           // candidates, sorted by (table, set), row ids ascending inside a set
-    const int64_t U32 = (U + 31) & ~31LL;
-    const int lane = threadIdx.x & 31;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < U32; j += (int64_t)gridDim.x * blockDim.x) {
-        bool head = false;
-        if (j < U) {
-            const uint32_t key = ckey[j];
-            const int t = find_segment(w.cstart, s.T, (int32_t)j);
-            head = j == w.cstart[t] || ckey[j - 1] != key;
-        }
-        const uint32_t m = __ballot_sync(0xffffffffU, head);
-        uint32_t base = 0;
-        if (lane == 0 && m) base = atomicAdd(&w.ctr->n_heads, (uint32_t)__popc(m));
-        base = __shfl_sync(0xffffffffU, base, 0);
-        if (head) w.heads[base + __popc(m & ((1u << lane) - 1u))] = (int32_t)j;
-    }
-}
-
-template <bool IND>
-__global__ void __launch_bounds__(256)
-k_policy(State s, Work w, const uint32_t* __restrict__ ckey, const uint32_t* __restrict__ cval, StepArgs av) {
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
-    if (w.ctr->abort) return;
-    const uint32_t step = (uint32_t)a.step, epoch = a.epoch;
-    const int ways = s.ways;
+    const int ways = s.ways, cap = bucket_cap(ways);
     const int lane = threadIdx.x & 31, way = lane & (ways - 1), gbase = lane & ~(ways - 1);
     const uint32_t gmask = group_mask(ways);
     const int64_t nheads = w.ctr->n_heads;
+    const int grp = threadIdx.x / ways;
     const int64_t gpb = blockDim.x / ways, ng = gpb * gridDim.x;
-    for (int64_t hi = blockIdx.x * gpb + threadIdx.x / ways; hi < nheads; hi += ng) {
-        const int64_t j = w.heads[hi];
-        const uint32_t key = ckey[j];
-        const int t = find_segment(w.cstart, s.T, (int32_t)j);
+    for (int64_t h = blockIdx.x * gpb + grp; h < nheads; h += ng) {
+        const int32_t k = w.heads[h];
+        const int t = w.uniq_t[k];
         const TableDev tb = s.tables[t];
-        const int64_t slot = (tb.set_base + key) * ways + way;
-        int32_t tag = s.tags[slot];
-        const int32_t resident = tag;
-        uint32_t pri = 0;
-        if (tag >= 0) pri = s.ts[slot];
-        int32_t cand = -1, vict = VICTIM_NONE;
-        uint32_t n_admit = 0, n_evict = 0, n_bypass = 0;
-        const int64_t jend = w.cstart[t + 1];
-        for (int64_t jj0 = j;; jj0 += ways) {
-            const int64_t jj = jj0 + way;
-            const bool valid = jj < jend && ckey[jj] == key;
-            int32_t ckk = 0, crow = 0; uint32_t cpv = step;
-            if (valid) {
-                ckk = (int32_t)cval[jj];
-                crow = w.uniq_row[ckk];
-                if (s.policy == 1) cpv = *count_of(s, tb.row_base + crow);
-            }
-            const int n = __popc(__ballot_sync(gmask, valid) & gmask);   // the valid lanes are a prefix of the group
-            // Between two replacements the set does not change, so every candidate that cannot beat the current
-            // minimum bypasses at once; only the candidates that replace are walked one by one.
-            int u = 0;
-            while (u < n) {
-                // empty ways rank below every priority; ties go to the lowest way
-                const uint32_t empties = __ballot_sync(gmask, tag < 0) & gmask;
-                int jw; bool jempty; uint32_t jpri = 0;
-                if (empties) { jw = __ffs(empties) - 1 - gbase; jempty = true; }
-                else {
-                    jpri = __reduce_min_sync(gmask, pri);
-                    jw = __ffs(__ballot_sync(gmask, pri == jpri) & gmask) - 1 - gbase;
-                    jempty = false;
-                }
-                // lane `way` holds candidate number `way` of this batch
-                const bool always = ways == 1 && s.policy == 0;                 // direct-mapped LRU never compares
-                const bool would = valid && way >= u && (jempty || always || cpv > jpri);
-                const uint32_t wm = (__ballot_sync(gmask, would) & gmask) >> gbase;
-                if (wm == 0) { n_bypass += (uint32_t)(n - u); break; }
-                const int f = __ffs(wm) - 1;                                    // the first candidate that replaces
-                n_bypass += (uint32_t)(f - u);
-                const int32_t kk = __shfl_sync(gmask, ckk, gbase + f);
-                const int32_t row = __shfl_sync(gmask, crow, gbase + f);
-                const uint32_t pv = __shfl_sync(gmask, cpv, gbase + f);
-                ++n_admit;
-                if (!jempty) ++n_evict;
-                if (way == jw) {
-                    if (tag >= 0 && cand < 0) {
-                        // a row that was resident when the step began leaves the cache
-                        if (s.hit_epoch[slot] == epoch) { w.final_loc[s.hit_k[slot]] = LOC_MISS; vict = VICTIM_DEFER; }
-                        else vict = tag;
-                    }
-                    tag = row; pri = pv; cand = kk;
-                }
-                u = f + 1;
-            }
-            if (n < ways) break;
-        }
-        {   // what the set's lowest priority value is now bounds it from below for good
-            const bool any_empty = (__ballot_sync(gmask, tag < 0) & gmask) != 0;
-            const uint32_t low = __reduce_min_sync(gmask, tag < 0 ? 0u : pri);
-            if (way == 0) s.floor[tb.set_base + key] = any_empty ? 0u : low;
-        }
-        if (cand >= 0) {
-            s.tags[slot] = tag;
-            s.ts[slot] = pri;                            // the newcomer's priority value (LRU: this step)
-            if (resident >= 0) *slot_of(s, tb.row_base + resident) = LOC_MISS;
-            *slot_of(s, tb.row_base + tag) = (int32_t)slot;
-            w.final_loc[cand] = (int32_t)slot;
-            w.victim[cand] = vict;
-            if (vict == VICTIM_DEFER) w.defer_k[atomicAdd(&w.ctr->deferred, 1u)] = cand;
-        }
+        const int32_t ub = w.ustart[t];
+        const PolicyCounts pc = policy_set(s, w, tb, tb.set_base + w.cand_key[k], ub, w.ustart[t + 1] - ub, (uint32_t)a.step, a.epoch, gmask,
+                                           gbase, way, scratch + grp * cap);
         if (way == 0) {
             unsigned long long* st = s.stats + (int64_t)t * 8;
-            if (n_admit) atomicAdd(st + 4, (unsigned long long)n_admit);
-            if (n_evict) atomicAdd(st + 5, (unsigned long long)n_evict);
-            if (n_bypass) atomicAdd(st + 6, (unsigned long long)n_bypass);
+            if (pc.admit) atomicAdd(st + 4, (unsigned long long)pc.admit);
+            if (pc.evict) atomicAdd(st + 5, (unsigned long long)pc.evict);
+            if (pc.bypass) atomicAdd(st + 6, (unsigned long long)pc.bypass);
         }
+        __syncwarp(gmask);
     }
 }
 
@@ -975,10 +888,9 @@ __device__ __forceinline__ float4 tree_reduce(const Term& term, int64_t first, i
 
 // rows with more than HOT_SPAN occurrences: one block per HOT_SPAN occurrences computes two tree levels
 // (8 groups of LANES lanes share the 32 chunks of a task)
-template <int LANES, bool IND>
+template <int LANES>
 __global__ void __launch_bounds__(8 * LANES, LANES == 32 ? 3 : 1)
-k_hot_partial(State s, Work w, StepArgs av) {
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
+k_hot_partial(State s, Work w, StepArgs a) {
     extern __shared__ float chunk_sums[];     // [32][dim]
     if (w.ctr->abort) return;
     const float* __restrict__ grad = a.grad;
@@ -1060,10 +972,9 @@ constexpr int UPD_SMEM = UPD_WARPS * (UPD_DEPTH * UPD_NB * 32 * 16 + 32 * 3 * 16
 // run four occurrences at a time: a batch of asynchronous 16-byte copies brings four gradient rows into shared memory
 // while the batch before it is added, and a row is finished (FP32 update, commit) the moment its last term has been added.
 
-template <int BITS, int LANES, bool IND>
+template <int BITS, int LANES>
 __global__ void __launch_bounds__(UPD_WARPS * 32, 8)
-k_update(State s, Work w, StepArgs av) {
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
+k_update(State s, Work w, StepArgs a) {
     extern __shared__ __align__(16) unsigned char upd_smem[];
     if (w.ctr->abort) return;
     const float* __restrict__ grad = a.grad;
@@ -1256,10 +1167,9 @@ k_update(State s, Work w, StepArgs av) {
 
 // Rows named by a list: the hot rows (gradient from the partial sums of k_hot_partial), and, in a
 // second launch, the newcomers whose slot had to be vacated by a row that was itself updated.
-template <int BITS, int LANES, bool IND>
+template <int BITS, int LANES>
 __global__ void __launch_bounds__(256)
-k_update_list(State s, Work w, const int32_t* __restrict__ list, const uint32_t* __restrict__ count, int deferred_pass, StepArgs av) {
-    StepArgs a = av; if (IND) a = *w.args;      // replayed from a graph: the arguments come from device memory
+k_update_list(State s, Work w, const int32_t* __restrict__ list, const uint32_t* __restrict__ count, int deferred_pass, StepArgs a) {
     if (w.ctr->abort) return;
     const float* __restrict__ grad = a.grad;
     const float lr = a.lr;
