@@ -256,7 +256,7 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags) {
     A(w.victim, nu); A(w.defer_k, nu); A(w.heads, nu);
     A(w.hot_base, nu); A(w.cand_key, nu);
     const int64_t max_tasks = hot_capacity(L);
-    A(w.task_k, max_tasks); A(w.partial, max_tasks * h->dim); A(w.hot_k, max_tasks);
+    A(w.task_k, max_tasks); A(w.partial, max_tasks * h->dim); A(w.hot_k, max_tasks); A(w.mid_k, L / MID_MIN + 1);
 #undef A
     CK(h, cudaMemset(w.ctr, 0, sizeof(Counters)));
     return MPE_OK;
@@ -594,7 +594,7 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool chain) {
             LAUNCH(h, "policy", k_policy, grid_for(h, std::min<int64_t>(L, h->total_sets), 256 / s.ways, resident_blocks(h, k_policy, 256, 0)), 256, 0, s, w, av);
     }
     if (rc != MPE_OK) return rc;
-    const int gu = grid_for(h, (L + 7) / 8, UPD_WARPS, 8);
+    const int gu = grid_for(h, (L + 7) / 8, UPD_WARPS, 7);
     const int gh = grid_for(h, hot_capacity(L), 256 / s.lanes, 4);
     dispatch(h->bits, s.lanes, [&](auto bc, auto lc) {
         constexpr int BITS = decltype(bc)::value, LANES = decltype(lc)::value;

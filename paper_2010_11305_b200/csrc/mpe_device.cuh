@@ -69,30 +69,19 @@ __device__ __forceinline__ uint2 load_codes4(const uint8_t* codes, int64_t grow,
     return make_uint2(q, 0u);
 }
 template <int BITS>
-__device__ __forceinline__ void store_codes4(uint8_t* codes, int64_t grow, int dim, int sub, uint32_t q0, uint32_t q1, uint32_t q2, uint32_t q3) {
+__device__ __forceinline__ void store_packed4(uint8_t* codes, int64_t grow, int dim, int sub, uint32_t q) {
     uint8_t* row = codes + grow * (dim * BITS / 8);
-    if (BITS == 16) { reinterpret_cast<uint2*>(row)[sub] = make_uint2(q0 | (q1 << 16), q2 | (q3 << 16)); return; }
-    const uint32_t q = q0 | (q1 << (BITS & 15)) | (q2 << ((2 * BITS) & 31)) | (q3 << ((3 * BITS) & 31));
     if (BITS == 8) reinterpret_cast<uint32_t*>(row)[sub] = q;
     else if (BITS == 4) reinterpret_cast<uint16_t*>(row)[sub] = (uint16_t)q;
     else row[sub] = (uint8_t)q;
 }
 
-// Element-wise IEEE additions / fused multiply-adds, two FP32 values per instruction (the packed f32x2 forms of sm_100):
-// every component is rounded to nearest exactly as the scalar instruction would round it.
+// element-wise IEEE additions / fused multiply-adds
 __device__ __forceinline__ float4 add4(float4 a, float4 b) {
     return make_float4(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z), __fadd_rn(a.w, b.w));
 }
-__device__ __forceinline__ float4 add4p(float4 a, float4 b) {
-    const float2 lo = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
-    const float2 hi = __fadd2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w));
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
-}
 __device__ __forceinline__ float4 fma4(float m, float4 g, float4 x) {       // m * g + x, fused, per component
-    const float2 mm = make_float2(m, m);
-    const float2 lo = __ffma2_rn(mm, make_float2(g.x, g.y), make_float2(x.x, x.y));
-    const float2 hi = __ffma2_rn(mm, make_float2(g.z, g.w), make_float2(x.z, x.w));
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
+    return make_float4(__fmaf_rn(m, g.x, x.x), __fmaf_rn(m, g.y, x.y), __fmaf_rn(m, g.z, x.z), __fmaf_rn(m, g.w, x.w));
 }
 // minimum / maximum over the lanes of `mask` in one instruction (floating-point warp reduction of sm_100a)
 __device__ __forceinline__ float group_min(float v, uint32_t mask) {
@@ -130,37 +119,31 @@ __device__ __forceinline__ float4 dequant4(const uint8_t* codes, const float2* s
     return decode4<BITS>(load_codes4<BITS, RO>(codes, grow, dim, sub), p);
 }
 
-__device__ __forceinline__ float4 mul4(float4 a, float4 b) {
-    const float2 lo = __fmul2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
-    const float2 hi = __fmul2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w));
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
-}
-
-// four values -> their codes; `stochastic` picks the rounding of Section 3 "Rounding" (it is the same for a whole kernel)
-struct Codes4 { uint32_t q0, q1, q2, q3; };
-__device__ __forceinline__ Codes4 quant4(float4 x, float mn, float inv, float qmax, uint32_t key, uint32_t column, bool stochastic) {
-    // (x - b)/s as (x - b) * (1/s); x - b is formed as x + (-b), which rounds identically
-    float4 y = mul4(add4p(x, make_float4(-mn, -mn, -mn, -mn)), make_float4(inv, inv, inv, inv));
-    y.x = fminf(fmaxf(y.x, 0.0f), qmax); y.y = fminf(fmaxf(y.y, 0.0f), qmax);
-    y.z = fminf(fmaxf(y.z, 0.0f), qmax); y.w = fminf(fmaxf(y.w, 0.0f), qmax);
-    Codes4 q;
-    if (stochastic) {
-        const float4 f = make_float4(floorf(y.x), floorf(y.y), floorf(y.z), floorf(y.w));
-        const float4 p = add4p(y, make_float4(-f.x, -f.y, -f.z, -f.w));          // y - floor(y), exact
-        float4 u;                                                                // 24 random bits each, scaled to [0, 1): exact
-        u.x = __uint2float_rn(mix32(key ^ (column * 0x9E3779B9U + 0x7F4A7C15U)) >> 8);
-        u.y = __uint2float_rn(mix32(key ^ ((column + 1u) * 0x9E3779B9U + 0x7F4A7C15U)) >> 8);
-        u.z = __uint2float_rn(mix32(key ^ ((column + 2u) * 0x9E3779B9U + 0x7F4A7C15U)) >> 8);
-        u.w = __uint2float_rn(mix32(key ^ ((column + 3u) * 0x9E3779B9U + 0x7F4A7C15U)) >> 8);
-        u = mul4(u, make_float4(0x1p-24f, 0x1p-24f, 0x1p-24f, 0x1p-24f));
-        q.q0 = (uint32_t)f.x + (u.x < p.x ? 1u : 0u);                            // x+ with probability p: expectation y
-        q.q1 = (uint32_t)f.y + (u.y < p.y ? 1u : 0u);
-        q.q2 = (uint32_t)f.z + (u.z < p.z ? 1u : 0u);
-        q.q3 = (uint32_t)f.w + (u.w < p.w ? 1u : 0u);
-    } else {                                                                     // nearest, ties to even
-        q.q0 = (uint32_t)rintf(y.x); q.q1 = (uint32_t)rintf(y.y); q.q2 = (uint32_t)rintf(y.z); q.q3 = (uint32_t)rintf(y.w);
+// Four values -> their codes, packed with the first in the lowest bits; `stochastic` picks the rounding of Section 3 "Rounding" (it
+// is the same for a whole kernel).  The integer part of y comes out of the mantissa of y + 2^23, rounded down (or to the nearest,
+// ties to even): two full-rate additions where a rounding and a conversion instruction run at a quarter of the rate.  The 2^23 that
+// stays in each term is taken off once, from the packed sum.  Scalar on purpose: with packed f32x2 arithmetic the moves that pair
+// and unpair registers outnumbered the instructions it saved.
+template <int BITS>
+__device__ __forceinline__ uint32_t quant_pack(float4 x, float mn, float inv, uint32_t key, uint32_t column, bool stochastic) {
+    constexpr float qmax = (float)((1 << BITS) - 1);
+    constexpr uint32_t BASE = 0x4B000000u;                                      // 2^23 as FP32
+    uint32_t packed = 0u - (BASE + (BASE << BITS) + (BASE << (2 * BITS)) + (BASE << (3 * BITS)));
+    const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        // (x - b)/s as (x - b) * (1/s)
+        const float y = fminf(fmaxf(__fmul_rn(__fsub_rn(v[i], mn), inv), 0.0f), qmax);
+        float t;
+        bool up = false;
+        if (stochastic) {
+            t = __fadd_rd(y, 8388608.0f);
+            const float p = __fsub_rn(y, __fsub_rn(t, 8388608.0f));             // y - floor(y), exact
+            up = uniform01(key, column + (uint32_t)i) < p;                      // x+ with probability p: expectation y
+        } else t = __fadd_rn(y, 8388608.0f);
+        packed += (__float_as_uint(t) + (up ? 1u : 0u)) << (BITS * i);
     }
-    return q;
+    return packed;
 }
 
 // one value -> FP16 bits: the nearer neighbour, or one of the two neighbours x- <= x <= x+ (one unit in the last
@@ -182,8 +165,9 @@ __device__ __forceinline__ void quantize_store(float4 x, uint8_t* __restrict__ c
                                                int64_t grow, int dim, int sub, int lanes_per_row, uint32_t key, bool stochastic) {
     if (BITS == 16) {       // FP16 table: element-wise, no scale or bias
         const uint32_t c = 4u * (uint32_t)sub;
-        store_codes4<BITS>(codes, grow, dim, sub, half1(x.x, key, c, stochastic), half1(x.y, key, c + 1, stochastic),
-                           half1(x.z, key, c + 2, stochastic), half1(x.w, key, c + 3, stochastic));
+        reinterpret_cast<uint2*>(codes + grow * (dim * 2))[sub] =
+            make_uint2(half1(x.x, key, c, stochastic) | (half1(x.y, key, c + 1, stochastic) << 16),
+                       half1(x.z, key, c + 2, stochastic) | (half1(x.w, key, c + 3, stochastic) << 16));
         return;
     }
     const uint32_t mask = group_mask(lanes_per_row);
@@ -200,33 +184,8 @@ __device__ __forceinline__ void quantize_store(float4 x, uint8_t* __restrict__ c
     if (s >= 1.17549435e-38f) inv = __fdiv_rn(1.0f, s);
     if (inv == 0.0f) s = 0.0f;
     const uint32_t c = 4u * (uint32_t)sub;
-    const Codes4 q = quant4(x, mn, inv, qmax, key, c, stochastic);
-    store_codes4<BITS>(codes, grow, dim, sub, q.q0, q.q1, q.q2, q.q3);
+    store_packed4<BITS>(codes, grow, dim, sub, quant_pack<BITS & 15>(x, mn, inv, key, c, stochastic));
     if (sub == 0) sb[grow] = make_float2(s, mn);
 }
-
-// ---- asynchronous 16-byte copies global -> shared (per thread; completion is waited for by group count) ----
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
-}
-// same with the shared-memory address already converted; `take` false copies nothing (the source is not read)
-__device__ __forceinline__ void cp_async16_if(uint32_t smem_addr, const void* gsrc, bool take) {
-    const uint32_t n = take ? 16u : 0u;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr), "l"(gsrc), "r"(n) : "memory");
-}
-// same, but the line is also kept in L1 (rows that many bags of one SM share)
-__device__ __forceinline__ void cp_async16_l1(void* smem_dst, const void* gsrc) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 
 }  // namespace mpe

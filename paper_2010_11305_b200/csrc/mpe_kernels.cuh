@@ -17,6 +17,10 @@ constexpr int HOT_SMALL_L = 1 << 20;  // "small": at most this many indices
 __host__ __device__ constexpr int64_t hot_capacity(int64_t L) {
     return (L < HOT_SMALL_L ? L : HOT_SMALL_L) / HOT_MIN_SMALL + L / HOT_MIN + L / HOT_SPAN + 4;
 }
+// Rows with more occurrences than this, but not hot, are handed to the warps of k_update one by one, ahead of the others: popular
+// rows can be neighbours (a vocabulary sorted by frequency), and a block of 32 of them kept one warp busy for 790 us where the
+// whole kernel should take 220 (8 tables of configuration 4).
+constexpr int MID_MIN = 16;
 // more occurrences than this: the multi-block path
 __host__ __device__ constexpr uint32_t hot_threshold(int64_t L) { return L <= HOT_SMALL_L ? (uint32_t)HOT_MIN_SMALL : (uint32_t)HOT_MIN; }
 constexpr int ERR_INDEX = 0, ERR_OFFSETS = 1;
@@ -36,6 +40,7 @@ struct Counters {
     uint32_t fwd_bad, fwd_done;      // of the running forward: offsets were inconsistent; blocks that have finished
     uint32_t hot_rows;
     uint32_t hot_tasks;
+    uint32_t mid_rows;
     uint32_t abort;        // offsets were inconsistent: every later kernel of the step returns at once
     uint32_t deferred;     // newcomers that wait for the write-back of an updated row
     uint32_t n_heads;      // cache sets that have miss candidates in this step
@@ -95,6 +100,7 @@ struct Work {
     int32_t *uniq_row, *uniq_t, *seg, *loc, *final_loc, *victim, *hot_base;   // per unique row
     int32_t* task_k;       // [hot tasks]
     int32_t* hot_k;        // [hot rows]
+    int32_t* mid_k;        // [rows with more than MID_MIN occurrences that are not hot]
     int32_t* cand_key;     // [distinct rows] the row's set if it is a candidate for admission, else CAND_NONE
     int32_t* defer_k;      // [deferred newcomers]
     int32_t* heads;        // [sets with candidates] one candidate of each (small steps: the set itself, table by table)
@@ -104,7 +110,7 @@ struct Work {
 
 // the counters of a step, as its first kernel leaves them
 __device__ __forceinline__ void reset_step(Counters* c, uint32_t L, uint32_t abort, unsigned long long dropped) {
-    c->L = L; c->U = 0; c->hot_rows = 0; c->hot_tasks = 0; c->abort = abort; c->dropped = dropped; c->hot_occ = 0; c->deferred = 0;
+    c->L = L; c->U = 0; c->hot_rows = 0; c->hot_tasks = 0; c->mid_rows = 0; c->abort = abort; c->dropped = dropped; c->hot_occ = 0; c->deferred = 0;
     c->n_heads = 0; c->upd_next = 0;
 }
 
@@ -191,6 +197,17 @@ __device__ __forceinline__ void list_hot_row(const Work& w, int32_t k, uint32_t 
     atomicAdd(&w.ctr->hot_occ, (unsigned long long)m);
     for (uint32_t j = 0; j < nt; ++j) w.task_k[hb + j] = k;
 }
+// a row with m occurrences joins the list it belongs on, if any (the lanes that call this together draw one number)
+__device__ __forceinline__ void list_long_row(const Work& w, int32_t k, uint32_t m, uint32_t hot_min, bool list_hot = true) {
+    if (m <= (uint32_t)MID_MIN) return;
+    if (m > hot_min) { if (list_hot) list_hot_row(w, k, m); return; }
+    const uint32_t mask = __activemask(), lane = threadIdx.x & 31;
+    const int leader = __ffs(mask) - 1;
+    uint32_t at = 0;
+    if (lane == (uint32_t)leader) at = atomicAdd(&w.ctr->mid_rows, (uint32_t)__popc(mask));
+    at = __shfl_sync(mask, at, leader) + (uint32_t)__popc(mask & ((1u << lane) - 1u));
+    w.mid_k[at] = k;
+}
 // One thread's SCAN_ITEMS consecutive sorted elements, starting at `base`: their keys, which of them begin a run of equal
 // (table, row) (bit i of *heads) and which end one (bit i of *lasts), and the table of the first.
 __device__ __forceinline__ void unique_items(const int32_t* __restrict__ table_start, int T, const uint32_t* __restrict__ skey, uint32_t n,
@@ -230,7 +247,7 @@ __device__ __forceinline__ void unique_items(const int32_t* __restrict__ table_s
 // ... and writes them out: the thread's first run has the index k.  The last occurrence of a row is marked in the sign bit of its
 // sample id (samples are below 2^31); ustart receives where each table's distinct rows begin.  A row with more occurrences than
 // the threshold (the element that many places behind its first one is still the same row) is listed for the multi-block
-// gradient path, HOT_SPAN occurrences per task; only for such a row the end of its run is searched for.
+// gradient path; only for such a row the end of its run is searched for.
 __device__ __forceinline__ void unique_write(const State& s, const Work& w, const uint32_t* __restrict__ skey, uint32_t n, uint32_t base, const uint32_t (&key)[SCAN_ITEMS], uint32_t heads,
                                              uint32_t lasts, int t, uint32_t k) {
     if (base >= n) return;
@@ -696,7 +713,7 @@ k_priority(State s, Work w, StepArgs a, int list_hot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int cap = bucket_cap(s.ways);
     const bool always = s.ways == 1 && s.policy == 0;
-    const uint32_t hot_min = list_hot ? hot_threshold(w.ctr->L) : 0xffffffffU;      // 0: the kernel that listed the distinct rows did it
+    const uint32_t hot_min = hot_threshold(w.ctr->L);
     // a block takes PRI_CHUNK consecutive rows at a time, thread i the rows i, i + 256, i + 512, i + 768 of them
     for (int64_t c0 = (int64_t)blockIdx.x * PRI_CHUNK; c0 < U; c0 += (int64_t)gridDim.x * PRI_CHUNK) {
         int t[Q], loc[Q]; int32_t row[Q], set[Q]; uint32_t mult[Q], old[Q]; int64_t rb[Q], sbase[Q]; int32_t nsets[Q];
@@ -740,7 +757,7 @@ k_priority(State s, Work w, StepArgs a, int list_hot) {
                     *count_of(s, rb[q] + row[q]) = pv;
                 }
                 bool hit = false, bypass = false;
-                if (mult[q] > hot_min) list_hot_row(w, (int32_t)k, mult[q]);
+                list_long_row(w, (int32_t)k, mult[q], hot_min, list_hot != 0);      // 0: the kernel that listed the distinct rows listed the hot ones
                 // the cached row's priority value, kept per slot: the LRU time stamp, or a copy of the LFU count (so
                 // that the policy kernel reads one line per set instead of one counter per resident row)
                 if (loc[q] >= 0) {
@@ -956,210 +973,191 @@ __device__ __forceinline__ void apply_update(const State& s, const TableDev& tb,
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-struct RawRow { float4 f; uint2 q; float2 sb; };
-
 constexpr int UPD_WARPS = 4;     // warps per block of k_update
-constexpr int UPD_NB = 4;        // gradient rows per batch of asynchronous copies
-constexpr int UPD_DEPTH = 2;     // batches in flight per group
 constexpr int UPD_SMALL_U = 524288;   // at most this many distinct rows: blocks of 8 rows instead of 32
-constexpr int UPD_SMEM = UPD_WARPS * (UPD_DEPTH * UPD_NB * 32 * 16 + 32 * 3 * 16);
+constexpr int UPD_SMEM = UPD_WARPS * 32 * (4 * 16 + 4);
 
 // Every distinct row that is not on the multi-block path, except newcomers that wait for a write-back.  A warp stages the
 // bookkeeping of 32 consecutive rows in shared memory, one row per lane (coalesced loads; the per-row scalar work --
-// addresses, the stochastic-rounding key -- is done there once, 32 rows at a time).  The distinct rows of a block are
-// consecutive in the sorted batch, so the gradient rows they need are one contiguous run of the sorted occurrence list
-// (broken only where a row is not this kernel's, or where the table changes).  Each group of LANES lanes walks such a
-// run four occurrences at a time: a batch of asynchronous 16-byte copies brings four gradient rows into shared memory
-// while the batch before it is added, and a row is finished (FP32 update, commit) the moment its last term has been added.
-
+// addresses, the stochastic-rounding key, the first four sample ids -- is done there once, 32 rows at a time).  Then its groups of
+// LANES lanes take a row each, side by side: the value and the first four gradient rows of the next row are on their way while a
+// row is finished (FP32 update, commit).  Few rows have more than four terms; the rest of a longer row is added eight terms at a time.
+// Bound by instruction issue.  Walking the rows' terms as one stream of asynchronous copies instead, every group at its own pace,
+// took 317 warp instructions per row at dim 128 and, with two groups of a warp out of step, 304 at dim 64.
 template <int BITS, int LANES>
-__global__ void __launch_bounds__(UPD_WARPS * 32, 8)
+__global__ void __launch_bounds__(UPD_WARPS * 32, 7)
 k_update(State s, Work w, StepArgs a) {
     extern __shared__ __align__(16) unsigned char upd_smem[];
     if (w.ctr->abort) return;
-    const float* __restrict__ grad = a.grad;
     const float lr = a.lr;
     const uint64_t step = a.step;
-    constexpr int dim = 4 * LANES, G = 32 / LANES, NB = LANES < UPD_NB ? LANES : UPD_NB, BPW = LANES / NB;
-    constexpr int SLOTS = UPD_DEPTH * NB;
+    constexpr int dim = 4 * LANES, G = 32 / LANES;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = lane & (LANES - 1), grp = lane / LANES, gbase = lane & ~(LANES - 1);
     const uint32_t gmask = group_mask(LANES);
-    float4* ring = reinterpret_cast<float4*>(upd_smem) + ((warp * G + grp) * SLOTS) * LANES + sub;       // slot i: ring[i * LANES]
-    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
-    // per staged row: A = {loc, final loc, global row lo, hi}, B = {rounding key, occurrences, first occurrence, victim},
-    // C = {victim's key, victim's global row lo, hi, gradient column}
-    int4* recs = reinterpret_cast<int4*>(upd_smem + UPD_WARPS * UPD_DEPTH * UPD_NB * 32 * 16) + warp * 96;
+    // per staged row: A = {loc, final loc, global row lo, hi}, B = {rounding key, occurrences (0: not ours), first occurrence, victim},
+    // C = {victim's key, victim's global row lo, hi, gradient column}, D = the first four sample ids; and its Adagrad accumulator
+    int4* recs = reinterpret_cast<int4*>(upd_smem) + warp * 128;
+    float* accums = reinterpret_cast<float*>(upd_smem + UPD_WARPS * 32 * 4 * 16) + warp * 32;
     const int64_t U = w.ctr->U;
-    const uint32_t hot_min = hot_threshold(w.ctr->L);
-    // rows per hand-out and per group: 32 per warp when there is plenty of work; a step with few distinct rows is cut
-    // finer, because there the kernel lasts as long as its longest chain of rows (each row ends in dependent loads)
-    const int rpt = U > UPD_SMALL_U ? 32 : (G > 8 ? G : 8);
-    const int rpg = rpt / G;
+    // rows per hand-out: first the rows with many terms, a row per group (two rows per warp); then 32 per warp when there is plenty of work; a step with few distinct rows is cut
+    // finer, because there the kernel lasts as long as its longest chain of rows
+    constexpr int rpm = G > 1 ? G : 2;
+    const int rpb = U > UPD_SMALL_U ? 32 : (G > 8 ? G : 8);
+    const int64_t mids = w.ctr->mid_rows, mid_blocks = (mids + rpm - 1) / rpm;
     const uint32_t stride_bytes = (uint32_t)s.T * (uint32_t)dim * 4u;
-    const char* gcol = reinterpret_cast<const char*>(grad + 4 * sub);
+    const char* gcol = reinterpret_cast<const char*>(a.grad + 4 * sub);
     const float NZ = __int_as_float(0x80000000);          // -0: adding it changes no value, not even a zero's sign
+    const float4 NZ4 = make_float4(NZ, NZ, NZ, NZ);
+    auto grad_row = [&](const char* col, uint32_t b) { return __ldg(reinterpret_cast<const float4*>(col + (size_t)b * stride_bytes)); };
     for (;;) {
-        // blocks of 32 rows are handed out on demand: their cost varies with the rows' multiplicities
+        // blocks of rows are handed out on demand: their cost varies with the rows' multiplicities
         uint32_t blk = 0;
         if (lane == 0) blk = atomicAdd(&w.ctr->upd_next, 1u);
-        const int64_t k0 = (int64_t)__shfl_sync(0xffffffffU, blk, 0) * rpt;
-        if (k0 >= U) break;
-        const int64_t k = k0 + lane;
-        bool skip = true; int myt = -1;
-        if (lane < rpt && k < U) {
-            const int32_t first = w.seg[k], row = w.uniq_row[k];
-            const int loc = w.loc[k], floc = w.final_loc[k], victim = w.victim[k], t = w.uniq_t[k];
-            const int32_t m = w.seg[k + 1] - first;
-            myt = t;
-            // pseudo rows, hot rows (own kernel) and newcomers that wait for a write-back are not ours
-            const bool newcomer = loc < 0 && floc >= 0;
-            skip = loc == LOC_INVALID || (uint32_t)m > hot_min || (newcomer && victim == VICTIM_DEFER);
-            int4 A = make_int4(loc, floc, 0, 0), Bq = make_int4(0, m, first, victim), C = make_int4(0, 0, 0, t * dim);
-            if (!skip) {
-                const int64_t rb = s.tables[t].row_base;
-                const int64_t grow = rb + row;
-                A.z = (int32_t)(uint32_t)grow; A.w = (int32_t)(grow >> 32);
-                Bq.x = (int32_t)rowkey(s.seed, DOMAIN_SR, (uint32_t)t, (uint32_t)row, step);
-                // pull this row's current value towards L2 now; it is needed when its gradient has been summed
-                if (loc >= 0) {
-                    const char* src = reinterpret_cast<const char*>(s.slab + (int64_t)loc * dim);
+        const int64_t b = __shfl_sync(0xffffffffU, blk, 0);
+        const bool mid = b < mid_blocks;
+        const int rpt = mid ? rpm : rpb;
+        const int64_t i = mid ? b * rpm + lane : (b - mid_blocks) * rpb + lane;
+        if (!mid && i - lane >= U) break;
+        if (lane < rpt) {
+            const int64_t k = mid ? (i < mids ? w.mid_k[i] : U) : i;
+            int4 A = make_int4(LOC_MISS, LOC_MISS, 0, 0), B = make_int4(0, 0, 0, VICTIM_NONE), C = make_int4(0, 0, 0, 0), D = C;
+            if (k < U) {
+                const int32_t first = w.seg[k], m = w.seg[k + 1] - first, row = w.uniq_row[k];
+                const int loc = w.loc[k], floc = w.final_loc[k], t = w.uniq_t[k];
+                const bool newcomer = loc < 0 && floc >= 0;
+                const int victim = newcomer ? w.victim[k] : VICTIM_NONE;
+                // pseudo rows, rows on a list (hot ones have their own kernel) and newcomers that wait for a write-back are not ours
+                if (loc != LOC_INVALID && (mid || m <= MID_MIN) && victim != VICTIM_DEFER) {
+                    const int64_t rb = s.tables[t].row_base, grow = rb + row;
+                    A = make_int4(loc, floc, (int32_t)(uint32_t)grow, (int32_t)(grow >> 32));
+                    B = make_int4((int32_t)rowkey(s.seed, DOMAIN_SR, (uint32_t)t, (uint32_t)row, step), m, first, victim);
+                    C.w = t * dim;
+                    D.x = w.occ_b[first] & 0x7fffffff;
+                    if (m > 1) D.y = w.occ_b[first + 1] & 0x7fffffff;
+                    if (m > 2) D.z = w.occ_b[first + 2] & 0x7fffffff;
+                    if (m > 3) D.w = w.occ_b[first + 3] & 0x7fffffff;
+                    if (s.optimizer == 1) accums[lane] = s.G[grow];
+                    // pull this row's current value towards L2 now; it is needed when its turn comes
+                    if (loc >= 0) {
+                        const char* src = reinterpret_cast<const char*>(s.slab + (int64_t)loc * dim);
 #pragma unroll
-                    for (int o = 0; o < dim * 4; o += 128) prefetch_l2(src + o);
-                } else {
-                    prefetch_l2(s.codes + grow * (dim * BITS / 8));
-                    if (BITS != 16) prefetch_l2(s.sb + grow);
-                }
-                if (newcomer && victim >= 0) {
-                    const int64_t vrow = rb + victim;
-                    C.x = (int32_t)rowkey(s.seed, DOMAIN_SR, (uint32_t)t, (uint32_t)victim, step);
-                    C.y = (int32_t)(uint32_t)vrow; C.z = (int32_t)(vrow >> 32);
-                    const char* src = reinterpret_cast<const char*>(s.slab + (int64_t)floc * dim);
+                        for (int o = 0; o < dim * 4; o += 128) prefetch_l2(src + o);
+                    } else {
+                        prefetch_l2(s.codes + grow * (dim * BITS / 8));
+                        if (BITS != 16) prefetch_l2(s.sb + grow);
+                    }
+                    if (victim >= 0) {
+                        const int64_t vrow = rb + victim;
+                        C.x = (int32_t)rowkey(s.seed, DOMAIN_SR, (uint32_t)t, (uint32_t)victim, step);
+                        C.y = (int32_t)(uint32_t)vrow; C.z = (int32_t)(vrow >> 32);
+                        const char* src = reinterpret_cast<const char*>(s.slab + (int64_t)floc * dim);
 #pragma unroll
-                    for (int o = 0; o < dim * 4; o += 128) prefetch_l2(src + o);
+                        for (int o = 0; o < dim * 4; o += 128) prefetch_l2(src + o);
+                    }
                 }
             }
-            recs[lane * 3] = A; recs[lane * 3 + 1] = Bq; recs[lane * 3 + 2] = C;
+            recs[lane * 4] = A; recs[lane * 4 + 1] = B; recs[lane * 4 + 2] = C; recs[lane * 4 + 3] = D;
         }
-        const int tprev = __shfl_up_sync(0xffffffffU, myt, 1);
-        const uint32_t skipmask = __ballot_sync(0xffffffffU, skip);                       // rows that are not ours (or past the end)
-        const uint32_t stopmask = skipmask | __ballot_sync(0xffffffffU, lane > 0 && myt != tprev);   // a run ends before these rows
         __syncwarp();
-        // this group's rows: rpg consecutive ones; their runs
-        const int gr0 = grp * rpg, gr1 = gr0 + rpg;
-        uint32_t avail = ~skipmask & (rpg == 32 ? 0xffffffffU : (((1U << rpg) - 1U) << gr0));
-        while (avail) {
-            const int rs = __ffs(avail) - 1;
-            const uint32_t above = stopmask & (rs == 31 ? 0u : (0xfffffffeU << rs));
-            int re = above ? __ffs(above) - 1 : 32;
-            re = min(re, gr1);
-            avail = re >= 32 ? 0u : (avail & (0xffffffffU << re));
-            // the run's occurrences and gradient column
-            const int4 Bs = recs[rs * 3 + 1], Be = recs[(re - 1) * 3 + 1];
-            const int32_t os = Bs.z, oe = Be.z + Be.y;
-            const char* src = gcol + (size_t)(uint32_t)recs[rs * 3 + 2].w * 4u;
-            const int nbatch = (oe - os + NB - 1) / NB;
-            uint32_t wb = 0, wlast = 0;                        // sample ids of LANES consecutive occurrences, one per lane; their row ends
-            uint32_t pend = 0;                                 // row-end bits of the batches in flight, NB bits per batch
-            auto issue = [&](int j) {                          // copies of batch j (none when j is past the end); always one group
-                if (j < nbatch) {
-                    const int jw = j % BPW;
-                    if (jw == 0) {
-                        const int32_t o = os + j * NB + sub;
-                        const uint32_t raw = o < oe ? (uint32_t)w.occ_b[o] : 0u;
-                        wlast = (__ballot_sync(gmask, (raw >> 31) != 0) & gmask) >> gbase;
-                        wb = raw & 0x7fffffffU;
-                    }
-                    constexpr uint32_t BM = (1u << NB) - 1u;
-                    const int f = (j % UPD_DEPTH) * NB;
-                    pend = (pend & ~(BM << f)) | (((wlast >> (jw * NB)) & BM) << f);
-                    const int32_t left = oe - (os + j * NB);
-                    const uint32_t dst = ring_s + (uint32_t)(((j % UPD_DEPTH) * NB) * LANES * 16);
-#pragma unroll
-                    for (int u = 0; u < NB; ++u) {
-                        const uint32_t b = __shfl_sync(gmask, wb, gbase + jw * NB + u);          // 0 (a valid sample) past the end
-                        cp_async16_if(dst + (uint32_t)(u * LANES * 16), src + (size_t)b * stride_bytes, u < left);
-                    }
-                }
-                cp_async_commit();
-            };
-            // current row: its records, its stored value, how many terms are still to come
-            int r = rs;
-            int4 A, Bq; RawRow xr;
-            auto open_row = [&]() {
-                A = recs[r * 3]; Bq = recs[r * 3 + 1];
-                if (A.x >= 0) {
-                    xr.f = reinterpret_cast<const float4*>(s.slab + (int64_t)A.x * dim)[sub];
-                } else {
-                    const int64_t grow = ((int64_t)A.w << 32) | (uint32_t)A.z;
-                    if (BITS != 16) xr.sb = s.sb[grow];
-                    xr.q = load_codes4<BITS, false>(s.codes, grow, dim, sub);
-                }
-            };
-            open_row();
-#pragma unroll
-            for (int j = 0; j < UPD_DEPTH; ++j) issue(j);
-            float4 chunkacc = make_float4(NZ, NZ, NZ, NZ), rowacc = chunkacc;
-            int c = 0;                                         // terms of the current row added so far
-            const int nocc = oe - os;
-            for (int j = 0; j < nbatch; ++j) {
-                if (j) issue(j - 1 + UPD_DEPTH);               // refill the slots just drained,
-                cp_async_wait<UPD_DEPTH - 1>();                // then wait for this batch
-                const uint32_t m = (pend >> ((j % UPD_DEPTH) * NB)) & ((1u << NB) - 1u);      // bit u: occurrence u ends its row
-                const float4* slot = ring + ((j % UPD_DEPTH) * NB) * LANES;
-                const int cnt = min(NB, nocc - j * NB);
-                if (NB == 4 && m == 0 && cnt == 4 && (c & 31) <= 28) {
-                    // four terms of one row and one chunk of 32 (the long rows are mostly made of these): no bookkeeping
-                    chunkacc = add4(add4(add4(add4(chunkacc, slot[0]), slot[LANES]), slot[2 * LANES]), slot[3 * LANES]);
-                    c += 4;
-                    if ((c & 31) == 0) { rowacc = add4(rowacc, chunkacc); chunkacc = make_float4(NZ, NZ, NZ, NZ); }
-                    continue;
-                }
-#pragma unroll 1
-                for (int u = 0; u < cnt; ++u) {
-                    chunkacc = add4(chunkacc, slot[u * LANES]);
-                    ++c;
-                    const bool last = (m >> u) & 1u;
-                    if (last || (c & 31) == 0) {               // a finished chunk joins the sum of chunk sums
-                        rowacc = add4(rowacc, chunkacc);
-                        chunkacc = make_float4(NZ, NZ, NZ, NZ);
-                    }
-                    if (last) {
-                        c = 0;
-                        const int loc = A.x, floc = A.y;
-                        float4 x = xr.f;
-                        if (loc < 0) x = decode4<BITS>(xr.q, xr.sb);
-                        const int64_t grow = ((int64_t)A.w << 32) | (uint32_t)A.z;
-                        float mult = lr;                                         // SGD: x <- x - lr * g
-                        if (s.optimizer == 1) {                                  // row-wise Adagrad
-                            float q = __fmul_rn(rowacc.x, rowacc.x);
-                            q = __fmaf_rn(rowacc.y, rowacc.y, q); q = __fmaf_rn(rowacc.z, rowacc.z, q); q = __fmaf_rn(rowacc.w, rowacc.w, q);
-#pragma unroll
-                            for (int o = LANES >> 1; o > 0; o >>= 1) q = __fadd_rn(q, __shfl_xor_sync(gmask, q, o));
-                            const float Gold = s.G[grow];
-                            __syncwarp(gmask);                                   // every lane has read G before lane 0 replaces it
-                            const float Gn = __fadd_rn(Gold, __fmul_rn(q, __fdiv_rn(1.0f, (float)dim)));
-                            if (sub == 0) s.G[grow] = Gn;
-                            mult = __fdiv_rn(lr, __fadd_rn(__fsqrt_rn(Gn), s.eps));
-                        }
-                        const float4 xn = fma4(-mult, rowacc, x);
-                        if (floc >= 0) {
-                            float4* dst = reinterpret_cast<float4*>(s.slab + (int64_t)floc * dim) + sub;
-                            if (loc < 0 && Bq.w >= 0) {          // the row this newcomer displaces is down-converted and placed back in T
-                                const int4 C = recs[r * 3 + 2];
-                                const int64_t vrow = ((int64_t)C.z << 32) | (uint32_t)C.y;
-                                quantize_store<BITS>(*dst, s.codes, s.sb, vrow, dim, sub, LANES, (uint32_t)C.x, s.rounding != 0);
-                            }
-                            *dst = xn;                           // cached rows keep full precision, a newcomer enters verbatim
-                        } else {
-                            quantize_store<BITS>(xn, s.codes, s.sb, grow, dim, sub, LANES, (uint32_t)Bq.x, s.rounding != 0);
-                        }
-                        rowacc = make_float4(NZ, NZ, NZ, NZ);
-                        if (++r < re) open_row();
-                    }
-                }
+        float4 g[4];                                       // first terms of the row whose turn comes next, and its stored value
+        uint4 raw;
+        auto fetch_row = [&](int r) {
+            const int4 A = recs[r * 4];
+            const int m = recs[r * 4 + 1].y;
+            if (m == 0) return;
+            if (A.x >= 0) {
+                raw = reinterpret_cast<const uint4*>(s.slab + (int64_t)A.x * dim)[sub];
+            } else {
+                const int64_t grow = ((int64_t)A.w << 32) | (uint32_t)A.z;
+                const uint2 q = load_codes4<BITS, false>(s.codes, grow, dim, sub);
+                raw.x = q.x; raw.y = q.y;
+                if (BITS != 16) { const float2 sb = s.sb[grow]; raw.z = __float_as_uint(sb.x); raw.w = __float_as_uint(sb.y); }
             }
-            cp_async_wait<0>();
+            const int4 D = recs[r * 4 + 3];
+            const char* col = gcol + (size_t)(uint32_t)recs[r * 4 + 2].w * 4u;
+            g[0] = grad_row(col, (uint32_t)D.x);
+            if (m > 1) {                                   // most rows have one term
+                g[1] = grad_row(col, (uint32_t)D.y);
+                g[2] = g[3] = NZ4;
+                if (m > 2) g[2] = grad_row(col, (uint32_t)D.z);
+                if (m > 3) g[3] = grad_row(col, (uint32_t)D.w);
+            }
+        };
+        fetch_row(grp);
+        for (int r = grp; r < rpt; r += G) {
+            const int4 A = recs[r * 4], B = recs[r * 4 + 1];
+            const int m = B.y;
+            float4 acc = g[0];
+            if (m > 1) acc = add4(add4(add4(acc, g[1]), g[2]), g[3]);
+            if (m > 4) {                                   // chunks of 32 terms left to right; the chunks' sums left to right
+                const char* col = gcol + (size_t)(uint32_t)recs[r * 4 + 2].w * 4u;
+                const int32_t* ids = w.occ_b + B.z;
+                float4 rows = NZ4;
+                // LANES consecutive sample ids at a time, one per lane, and the LANES behind them on their way
+                int32_t cur = ids[min(sub, m - 1)], nxt = ids[min(LANES + sub, m - 1)];
+                auto id_at = [&](int j) {                  // j moves forward by one; for rows of less than four lanes the ids are read one by one
+                    if (LANES < 4) return (uint32_t)ids[min(j, m - 1)] & 0x7fffffffu;
+                    return (uint32_t)__shfl_sync(gmask, cur, gbase + (j & (LANES - 1))) & 0x7fffffffu;
+                };
+                auto step4 = [&](int j) {                  // j, a multiple of four, is where the next ids begin
+                    if (LANES >= 4 && (j & (LANES - 1)) == 0) { cur = nxt; nxt = ids[min(j + LANES + sub, m - 1)]; }
+                };
+                step4(4);
+                for (int c = 4; c < m; c += 8) {
+                    float4 h[4];                           // g is free: eight rows in flight
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t id = id_at(c + u);
+                        g[u] = NZ4;
+                        if (c + u < m) g[u] = grad_row(col, id);
+                    }
+                    step4(c + 4);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t id = id_at(c + 4 + u);
+                        h[u] = NZ4;
+                        if (c + 4 + u < m) h[u] = grad_row(col, id);
+                    }
+                    step4(c + 8);
+                    if ((c & 31) == 0) { rows = add4(rows, acc); acc = NZ4; }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc = add4(acc, g[u]);
+                    if (((c + 4) & 31) == 0) { rows = add4(rows, acc); acc = NZ4; }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc = add4(acc, h[u]);
+                }
+                acc = add4(rows, acc);
+            }
+            const int loc = A.x, floc = A.y;
+            float4 x;
+            if (loc >= 0) x = make_float4(__uint_as_float(raw.x), __uint_as_float(raw.y), __uint_as_float(raw.z), __uint_as_float(raw.w));
+            else x = decode4<BITS>(make_uint2(raw.x, raw.y), make_float2(__uint_as_float(raw.z), __uint_as_float(raw.w)));
+            if (r + G < rpt) fetch_row(r + G);
+            if (m == 0) continue;
+            const int64_t grow = ((int64_t)A.w << 32) | (uint32_t)A.z;
+            float mult = lr;                                         // SGD: x <- x - lr * g
+            if (s.optimizer == 1) {                                  // row-wise Adagrad
+                float q = __fmul_rn(acc.x, acc.x);
+                q = __fmaf_rn(acc.y, acc.y, q); q = __fmaf_rn(acc.z, acc.z, q); q = __fmaf_rn(acc.w, acc.w, q);
+#pragma unroll
+                for (int o = LANES >> 1; o > 0; o >>= 1) q = __fadd_rn(q, __shfl_xor_sync(gmask, q, o));
+                const float Gn = __fadd_rn(accums[r], __fmul_rn(q, __fdiv_rn(1.0f, (float)dim)));
+                if (sub == 0) s.G[grow] = Gn;
+                mult = __fdiv_rn(lr, __fadd_rn(__fsqrt_rn(Gn), s.eps));
+            }
+            const float4 xn = fma4(-mult, acc, x);
+            if (floc >= 0) {
+                float4* dst = reinterpret_cast<float4*>(s.slab + (int64_t)floc * dim) + sub;
+                if (loc < 0 && B.w >= 0) {           // the row this newcomer displaces is down-converted and placed back in T
+                    const int4 C = recs[r * 4 + 2];
+                    const int64_t vrow = ((int64_t)C.z << 32) | (uint32_t)C.y;
+                    quantize_store<BITS>(*dst, s.codes, s.sb, vrow, dim, sub, LANES, (uint32_t)C.x, s.rounding != 0);
+                }
+                *dst = xn;                           // cached rows keep full precision, a newcomer enters verbatim
+            } else {
+                quantize_store<BITS>(xn, s.codes, s.sb, grow, dim, sub, LANES, (uint32_t)B.x, s.rounding != 0);
+            }
         }
         __syncwarp();                                          // the records are rewritten by the next block
     }

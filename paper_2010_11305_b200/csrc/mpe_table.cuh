@@ -439,7 +439,7 @@ __device__ void table_state(TableShared& sh, int32_t* scratch, const State& s, c
                         if (!always && pv <= low[j]) ++n_byp;
                         else { ckey = set[j]; lists = bucket_put(s, tb.set_base + set[j], cap, (int32_t)k); }
                     }
-                    if (mult[j] > hot_min) list_hot_row(w, (int32_t)k, mult[j]);
+                    list_long_row(w, (int32_t)k, mult[j], hot_min);
                 }
                 w.loc[k] = loc[j]; w.final_loc[k] = loc[j];
                 w.cand_key[k] = ckey;
