@@ -254,7 +254,7 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags) {
     A(w.occ_b, n);
     A(w.uniq_row, nu); A(w.uniq_t, nu); A(w.seg, nu + 1); A(w.loc, nu); A(w.final_loc, nu);
     A(w.victim, nu); A(w.defer_k, nu); A(w.heads, nu);
-    A(w.hot_base, nu); A(w.cand_key, nu);
+    A(w.hot_base, nu); A(w.hot_left, nu); A(w.cand_key, nu);
     const int64_t max_tasks = hot_capacity(L);
     A(w.task_k, max_tasks); A(w.partial, max_tasks * h->dim); A(w.hot_k, max_tasks); A(w.mid_k, L / MID_MIN + 1);
 #undef A
@@ -574,14 +574,22 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool chain) {
         CK(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
         dispatch(h->bits, s.lanes, [&](auto bc, auto lc) {
             constexpr int LANES = decltype(lc)::value;
-            LAUNCH_ON(h, h->side, "hot_partial", k_hot_partial<LANES>, grid_for(h, hot_capacity(L), 1, 2), 8 * LANES, 32 * s.dim * sizeof(float), s, w, av);
+            LAUNCH_ON(h, h->side, "hot_partial", k_hot_partial<LANES>, grid_for(h, hot_capacity(L), 1, 2), HOT_THREADS, 32 * s.dim * sizeof(float), s, w, av);
         });
         CK(h, cudaEventRecord(h->ev_join, h->side));
         return MPE_OK;
     };
     if (plan.blocks == 1 && plan.items == TBL_ITEMS_SMALL && chain) {
         rc = enqueue_table(h, plan, av, true);
-        if (rc == MPE_OK) rc = hot_partial();
+        if (rc != MPE_OK) return rc;
+        if (L <= UPD_ONE_LAUNCH_L) {
+            dispatch(h->bits, s.lanes, [&](auto bc, auto lc) {
+                auto kern = k_update_small<decltype(bc)::value, decltype(lc)::value>;
+                LAUNCH(h, "update", kern, grid_for(h, L, HOT_THREADS / s.lanes, 2), HOT_THREADS, 32 * s.dim * sizeof(float), s, w, av);
+            });
+            return check_launch(h);
+        }
+        rc = hot_partial();
     } else {
         // (the cluster kernel leaves the hot rows to k_priority; the grid-wide kernels list them with the distinct rows, so that
         // their partial sums can start before it)

@@ -97,7 +97,7 @@ struct Work {
     Counters* ctr;
     int32_t *table_start, *tile_base, *ustart;   // [T+1]
     int32_t* occ_b;        // [L] by sorted order: sample of the element; sign bit: last occurrence of its row
-    int32_t *uniq_row, *uniq_t, *seg, *loc, *final_loc, *victim, *hot_base;   // per unique row
+    int32_t *uniq_row, *uniq_t, *seg, *loc, *final_loc, *victim, *hot_base, *hot_left;   // per unique row
     int32_t* task_k;       // [hot tasks]
     int32_t* hot_k;        // [hot rows]
     int32_t* mid_k;        // [rows with more than MID_MIN occurrences that are not hot]
@@ -192,7 +192,7 @@ k_make_keys(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
 __device__ __forceinline__ void list_hot_row(const Work& w, int32_t k, uint32_t m) {
     const uint32_t nt = (m + HOT_SPAN - 1) / HOT_SPAN;
     const uint32_t hb = atomicAdd(&w.ctr->hot_tasks, nt);
-    w.hot_base[k] = (int32_t)hb;
+    w.hot_base[k] = (int32_t)hb; w.hot_left[k] = (int32_t)nt;
     w.hot_k[atomicAdd(&w.ctr->hot_rows, 1u)] = k;
     atomicAdd(&w.ctr->hot_occ, (unsigned long long)m);
     for (uint32_t j = 0; j < nt; ++j) w.task_k[hb + j] = k;
@@ -834,26 +834,39 @@ k_policy(State s, Work w, StepArgs a) {
 // ---------------------------------------------------------------------------------------------
 // backward 3: merged gradient of one distinct row (Section 5.1), radix-32 tree over index positions
 // ---------------------------------------------------------------------------------------------
-// up to 32 consecutive occurrences, added left to right; the group reads LANES sample ids at a time.
+// Up to 32 consecutive occurrences, added left to right.  The sample ids are fetched all at once, LANES per register, and handed
+// round with shuffles; eight gradient rows are in flight, four of them being added.
 // gcol points at the group's lane-th float4 of column block t; stride_bytes is the size of one sample's row of grad_out.
-template <int LANES>
-__device__ __forceinline__ float4 sum_chunk(const int32_t* __restrict__ occ_b, const char* __restrict__ gcol, uint32_t stride_bytes,
-                                            int32_t first, int len, uint32_t gmask, int gbase, int sub) {
-    constexpr int NB = LANES < 8 ? LANES : 8;
-    float4 acc;
-    if (LANES == 32 && len == 32) {       // a full chunk handled by a whole warp: no bounds to check, 8 rows in flight
-        const uint32_t myb = (uint32_t)occ_b[first + sub] & 0x7fffffffU;
-        float4 va[4], vb[4];
-        auto row = [&](int u) { return __ldg(reinterpret_cast<const float4*>(gcol + (size_t)__shfl_sync(0xffffffffU, myb, u) * stride_bytes)); };
+// FULL: the chunk has all 32 (most chunks of a hot row do): no bounds to check.
+template <int LANES, bool FULL>
+__device__ __forceinline__ float4 sum_chunk_of(const int32_t* __restrict__ occ_b, const char* __restrict__ gcol, uint32_t stride_bytes,
+                                               int32_t first, int len, uint32_t gmask, int gbase, int sub) {
+    if (FULL) len = 32;
+    constexpr int NW = LANES >= 4 ? 32 / LANES : 1;        // groups of one or two lanes read the ids one by one
+    uint32_t id[NW];
+    if (LANES >= 4) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) va[u] = row(u);
+        for (int j = 0; j < NW; ++j) id[j] = (uint32_t)occ_b[first + min(j * LANES + sub, len - 1)] & 0x7fffffffu;
+    }
+    const float NZ = __int_as_float(0x80000000);           // -0: adding it changes no value, not even a zero's sign
+    auto row = [&](int u) {
+        const uint32_t b = LANES >= 4 ? __shfl_sync(gmask, id[LANES >= 4 ? u / LANES : 0], gbase + (u & (LANES - 1)))
+                                      : (uint32_t)occ_b[first + min(u, len - 1)] & 0x7fffffffu;
+        float4 v = make_float4(NZ, NZ, NZ, NZ);
+        if (FULL || u < len) v = __ldg(reinterpret_cast<const float4*>(gcol + (size_t)b * stride_bytes));
+        return v;
+    };
+    float4 va[4], vb[4], acc;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) vb[u] = row(4 + u);
-        acc = va[0];
+    for (int u = 0; u < 4; ++u) va[u] = row(u);
 #pragma unroll
-        for (int u = 1; u < 4; ++u) acc = add4(acc, va[u]);
+    for (int u = 0; u < 4; ++u) vb[u] = row(4 + u);
+    acc = va[0];
 #pragma unroll
-        for (int g = 1; g < 4; ++g) {
+    for (int u = 1; u < 4; ++u) acc = add4(acc, va[u]);
+#pragma unroll
+    for (int g = 1; g < 4; ++g) {
+        if (FULL || len > 8 * g - 4) {                     // the same for the whole group
 #pragma unroll
             for (int u = 0; u < 4; ++u) va[u] = row(8 * g + u);
 #pragma unroll
@@ -863,27 +876,18 @@ __device__ __forceinline__ float4 sum_chunk(const int32_t* __restrict__ occ_b, c
 #pragma unroll
             for (int u = 0; u < 4; ++u) acc = add4(acc, va[u]);
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc = add4(acc, vb[u]);
-        return acc;
     }
-    acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int j0 = 0; j0 < len; j0 += LANES) {
-        const int n = min(LANES, len - j0);
-        const uint32_t myb = sub < n ? (uint32_t)occ_b[first + j0 + sub] & 0x7fffffffU : 0u;
-        for (int u0 = 0; u0 < n; u0 += NB) {
-            float4 v[NB];
+    // the last batch fetched has not been added yet (it is all -0 where the chunk ended before it)
 #pragma unroll
-            for (int u = 0; u < NB; ++u) {
-                const uint32_t b = __shfl_sync(gmask, myb, gbase + u0 + u);
-                if (u0 + u < n) v[u] = __ldg(reinterpret_cast<const float4*>(gcol + (size_t)b * stride_bytes));
-            }
-#pragma unroll
-            for (int u = 0; u < NB; ++u)
-                if (u0 + u < n) acc = (j0 + u0 + u == 0) ? v[u] : add4(acc, v[u]);
-        }
-    }
+    for (int u = 0; u < 4; ++u) acc = add4(acc, vb[u]);
     return acc;
+}
+
+template <int LANES>
+__device__ __forceinline__ float4 sum_chunk(const int32_t* __restrict__ occ_b, const char* __restrict__ gcol, uint32_t stride_bytes,
+                                            int32_t first, int len, uint32_t gmask, int gbase, int sub) {
+    return len == 32 ? sum_chunk_of<LANES, true>(occ_b, gcol, stride_bytes, first, len, gmask, gbase, sub)
+                     : sum_chunk_of<LANES, false>(occ_b, gcol, stride_bytes, first, len, gmask, gbase, sub);
 }
 
 // LEVEL 0 adds up to 32 terms left to right; LEVEL l adds up to 32 results of LEVEL l-1
@@ -903,38 +907,45 @@ __device__ __forceinline__ float4 tree_reduce(const Term& term, int64_t first, i
     }
 }
 
-// rows with more than HOT_SPAN occurrences: one block per HOT_SPAN occurrences computes two tree levels
-// (8 groups of LANES lanes share the 32 chunks of a task)
+// One task of a hot row, by a whole block: two tree levels over HOT_SPAN occurrences, a chunk of 32 per group of LANES lanes.  The
+// sum is left with group 0.
+constexpr int HOT_THREADS = 256;
 template <int LANES>
-__global__ void __launch_bounds__(8 * LANES, LANES == 32 ? 3 : 1)
-k_hot_partial(State s, Work w, StepArgs a) {
-    extern __shared__ float chunk_sums[];     // [32][dim]
-    if (w.ctr->abort) return;
-    const float* __restrict__ grad = a.grad;
-    const int dim = s.dim;
-    const int sub = threadIdx.x & (LANES - 1), grp = threadIdx.x / LANES, ngrp = blockDim.x / LANES;
+__device__ __forceinline__ float4 hot_task_sum(const State& s, const Work& w, const float* __restrict__ grad, uint32_t task, int32_t k, float* chunk_sums /* [32][dim] */) {
+    constexpr int dim = 4 * LANES, ngrp = HOT_THREADS / LANES;
+    const int sub = threadIdx.x & (LANES - 1), grp = threadIdx.x / LANES;
     const int gbase = (threadIdx.x & 31) & ~(LANES - 1);
     const uint32_t gmask = group_mask(LANES);
-    const uint32_t ntask = w.ctr->hot_tasks;
     const uint32_t stride_bytes = (uint32_t)s.T * (uint32_t)dim * 4u;
+    const int32_t j = (int32_t)task - w.hot_base[k];
+    const int32_t first = w.seg[k] + j * HOT_SPAN;
+    const int32_t n = min(HOT_SPAN, w.seg[k + 1] - first);
+    const int nchunk = (n + 31) >> 5;
+    const char* gcol = reinterpret_cast<const char*>(grad + (int64_t)w.uniq_t[k] * dim + 4 * sub);
+    for (int c = grp; c < nchunk; c += ngrp) {
+        const float4 v = sum_chunk<LANES>(w.occ_b, gcol, stride_bytes, first + 32 * c, min(32, n - 32 * c), gmask, gbase, sub);
+        reinterpret_cast<float4*>(chunk_sums + c * dim)[sub] = v;
+    }
+    __syncthreads();
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (grp == 0) {
+        acc = reinterpret_cast<const float4*>(chunk_sums)[sub];
+        for (int c = 1; c < nchunk; ++c) acc = add4(acc, reinterpret_cast<const float4*>(chunk_sums + c * dim)[sub]);
+    }
+    __syncthreads();
+    return acc;
+}
+
+// the hot rows' tasks -> their partial sums
+template <int LANES>
+__global__ void __launch_bounds__(HOT_THREADS, 2)
+k_hot_partial(State s, Work w, StepArgs a) {
+    extern __shared__ float chunk_sums[];
+    if (w.ctr->abort) return;
+    const uint32_t ntask = w.ctr->hot_tasks;
     for (uint32_t task = blockIdx.x; task < ntask; task += gridDim.x) {
-        const int32_t k = w.task_k[task];
-        const int32_t j = (int32_t)task - w.hot_base[k];
-        const int32_t first = w.seg[k] + j * HOT_SPAN;
-        const int32_t n = min(HOT_SPAN, w.seg[k + 1] - first);
-        const int nchunk = (n + 31) >> 5;
-        const char* gcol = reinterpret_cast<const char*>(grad + (int64_t)w.uniq_t[k] * dim + 4 * sub);
-        for (int c = grp; c < nchunk; c += ngrp) {
-            const float4 v = sum_chunk<LANES>(w.occ_b, gcol, stride_bytes, first + 32 * c, min(32, n - 32 * c), gmask, gbase, sub);
-            reinterpret_cast<float4*>(chunk_sums + c * dim)[sub] = v;
-        }
-        __syncthreads();
-        if (grp == 0) {
-            float4 acc = reinterpret_cast<const float4*>(chunk_sums)[sub];
-            for (int c = 1; c < nchunk; ++c) acc = add4(acc, reinterpret_cast<const float4*>(chunk_sums + c * dim)[sub]);
-            reinterpret_cast<float4*>(w.partial + (int64_t)task * dim)[sub] = acc;
-        }
-        __syncthreads();
+        const float4 acc = hot_task_sum<LANES>(s, w, a.grad, task, w.task_k[task], chunk_sums);
+        if (threadIdx.x < LANES) reinterpret_cast<float4*>(w.partial + (int64_t)task * 4 * LANES)[threadIdx.x] = acc;
     }
 }
 
@@ -975,6 +986,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 
 constexpr int UPD_WARPS = 4;     // warps per block of k_update
 constexpr int UPD_SMALL_U = 524288;   // at most this many distinct rows: blocks of 8 rows instead of 32
+constexpr int64_t UPD_ONE_LAUNCH_L = 131072;   // steps of at most this many indices: k_update_small
 constexpr int UPD_SMEM = UPD_WARPS * 32 * (4 * 16 + 4);
 
 // Every distinct row that is not on the multi-block path, except newcomers that wait for a write-back.  A warp stages the
@@ -1203,6 +1215,86 @@ k_update_list(State s, Work w, const int32_t* __restrict__ list, const uint32_t*
             g = tree_reduce<4>(term, 0, (m + HOT_SPAN - 1) / HOT_SPAN);
         }
         apply_update<BITS, LANES>(s, tb, t, row, loc, floc, victim, g, x, lr, step, sub, gmask);
+    }
+}
+
+// The whole of backward 3 and 4 in one launch, for steps of few indices: with few rows there is nothing to gain from staging and
+// handing out (k_update), and each of its neighbours (k_hot_partial, two of k_update_list) lasts as long as a launch does.  A block
+// takes the tasks of hot rows first -- the last of a row's tasks to finish updates the row -- then rows, one per group of LANES
+// lanes; the block that finishes last updates the newcomers that had to wait for a write-back.
+template <int BITS, int LANES>
+__global__ void __launch_bounds__(HOT_THREADS, 2)
+k_update_small(State s, Work w, StepArgs a) {
+    extern __shared__ float chunk_sums[];
+    __shared__ uint32_t s_last;
+    if (w.ctr->abort) return;
+    constexpr int dim = 4 * LANES, ngrp = HOT_THREADS / LANES;
+    const int sub = threadIdx.x & (LANES - 1), grp = threadIdx.x / LANES;
+    const int gbase = (threadIdx.x & 31) & ~(LANES - 1);
+    const uint32_t gmask = group_mask(LANES);
+    const uint32_t hot_min = hot_threshold(w.ctr->L);
+    const uint32_t ntask = w.ctr->hot_tasks;
+    const uint32_t items = ntask + (w.ctr->U + ngrp - 1) / ngrp;
+    const uint32_t stride_bytes = (uint32_t)s.T * (uint32_t)dim * 4u;
+    auto tree = [&](int32_t k, int32_t m) {                // merged gradient of a hot row from its tasks' sums
+        const float* part = w.partial + (int64_t)w.hot_base[k] * dim + 4 * sub;
+        auto term = [&](int64_t j) { return __ldcg(reinterpret_cast<const float4*>(part + j * dim)); };
+        return tree_reduce<4>(term, 0, (m + HOT_SPAN - 1) / HOT_SPAN);
+    };
+    auto merged = [&](int32_t k, int t, int32_t first, int32_t m) {       // ... of any other row
+        const char* gcol = reinterpret_cast<const char*>(a.grad + (int64_t)t * dim + 4 * sub);
+        float4 g = sum_chunk<LANES>(w.occ_b, gcol, stride_bytes, first, min(32, m), gmask, gbase, sub);
+        for (int32_t c = 32; c < m; c += 32) g = add4(g, sum_chunk<LANES>(w.occ_b, gcol, stride_bytes, first + c, min(32, m - c), gmask, gbase, sub));
+        return g;
+    };
+    for (uint32_t item = blockIdx.x; item < items; item += gridDim.x) {
+        if (item < ntask) {
+            const int32_t k = w.task_k[item];
+            const float4 acc = hot_task_sum<LANES>(s, w, a.grad, item, k, chunk_sums);
+            const int loc = w.loc[k], floc = w.final_loc[k], victim = loc < 0 && floc >= 0 ? w.victim[k] : VICTIM_NONE;
+            const int32_t m = w.seg[k + 1] - w.seg[k];
+            const bool single = m <= HOT_SPAN && victim != VICTIM_DEFER;
+            if (!single) {
+                if (grp == 0) { reinterpret_cast<float4*>(w.partial + (int64_t)item * dim)[sub] = acc; __threadfence(); }
+                __syncthreads();
+                if (threadIdx.x == 0) s_last = atomicSub(w.hot_left + k, 1);
+                __syncthreads();
+                if (s_last != 1u || victim == VICTIM_DEFER) continue;
+                __threadfence();
+            }
+            if (grp == 0) {
+                const int t = w.uniq_t[k];
+                const int32_t row = w.uniq_row[k];
+                const TableDev tb = s.tables[t];
+                const float4 x = fetch4<BITS, false>(s, tb, row, loc, sub);
+                apply_update<BITS, LANES>(s, tb, t, row, loc, floc, victim, single ? acc : tree(k, m), x, a.lr, a.step, sub, gmask);
+            }
+        } else {
+            const int64_t k = (int64_t)(item - ntask) * ngrp + grp;
+            if (k >= w.ctr->U) continue;
+            const int32_t first = w.seg[k], m = w.seg[k + 1] - first, row = w.uniq_row[k];
+            const int loc = w.loc[k], floc = w.final_loc[k], t = w.uniq_t[k];
+            const int victim = loc < 0 && floc >= 0 ? w.victim[k] : VICTIM_NONE;
+            if (loc == LOC_INVALID || (uint32_t)m > hot_min || victim == VICTIM_DEFER) continue;
+            const TableDev tb = s.tables[t];
+            const float4 x = fetch4<BITS, false>(s, tb, row, loc, sub);
+            apply_update<BITS, LANES>(s, tb, t, row, loc, floc, victim, merged((int32_t)k, t, first, m), x, a.lr, a.step, sub, gmask);
+        }
+    }
+    __syncthreads();                                       // the block's stores have been issued
+    if (threadIdx.x == 0) { __threadfence(); s_last = atomicAdd(&w.ctr->upd_next, 1u) == gridDim.x - 1u; }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const uint32_t n = __ldcg(&w.ctr->deferred);
+    for (uint32_t i = grp; i < n; i += ngrp) {             // the rows they displace have been written back by now
+        const int32_t k = w.defer_k[i];
+        const int t = w.uniq_t[k];
+        const int32_t row = w.uniq_row[k], first = w.seg[k], m = w.seg[k + 1] - first;
+        const TableDev tb = s.tables[t];
+        const float4 x = fetch4<BITS, false>(s, tb, row, w.loc[k], sub);
+        const float4 g = (uint32_t)m > hot_min ? tree(k, m) : merged(k, t, first, m);
+        apply_update<BITS, LANES>(s, tb, t, row, w.loc[k], w.final_loc[k], w.victim[k], g, x, a.lr, a.step, sub, gmask);
     }
 }
 
