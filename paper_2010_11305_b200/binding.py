@@ -219,9 +219,9 @@ class Mpe:
     def export_rows(self, table, rows):
         rows = np.ascontiguousarray(rows, np.int64)
         n = rows.size
-        codes = np.zeros((n, self.dim * self.bits // 8), np.uint8)
-        scale = np.zeros(n, np.float32)
-        bias = np.zeros(n, np.float32)
+        codes = np.empty((n, self.dim * self.bits // 8), np.uint8)       # the call writes every entry
+        scale = np.empty(n, np.float32)
+        bias = np.empty(n, np.float32)
         _check(_lib.mpe_export_rows(self._h, table, rows.ctypes.data, n, codes.ctypes.data, scale.ctypes.data,
                                     bias.ctypes.data), "mpe_export_rows")
         return codes, scale, bias
@@ -237,10 +237,10 @@ class Mpe:
 
     def export_aux(self, table, rows):
         rows = np.ascontiguousarray(rows, np.int64)
-        cnt = np.zeros(max(rows.size, 1), np.uint32)
-        G = np.zeros(max(rows.size, 1), np.float32)
+        cnt = np.empty(rows.size, np.uint32)
+        G = np.empty(rows.size, np.float32)
         _check(_lib.mpe_export_aux(self._h, table, rows.ctypes.data, rows.size, cnt.ctypes.data, G.ctypes.data), "mpe_export_aux")
-        return cnt[:rows.size], G[:rows.size]
+        return cnt, G
 
     def set_rounding(self, mode):
         _check(_lib.mpe_set_rounding(self._h, mode), "mpe_set_rounding")

@@ -5,6 +5,7 @@
 #include "mpe_table.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -12,6 +13,7 @@
 #include <mutex>
 #include <set>
 #include <string>
+#include <thread>
 #include <type_traits>
 #include <vector>
 
@@ -69,6 +71,10 @@ struct mpe_handle {
         cudaEvent_t ev_idx = nullptr, ev_grad = nullptr, ev_fwd = nullptr, ev_done = nullptr, ev_down = nullptr;
         bool used = false;
     } slot[2];
+    // staging of the exports: two slots of pinned host memory and of device memory, so that one chunk of rows crosses the link
+    // while the chunk before it is copied into the caller's arrays
+    struct ExportSlot { unsigned char *pin = nullptr, *dev = nullptr; } xslot[2];
+    size_t x_cap = 0;
     int64_t sh_cap_L = 0, sh_cap_off = 0, sh_cap_out = 0;
     uint64_t submitted = 0;
     // step state
@@ -720,6 +726,100 @@ int send_route(mpe_handle* h, const void* const* ptrs, int32_t n_ranks, int32_t 
     return MPE_OK;
 }
 
+void free_export_slots(mpe_handle* h) {
+    for (auto& sl : h->xslot) { if (sl.pin) cudaFreeHost(sl.pin); if (sl.dev) cudaFree(sl.dev); sl = {}; }
+    h->x_cap = 0;
+}
+
+// Copies between the caller's arrays and a pinned slot, by up to EXPORT_THREADS threads: a fresh array of the caller's is mapped in
+// page by page as it is written, which is what bounds a large export (one thread: about 2 GB/s).
+constexpr int EXPORT_THREADS = 8;
+constexpr size_t EXPORT_SLOT_BYTES = 16u << 20, EXPORT_PIECE = 1u << 20;
+struct CopyJob { unsigned char* dst; const unsigned char* src; size_t n; };
+class Copier {
+public:
+    ~Copier() { wait(); }
+    // starts on the copies; `big` ones are shared out among threads, small ones are made here
+    void start(std::vector<CopyJob>&& whole) {
+        wait();
+        size_t total = 0;
+        jobs_.clear();
+        for (const CopyJob& j : whole)
+            for (size_t o = 0; o < j.n; o += EXPORT_PIECE) jobs_.push_back({j.dst + o, j.src + o, std::min(EXPORT_PIECE, j.n - o)});
+        for (const CopyJob& j : jobs_) total += j.n;
+        next_ = 0;
+        const int want = (int)std::min<size_t>({(size_t)EXPORT_THREADS, total / EXPORT_PIECE, (size_t)std::max(1u, std::thread::hardware_concurrency())});
+        if (want < 2) { work(); return; }
+        try { for (int i = 0; i < want; ++i) threads_.emplace_back([this] { work(); }); }
+        catch (...) { work(); }                  // no thread to be had: what is left is done here
+    }
+    void wait() { for (auto& t : threads_) t.join(); threads_.clear(); }
+private:
+    void work() { for (size_t i; (i = next_.fetch_add(1)) < jobs_.size();) std::memcpy(jobs_[i].dst, jobs_[i].src, jobs_[i].n); }
+    std::vector<CopyJob> jobs_;
+    std::atomic<size_t> next_{0};
+    std::vector<std::thread> threads_;
+};
+
+// codes / scale / bias, or counters / accumulators, of n rows into the caller's arrays (null: not wanted)
+int export_rows(mpe_handle* h, int32_t table, const int64_t* h_rows, int64_t n, uint8_t* h_codes, float* h_scale, float* h_bias,
+                uint32_t* h_cnt, float* h_G) {
+    DeviceGuard guard(h->device);
+    CK(h, cudaStreamSynchronize(h->stream));
+    const size_t cb = (size_t)h->code_bytes;
+    struct Part { unsigned char* host; size_t bytes; size_t at; };
+    std::vector<Part> parts{{reinterpret_cast<unsigned char*>(h_codes), cb, 0}, {reinterpret_cast<unsigned char*>(h_scale), 4, 0},
+                            {reinterpret_cast<unsigned char*>(h_bias), 4, 0}, {reinterpret_cast<unsigned char*>(h_cnt), 4, 0},
+                            {reinterpret_cast<unsigned char*>(h_G), 4, 0}};
+    auto padded = [](size_t v) { return (v + 255) & ~size_t(255); };
+    size_t per_row = sizeof(int64_t);
+    for (const Part& p : parts) if (p.host) per_row += p.bytes;
+    const int64_t chunk = std::min<int64_t>(n, (int64_t)((EXPORT_SLOT_BYTES - 8 * 256) / per_row));
+    const size_t need = per_row * (size_t)chunk + 8 * 256;
+    if (need > h->x_cap) {
+        free_export_slots(h);
+        // small exports get a small slot; the larger of the two kinds is kept until the handle goes
+        const size_t cap = std::min(EXPORT_SLOT_BYTES, std::max<size_t>(need, 64u << 10));
+        for (auto& sl : h->xslot)
+            if (cudaHostAlloc((void**)&sl.pin, cap, cudaHostAllocDefault) != cudaSuccess || cudaMalloc((void**)&sl.dev, cap) != cudaSuccess) {
+                cudaGetLastError();
+                free_export_slots(h);
+                return MPE_ERR_NOMEM;
+            }
+        h->x_cap = cap;
+    }
+    Copier copier;
+    int rc = MPE_OK;
+    int turn = 0;
+    for (int64_t r0 = 0; r0 < n; r0 += chunk, turn ^= 1) {
+        const int64_t m = std::min(chunk, n - r0);
+        auto& sl = h->xslot[turn];               // its last contents were copied out before the chunk before this one was started on
+        const size_t out0 = padded(sizeof(int64_t) * (size_t)m);
+        size_t at = out0;
+        for (Part& p : parts) if (p.host) { p.at = at; at = padded(at + p.bytes * (size_t)m); }
+        std::memcpy(sl.pin, h_rows + r0, sizeof(int64_t) * (size_t)m);
+        CK(h, cudaMemcpyAsync(sl.dev, sl.pin, sizeof(int64_t) * (size_t)m, cudaMemcpyHostToDevice, h->stream));
+        const int64_t* d_rows = reinterpret_cast<const int64_t*>(sl.dev);
+        auto dev = [&](int i) { return parts[i].host ? sl.dev + parts[i].at : nullptr; };
+        if (h_codes) {
+            const int words = (int)(cb % 16 == 0 ? cb / 16 : cb % 4 == 0 ? cb / 4 : cb);
+            const int g = grid_for(h, m * words, 256, 8);
+            if (cb % 16 == 0) LAUNCH(h, "gather_rows", k_gather_codes<uint4>, g, 256, 0, h->st, table, d_rows, m, words, reinterpret_cast<uint4*>(dev(0)));
+            else if (cb % 4 == 0) LAUNCH(h, "gather_rows", k_gather_codes<uint32_t>, g, 256, 0, h->st, table, d_rows, m, words, reinterpret_cast<uint32_t*>(dev(0)));
+            else LAUNCH(h, "gather_rows", k_gather_codes<uint8_t>, g, 256, 0, h->st, table, d_rows, m, words, dev(0));
+        }
+        LAUNCH(h, "gather_rows", k_gather_scalars, grid_for(h, m, 256, 8), 256, 0, h->st, table, d_rows, m, reinterpret_cast<float*>(dev(1)),
+               reinterpret_cast<float*>(dev(2)), reinterpret_cast<uint32_t*>(dev(3)), reinterpret_cast<float*>(dev(4)));
+        CK(h, cudaMemcpyAsync(sl.pin + out0, sl.dev + out0, at - out0, cudaMemcpyDeviceToHost, h->stream));
+        CK(h, cudaStreamSynchronize(h->stream));
+        if ((rc = check_launch(h)) != MPE_OK) break;
+        std::vector<CopyJob> jobs;
+        for (const Part& p : parts) if (p.host) jobs.push_back({p.host + p.bytes * (size_t)r0, sl.pin + p.at, p.bytes * (size_t)m});
+        copier.start(std::move(jobs));           // waits for the chunk before this one
+    }
+    return rc;
+}
+
 }  // namespace
 
 extern "C" {
@@ -950,6 +1050,7 @@ int mpe_destroy(mpe_handle* h) {
     for (cudaEvent_t e : {h->ev_free, h->alt.ev_free, h->ev_keys, h->ev_prep, h->alt.ev_keys, h->alt.ev_prep}) if (e) cudaEventDestroy(e);
     if (h->copy_in) { cudaStreamSynchronize(h->copy_in); cudaStreamDestroy(h->copy_in); }
     if (h->copy_out) { cudaStreamSynchronize(h->copy_out); cudaStreamDestroy(h->copy_out); }
+    free_export_slots(h);
     for (auto& sl : h->slot) {
         for (cudaEvent_t e : {sl.ev_idx, sl.ev_grad, sl.ev_fwd, sl.ev_done, sl.ev_down}) if (e) cudaEventDestroy(e);
         cudaFree(sl.idx); cudaFree(sl.off); cudaFree(sl.grad); cudaFree(sl.out);
@@ -1090,23 +1191,7 @@ int mpe_export_rows(mpe_handle* h, int32_t table, const int64_t* h_rows, int64_t
                     float* h_scale, float* h_bias) {
     if (!h || table < 0 || table >= h->T || n < 0 || (n > 0 && (!h_rows || !h_codes || !h_scale || !h_bias))) return MPE_ERR_ARG;
     if (n == 0) return MPE_OK;
-    DeviceGuard guard(h->device);
-    CK(h, cudaStreamSynchronize(h->stream));
-    int64_t* d_rows = nullptr; uint8_t* d_codes = nullptr; float *d_s = nullptr, *d_b = nullptr;
-    int rc = MPE_OK;
-    if ((rc = dmalloc(h, &d_rows, n, nullptr)) == MPE_OK && (rc = dmalloc(h, &d_codes, n * h->code_bytes, nullptr)) == MPE_OK &&
-        (rc = dmalloc(h, &d_s, n, nullptr)) == MPE_OK && (rc = dmalloc(h, &d_b, n, nullptr)) == MPE_OK) {
-        cudaMemcpy(d_rows, h_rows, sizeof(int64_t) * n, cudaMemcpyHostToDevice);
-        cudaMemset(d_codes, 0, (size_t)n * h->code_bytes); cudaMemset(d_s, 0, sizeof(float) * n); cudaMemset(d_b, 0, sizeof(float) * n);
-        LAUNCH(h, "gather_rows", k_gather_rows, grid_for(h, n, 256, 8), 256, 0, h->st, table, (const int64_t*)d_rows, n, h->code_bytes,
-               d_codes, d_s, d_b, (uint32_t*)nullptr, (float*)nullptr);
-        cudaMemcpy(h_codes, d_codes, (size_t)n * h->code_bytes, cudaMemcpyDeviceToHost);
-        cudaMemcpy(h_scale, d_s, sizeof(float) * n, cudaMemcpyDeviceToHost);
-        cudaMemcpy(h_bias, d_b, sizeof(float) * n, cudaMemcpyDeviceToHost);
-        rc = check_launch(h);
-    }
-    cudaFree(d_rows); cudaFree(d_codes); cudaFree(d_s); cudaFree(d_b);
-    return rc;
+    return export_rows(h, table, h_rows, n, h_codes, h_scale, h_bias, nullptr, nullptr);
 }
 
 int mpe_export_cache(mpe_handle* h, int32_t table, int32_t* h_tags, float* h_rows, uint32_t* h_ts) {
@@ -1128,22 +1213,7 @@ int mpe_export_cache(mpe_handle* h, int32_t table, int32_t* h_tags, float* h_row
 int mpe_export_aux(mpe_handle* h, int32_t table, const int64_t* h_rows, int64_t n, uint32_t* h_cnt, float* h_adagrad) {
     if (!h || table < 0 || table >= h->T || n < 0 || (n > 0 && !h_rows)) return MPE_ERR_ARG;
     if (n == 0 || (!h_cnt && !h_adagrad)) return MPE_OK;
-    DeviceGuard guard(h->device);
-    CK(h, cudaStreamSynchronize(h->stream));
-    int64_t* d_rows = nullptr; uint32_t* d_c = nullptr; float* d_g = nullptr;
-    int rc = MPE_OK;
-    if ((rc = dmalloc(h, &d_rows, n, nullptr)) == MPE_OK && (rc = dmalloc(h, &d_c, n, nullptr)) == MPE_OK &&
-        (rc = dmalloc(h, &d_g, n, nullptr)) == MPE_OK) {
-        cudaMemcpy(d_rows, h_rows, sizeof(int64_t) * n, cudaMemcpyHostToDevice);
-        cudaMemset(d_c, 0, sizeof(uint32_t) * n); cudaMemset(d_g, 0, sizeof(float) * n);
-        LAUNCH(h, "gather_rows", k_gather_rows, grid_for(h, n, 256, 8), 256, 0, h->st, table, (const int64_t*)d_rows, n, h->code_bytes,
-               (uint8_t*)nullptr, (float*)nullptr, (float*)nullptr, d_c, d_g);
-        if (h_cnt) cudaMemcpy(h_cnt, d_c, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost);
-        if (h_adagrad) cudaMemcpy(h_adagrad, d_g, sizeof(float) * n, cudaMemcpyDeviceToHost);
-        rc = check_launch(h);
-    }
-    cudaFree(d_rows); cudaFree(d_c); cudaFree(d_g);
-    return rc;
+    return export_rows(h, table, h_rows, n, nullptr, nullptr, nullptr, h_cnt, h_adagrad);
 }
 
 int mpe_kernel_launches(mpe_handle* h, uint64_t* count) {

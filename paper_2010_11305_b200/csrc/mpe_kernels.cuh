@@ -69,7 +69,7 @@ struct State {
     uint32_t* hit_epoch;   // [slots] forward call in which the slot was last hit
     int32_t* hit_k;        // [slots] unique-row index of that hit
     uint32_t* set_cnt;     // [sets] candidates for admission dropped into the set's bucket in this step; zero between steps
-    int32_t* bucket;       // [sets][bucket_cap(ways)] their distinct-row indices
+    int2* bucket;          // [sets][bucket_cap(ways)] their {distinct-row index, row id}
     uint32_t* floor;       // [sets] a lower bound of the lowest priority value among the set's residents (0: none known)
     unsigned long long* stats;   // [T][8]
 };
@@ -103,7 +103,7 @@ struct Work {
     int32_t* mid_k;        // [rows with more than MID_MIN occurrences that are not hot]
     int32_t* cand_key;     // [distinct rows] the row's set if it is a candidate for admission, else CAND_NONE
     int32_t* defer_k;      // [deferred newcomers]
-    int32_t* heads;        // [sets with candidates] one candidate of each (small steps: the set itself, table by table)
+    int2* heads;           // [sets with candidates] {set of the concatenated cache, table}
     float* partial;        // [hot tasks][dim]
     int32_t sort_tile;     // keys per tile of the sorts of this workspace
 };
@@ -535,18 +535,18 @@ constexpr int BUCKET_CAP_MAX = 64;
 constexpr int BUCKET_PER_LANE = 4;    // bucket_cap(ways) / ways is at most this
 
 // the candidate k joins the bucket of set `gset`; true if it is the set's first one in this step
-__device__ __forceinline__ bool bucket_put(const State& s, int64_t gset, int cap, int32_t k) {
+__device__ __forceinline__ bool bucket_put(const State& s, int64_t gset, int cap, int32_t k, int32_t row) {
     const uint32_t pos = atomicAdd(s.set_cnt + gset, 1u);
-    if (pos < (uint32_t)cap) s.bucket[gset * cap + pos] = k;
+    if (pos < (uint32_t)cap) s.bucket[gset * cap + pos] = make_int2(k, row);
     return pos == 0;
 }
 
 struct PolicyCounts { uint32_t admit, evict, bypass; };
 
 // One set.  All lanes of the group (`gmask`, first lane `gbase`) take part; `sorted` is the group's own piece of shared memory,
-// bucket_cap(ways) words.  The table's distinct rows are [ub, ub + n_rows).
+// bucket_cap(ways) pairs.  The table's distinct rows are [ub, ub + n_rows).
 __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w, const TableDev& tb, int64_t gset, int32_t ub, int32_t n_rows,
-                                                   uint32_t step, uint32_t epoch, uint32_t gmask, int gbase, int way, volatile int32_t* sorted) {
+                                                   uint32_t step, uint32_t epoch, uint32_t gmask, int gbase, int way, int2* sorted) {
     const int ways = s.ways, cap = bucket_cap(ways);
     const int64_t slot = gset * ways + way;
     const int32_t set = (int32_t)(gset - tb.set_base);
@@ -554,11 +554,11 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
     int32_t tag = s.tags[slot];
     uint32_t pri = s.ts[slot];
     const bool in_bucket = n <= cap;
-    int32_t c[BUCKET_PER_LANE];
+    int2 c[BUCKET_PER_LANE];                                       // fetched before it is known how many there are: one latency less
 #pragma unroll
     for (int j = 0; j < BUCKET_PER_LANE; ++j) {
-        c[j] = 0x7fffffff;
-        if (in_bucket && way + j * ways < n) c[j] = __ldcg(s.bucket + gset * cap + way + j * ways);
+        c[j] = j * ways < cap ? __ldcg(s.bucket + gset * cap + way + j * ways) : make_int2(0, 0);
+        if (!in_bucket || way + j * ways >= n) c[j].x = 0x7fffffff;
     }
     const int32_t resident = tag;
     if (tag < 0) pri = 0;
@@ -568,9 +568,9 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
         for (int j = 0; j < BUCKET_PER_LANE; ++j) {
             const int live = min(ways, n - j * ways);
             for (int u = 0; u < live; ++u) {
-                const int32_t v = __shfl_sync(gmask, c[j], gbase + u);
+                const int32_t v = __shfl_sync(gmask, c[j].x, gbase + u);
 #pragma unroll
-                for (int i = 0; i < BUCKET_PER_LANE; ++i) place[i] += v < c[i];
+                for (int i = 0; i < BUCKET_PER_LANE; ++i) place[i] += v < c[i].x;
             }
         }
 #pragma unroll
@@ -580,22 +580,22 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
     if (way == 0) s.set_cnt[gset] = 0;                             // every lane has read it; empty again for the next step
     // next `ways` candidates in row order, one per lane: from the sorted bucket, or by walking the table's distinct rows
     int taken = 0, cursor = 0;                                     // candidates handed out; distinct rows walked
-    auto next_batch = [&](int32_t* k) {
+    auto next_batch = [&](int2* k) {
         if (in_bucket) {
-            *k = taken + way < n ? sorted[taken + way] : -1;
+            *k = taken + way < n ? sorted[taken + way] : make_int2(-1, 0);
             const int m = min(ways, n - taken);
             taken += m;
             return m;
         }
         int m = 0;                                                 // found so far; the first `ways` of them wait in `sorted`
-        *k = -1;
+        *k = make_int2(-1, 0);
         while (m < ways && cursor < n_rows) {
             const int i = cursor + way;
             const bool mine = i < n_rows && __ldcg(w.cand_key + ub + i) == set;
             const uint32_t found = (__ballot_sync(gmask, mine) & gmask) >> gbase;
             const int at = m + __popc(found & ((1u << way) - 1u));
             const bool take = mine && at < ways;
-            if (take) sorted[at] = ub + i;
+            if (take) sorted[at] = make_int2(ub + i, w.uniq_row[ub + i]);
             const uint32_t taken_m = (__ballot_sync(gmask, take) & gmask) >> gbase;
             m += __popc(taken_m);
             // a batch that is full ends the walk behind its last candidate
@@ -625,25 +625,26 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
                 const uint32_t v = __shfl_sync(gmask, age, gbase + u);
                 order += ((opens >> u) & 1u) && (v < age || (v == age && u < way));
             }
-            int32_t k;
+            int2 k;
             next_batch(&k);
-            const int32_t mine = __shfl_sync(gmask, k, gbase + min(order, ways - 1));
+            const int32_t mine = __shfl_sync(gmask, k.x, gbase + min(order, ways - 1));
+            const int32_t mrow = __shfl_sync(gmask, k.y, gbase + min(order, ways - 1));
             if (open && order < m) {
                 if (tag >= 0) displace();
-                cand = mine; tag = w.uniq_row[mine]; pri = step;
+                cand = mine; tag = mrow; pri = step;
             }
         }
         const int empties = __popc((__ballot_sync(gmask, resident < 0) & gmask) >> gbase);
         pc.admit = (uint32_t)m; pc.evict = (uint32_t)max(0, m - empties); pc.bypass = (uint32_t)(n - m);
     } else {
         for (int left = n; left > 0;) {
-            int32_t ckk; int32_t crow = 0; uint32_t cpv = step;
-            const int nb = next_batch(&ckk);
+            int2 batch; uint32_t cpv = step;
+            const int nb = next_batch(&batch);
             if (nb == 0) break;
             left -= nb;
             const bool valid = way < nb;
+            const int32_t ckk = batch.x, crow = batch.y;
             if (valid) {
-                crow = w.uniq_row[ckk];
                 if (s.policy == 1) cpv = *count_of(s, tb.row_base + crow);
             }
             // Between two replacements the set does not change, so every candidate that cannot beat the current
@@ -769,7 +770,7 @@ k_priority(State s, Work w, StepArgs a, int list_hot) {
                     // puts a larger value in the place of the lowest, no way is ever emptied), so a row that does not
                     // beat a bound recorded earlier is bypassed whatever happens in this step (Algorithm 2's test).
                     if (!always && pv <= low[q]) bypass = true;
-                    else { ckey = set[q]; lists = bucket_put(s, sbase[q] + set[q], cap, (int32_t)k); }
+                    else { ckey = set[q]; lists = bucket_put(s, sbase[q] + set[q], cap, (int32_t)k, row[q]); }
                 }
                 if (one_table) { m += mult[q]; ++un; if (hit) { hitm += mult[q]; ++uh; } byp += bypass; }
                 else {
@@ -785,7 +786,7 @@ k_priority(State s, Work w, StepArgs a, int list_hot) {
                 uint32_t at = 0;
                 if (lane == 0) at = atomicAdd(&w.ctr->n_heads, (uint32_t)__popc(lm));
                 at = __shfl_sync(0xffffffffU, at, 0) + (uint32_t)__popc(lm & ((1u << lane) - 1u));
-                if (lists) w.heads[at] = (int32_t)k;
+                if (lists) w.heads[at] = make_int2((int32_t)(sbase[q] + set[q]), t[q]);
             }
         }
         if (one_table) {
@@ -803,10 +804,10 @@ k_priority(State s, Work w, StepArgs a, int list_hot) {
     }
 }
 
-// every set that has candidates (w.heads: the first candidate each of them got)
+// every set that has candidates
 __global__ void __launch_bounds__(256)
 k_policy(State s, Work w, StepArgs a) {
-    __shared__ int32_t scratch[256 * BUCKET_PER_LANE];             // a group of `ways` lanes has bucket_cap(ways) <= BUCKET_PER_LANE * ways words
+    __shared__ int2 scratch[256 * BUCKET_PER_LANE];                // a group of `ways` lanes has bucket_cap(ways) <= BUCKET_PER_LANE * ways pairs
     if (w.ctr->abort) return;
     const int ways = s.ways, cap = bucket_cap(ways);
     const int lane = threadIdx.x & 31, way = lane & (ways - 1), gbase = lane & ~(ways - 1);
@@ -815,11 +816,11 @@ k_policy(State s, Work w, StepArgs a) {
     const int grp = threadIdx.x / ways;
     const int64_t gpb = blockDim.x / ways, ng = gpb * gridDim.x;
     for (int64_t h = blockIdx.x * gpb + grp; h < nheads; h += ng) {
-        const int32_t k = w.heads[h];
-        const int t = w.uniq_t[k];
+        const int2 head = w.heads[h];
+        const int t = head.y;
         const TableDev tb = s.tables[t];
         const int32_t ub = w.ustart[t];
-        const PolicyCounts pc = policy_set(s, w, tb, tb.set_base + w.cand_key[k], ub, w.ustart[t + 1] - ub, (uint32_t)a.step, a.epoch, gmask,
+        const PolicyCounts pc = policy_set(s, w, tb, head.x, ub, w.ustart[t + 1] - ub, (uint32_t)a.step, a.epoch, gmask,
                                            gbase, way, scratch + grp * cap);
         if (way == 0) {
             unsigned long long* st = s.stats + (int64_t)t * 8;
@@ -1354,20 +1355,34 @@ k_flush(State s, int64_t total_slots, uint64_t step) {
     }
 }
 
-__global__ void k_gather_rows(State s, int t, const int64_t* __restrict__ rows, int64_t n, int code_bytes,
-                              uint8_t* __restrict__ codes, float* __restrict__ scale, float* __restrict__ bias,
-                              uint32_t* __restrict__ cnt, float* __restrict__ G) {
+// Rows named by the caller -> contiguous arrays (zeros for a row outside the table): the codes, moved in words of V, and
+// what goes with them.
+template <class V>
+__global__ void __launch_bounds__(256)
+k_gather_codes(State s, int t, const int64_t* __restrict__ rows, int64_t n, int words, V* __restrict__ codes) {
+    const TableDev tb = s.tables[t];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n * words; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = rows[i / words];
+        V v{};
+        if (r >= 0 && r < tb.N) v = reinterpret_cast<const V*>(s.codes)[(tb.row_base + r) * words + i % words];
+        codes[i] = v;
+    }
+}
+__global__ void __launch_bounds__(256)
+k_gather_scalars(State s, int t, const int64_t* __restrict__ rows, int64_t n, float* __restrict__ scale, float* __restrict__ bias,
+                 uint32_t* __restrict__ cnt, float* __restrict__ G) {
     const TableDev tb = s.tables[t];
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = rows[i];
-        if (r < 0 || r >= tb.N) continue;
-        const int64_t g = tb.row_base + r;
-        if (codes) {
-            for (int c = 0; c < code_bytes; ++c) codes[i * code_bytes + c] = s.codes[g * code_bytes + c];
-            scale[i] = s.sb ? s.sb[g].x : 1.0f; bias[i] = s.sb ? s.sb[g].y : 0.0f;
+        const bool ok = r >= 0 && r < tb.N;
+        const int64_t g = tb.row_base + (ok ? r : 0);
+        if (scale) {
+            float2 p = make_float2(0.0f, 0.0f);
+            if (ok) p = s.sb ? s.sb[g] : make_float2(1.0f, 0.0f);
+            scale[i] = p.x; bias[i] = p.y;
         }
-        if (cnt) cnt[i] = s.policy == 1 ? *count_of(s, g) : 0u;
-        if (G) G[i] = s.G ? s.G[g] : 0.0f;
+        if (cnt) cnt[i] = ok && s.policy == 1 ? *count_of(s, g) : 0u;
+        if (G) G[i] = ok && s.G ? s.G[g] : 0.0f;
     }
 }
 

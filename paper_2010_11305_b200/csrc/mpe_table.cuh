@@ -383,7 +383,7 @@ __device__ uint32_t table_unique(TableShared& sh, const State& s, const Work& w,
 // (One block.)  Where the table's distinct rows live, their new priority values, the candidates for admission in their sets' buckets, the hot
 // rows' tasks; then the admission test for every set that has candidates.
 template <int BATCH>
-__device__ void table_state(TableShared& sh, int32_t* scratch, const State& s, const Work& w, const TableJob& job, uint32_t ubase, uint32_t U,
+__device__ void table_state(TableShared& sh, int2* scratch, const State& s, const Work& w, const TableJob& job, uint32_t ubase, uint32_t U,
                             uint32_t step, uint32_t epoch) {
     const int lane = threadIdx.x & 31;
     const TableDev tb = s.tables[job.t];
@@ -437,7 +437,7 @@ __device__ void table_state(TableShared& sh, int32_t* scratch, const State& s, c
                     } else if (tb.n_sets > 0) {
                         // the early bypass: see k_priority
                         if (!always && pv <= low[j]) ++n_byp;
-                        else { ckey = set[j]; lists = bucket_put(s, tb.set_base + set[j], cap, (int32_t)k); }
+                        else { ckey = set[j]; lists = bucket_put(s, tb.set_base + set[j], cap, (int32_t)k, row[j]); }
                     }
                     list_long_row(w, (int32_t)k, mult[j], hot_min);
                 }
@@ -449,7 +449,7 @@ __device__ void table_state(TableShared& sh, int32_t* scratch, const State& s, c
                 uint32_t at = 0;
                 if (lane == __ffs(lm) - 1) at = atomicAdd(&sh.n_heads, (uint32_t)__popc(lm));
                 at = __shfl_sync(0xffffffffU, at, __ffs(lm) - 1);
-                if (lists) w.heads[ubase + at + (uint32_t)__popc(lm & ((1u << lane) - 1u))] = set[j];
+                if (lists) w.heads[ubase + at + (uint32_t)__popc(lm & ((1u << lane) - 1u))] = make_int2((int32_t)(tb.set_base + set[j]), job.t);
             }
         }
     }
@@ -468,8 +468,7 @@ __device__ void table_state(TableShared& sh, int32_t* scratch, const State& s, c
         const uint32_t gpb = TBL_THREADS / (uint32_t)ways, grp = threadIdx.x / (uint32_t)ways;
         uint32_t n_admit = 0, n_evict = 0, n_more = 0;
         for (uint32_t h = grp; h < heads; h += gpb) {
-            const int32_t set = __ldcg(w.heads + ubase + h);
-            const PolicyCounts pc = policy_set(s, w, tb, tb.set_base + set, (int32_t)ubase, (int32_t)U, step, epoch, gmask, gbase, way,
+            const PolicyCounts pc = policy_set(s, w, tb, __ldcg(w.heads + ubase + h).x, (int32_t)ubase, (int32_t)U, step, epoch, gmask, gbase, way,
                                                scratch + grp * cap);
             n_admit += pc.admit; n_evict += pc.evict; n_more += pc.bypass;
             __syncwarp(gmask);
@@ -544,7 +543,7 @@ k_table(State s, Work w, uint2* __restrict__ records, uint2* __restrict__ spill,
     cluster_sync(job.blocks);                                  // the lists are complete
     finished();
     if (!ok) return;
-    if (STATE) table_state<2>(sh, reinterpret_cast<int32_t*>(buf), s, w, job, ubase, U, step, epoch);
+    if (STATE) table_state<2>(sh, reinterpret_cast<int2*>(buf), s, w, job, ubase, U, step, epoch);
 }
 
 }  // namespace mpe
