@@ -58,9 +58,18 @@ __device__ __forceinline__ uint32_t ld_once_u32(const void* p) { uint32_t v; asm
 __device__ __forceinline__ uint2 ld_once_u32x2(const void* p) { uint2 v; asm("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p)); return v; }
 __device__ __forceinline__ float2 ld_once_f32x2(const void* p) { float2 v; asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p)); return v; }
 
+// Where the low-precision rows are: codes and (scale, bias) of row r at codes + r * code_stride and sb + r * sb_stride.  On the GPU
+// both usually are parts of one record per row (see mpe_create_placed).
+struct LowRows {
+    uint8_t *codes, *sb;
+    uint32_t code_stride, sb_stride;
+    __host__ __device__ uint8_t* codes_of(int64_t r) const { return codes + r * (int64_t)code_stride; }
+    __host__ __device__ float2* sb_of(int64_t r) const { return reinterpret_cast<float2*>(sb + r * (int64_t)sb_stride); }
+};
+
 template <int BITS, bool RO>
-__device__ __forceinline__ uint2 load_codes4(const uint8_t* codes, int64_t grow, int dim, int sub) {
-    const uint8_t* row = codes + grow * (dim * BITS / 8);
+__device__ __forceinline__ uint2 load_codes4(const LowRows& low, int64_t grow, int sub) {
+    const uint8_t* row = low.codes_of(grow);
     if (BITS == 16) return RO ? ld_once_u32x2(reinterpret_cast<const uint2*>(row) + sub) : reinterpret_cast<const uint2*>(row)[sub];
     uint32_t q;
     if (BITS == 8) q = RO ? ld_once_u32(reinterpret_cast<const uint32_t*>(row) + sub) : reinterpret_cast<const uint32_t*>(row)[sub];
@@ -69,8 +78,8 @@ __device__ __forceinline__ uint2 load_codes4(const uint8_t* codes, int64_t grow,
     return make_uint2(q, 0u);
 }
 template <int BITS>
-__device__ __forceinline__ void store_packed4(uint8_t* codes, int64_t grow, int dim, int sub, uint32_t q) {
-    uint8_t* row = codes + grow * (dim * BITS / 8);
+__device__ __forceinline__ void store_packed4(const LowRows& low, int64_t grow, int sub, uint32_t q) {
+    uint8_t* row = low.codes_of(grow);
     if (BITS == 8) reinterpret_cast<uint32_t*>(row)[sub] = q;
     else if (BITS == 4) reinterpret_cast<uint16_t*>(row)[sub] = (uint16_t)q;
     else row[sub] = (uint8_t)q;
@@ -113,10 +122,10 @@ __device__ __forceinline__ float4 decode4(uint2 qq, float2 p) {
 
 // RO = the table is not written by the running kernel, so the read-only data path may serve the loads
 template <int BITS, bool RO>
-__device__ __forceinline__ float4 dequant4(const uint8_t* codes, const float2* sb, int64_t grow, int dim, int sub) {
+__device__ __forceinline__ float4 dequant4(const LowRows& low, int64_t grow, int sub) {
     float2 p = make_float2(1.0f, 0.0f);
-    if (BITS != 16) p = RO ? ld_once_f32x2(sb + grow) : sb[grow];
-    return decode4<BITS>(load_codes4<BITS, RO>(codes, grow, dim, sub), p);
+    if (BITS != 16) p = RO ? ld_once_f32x2(low.sb_of(grow)) : *low.sb_of(grow);
+    return decode4<BITS>(load_codes4<BITS, RO>(low, grow, sub), p);
 }
 
 // Four values -> their codes, packed with the first in the lowest bits; `stochastic` picks the rounding of Section 3 "Rounding" (it
@@ -161,11 +170,10 @@ __device__ __forceinline__ uint32_t half1(float x, uint32_t key, uint32_t column
 
 // Down-convert one FP32 row (four columns per lane) into the low-precision table.
 template <int BITS>
-__device__ __forceinline__ void quantize_store(float4 x, uint8_t* __restrict__ codes, float2* __restrict__ sb,
-                                               int64_t grow, int dim, int sub, int lanes_per_row, uint32_t key, bool stochastic) {
+__device__ __forceinline__ void quantize_store(float4 x, const LowRows& low, int64_t grow, int sub, int lanes_per_row, uint32_t key, bool stochastic) {
     if (BITS == 16) {       // FP16 table: element-wise, no scale or bias
         const uint32_t c = 4u * (uint32_t)sub;
-        reinterpret_cast<uint2*>(codes + grow * (dim * 2))[sub] =
+        reinterpret_cast<uint2*>(low.codes_of(grow))[sub] =
             make_uint2(half1(x.x, key, c, stochastic) | (half1(x.y, key, c + 1, stochastic) << 16),
                        half1(x.z, key, c + 2, stochastic) | (half1(x.w, key, c + 3, stochastic) << 16));
         return;
@@ -184,8 +192,8 @@ __device__ __forceinline__ void quantize_store(float4 x, uint8_t* __restrict__ c
     if (s >= 1.17549435e-38f) inv = __fdiv_rn(1.0f, s);
     if (inv == 0.0f) s = 0.0f;
     const uint32_t c = 4u * (uint32_t)sub;
-    store_packed4<BITS>(codes, grow, dim, sub, quant_pack<BITS & 15>(x, mn, inv, key, c, stochastic));
-    if (sub == 0) sb[grow] = make_float2(s, mn);
+    store_packed4<BITS>(low, grow, sub, quant_pack<BITS & 15>(x, mn, inv, key, c, stochastic));
+    if (sub == 0) *low.sb_of(grow) = make_float2(s, mn);
 }
 
 }  // namespace mpe

@@ -57,14 +57,12 @@ struct State {
     uint64_t seed;
     float eps;
     const TableDev* tables;
-    uint8_t* codes;        // [sum N][dim*bits/8]
-    float2* sb;            // [sum N] (scale, bias)
+    LowRows low;           // [sum N] codes, (scale, bias)
     float* G;              // Adagrad: [sum N]
     float* slab;           // [slots][dim]
     int32_t* tags;         // [slots], -1 empty
-    int32_t* home;         // per row: its cache slot, or LOC_MISS (the inverse of tags); LFU: {slot, access count} in one 8-byte
-                           // record, so that a row's slot and count are one memory access
-    int home_shift;        // 0, or 1 where a record holds the count too
+    uint8_t* home;         // per row: its cache slot, or LOC_MISS (the inverse of tags), and under LFU its access count behind it, so that
+    uint32_t home_stride;  // both are one memory access; row r at home + r * home_stride
     uint32_t* ts;          // [slots] priority value of the resident row: LRU time stamp, or a copy of its LFU count
     uint32_t* hit_epoch;   // [slots] forward call in which the slot was last hit
     int32_t* hit_k;        // [slots] unique-row index of that hit
@@ -74,8 +72,8 @@ struct State {
     unsigned long long* stats;   // [T][8]
 };
 
-__device__ __forceinline__ int32_t* slot_of(const State& s, int64_t row) { return s.home + (row << s.home_shift); }
-__device__ __forceinline__ uint32_t* count_of(const State& s, int64_t row) { return reinterpret_cast<uint32_t*>(s.home + 2 * row + 1); }   // LFU
+__device__ __forceinline__ int32_t* slot_of(const State& s, int64_t row) { return reinterpret_cast<int32_t*>(s.home + row * (int64_t)s.home_stride); }
+__device__ __forceinline__ uint32_t* count_of(const State& s, int64_t row) { return reinterpret_cast<uint32_t*>(slot_of(s, row) + 1); }   // LFU
 
 // Destination of the pooled vectors when the tables are partitioned over several GPUs (Section 1: model parallelism
 // with no replication): sample b belongs to rank b / B_local, whose buffer is [B_local][T_global * dim].
@@ -328,7 +326,7 @@ __device__ __forceinline__ float4 fetch4(const State& s, const TableDev& tb, int
         const float4* src = reinterpret_cast<const float4*>(s.slab + (int64_t)loc * s.dim) + sub;
         return RO ? __ldg(src) : *src;
     }
-    return dequant4<BITS, RO>(s.codes, s.sb, tb.row_base + row, s.dim, sub);
+    return dequant4<BITS, RO>(s.low, tb.row_base + row, sub);
 }
 
 // What a forward leaves behind besides the pooled vectors.
@@ -450,7 +448,7 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
                 x = __ldg(reinterpret_cast<const float4*>(slab_col + (size_t)(uint32_t)lc * (size_t)(dim * 4)));
             } else if (lc == LOC_MISS) {
                 const int32_t rw = __shfl_sync(gmask, myrow, gbase + src_lane);
-                x = dequant4<BITS, true>(s.codes, s.sb, row_base + rw, dim, sub);
+                x = dequant4<BITS, true>(s.low, row_base + rw, sub);
             }
             return x;
         };
@@ -543,44 +541,63 @@ __device__ __forceinline__ bool bucket_put(const State& s, int64_t gset, int cap
 
 struct PolicyCounts { uint32_t admit, evict, bypass; };
 
+// ascending over the group's lanes (a power of two of them); `extra` goes with its key
+template <int WAYS>
+__device__ __forceinline__ void group_sort(int32_t& key, int32_t& extra, int ways, int way, uint32_t gmask) {
+#pragma unroll
+    for (int k = 2; k <= (WAYS ? WAYS : 32); k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (!WAYS && k > ways) continue;
+            const int32_t ok = __shfl_xor_sync(gmask, key, j), oe = __shfl_xor_sync(gmask, extra, j);
+            const bool low = (way & j) == 0, up = (way & k) == 0;
+            if (low == up ? ok < key : ok > key) { key = ok; extra = oe; }
+        }
+}
+
 // One set.  All lanes of the group (`gmask`, first lane `gbase`) take part; `sorted` is the group's own piece of shared memory,
 // bucket_cap(ways) pairs.  The table's distinct rows are [ub, ub + n_rows).
+template <int WAYS>          // the number of ways, 0 if it is to be read from the state
 __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w, const TableDev& tb, int64_t gset, int32_t ub, int32_t n_rows,
                                                    uint32_t step, uint32_t epoch, uint32_t gmask, int gbase, int way, int2* sorted) {
-    const int ways = s.ways, cap = bucket_cap(ways);
+    const int ways = WAYS ? WAYS : s.ways, cap = bucket_cap(ways);
+    constexpr int PER_LANE = WAYS >= 8 ? 2 : BUCKET_PER_LANE;
     const int64_t slot = gset * ways + way;
     const int32_t set = (int32_t)(gset - tb.set_base);
     const int n = (int)__ldcg(s.set_cnt + gset);                   // candidates
     int32_t tag = s.tags[slot];
     uint32_t pri = s.ts[slot];
     const bool in_bucket = n <= cap;
-    int2 c[BUCKET_PER_LANE];                                       // fetched before it is known how many there are: one latency less
+    int2 c[PER_LANE];                                       // fetched before it is known how many there are: one latency less
 #pragma unroll
-    for (int j = 0; j < BUCKET_PER_LANE; ++j) {
+    for (int j = 0; j < PER_LANE; ++j) {
         c[j] = j * ways < cap ? __ldcg(s.bucket + gset * cap + way + j * ways) : make_int2(0, 0);
         if (!in_bucket || way + j * ways >= n) c[j].x = 0x7fffffff;
     }
     const int32_t resident = tag;
     if (tag < 0) pri = 0;
-    if (in_bucket) {                                               // distinct rows are numbered in row order: a candidate's place is the number of smaller ones
-        int place[BUCKET_PER_LANE] = {};
+    const bool one_batch = n <= ways;                              // the usual case: sorted in registers
+    if (one_batch) group_sort<WAYS>(c[0].x, c[0].y, ways, way, gmask);
+    else if (in_bucket) {                                          // distinct rows are numbered in row order: a candidate's place is the number of smaller ones
+        int place[PER_LANE] = {};
 #pragma unroll
-        for (int j = 0; j < BUCKET_PER_LANE; ++j) {
-            const int live = min(ways, n - j * ways);
+        for (int j = 0; j < PER_LANE; ++j) {
+            const int live = min(ways, n - j * ways);              // none for the places a set's bucket does not have
             for (int u = 0; u < live; ++u) {
                 const int32_t v = __shfl_sync(gmask, c[j].x, gbase + u);
 #pragma unroll
-                for (int i = 0; i < BUCKET_PER_LANE; ++i) place[i] += v < c[i].x;
+                for (int i = 0; i < PER_LANE; ++i) place[i] += v < c[i].x;
             }
         }
 #pragma unroll
-        for (int j = 0; j < BUCKET_PER_LANE; ++j) if (way + j * ways < n) sorted[place[j]] = c[j];
+        for (int j = 0; j < PER_LANE; ++j) if (way + j * ways < n) sorted[place[j]] = c[j];
     }
     __syncwarp(gmask);
     if (way == 0) s.set_cnt[gset] = 0;                             // every lane has read it; empty again for the next step
     // next `ways` candidates in row order, one per lane: from the sorted bucket, or by walking the table's distinct rows
     int taken = 0, cursor = 0;                                     // candidates handed out; distinct rows walked
     auto next_batch = [&](int2* k) {
+        if (one_batch) { *k = way < n ? c[0] : make_int2(-1, 0); taken = n; return n; }
         if (in_bucket) {
             *k = taken + way < n ? sorted[taken + way] : make_int2(-1, 0);
             const int m = min(ways, n - taken);
@@ -621,9 +638,24 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
         const int m = min(n, __popc(opens));
         int order = 0;
         if (m > 0) {
-            for (int u = 0; u < ways; ++u) {
-                const uint32_t v = __shfl_sync(gmask, age, gbase + u);
-                order += ((opens >> u) & 1u) && (v < age || (v == age && u < way));
+            // the place of this way among those that are open, by (age, way): sorted as one number per way while the ages, counted
+            // back from this step, leave room for the way in 32 bits, which is anything but a row untouched for 2^26 steps
+            const uint32_t back = !open ? 0u : tag < 0 ? 0x03ffffffu : step - pri;         // 1 = touched in the step before
+            if (__all_sync(gmask, tag < 0 || back < 0x03ffffffu)) {
+                int32_t key = open ? (int32_t)(((0x03ffffffu - back) << 5) | (uint32_t)way) : 0x7fffffff, whose = way;
+                group_sort<WAYS>(key, whose, ways, way, gmask);    // lane i: the way that is i-th
+                uint32_t at = 0xffffffffu;                         // and back: which place has this way?  (bit by bit)
+#pragma unroll
+                for (int o = 0; o < 5; ++o) {
+                    const uint32_t lanes = (__ballot_sync(gmask, (whose >> o) & 1) & gmask) >> gbase;
+                    at &= ((way >> o) & 1) ? lanes : ~lanes;
+                }
+                order = __ffs((int)(at & (gmask >> gbase))) - 1;
+            } else {
+                for (int u = 0; u < ways; ++u) {
+                    const uint32_t v = __shfl_sync(gmask, age, gbase + u);
+                    order += ((opens >> u) & 1u) && (v < age || (v == age && u < way));
+                }
             }
             int2 k;
             next_batch(&k);
@@ -805,11 +837,12 @@ k_priority(State s, Work w, StepArgs a, int list_hot) {
 }
 
 // every set that has candidates
+template <int WAYS>
 __global__ void __launch_bounds__(256)
 k_policy(State s, Work w, StepArgs a) {
-    __shared__ int2 scratch[256 * BUCKET_PER_LANE];                // a group of `ways` lanes has bucket_cap(ways) <= BUCKET_PER_LANE * ways pairs
+    __shared__ int2 scratch[256 / WAYS * bucket_cap(WAYS)];
     if (w.ctr->abort) return;
-    const int ways = s.ways, cap = bucket_cap(ways);
+    constexpr int ways = WAYS, cap = bucket_cap(WAYS);
     const int lane = threadIdx.x & 31, way = lane & (ways - 1), gbase = lane & ~(ways - 1);
     const uint32_t gmask = group_mask(ways);
     const int64_t nheads = w.ctr->n_heads;
@@ -820,7 +853,7 @@ k_policy(State s, Work w, StepArgs a) {
         const int t = head.y;
         const TableDev tb = s.tables[t];
         const int32_t ub = w.ustart[t];
-        const PolicyCounts pc = policy_set(s, w, tb, head.x, ub, w.ustart[t + 1] - ub, (uint32_t)a.step, a.epoch, gmask,
+        const PolicyCounts pc = policy_set<WAYS>(s, w, tb, head.x, ub, w.ustart[t + 1] - ub, (uint32_t)a.step, a.epoch, gmask,
                                            gbase, way, scratch + grp * cap);
         if (way == 0) {
             unsigned long long* st = s.stats + (int64_t)t * 8;
@@ -937,6 +970,13 @@ __device__ __forceinline__ float4 hot_task_sum(const State& s, const Work& w, co
     return acc;
 }
 
+// merged gradient of a hot row from its tasks' sums (this lane's four columns of them), which other blocks may just have written
+template <int LANES>
+__device__ __forceinline__ float4 hot_row_sum(const float* part, int32_t m) {
+    auto term = [&](int64_t j) { return __ldcg(reinterpret_cast<const float4*>(part + j * 4 * LANES)); };
+    return tree_reduce<4>(term, 0, (m + HOT_SPAN - 1) / HOT_SPAN);
+}
+
 // the hot rows' tasks -> their partial sums
 template <int LANES>
 __global__ void __launch_bounds__(HOT_THREADS, 2)
@@ -974,11 +1014,11 @@ __device__ __forceinline__ void apply_update(const State& s, const TableDev& tb,
     if (floc >= 0) {
         float4* dst = reinterpret_cast<float4*>(s.slab + (int64_t)floc * dim) + sub;
         if (loc < 0 && victim >= 0)     // the row this newcomer displaces is down-converted and placed back in T
-            quantize_store<BITS>(*dst, s.codes, s.sb, tb.row_base + victim, dim, sub, LANES,
+            quantize_store<BITS>(*dst, s.low, tb.row_base + victim, sub, LANES,
                                 rowkey(s.seed, DOMAIN_SR, (uint32_t)t, (uint32_t)victim, step), s.rounding != 0);
         *dst = xn;                      // cached rows keep full precision, a newcomer enters verbatim
     } else {
-        quantize_store<BITS>(xn, s.codes, s.sb, grow, dim, sub, LANES,
+        quantize_store<BITS>(xn, s.low, grow, sub, LANES,
                             rowkey(s.seed, DOMAIN_SR, (uint32_t)t, (uint32_t)row, step), s.rounding != 0);
     }
 }
@@ -1057,8 +1097,10 @@ k_update(State s, Work w, StepArgs a) {
 #pragma unroll
                         for (int o = 0; o < dim * 4; o += 128) prefetch_l2(src + o);
                     } else {
-                        prefetch_l2(s.codes + grow * (dim * BITS / 8));
-                        if (BITS != 16) prefetch_l2(s.sb + grow);
+                        const uint8_t* src = s.low.codes_of(grow);
+                        prefetch_l2(src);
+                        if (dim * BITS / 8 > 16) prefetch_l2(src + dim * BITS / 8 - 1);          // a row can straddle two lines
+                        if (BITS != 16) prefetch_l2(s.low.sb_of(grow));
                     }
                     if (victim >= 0) {
                         const int64_t vrow = rb + victim;
@@ -1083,9 +1125,9 @@ k_update(State s, Work w, StepArgs a) {
                 raw = reinterpret_cast<const uint4*>(s.slab + (int64_t)A.x * dim)[sub];
             } else {
                 const int64_t grow = ((int64_t)A.w << 32) | (uint32_t)A.z;
-                const uint2 q = load_codes4<BITS, false>(s.codes, grow, dim, sub);
+                const uint2 q = load_codes4<BITS, false>(s.low, grow, sub);
                 raw.x = q.x; raw.y = q.y;
-                if (BITS != 16) { const float2 sb = s.sb[grow]; raw.z = __float_as_uint(sb.x); raw.w = __float_as_uint(sb.y); }
+                if (BITS != 16) { const float2 sb = *s.low.sb_of(grow); raw.z = __float_as_uint(sb.x); raw.w = __float_as_uint(sb.y); }
             }
             const int4 D = recs[r * 4 + 3];
             const char* col = gcol + (size_t)(uint32_t)recs[r * 4 + 2].w * 4u;
@@ -1165,11 +1207,11 @@ k_update(State s, Work w, StepArgs a) {
                 if (loc < 0 && B.w >= 0) {           // the row this newcomer displaces is down-converted and placed back in T
                     const int4 C = recs[r * 4 + 2];
                     const int64_t vrow = ((int64_t)C.z << 32) | (uint32_t)C.y;
-                    quantize_store<BITS>(*dst, s.codes, s.sb, vrow, dim, sub, LANES, (uint32_t)C.x, s.rounding != 0);
+                    quantize_store<BITS>(*dst, s.low, vrow, sub, LANES, (uint32_t)C.x, s.rounding != 0);
                 }
                 *dst = xn;                           // cached rows keep full precision, a newcomer enters verbatim
             } else {
-                quantize_store<BITS>(xn, s.codes, s.sb, grow, dim, sub, LANES, (uint32_t)B.x, s.rounding != 0);
+                quantize_store<BITS>(xn, s.low, grow, sub, LANES, (uint32_t)B.x, s.rounding != 0);
             }
         }
         __syncwarp();                                          // the records are rewritten by the next block
@@ -1211,9 +1253,7 @@ k_update_list(State s, Work w, const int32_t* __restrict__ list, const uint32_t*
             for (int32_t c = 32; c < m; c += 32)
                 g = add4(g, sum_chunk<LANES>(w.occ_b, gcol, stride_bytes, first + c, min(32, m - c), gmask, gbase, sub));
         } else {
-            const float* part = w.partial + (int64_t)w.hot_base[k] * dim + 4 * sub;
-            auto term = [&](int64_t j) { return *reinterpret_cast<const float4*>(part + j * dim); };
-            g = tree_reduce<4>(term, 0, (m + HOT_SPAN - 1) / HOT_SPAN);
+            g = hot_row_sum<LANES>(w.partial + (int64_t)w.hot_base[k] * dim + 4 * sub, m);
         }
         apply_update<BITS, LANES>(s, tb, t, row, loc, floc, victim, g, x, lr, step, sub, gmask);
     }
@@ -1237,11 +1277,7 @@ k_update_small(State s, Work w, StepArgs a) {
     const uint32_t ntask = w.ctr->hot_tasks;
     const uint32_t items = ntask + (w.ctr->U + ngrp - 1) / ngrp;
     const uint32_t stride_bytes = (uint32_t)s.T * (uint32_t)dim * 4u;
-    auto tree = [&](int32_t k, int32_t m) {                // merged gradient of a hot row from its tasks' sums
-        const float* part = w.partial + (int64_t)w.hot_base[k] * dim + 4 * sub;
-        auto term = [&](int64_t j) { return __ldcg(reinterpret_cast<const float4*>(part + j * dim)); };
-        return tree_reduce<4>(term, 0, (m + HOT_SPAN - 1) / HOT_SPAN);
-    };
+    auto tree = [&](int32_t k, int32_t m) { return hot_row_sum<LANES>(w.partial + (int64_t)w.hot_base[k] * dim + 4 * sub, m); };
     auto merged = [&](int32_t k, int t, int32_t first, int32_t m) {       // ... of any other row
         const char* gcol = reinterpret_cast<const char*>(a.grad + (int64_t)t * dim + 4 * sub);
         float4 g = sum_chunk<LANES>(w.occ_b, gcol, stride_bytes, first, min(32, m), gmask, gbase, sub);
@@ -1316,7 +1352,7 @@ __global__ void k_init_table(State s, int t, float lo, float hi) {
         x.y = __fmaf_rn(uniform01(key, 4 * sub + 1), width, lo);
         x.z = __fmaf_rn(uniform01(key, 4 * sub + 2), width, lo);
         x.w = __fmaf_rn(uniform01(key, 4 * sub + 3), width, lo);
-        quantize_store<BITS>(x, s.codes, s.sb, tb.row_base + row, s.dim, sub, lanes, 0u, false);
+        quantize_store<BITS>(x, s.low, tb.row_base + row, sub, lanes, 0u, false);
     }
 }
 
@@ -1349,7 +1385,7 @@ k_flush(State s, int64_t total_slots, uint64_t step) {
                 if (s.tables[mid].set_base <= set) lo = mid; else hi = mid;
             }
             const int t = lo;
-            quantize_store<BITS>(x[q], s.codes, s.sb, s.tables[t].row_base + tag[q], s.dim, sub, lanes,
+            quantize_store<BITS>(x[q], s.low, s.tables[t].row_base + tag[q], sub, lanes,
                                  rowkey(s.seed, DOMAIN_FLUSH, (uint32_t)t, (uint32_t)tag[q], step), s.rounding != 0);
         }
     }
@@ -1364,7 +1400,7 @@ k_gather_codes(State s, int t, const int64_t* __restrict__ rows, int64_t n, int 
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n * words; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = rows[i / words];
         V v{};
-        if (r >= 0 && r < tb.N) v = reinterpret_cast<const V*>(s.codes)[(tb.row_base + r) * words + i % words];
+        if (r >= 0 && r < tb.N) v = reinterpret_cast<const V*>(s.low.codes_of(tb.row_base + r))[i % words];
         codes[i] = v;
     }
 }
@@ -1378,7 +1414,7 @@ k_gather_scalars(State s, int t, const int64_t* __restrict__ rows, int64_t n, fl
         const int64_t g = tb.row_base + (ok ? r : 0);
         if (scale) {
             float2 p = make_float2(0.0f, 0.0f);
-            if (ok) p = s.sb ? s.sb[g] : make_float2(1.0f, 0.0f);
+            if (ok) p = s.low.sb ? *s.low.sb_of(g) : make_float2(1.0f, 0.0f);
             scale[i] = p.x; bias[i] = p.y;
         }
         if (cnt) cnt[i] = ok && s.policy == 1 ? *count_of(s, g) : 0u;

@@ -468,7 +468,7 @@ __device__ void table_state(TableShared& sh, int2* scratch, const State& s, cons
         const uint32_t gpb = TBL_THREADS / (uint32_t)ways, grp = threadIdx.x / (uint32_t)ways;
         uint32_t n_admit = 0, n_evict = 0, n_more = 0;
         for (uint32_t h = grp; h < heads; h += gpb) {
-            const PolicyCounts pc = policy_set(s, w, tb, __ldcg(w.heads + ubase + h).x, (int32_t)ubase, (int32_t)U, step, epoch, gmask, gbase, way,
+            const PolicyCounts pc = policy_set<0>(s, w, tb, __ldcg(w.heads + ubase + h).x, (int32_t)ubase, (int32_t)U, step, epoch, gmask, gbase, way,
                                                scratch + grp * cap);
             n_admit += pc.admit; n_evict += pc.evict; n_more += pc.bypass;
             __syncwarp(gmask);
