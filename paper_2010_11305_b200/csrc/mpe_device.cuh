@@ -58,6 +58,13 @@ __device__ __forceinline__ uint32_t ld_once_u32(const void* p) { uint32_t v; asm
 __device__ __forceinline__ uint2 ld_once_u32x2(const void* p) { uint2 v; asm("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p)); return v; }
 __device__ __forceinline__ float2 ld_once_f32x2(const void* p) { float2 v; asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p)); return v; }
 
+// First statement of every kernel that is launched by LAUNCH_NEXT: lets the kernel behind it in the stream be set up from now on,
+// and waits until the one before it has finished and its writes are visible.  Nothing of memory may be touched before.
+__device__ __forceinline__ void after_previous_kernel() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Where the low-precision rows are: codes and (scale, bias) of row r at codes + r * code_stride and sb + r * sb_stride.  On the GPU
 // both usually are parts of one record per row (see mpe_create_placed).
 struct LowRows {

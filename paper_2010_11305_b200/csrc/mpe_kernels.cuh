@@ -387,6 +387,7 @@ __device__ __forceinline__ void forward_close(const State& s, const Work& w, con
 template <int BITS, int LANES, int MODE>
 __global__ void __launch_bounds__(256, 4)
 k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
+    after_previous_kernel();
     const int32_t* __restrict__ indices = a.indices;
     const int32_t* __restrict__ offsets = a.offsets;
     float* __restrict__ out = a.out;
@@ -739,6 +740,7 @@ constexpr int PRI_CHUNK = PRI_Q * 256;   // rows per block and round
 __global__ void __launch_bounds__(256, 3)
 k_priority(State s, Work w, StepArgs a, int list_hot) {
     __shared__ uint32_t sums[8][5];
+    after_previous_kernel();
     if (w.ctr->abort) return;
     const uint32_t step = (uint32_t)a.step;
     constexpr int Q = PRI_Q;
@@ -1268,6 +1270,7 @@ __global__ void __launch_bounds__(HOT_THREADS, 2)
 k_update_small(State s, Work w, StepArgs a) {
     extern __shared__ float chunk_sums[];
     __shared__ uint32_t s_last;
+    after_previous_kernel();
     if (w.ctr->abort) return;
     constexpr int dim = 4 * LANES, ngrp = HOT_THREADS / LANES;
     const int sub = threadIdx.x & (LANES - 1), grp = threadIdx.x / LANES;

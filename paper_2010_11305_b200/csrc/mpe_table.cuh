@@ -494,6 +494,7 @@ k_table(State s, Work w, uint2* __restrict__ records, uint2* __restrict__ spill,
     extern __shared__ __align__(16) unsigned char table_smem[];
     uint2* buf = reinterpret_cast<uint2*>(table_smem);
     TableShared& sh = *reinterpret_cast<TableShared*>(table_smem + (size_t)ITEMS * TBL_THREADS * sizeof(uint2));
+    after_previous_kernel();
     TableJob job;
     job.blocks = cluster_size(); job.rank = job.blocks == 1 ? 0u : cluster_rank();
     job.t = (int)(blockIdx.x / job.blocks);
