@@ -1,0 +1,109 @@
+"""Each kernel variant at the sizes where it begins, ends or has a remainder, against the CPU oracle.
+
+The library chooses by sizes alone: a thread-block cluster per table sorts a batch (4096 or 12288 elements per block; a table with
+more than its cluster holds goes through global memory) until the tables average over 150000 indices, then grid-wide kernels do; up
+to 131072 indices one launch updates every row; a row's gradient is summed by its group of lanes, by a warp's list of mid rows (from
+16 occurrences) or by whole blocks (from 64 or 256); a cache set finds its candidates in a bucket until that overflows."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2010_11305_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _cfg(num_rows, batch, **kw):
+    base = dict(name="paths", num_rows=num_rows, dim=4, bits=8, cache_fraction=0.05, ways=8, policy=wl.LFU, optimizer=wl.SGD, lr=0.05,
+                batch=batch, bag=("fixed", 1), zipf=[None] * len(num_rows), steps=2, seed=3)
+    base.update(kw)
+    return wl.Config(**base)
+
+
+def _batch(rng, ids, batch, dim):
+    """One batch from a list of ids per table, the ids cut into `batch` bags at random places."""
+    lens = []
+    for x in ids:
+        cuts = np.sort(rng.integers(0, len(x) + 1, batch - 1))
+        lens.append(np.diff(np.concatenate([[0], cuts, [len(x)]])))
+    off = np.concatenate([[0], np.cumsum(np.concatenate(lens))]).astype(np.int32)
+    grad = rng.uniform(-1, 1, (batch, len(ids) * dim)).astype(np.float32)
+    return np.concatenate(ids).astype(np.int32), off, grad
+
+
+def _check(cfg, make_ids, steps=2):
+    from parity_util import compare_state, make_pair
+    h, o = make_pair(cfg)
+    rng = np.random.default_rng(cfg.seed)
+    for step in range(1, steps + 1):
+        idx, off, grad = _batch(rng, make_ids(rng), cfg.batch, cfg.dim)
+        out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, device="cuda")
+        h.forward(torch.from_numpy(idx).cuda(), torch.from_numpy(off).cuda(), cfg.batch, out)
+        ref = o.forward(idx, off, cfg.batch)
+        assert np.array_equal(out.cpu().numpy(), ref), f"step {step}"
+        h.backward(torch.from_numpy(grad).cuda(), cfg.lr, step)
+        o.backward(grad, cfg.lr, step)
+    assert h.last_error() == (0, 0)
+    compare_state(h, o, cfg, range(cfg.num_tables), rng)
+    h.close()
+
+
+def _skewed(rng, n_rows, count):
+    return np.minimum((n_rows * rng.random(count) ** 3).astype(np.int64), n_rows - 1)
+
+
+@pytest.mark.parametrize("counts", [
+    (0, 1, 31, 33, 1023, 1025, 3000),           # one block per table, tables without indices among them
+    (3641,), (3642,), (4097,),                  # the last size of one block, the first of two
+    (8000, 10, 0),                              # more than the one block holds
+    (7281,), (7283, 7290), (57000,),            # two, four and sixteen blocks
+    (60000, 5, 5),                              # more than the cluster's blocks hold
+    (5000,) * 99 + (12289,),                    # 12288 elements per block, and one table beyond
+    (100003,), (199000, 900),                   # sixteen large blocks: within, and one table beyond
+    (150000,), (150001,),                       # the last average of the cluster kernel, the first of the grid-wide ones
+    (320000, 7, 0), (1048576 + 9,),             # grid-wide: a few tiles and none, large tiles
+])
+def test_index_work_at_its_boundaries(counts):
+    num_rows = [max(3, c // 3) for c in counts]
+    num_rows[0] = 70001                         # keys of three digits
+    _check(_cfg(num_rows, 16), lambda rng: [_skewed(rng, n, c) for n, c in zip(num_rows, counts)])
+
+
+@pytest.mark.parametrize("total", [131072, 131073])
+def test_one_launch_update_at_its_last_size(total):
+    counts = [total // 36 + (t < total % 36) for t in range(36)]
+    _check(_cfg([9000] * 36, 64, dim=8), lambda rng: [_skewed(rng, 9000, c) for c in counts])
+
+
+@pytest.mark.parametrize("dim,bits,rest,tables", [(4, 8, 300, 1), (64, 4, 400, 3), (128, 16, 300, 1), (4, 8, 140000, 1), (64, 4, 140000, 1),
+                                                  (128, 16, 140000, 1), (4, 8, 1 << 20, 1)])
+def test_rows_with_few_and_many_occurrences(dim, bits, rest, tables):
+    """Multiplicities around every limit of the gradient sums, beside rows that occur once or twice."""
+    times = [1, 2, 15, 16, 17, 31, 32, 33, 63, 64, 65, 255, 256, 257, 1023, 1024, 1025, 2100]
+    hot = np.repeat(np.arange(len(times)), times)
+    cfg = _cfg([900000] * tables, 512, dim=dim, bits=bits, cache_fraction=0.001, optimizer=wl.ROWWISE_ADAGRAD)
+    _check(cfg, lambda rng: [rng.permutation(np.concatenate([hot, rng.integers(100, 900000, rest)])) for _ in range(tables)])
+
+
+@pytest.mark.parametrize("ways", [1, 2, 4, 8, 16, 32])
+@pytest.mark.parametrize("policy", [wl.LRU, wl.LFU])
+@pytest.mark.parametrize("count", [3000, 9000])
+def test_sets_with_few_and_with_too_many_candidates(ways, policy, count):
+    """Per set about half as many candidates as ways, one and a half times, and five times as many; one block per table (which
+    admits by itself) and several."""
+    sizes = [40000, 8000, 2500]
+    cfg = _cfg(sizes, 128, ways=ways, policy=policy, cache_fraction=0.2, dim=8, bits=4)
+    _check(cfg, lambda rng: [_skewed(rng, n, count) for n in sizes], steps=4)
+
+
+@pytest.mark.parametrize("dim,bits,n", [(64, 8, 400001), (4, 2, 5000003)])
+def test_exports_of_many_pieces(dim, bits, n):
+    """More rows than one staging slot takes, in any order and more than once; rows that are whole words, and of one byte."""
+    from parity_util import make_pair
+    cfg = _cfg([300000], 16, dim=dim, bits=bits)
+    h, o = make_pair(cfg)
+    rows = np.random.default_rng(1).integers(0, 300000, n)
+    every = np.arange(300000, dtype=np.int64)
+    for got, ref in zip(h.export_rows(0, rows), o.rows(0, every)):
+        assert np.array_equal(got, ref[rows])
+    h.close()
