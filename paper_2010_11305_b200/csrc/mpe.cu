@@ -497,6 +497,7 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
     if ((rc = dmalloc(h, &s.ts, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.hit_epoch, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.hit_k, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
+    if ((rc = dmalloc(h, &s.chain, h->total_slots, nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.set_cnt, std::max<int64_t>(1, h->total_sets), nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.bucket, h->total_sets * bucket_cap(ways), nullptr)) != MPE_OK) return fail(rc);
     if ((rc = dmalloc(h, &s.floor, std::max<int64_t>(1, h->total_sets), nullptr)) != MPE_OK) return fail(rc);
@@ -512,6 +513,7 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
     CKC(cudaMemset(s.stats, 0, sizeof(unsigned long long) * 8 * num_tables));
     LAUNCH(h, "init_home", k_init_home, grid_for(h, h->total_rows, 256, 8), 256, 0, s, h->total_rows);
     LAUNCH(h, "fill_tags", k_fill_i32, grid_for(h, h->total_slots, 256, 8), 256, 0, s.tags, h->total_slots, -1);
+    LAUNCH(h, "fill_chain", k_fill_i32, grid_for(h, h->total_slots, 256, 8), 256, 0, s.chain, h->total_slots, -1);
     for (int t = 0; t < num_tables; ++t) {
         const int g = grid_for(h, h->tables[t].N, 256 / s.lanes, 8);
         if (bits == 8) LAUNCH(h, "init_table", k_init_table<8>, g, 256, 0, s, t, init_lo, init_hi);
@@ -1114,7 +1116,7 @@ int mpe_destroy(mpe_handle* h) {
     else { cudaFree(s.low.codes); cudaFree(s.low.sb); cudaFree(s.home); }
     cudaFree(h->d_route);
     cudaFree(h->d_tables); cudaFree(s.G); cudaFree(s.slab);
-    cudaFree(s.tags); cudaFree(s.ts); cudaFree(s.hit_epoch); cudaFree(s.hit_k); cudaFree(s.floor); cudaFree(s.set_cnt); cudaFree(s.bucket); cudaFree(s.stats);
+    cudaFree(s.tags); cudaFree(s.ts); cudaFree(s.hit_epoch); cudaFree(s.hit_k); cudaFree(s.floor); cudaFree(s.set_cnt); cudaFree(s.chain); cudaFree(s.bucket); cudaFree(s.stats);
     for (auto& r : h->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (auto e : h->event_pool) cudaEventDestroy(e);
     delete h;

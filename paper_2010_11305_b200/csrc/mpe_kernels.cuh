@@ -66,6 +66,7 @@ struct State {
     uint32_t* ts;          // [slots] priority value of the resident row: LRU time stamp, or a copy of its LFU count
     uint32_t* hit_epoch;   // [slots] forward call in which the slot was last hit
     int32_t* hit_k;        // [slots] unique-row index of that hit
+    int32_t* chain;        // [slots] per set, `ways` lists of the candidates its bucket has no room for; -1 between steps
     uint32_t* set_cnt;     // [sets] candidates for admission dropped into the set's bucket in this step; zero between steps
     int2* bucket;          // [sets][bucket_cap(ways)] their {distinct-row index, row id}
     uint32_t* floor;       // [sets] a lower bound of the lowest priority value among the set's residents (0: none known)
@@ -523,8 +524,9 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
 // in ascending row order and applies Algorithm 2's admission test (a candidate whose priority value does
 // not exceed the lowest one among the residents bypasses, otherwise it takes that resident's place).  No row value is read or
 // written here.
-// A bucket holds twice as many candidates as the set has ways (a few more for narrow sets).  A set with more candidates than that
-// finds them by walking its table's distinct rows, which are in row order, and picking those whose candidate key is the set.
+// A bucket holds twice as many candidates as the set has ways (a few more for narrow sets).  What a bucket has no room for goes into
+// one of `ways` linked lists of the set, so that each lane of the group follows a list of its own; the links stand in `victim`, which
+// the policy writes only afterwards.
 // ---------------------------------------------------------------------------------------------
 constexpr int VICTIM_NONE = -1;       // the way was empty, or the displaced row writes itself back
 constexpr int VICTIM_DEFER = -2;      // the displaced row was hit in this step: the newcomer waits for its write-back
@@ -534,9 +536,10 @@ constexpr int BUCKET_CAP_MAX = 64;
 constexpr int BUCKET_PER_LANE = 4;    // bucket_cap(ways) / ways is at most this
 
 // the candidate k joins the bucket of set `gset`; true if it is the set's first one in this step
-__device__ __forceinline__ bool bucket_put(const State& s, int64_t gset, int cap, int32_t k, int32_t row) {
+__device__ __forceinline__ bool bucket_put(const State& s, const Work& w, int64_t gset, int cap, int32_t k, int32_t row) {
     const uint32_t pos = atomicAdd(s.set_cnt + gset, 1u);
     if (pos < (uint32_t)cap) s.bucket[gset * cap + pos] = make_int2(k, row);
+    else w.victim[k] = atomicExch(s.chain + gset * s.ways + (pos & (uint32_t)(s.ways - 1)), k);
     return pos == 0;
 }
 
@@ -556,11 +559,27 @@ __device__ __forceinline__ void group_sort(int32_t& key, int32_t& extra, int way
         }
 }
 
+// the same for keys alone; MERGE: of keys that already rise and then fall
+template <int WAYS, bool MERGE>
+__device__ __forceinline__ int32_t group_sort_keys(int32_t key, int ways, int way, uint32_t gmask) {
+#pragma unroll
+    for (int k = MERGE && WAYS ? WAYS : 2; k <= (WAYS ? WAYS : 32); k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (!WAYS && (k > ways || (MERGE && k < ways))) continue;
+            const int32_t other = __shfl_xor_sync(gmask, key, j);
+            const bool low = (way & j) == 0, up = (way & k) == 0;
+            key = low == up ? min(key, other) : max(key, other);
+        }
+    return key;
+}
+
 // One set.  All lanes of the group (`gmask`, first lane `gbase`) take part; `sorted` is the group's own piece of shared memory,
 // bucket_cap(ways) pairs.  The table's distinct rows are [ub, ub + n_rows).
 template <int WAYS>          // the number of ways, 0 if it is to be read from the state
 __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w, const TableDev& tb, int64_t gset, int32_t ub, int32_t n_rows,
                                                    uint32_t step, uint32_t epoch, uint32_t gmask, int gbase, int way, int2* sorted) {
+    constexpr int32_t NO_CAND = 0x7fffffff;
     const int ways = WAYS ? WAYS : s.ways, cap = bucket_cap(ways);
     constexpr int PER_LANE = WAYS >= 8 ? 2 : BUCKET_PER_LANE;
     const int64_t slot = gset * ways + way;
@@ -573,8 +592,10 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
 #pragma unroll
     for (int j = 0; j < PER_LANE; ++j) {
         c[j] = j * ways < cap ? __ldcg(s.bucket + gset * cap + way + j * ways) : make_int2(0, 0);
-        if (!in_bucket || way + j * ways >= n) c[j].x = 0x7fffffff;
+        if (way + j * ways >= min(n, cap)) c[j].x = NO_CAND;
     }
+    int32_t chain = -1;
+    if (!in_bucket) { chain = __ldcg(s.chain + slot); s.chain[slot] = -1; }
     const int32_t resident = tag;
     if (tag < 0) pri = 0;
     const bool one_batch = n <= ways;                              // the usual case: sorted in registers
@@ -595,14 +616,44 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
     }
     __syncwarp(gmask);
     if (way == 0) s.set_cnt[gset] = 0;                             // every lane has read it; empty again for the next step
-    // next `ways` candidates in row order, one per lane: from the sorted bucket, or by walking the table's distinct rows
+    // next `ways` candidates in row order, one per lane: from the sorted bucket; or the lowest ones behind those handed out already,
+    // from the bucket and the lists; or by walking the table's distinct rows
     int taken = 0, cursor = 0;                                     // candidates handed out; distinct rows walked
+    int32_t last = -1;                                             // the last candidate handed out
+    // Going through bucket and lists takes n / ways rounds for each batch handed out, a round costing about two of the walk's.  Under LRU
+    // one batch is all that is needed, and the walk finds it among the first ways * n_rows / n rows; under LFU the walk goes through
+    // all rows.  (A cold 32-way LFU cache of 1562 sets per table, 128 candidates each among 200,000 distinct rows of a table, walked in
+    // 7 ms; 13 tables of FP16 rows, some with a handful of sets: 149 us per step by lists alone, 144 by this rule.)
+    const int64_t need = s.policy == 0 ? 2 * (int64_t)n * n : 2 * (int64_t)n * ((n + ways - 1) / ways);
+    const bool by_lists = need < (s.policy == 0 ? (int64_t)ways * n_rows : (int64_t)n_rows);
     auto next_batch = [&](int2* k) {
         if (one_batch) { *k = way < n ? c[0] : make_int2(-1, 0); taken = n; return n; }
         if (in_bucket) {
             *k = taken + way < n ? sorted[taken + way] : make_int2(-1, 0);
             const int m = min(ways, n - taken);
             taken += m;
+            return m;
+        }
+        if (by_lists) {
+            int32_t kept = NO_CAND;                                    // the lowest so far, ascending over the lanes
+            auto merge = [&](int32_t x) {
+                if (x <= last) x = NO_CAND;
+                const int32_t highest = __shfl_sync(gmask, kept, gbase + ways - 1);
+                if (!(__ballot_sync(gmask, x < highest) & gmask)) return;
+                x = group_sort_keys<WAYS, false>(x, ways, way, gmask);
+                kept = min(kept, __shfl_sync(gmask, x, gbase + ways - 1 - way));     // the lowest `ways` of the two, rising, then falling
+                kept = group_sort_keys<WAYS, true>(kept, ways, way, gmask);
+            };
+#pragma unroll
+            for (int j = 0; j < PER_LANE; ++j) merge(c[j].x);
+            for (int32_t p = chain; __ballot_sync(gmask, p >= 0) & gmask;) {
+                const int32_t x = p >= 0 ? p : NO_CAND;
+                if (p >= 0) p = __ldcg(w.victim + p);
+                merge(x);
+            }
+            const int m = __popc(__ballot_sync(gmask, kept != NO_CAND) & gmask);
+            *k = kept != NO_CAND ? make_int2(kept, w.uniq_row[kept]) : make_int2(-1, 0);
+            if (m > 0) last = __shfl_sync(gmask, kept, gbase + m - 1);
             return m;
         }
         int m = 0;                                                 // found so far; the first `ways` of them wait in `sorted`
@@ -630,7 +681,18 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
         if (s.hit_epoch[slot] == epoch) { w.final_loc[s.hit_k[slot]] = LOC_MISS; vict = VICTIM_DEFER; }
         else vict = tag;
     };
-    if (s.policy == 0 && ways > 1) {
+    if (s.policy == 0 && ways == 1) {
+        // direct-mapped LRU never compares: every candidate replaces the one before, the last in row order stays
+        int32_t hi = -1;
+#pragma unroll
+        for (int j = 0; j < PER_LANE; ++j) if (c[j].x != NO_CAND) hi = max(hi, c[j].x);
+        for (int32_t p = chain; p >= 0; p = __ldcg(w.victim + p)) hi = max(hi, p);
+        if (hi >= 0) {
+            pc.admit = (uint32_t)n; pc.evict = (uint32_t)(n - (tag < 0));
+            if (tag >= 0) displace();
+            cand = hi; tag = w.uniq_row[hi]; pri = step;
+        }
+    } else if (s.policy == 0) {
         // LRU: every candidate has the time stamp of this step, the highest there is.  So the candidates, in row order, take the
         // empty ways and then the ways with the oldest stamps (ties: lowest way), and bypass once every way was touched in this step.
         const bool open = tag < 0 || pri < step;
@@ -694,8 +756,7 @@ __device__ __forceinline__ PolicyCounts policy_set(const State& s, const Work& w
                     jempty = false;
                 }
                 // lane `way` holds candidate number `way` of this batch
-                const bool always = ways == 1 && s.policy == 0;                 // direct-mapped LRU never compares
-                const bool would = valid && way >= u && (jempty || always || cpv > jpri);
+                const bool would = valid && way >= u && (jempty || cpv > jpri);
                 const uint32_t wm = (__ballot_sync(gmask, would) & gmask) >> gbase;
                 if (wm == 0) { pc.bypass += (uint32_t)(nb - u); break; }
                 const int f = __ffs(wm) - 1;                                    // the first candidate that replaces
@@ -804,7 +865,7 @@ k_priority(State s, Work w, StepArgs a, int list_hot) {
                     // puts a larger value in the place of the lowest, no way is ever emptied), so a row that does not
                     // beat a bound recorded earlier is bypassed whatever happens in this step (Algorithm 2's test).
                     if (!always && pv <= low[q]) bypass = true;
-                    else { ckey = set[q]; lists = bucket_put(s, sbase[q] + set[q], cap, (int32_t)k, row[q]); }
+                    else { ckey = set[q]; lists = bucket_put(s, w, sbase[q] + set[q], cap, (int32_t)k, row[q]); }
                 }
                 if (one_table) { m += mult[q]; ++un; if (hit) { hitm += mult[q]; ++uh; } byp += bypass; }
                 else {
@@ -840,7 +901,7 @@ k_priority(State s, Work w, StepArgs a, int list_hot) {
 
 // every set that has candidates
 template <int WAYS>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 k_policy(State s, Work w, StepArgs a) {
     __shared__ int2 scratch[256 / WAYS * bucket_cap(WAYS)];
     if (w.ctr->abort) return;

@@ -437,7 +437,7 @@ __device__ void table_state(TableShared& sh, int2* scratch, const State& s, cons
                     } else if (tb.n_sets > 0) {
                         // the early bypass: see k_priority
                         if (!always && pv <= low[j]) ++n_byp;
-                        else { ckey = set[j]; lists = bucket_put(s, tb.set_base + set[j], cap, (int32_t)k, row[j]); }
+                        else { ckey = set[j]; lists = bucket_put(s, w, tb.set_base + set[j], cap, (int32_t)k, row[j]); }
                     }
                     list_long_row(w, (int32_t)k, mult[j], hot_min);
                 }
