@@ -798,8 +798,9 @@ void free_export_slots(mpe_handle* h) {
 
 // Copies between the caller's arrays and a pinned slot, by up to EXPORT_THREADS threads: a fresh array of the caller's is mapped in
 // page by page as it is written, which is what bounds a large export (one thread: about 2 GB/s).
+// Slots of 4 / 8 / 16 MB: a snapshot of 174 MB in 14.2 / 12.4 / 12.4 ms; page-locking them costs a handle's first export 2.5 ms per MB.
 constexpr int EXPORT_THREADS = 8;
-constexpr size_t EXPORT_SLOT_BYTES = 4u << 20, EXPORT_SLOT_SMALL = 64u << 10, EXPORT_PIECE = 512u << 10;
+constexpr size_t EXPORT_SLOT_BYTES = 8u << 20, EXPORT_SLOT_SMALL = 64u << 10, EXPORT_PIECE = 1u << 20;
 struct CopyJob { unsigned char* dst; const unsigned char* src; size_t n; };
 class Copier {
 public:
