@@ -35,15 +35,15 @@ NOMINAL_HBM_GBS = 8000.0
 # proportion to the indices processed): dram__bytes_read.sum + dram__bytes_write.sum per index of the batch, and the
 # limiter the counters point at.  The summaries under profiles/ give the commands and the counters.
 KERNEL_EVIDENCE = {
-    "update": {"dram_bytes_per_index": 112.7, "bound": "issue",
-               "evidence": "80 % of the issue slots used, 317 warp instructions per distinct row; DRAM 29 %, L2 26 % of peak",
-               "profile": "profiles/k_update_cfg4_8tables.md"},
-    "pool": {"dram_bytes_per_index": 72.8, "bound": "latency",
-             "evidence": "7.3 long-scoreboard stall cycles per issue at 46 % of the warp slots (64 registers); L1 50 %, DRAM 22 % of peak; 61 % of the sectors hit in L1",
-             "profile": "profiles/k_pool_cfg4_8tables.md"},
-    "hot_partial": {"dram_bytes_per_index": 20.9, "bound": "l2-latency",
-                    "evidence": "gradient rows come from L2 (83 % hits, 36 % of its throughput), 11.2 long-scoreboard stall cycles per issue at 24 % of the warp slots (kept small on purpose: it runs beside other kernels)",
-                    "profile": "profiles/k_hot_partial_cfg4_8tables.md"},
+    "update": {"dram_bytes_per_index": 103.6, "bound": "issue",
+               "evidence": "74 % of the issue slots used, 321 warp instructions per distinct row; DRAM 25 %, L2 30 % of peak",
+               "profile": "profiles/step_kernels_cfg4_8tables.md"},
+    "pool": {"dram_bytes_per_index": 67.6, "bound": "latency",
+             "evidence": "6.1 long-scoreboard stall cycles per issue at 49 % of the warp slots (64 registers); DRAM 18 %, L2 20 % of peak; 60 % of the sectors hit in L1",
+             "profile": "profiles/step_kernels_cfg4_8tables.md"},
+    "hot_partial": {"dram_bytes_per_index": 22.8, "bound": "l2-latency",
+                    "evidence": "gradient rows come from L2 (82 % hits, 37 % of its throughput), 7.5 long-scoreboard stall cycles per issue at 24 % of the warp slots (kept small on purpose: it runs beside other kernels)",
+                    "profile": "profiles/step_kernels_cfg4_8tables.md"},
     # on the small case a pass of the sort is L2 resident, so its DRAM traffic does not scale to the full size: none given
     "sort_scatter": {"dram_bytes_per_index": None, "bound": "latency",
                      "evidence": "short scoreboard 6.1 (ranking through shared-memory counters), long scoreboard 5.6 (tile load, look-back) and barrier 2.6 stall cycles per issue; 35 % of the issue slots; DRAM 14 %, L2 24 % of peak",
@@ -259,10 +259,9 @@ def run_ours(args, cfg, rank, world, local_rank):
     maxL = max(b[0].numel() for b in batches)
     h.reserve(cfg.batch, maxL)
     out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, dtype=torch.float32, device=dev)
-    # The step runs on a stream of higher priority than the one the next batch is prepared on (and than the library's own
-    # second stream): when both have blocks ready, the step's kernels get the SMs first and the others fill the gaps.
-    torch.cuda.synchronize(dev)
-    torch.cuda.set_stream(torch.cuda.Stream(dev, priority=-1))
+    # A stream of its own for the step, of the priority of the one the next batch is prepared on: with the step's ahead, the next
+    # batch's sort starves and the step after waits for it (5.04 against 4.89 ms).
+    torch.cuda.set_stream(torch.cuda.Stream(dev, priority=0))
     cs = torch.cuda.current_stream(dev)
     sp = cs.cuda_stream
 
@@ -385,7 +384,7 @@ def run_ours(args, cfg, rank, world, local_rank):
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": describe(cfg), "l2": "inputs larger than L2; a new batch every step",
                    "launch": "plain launches; per-kernel times from a second pass without the preparation",
-                   "next_batch": "sorted ahead on a second stream of lower priority (mpe_prepare) while the current step runs" if ahead else "not prepared ahead",
+                   "next_batch": "sorted ahead on a second stream (mpe_prepare) while the current step runs" if ahead else "not prepared ahead",
                    "sharding": "each rank trains its own tables (no data-path collective)" if world > 1 else "one GPU"},
         "clocks": clocks,
         "e2e": {"value": e2e_rows / e2e_s if e2e_s > 0 else None, "unit": "rows/s", "h2d_bytes_per_step": h2d,
