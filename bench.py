@@ -261,6 +261,7 @@ def run_ours(args, cfg, rank, world, local_rank):
     out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, dtype=torch.float32, device=dev)
     # A stream of its own for the step, of the priority of the one the next batch is prepared on: with the step's ahead, the next
     # batch's sort starves and the step after waits for it (5.04 against 4.89 ms).
+    torch.cuda.synchronize(dev)         # the batches have been generated, on the default stream
     torch.cuda.set_stream(torch.cuda.Stream(dev, priority=0))
     cs = torch.cuda.current_stream(dev)
     sp = cs.cuda_stream

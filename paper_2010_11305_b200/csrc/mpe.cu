@@ -215,7 +215,7 @@ void free_workspace(mpe_handle* h) {
 // Batches up to this size are sorted in small tiles: large ones would leave SMs without a tile.
 constexpr int64_t SMALL_TILE_MAX_INDICES = 4 << 20;
 
-int alloc_set(mpe_handle* h, int64_t L, int64_t bags);
+int alloc_set(mpe_handle* h, int64_t L, int64_t bags, cudaStream_t first_use);
 
 int64_t sort_max_tiles(const mpe_handle* h, int64_t L) {
     const int tile = sort_tile(L <= SMALL_TILE_MAX_INDICES);
@@ -233,19 +233,24 @@ int renew_sort_tags(mpe_handle* h) {
         }
         swap_sets(h);
     }
+    // the clears are on the default stream, which the streams of the next step and the next mpe_prepare need not wait for
+    CK(h, cudaDeviceSynchronize());
     h->sort_passes_bound = 0;
     return MPE_OK;
 }
 
 int alloc_workspace(mpe_handle* h, int64_t L, int64_t bags) {
     free_workspace(h);
-    int rc = alloc_set(h, L, bags);
+    int rc = alloc_set(h, L, bags, h->stream);       // a change of stream waits for the old one
     if (rc != MPE_OK) return rc;
     h->cap_L = L; h->cap_bags = bags;
     return MPE_OK;
 }
 
-int alloc_set(mpe_handle* h, int64_t L, int64_t bags) {
+// first_use: the stream that works in the new workspace first.  What has to start from zero is cleared there, in front of that work:
+// a clear on any other stream -- the default one, which a non-blocking stream does not wait for -- can still be queued behind other
+// kernels while the sort already counts in the array.
+int alloc_set(mpe_handle* h, int64_t L, int64_t bags, cudaStream_t first_use) {
     // everything a step needs between its first and last kernel, sized for L indices
     (void)bags;
     free_set(h);
@@ -262,16 +267,16 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags) {
     struct Piece { void* p; int64_t bytes; };             // where the pointer to it goes
     std::vector<Piece> pieces;
 #define A(ptr, count) pieces.push_back({&(ptr), std::max<int64_t>((count), 1) * (int64_t)sizeof(*(ptr))})
-    // the sort's two buffers; the second sort (miss candidates by cache set) runs in backward, when the first sort's
-    // results have been consumed, and uses the same two
-    h->sort_n = (n + 3) & ~int64_t(3);
-    A(h->sortA, 2 * h->sort_n); A(h->sortB, 2 * h->sort_n);
     // small batches get small tiles, so that every SM has one
     w.sort_tile = sort_tile(L <= SMALL_TILE_MAX_INDICES);
     const int64_t max_tiles = sort_max_tiles(h, L);
-    A(h->sort_status, 256 * max_tiles); A(h->ghist, (int64_t)T * SORT_MAX_PASSES * 256); A(h->sort_ctl, 1);
+    // these start from zero and are kept consistent from one step to the next by the kernels that use them
+    A(h->sort_status, 256 * max_tiles); A(h->ghist, (int64_t)T * SORT_MAX_PASSES * 256); A(h->sort_ctl, 1); A(w.ctr, 1);
+    const size_t n_zeroed = pieces.size();
+    // the sort's two buffers
+    h->sort_n = (n + 3) & ~int64_t(3);
+    A(h->sortA, 2 * h->sort_n); A(h->sortB, 2 * h->sort_n);
     A(h->block_sums, n / SCAN_TILE + 2);
-    A(w.ctr, 1);
     A(w.table_start, T + 1); A(w.tile_base, T + 1); A(w.ustart, T + 1);
     A(w.occ_b, n);
     A(w.uniq_row, nu); A(w.uniq_t, nu); A(w.seg, nu + 1); A(w.loc, nu); A(w.final_loc, nu);
@@ -280,20 +285,20 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags) {
     const int64_t max_tasks = hot_capacity(L);
     A(w.task_k, max_tasks); A(w.partial, max_tasks * h->dim); A(w.hot_k, max_tasks); A(w.mid_k, L / MID_MIN + 1);
 #undef A
-    int64_t total = 0;
-    for (const Piece& x : pieces) total += (x.bytes + 255) / 256 * 256;
+    int64_t total = 0, zeroed = 0;
+    for (size_t i = 0; i < pieces.size(); ++i) {
+        total += (pieces[i].bytes + 255) / 256 * 256;
+        if (i + 1 == n_zeroed) zeroed = total;
+    }
     uint8_t* base = nullptr;
     if ((rc = dmalloc(h, &base, total, tr)) != MPE_OK) return rc;
+    CK(h, cudaMemsetAsync(base, 0, (size_t)zeroed, first_use));
+    CK(h, cudaEventRecord(h->ev_prep, first_use));       // whoever prepares a batch here on another stream waits for this
     for (const Piece& x : pieces) {
         std::memcpy(x.p, &base, sizeof(base));
         base += (x.bytes + 255) / 256 * 256;
         h->ws_bytes += (uint64_t)x.bytes;
     }
-    // the sort keeps these consistent by itself from one pass to the next; they start from zero
-    CK(h, cudaMemset(h->sort_status, 0, sizeof(unsigned long long) * 256 * max_tiles));
-    CK(h, cudaMemset(h->ghist, 0, sizeof(uint32_t) * T * SORT_MAX_PASSES * 256));
-    CK(h, cudaMemset(h->sort_ctl, 0, sizeof(SortCtl)));
-    CK(h, cudaMemset(w.ctr, 0, sizeof(Counters)));
     return MPE_OK;
 }
 
@@ -743,7 +748,7 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
     if (!h->alt.wk.ctr) {                    // first use: the second workspace; from here on the steps record when they leave theirs
         CK(h, cudaEventRecord(h->ev_free, h->stream));
         swap_sets(h);
-        int rc = alloc_set(h, h->cap_L, h->cap_bags);
+        int rc = alloc_set(h, h->cap_L, h->cap_bags, stream);
         if (rc != MPE_OK) free_set(h);
         swap_sets(h);
         if (rc != MPE_OK) return rc;
@@ -1109,6 +1114,7 @@ int mpe_destroy(mpe_handle* h) {
     if (!h) return MPE_ERR_ARG;
     DeviceGuard guard(h->device);
     cudaStreamSynchronize(h->stream);
+    for (cudaEvent_t e : {h->ev_prep, h->alt.ev_prep}) if (e) cudaEventSynchronize(e);       // a batch may still be prepared on a stream of the caller's
     if (h->side) { cudaStreamSynchronize(h->side); cudaStreamDestroy(h->side); }
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
@@ -1144,11 +1150,12 @@ int mpe_last_error(mpe_handle* h, int32_t* code, int64_t* detail) {
     if (h->prep_running) CK(h, cudaEventSynchronize(h->ev_prep));
     Counters c;
     CK(h, cudaMemcpy(&c, h->wk.ctr, sizeof(c), cudaMemcpyDeviceToHost));
-    CK(h, cudaMemset(&h->wk.ctr->err[0], 0, sizeof(c.err)));
+    CK(h, cudaMemsetAsync(&h->wk.ctr->err[0], 0, sizeof(c.err), h->stream));
     if (h->alt.wk.ctr && !h->prepared) {     // steps alternate between the two workspaces: conditions seen in either count
         Counters c2;                         // (a batch that is prepared but not yet taken over reports with its own step)
+        CK(h, cudaEventSynchronize(h->alt.ev_prep));     // a batch that was prepared and then discarded may still be sorted there
         CK(h, cudaMemcpy(&c2, h->alt.wk.ctr, sizeof(c2), cudaMemcpyDeviceToHost));
-        CK(h, cudaMemset(&h->alt.wk.ctr->err[0], 0, sizeof(c2.err)));
+        CK(h, cudaMemsetAsync(&h->alt.wk.ctr->err[0], 0, sizeof(c2.err), h->stream));
         c.err[ERR_OFFSETS] += c2.err[ERR_OFFSETS]; c.err[ERR_INDEX] += c2.err[ERR_INDEX];
     }
     // a wait inside the sort that ran out (its step was abandoned) outranks the conditions of the inputs
@@ -1157,8 +1164,9 @@ int mpe_last_error(mpe_handle* h, int32_t* code, int64_t* detail) {
         if (!ctl) continue;
         SortCtl sc;
         CK(h, cudaMemcpy(&sc, ctl, sizeof(sc), cudaMemcpyDeviceToHost));
-        if (sc.timeout) { timeouts += sc.timeout; CK(h, cudaMemset(&ctl->timeout, 0, sizeof(uint32_t))); }
+        if (sc.timeout) { timeouts += sc.timeout; CK(h, cudaMemsetAsync(&ctl->timeout, 0, sizeof(uint32_t), h->stream)); }
     }
+    CK(h, cudaStreamSynchronize(h->stream));     // the clears are done before a later call, on whatever stream, counts there again
     if (timeouts) { *code = MPE_ERR_TIMEOUT; *detail = (int64_t)timeouts; }
     else if (c.err[ERR_OFFSETS]) { *code = MPE_ERR_OFFSETS; *detail = (int64_t)c.err[ERR_OFFSETS]; }
     else if (c.err[ERR_INDEX]) { *code = MPE_ERR_INDEX; *detail = (int64_t)c.err[ERR_INDEX]; }

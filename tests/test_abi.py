@@ -69,3 +69,18 @@ def test_bench_evidence_points_at_committed_summaries():
         path = os.path.join(ROOT, ev["profile"])
         assert os.path.isfile(path) and path.endswith(".md"), f"{name}: {ev['profile']}"
         assert "--clock-control none" in open(path).read(), f"{name}: the summary does not give its command"
+
+
+def test_device_memory_is_cleared_in_front_of_its_first_use():
+    """cudaMemset goes to the default stream, which a non-blocking stream does not wait for: the sort of a batch prepared on such a
+    stream once counted in a workspace whose clear was still queued behind the running forward.  A clear either names the stream
+    that uses the memory next, or the function it stands in waits for the device before it returns."""
+    src = open(os.path.join(ROOT, "paper_2010_11305_b200", "csrc", "mpe.cu")).read()
+    clears = [m.start() for m in re.finditer(r"\bcudaMemset\(", src)]
+    assert clears
+    for at in clears:
+        rest = src[at:src.index("\n}\n", at)]
+        assert "cudaDeviceSynchronize()" in rest, f"not waited for: {src[at:src.index(chr(10), at)]}"
+    bench = open(os.path.join(ROOT, "bench.py")).read()
+    made, switched = bench.index("stream_gen.batch(s) for s in"), bench.index("torch.cuda.set_stream(")
+    assert "torch.cuda.synchronize(" in bench[made:switched]           # the batches are made on the default stream

@@ -107,3 +107,48 @@ def test_exports_of_many_pieces(dim, bits, n):
     for got, ref in zip(h.export_rows(0, rows), o.rows(0, every)):
         assert np.array_equal(got, ref[rows])
     h.close()
+
+
+def _ahead(cfg, counts, stream, busy):
+    """The loop forward(k); prepare(k + 1); backward(k) with no wait of the host between them, against the oracle; counts[k] indices
+    per table in step k, the workspace reserved when it grows.  `busy`: clock cycles of other work in front of every forward, so
+    that all that follows is queued behind it."""
+    from parity_util import compare_state, make_pair
+    h, o = make_pair(cfg)
+    rng = np.random.default_rng(cfg.seed)
+    T, steps = cfg.num_tables, len(counts)
+    batches = [_batch(rng, [_skewed(rng, r, c) for r in cfg.num_rows], cfg.batch, cfg.dim) for c in counts]
+    dev = [tuple(torch.from_numpy(x).cuda() for x in b) for b in batches]
+    outs = [torch.empty(cfg.batch, T * cfg.dim, device="cuda") for _ in range(steps)]
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for k, (idx, off, grad) in enumerate(dev):
+            h.reserve(cfg.batch, T * counts[k])
+            if busy:
+                torch.cuda._sleep(busy)
+            h.forward(idx, off, cfg.batch, outs[k], stream.cuda_stream)
+            if k + 1 < steps:
+                h.prepare(dev[k + 1][0], dev[k + 1][1], cfg.batch, side.cuda_stream)
+            h.backward(grad, cfg.lr, k + 1)
+    assert h.last_error() == (0, 0)
+    for k, (idx, off, grad) in enumerate(batches):
+        assert np.array_equal(outs[k].cpu().numpy(), o.forward(idx, off, cfg.batch)), f"step {k + 1}"
+        o.backward(grad, cfg.lr, k + 1)
+    compare_state(h, o, cfg, range(T), rng)
+    h.close()
+
+
+@pytest.mark.parametrize("count", [300, 155000])
+def test_first_prepared_batch_of_a_handle_whose_memory_was_used_before(count):
+    """The second workspace is allocated by the first prepare, in memory that an earlier handle has left full, while the default
+    stream is busy with the forward: its counters have to be zero before the sort on the other stream begins."""
+    for seed in (3, 4, 5):
+        _ahead(_cfg([70001, 900], 64, seed=seed), [count] * 3, torch.cuda.default_stream(), 20_000_000)
+
+
+@pytest.mark.parametrize("count", [300, 155000])
+def test_step_on_a_non_blocking_stream_straight_after_reserve(count):
+    """The workspace grows between two steps of a stream that does not wait for the default one."""
+    for seed in (6, 7):
+        _ahead(_cfg([70001, 900], 64, seed=seed), [count // 3, count, count, 2 * count, 2 * count], torch.cuda.Stream(), 0)
