@@ -258,9 +258,13 @@ int mpe_workspace_bytes(mpe_handle* h, uint64_t* out2);
  *     up as designed: the next mpe_last_error reports MPE_ERR_TIMEOUT with detail 1, exactly as after a real one, and
  *     the handle goes on working.  Nothing hangs or faults.  Not between a forward and its backward.
  *   MPE_SELFTEST_RENEW_TAGS: the next mpe_forward starts the sort's pass numbers over (waits for the device, clears the
- *     per-tile words), which otherwise happens once in hundreds of millions of steps. */
+ *     per-tile words), which otherwise happens once in hundreds of millions of steps.
+ *   MPE_SELFTEST_ABANDON_NEXT_SORT: in the next grid-wide sort of a table of several tiles, the look-backs give up at once, so
+ *     that the step it belongs to is abandoned.  (Steps whose tables are sorted inside thread-block clusters have no such waits
+ *     and are not affected.)  Not between a forward and its backward, nor with a batch prepared. */
 #define MPE_SELFTEST_LOOK_BACK_TIMEOUT 1
 #define MPE_SELFTEST_RENEW_TAGS 2
+#define MPE_SELFTEST_ABANDON_NEXT_SORT 3
 int mpe_selftest(mpe_handle* h, int32_t which);
 /* Geometry of table `table`'s cache. */
 int mpe_cache_geometry(mpe_handle* h, int32_t table, int32_t* n_sets, int32_t* ways);

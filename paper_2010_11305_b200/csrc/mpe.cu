@@ -258,8 +258,8 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags, cudaStream_t first_use) {
     const int T = h->T;
     const int64_t n = L + 1;
     // arrays with one entry per distinct row: there are at most as many distinct rows as indices, and at most as many
-    // as the tables have rows (plus one pseudo row per table that collects its out-of-range ids)
-    const int64_t nu = std::min<int64_t>(L, h->total_rows + T) + 2;
+    // as the tables have rows (plus one pseudo row per table that collects its out-of-range ids), and an entry behind each table's
+    const int64_t nu = std::min<int64_t>(L, h->total_rows + T) + T + 2;
     Work& w = h->wk;
     int rc = MPE_OK;
     h->ws_bytes = 0;
@@ -277,7 +277,7 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags, cudaStream_t first_use) {
     h->sort_n = (n + 3) & ~int64_t(3);
     A(h->sortA, 2 * h->sort_n); A(h->sortB, 2 * h->sort_n);
     A(h->block_sums, n / SCAN_TILE + 2);
-    A(w.table_start, T + 1); A(w.tile_base, T + 1); A(w.ustart, T + 1);
+    A(w.table_start, T + 1); A(w.tile_base, T + 1); A(w.ustart, 2 * T + 1);
     A(w.occ_b, n);
     A(w.uniq_row, nu); A(w.uniq_t, nu); A(w.seg, nu + 1); A(w.loc, nu); A(w.final_loc, nu);
     A(w.victim, nu); A(w.defer_k, nu); A(w.heads, nu);
@@ -595,12 +595,12 @@ int launch_table(mpe_handle* h, int blocks, const StepArgs& av) {
         h->table_ready.insert(reinterpret_cast<const void*>(kern));
     }
     LaunchScope ls(h, STATE ? "table" : "table_sort", h->stream);
-    CK(h, cudaLaunchKernelEx(&cfg, kern, h->st, h->wk, sort_input(sort_bufs(h)), reinterpret_cast<uint2*>(h->sortA), h->sort_status, h->sort_ctl,
-                             (uint32_t)av.step, av.epoch));
+    CK(h, cudaLaunchKernelEx(&cfg, kern, h->st, h->wk, sort_input(sort_bufs(h)), reinterpret_cast<uint2*>(h->sortA), (uint32_t)av.step, av.epoch));
     return MPE_OK;
 }
 // the sort and the distinct rows; `state`: the priorities and the admission too (a cluster of one block)
 int enqueue_table(mpe_handle* h, const TablePlan& plan, const StepArgs& av, bool state) {
+    h->wk.uend = h->wk.ustart + h->T + 1;            // the tables' lists stand in any order
     if (plan.items == TBL_ITEMS_LARGE) return launch_table<TBL_ITEMS_LARGE, false>(h, plan.blocks, av);
     return state ? launch_table<TBL_ITEMS_SMALL, true>(h, plan.blocks, av) : launch_table<TBL_ITEMS_SMALL, false>(h, plan.blocks, av);
 }
@@ -612,6 +612,7 @@ int enqueue_index_chain(mpe_handle* h, int64_t L) {
     Work& w = h->wk;
     const TablePlan plan = table_plan(h, L);
     if (plan.blocks) return enqueue_table(h, plan, StepArgs{}, false);
+    w.uend = w.ustart + 1;                           // a table's distinct rows end where the next one's begin
     // sort the row indices of the mini-batch (Section 5.1), table by table
     seg_sort(h, sort_bufs(h), w.table_start, w.tile_base, bits_for((uint32_t)h->max_rows), L, reinterpret_cast<uint32_t*>(w.occ_b), &h->skey);
     // distinct rows
@@ -1207,6 +1208,11 @@ int mpe_selftest(mpe_handle* h, int32_t which) {
         ++h->sort_passes_bound;
         return check_launch(h);
     }
+    if (which == MPE_SELFTEST_ABANDON_NEXT_SORT) {
+        if (h->have_forward || h->prepared) return MPE_ERR_SEQUENCE;
+        LAUNCH(h, "selftest", k_selftest_cut, 1, 1, 0, h->sort_ctl);
+        return check_launch(h);
+    }
     if (which == MPE_SELFTEST_RENEW_TAGS) {
         h->sort_passes_bound = SORT_TAG_MASK;           // the next forward starts the pass numbers over
         return MPE_OK;
@@ -1242,20 +1248,19 @@ int mpe_step_info(mpe_handle* h, int64_t* out6) {
     if (h->prep_running) CK(h, cudaEventSynchronize(h->ev_prep));
     Counters c;
     CK(h, cudaMemcpy(&c, h->wk.ctr, sizeof(c), cudaMemcpyDeviceToHost));
-    if (c.abort) return MPE_OK;
-    std::vector<int32_t> us(h->T + 1), urow(1);
+    if (c.abort || !h->wk.uend) return MPE_OK;
+    std::vector<int32_t> us(h->T), ue(h->T);
+    CK(h, cudaMemcpy(us.data(), h->wk.ustart, sizeof(int32_t) * h->T, cudaMemcpyDeviceToHost));
+    CK(h, cudaMemcpy(ue.data(), h->wk.uend, sizeof(int32_t) * h->T, cudaMemcpyDeviceToHost));
     out4[0] = (int64_t)c.L - (int64_t)c.dropped;
-    // distinct rows: the sort puts each table's out-of-range ids into one pseudo row; leave those out
-    int64_t pseudo = 0;
-    if (c.dropped) {
-        CK(h, cudaMemcpy(us.data(), h->wk.ustart, sizeof(int32_t) * (h->T + 1), cudaMemcpyDeviceToHost));
-        for (int t = 0; t < h->T; ++t) {
-            if (us[t + 1] == us[t]) continue;
-            CK(h, cudaMemcpy(urow.data(), h->wk.uniq_row + us[t + 1] - 1, sizeof(int32_t), cudaMemcpyDeviceToHost));
-            if (urow[0] >= h->tables[t].N) ++pseudo;
+    for (int t = 0; t < h->T; ++t) {
+        out4[1] += ue[t] - us[t];
+        if (c.dropped && ue[t] > us[t]) {        // the sort puts a table's out-of-range ids into one pseudo row behind the others; leave it out
+            int32_t last = 0;
+            CK(h, cudaMemcpy(&last, h->wk.uniq_row + ue[t] - 1, sizeof(int32_t), cudaMemcpyDeviceToHost));
+            if (last >= h->tables[t].N) --out4[1];
         }
     }
-    out4[1] = (int64_t)c.U - pseudo;
     out4[2] = (int64_t)c.dropped;
     out4[3] = (int64_t)c.hot_rows;
     out6[4] = (int64_t)c.hot_occ;

@@ -36,7 +36,8 @@ struct TableDev {
 
 struct Counters {
     uint32_t L;            // indices in this batch
-    uint32_t U;            // distinct (table,row) pairs incl. one pseudo row per table that had bad indices
+    uint32_t U;            // entries in the list of distinct (table,row) pairs: with one pseudo row per table that had bad indices, and
+                           // where a cluster took each table, one entry behind each table's rows
     uint32_t fwd_bad, fwd_done;      // of the running forward: offsets were inconsistent; blocks that have finished
     uint32_t hot_rows;
     uint32_t hot_tasks;
@@ -94,7 +95,8 @@ struct StepArgs {
 
 struct Work {
     Counters* ctr;
-    int32_t *table_start, *tile_base, *ustart;   // [T+1]
+    int32_t *table_start, *tile_base;            // [T+1]
+    int32_t *ustart, *uend;                      // [T] where each table's distinct rows are listed
     int32_t* occ_b;        // [L] by sorted order: sample of the element; sign bit: last occurrence of its row
     int32_t *uniq_row, *uniq_t, *seg, *loc, *final_loc, *victim, *hot_base, *hot_left;   // per unique row
     int32_t* task_k;       // [hot tasks]
@@ -915,8 +917,8 @@ k_policy(State s, Work w, StepArgs a) {
         const int2 head = w.heads[h];
         const int t = head.y;
         const TableDev tb = s.tables[t];
-        const int32_t ub = w.ustart[t];
-        const PolicyCounts pc = policy_set<WAYS>(s, w, tb, head.x, ub, w.ustart[t + 1] - ub, (uint32_t)a.step, a.epoch, gmask,
+        const int32_t ub = w.ustart[t], ue = w.uend[t];
+        const PolicyCounts pc = policy_set<WAYS>(s, w, tb, head.x, ub, ue - ub, (uint32_t)a.step, a.epoch, gmask,
                                            gbase, way, scratch + grp * cap);
         if (way == 0) {
             unsigned long long* st = s.stats + (int64_t)t * 8;

@@ -105,7 +105,7 @@ struct SortCtl {
     uint32_t seq;        // passes completed on this workspace; pass tags are seq + 1
     uint32_t ticket;     // next tile to hand out; the block that draws the last ticket of a pass puts it back to 0
     uint32_t timeout;    // sticky: look-backs that gave up
-    uint32_t done;       // blocks that have finished the current pass
+    uint32_t cut;        // self-check: the look-backs of the next pass give up
 };
 constexpr uint32_t SORT_TAG_MASK = 0x3fffffffU;
 constexpr unsigned long long SORT_PREFIX = 1ULL << 32, SORT_POISON = 1ULL << 33;
@@ -125,63 +125,21 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned l
 
 // Hands the calling block its next tile (all threads call); false when none is left.
 // Tickets are drawn when the block is ready for the tile, never ahead of time: the tiles behind a ticket wait for its tile.
-__device__ __forceinline__ bool draw_tile(SortCtl* ctl, uint32_t ntiles, uint32_t* s_turn /* [2], shared */, uint32_t* tile, uint32_t* tag) {
+__device__ __forceinline__ bool draw_tile(SortCtl* ctl, uint32_t ntiles, uint32_t* s_turn /* [3], shared */, uint32_t* tile, uint32_t* tag) {
     __syncthreads();
-    if (threadIdx.x == 0) { s_turn[0] = atomicAdd(&ctl->ticket, 1u); s_turn[1] = (ctl->seq + 1u) & SORT_TAG_MASK; }
+    if (threadIdx.x == 0) { s_turn[0] = atomicAdd(&ctl->ticket, 1u); s_turn[1] = (ctl->seq + 1u) & SORT_TAG_MASK; s_turn[2] = ctl->cut; }
     __syncthreads();
     *tile = s_turn[0]; *tag = s_turn[1];
     return *tile < ntiles;
 }
-// After its last draw: true in exactly one block of the grid, the last one to get here.  Every other block's writes are
-// visible to that block (through L2: read them with __ldcg), which ends the pass with close_pass() when it is done.
-__device__ __forceinline__ bool last_block_of_pass(SortCtl* ctl, uint32_t* s_turn) {
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_turn[0] = atomicAdd(&ctl->done, 1u);
-    __syncthreads();
-    return s_turn[0] == gridDim.x - 1u;
-}
 __device__ __forceinline__ void close_pass(SortCtl* ctl, uint32_t tag) {
-    if (threadIdx.x == 0) { ctl->ticket = 0; ctl->done = 0; ctl->seq = tag; }
-}
-
-// One word per tile (the compactions).  tile_publish (one thread): how many items the tile holds, as soon as it is known.
-// tile_look_back (one whole warp, any time later): the sum of `total` over the tiles before `tile`, reading 32 predecessors'
-// words at a time; it leaves the tile's prefix in its word.
-__device__ __forceinline__ void tile_publish(unsigned long long* words, uint32_t tile, uint32_t total, uint32_t tag) {
-    st_relaxed_u64(words + tile, sort_word(tag, tile == 0 ? SORT_PREFIX : 0ULL, total));
-}
-__device__ __forceinline__ uint32_t tile_look_back(unsigned long long* words, uint32_t tile, uint32_t total, uint32_t tag, bool* poison,
-                                                   int poll_limit = SORT_POLL_LIMIT) {
-    const int lane = threadIdx.x & 31;
-    uint32_t sum = 0;
-    bool bad = false;
-    if (tile > 0) {
-        for (int64_t base = (int64_t)tile - 1;; base -= 32) {
-            const int64_t j = base - lane;
-            unsigned long long v = sort_word(tag, SORT_PREFIX, 0);            // before the first tile: nothing
-            if (j >= 0) {
-                v = ld_relaxed_u64(words + j);
-                for (int polls = 0; (uint32_t)(v >> 34) != tag; v = ld_relaxed_u64(words + j)) {
-                    if (++polls > poll_limit) { v = SORT_PREFIX | SORT_POISON; break; }
-                    if (polls > 32) __nanosleep(200);
-                }
-            }
-            const uint32_t pm = __ballot_sync(0xffffffffU, (v & SORT_PREFIX) != 0);
-            const int stop = pm ? __ffs(pm) - 1 : 31;                          // nearest predecessor that knows its prefix
-            sum += __reduce_add_sync(0xffffffffU, lane <= stop ? (uint32_t)v : 0u);
-            bad |= __any_sync(0xffffffffU, lane <= stop && (v & SORT_POISON) != 0);
-            if (pm) break;
-        }
-        if (lane == 0) st_relaxed_u64(words + tile, sort_word(tag, SORT_PREFIX | (bad ? SORT_POISON : 0ULL), sum + total));
-    }
-    *poison = bad;
-    return sum;
+    if (threadIdx.x == 0) { ctl->ticket = 0; ctl->cut = 0; ctl->seq = tag; }
 }
 
 // Sum of what the `left` tiles before the one that owns `word` hold of this thread's digit, plus where the first of them
 // begins: walks back over their words until it meets a prefix.
-__device__ __forceinline__ uint32_t sort_look_back(const unsigned long long* word, int left, uint32_t tag, bool* poison) {
+__device__ __forceinline__ uint32_t sort_look_back(const unsigned long long* word, int left, uint32_t tag, bool* poison,
+                                                   int poll_limit = SORT_POLL_LIMIT) {
     uint32_t sum = 0;
     bool bad = false;
     const unsigned long long* q = word - 256;
@@ -194,7 +152,7 @@ __device__ __forceinline__ uint32_t sort_look_back(const unsigned long long* wor
         for (int u = 0; u < SORT_LOOK; ++u) {
             if (done) break;
             for (int polls = 0; (uint32_t)(v[u] >> 34) != tag; v[u] = ld_relaxed_u64(q - 256 * u)) {
-                if (++polls > SORT_POLL_LIMIT) { v[u] = SORT_PREFIX | SORT_POISON; break; }
+                if (++polls > poll_limit) { v[u] = SORT_PREFIX | SORT_POISON; break; }
                 if (polls > 32) __nanosleep(200);
             }
             sum += (uint32_t)v[u];
@@ -268,7 +226,7 @@ k_sort_scatter(const uint2* __restrict__ pairs_in, uint2* __restrict__ pairs_out
     __shared__ uint32_t goff[256];             // first global position of each digit of this tile minus its tile-local start
     __shared__ uint2 skv[SORT_TILE];
     __shared__ uint32_t scan_tmp[SORT_THREADS / 32 + 1];
-    __shared__ uint32_t s_ticket[2];
+    __shared__ uint32_t s_ticket[3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const bool off = *abort_flag != 0;          // the step was abandoned before this pass: nothing to sort
@@ -363,6 +321,7 @@ k_sort_scatter(const uint2* __restrict__ pairs_in, uint2* __restrict__ pairs_out
             gb = (uint32_t)seg_start[t] + block_exclusive_scan<SORT_THREADS>(mine, &all, scan_tmp);
         } else {
             gb = sort_look_back(word, local, tag, &poison);
+            poison |= s_ticket[2] != 0;
         }
         st_relaxed_u64(word, sort_word(tag, SORT_PREFIX | (poison ? SORT_POISON : 0ULL), gb + tot));
         goff[threadIdx.x] = gb - ds;                                           // global position = goff + tile-local position
@@ -407,17 +366,16 @@ k_scan_block_sums(uint32_t* __restrict__ block_sums, const uint32_t* __restrict_
 
 // ---- self-check of the bounded wait ----------------------------------------------------------
 // One warp plays tile 1 of a pass whose tile 0 belongs to nobody, with the wait cut to a few thousand polls (about a
-// millisecond): the look-back has to give up and say so.  The pass number moves on afterwards, so the word it leaves
-// can never be taken for one of a real pass.
-__global__ void k_selftest_look_back(unsigned long long* words, SortCtl* ctl) {
+// millisecond): the look-back has to give up and say so.  The pass number moves on afterwards.
+__global__ void k_selftest_look_back(const unsigned long long* words, SortCtl* ctl) {
     if (blockIdx.x != 0 || threadIdx.x >= 32) return;
     const uint32_t tag = (ctl->seq + 1u) & SORT_TAG_MASK;
     bool poison = false;
-    tile_look_back(words, 1u, 0u, tag, &poison, 4096);
-    if (threadIdx.x == 0) {
-        if (poison) atomicAdd(&ctl->timeout, 1u);
-        ctl->seq = tag;
-    }
+    sort_look_back(words + 256 + threadIdx.x, 1, tag, &poison, 4096);
+    if (__any_sync(0xffffffffU, poison) && threadIdx.x == 0) atomicAdd(&ctl->timeout, 1u);
+    if (threadIdx.x == 0) ctl->seq = tag;
 }
+// The look-backs of the next pass give up, so that the step it belongs to is abandoned.
+__global__ void k_selftest_cut(SortCtl* ctl) { ctl->cut = 1; }
 
 }  // namespace mpe

@@ -53,8 +53,7 @@ struct TableShared {
     uint32_t tmp[TBL_WARPS + 1];
     uint32_t wsum[TBL_WARPS];
     uint32_t heads[TBL_MAX_CLUSTER];              // distinct rows that begin in each block
-    alignas(8) uint32_t base[2];                  // first distinct row of the table; a look-back that gave up
-    uint32_t table;                               // (block 0) the table drawn
+    uint32_t base;                                // first distinct row of the table
     uint32_t n_heads;                             // (block 0) sets with candidates
     uint32_t stats[8];
 };
@@ -275,12 +274,14 @@ __device__ void table_sort_spilled(TableShared& sh, uint2** src, uint2* other, c
     }
 }
 
-// The distinct rows of the table: lists them at their place among all tables' distinct rows (the tables before this one say how many
-// they have through one word each), marks each row's last occurrence.  Returns the number of distinct rows of the table and sets
-// *first to the first one's index; false in *ok if a look-back gave up.
+// The distinct rows of the table: lists them, marks each row's last occurrence.  Returns the number of distinct rows of the table and
+// sets *first to the first one's index.
+// The tables' lists stand in whatever order the clusters get here: a cluster takes its place with one addition and waits for no other,
+// so that nothing can run out or be abandoned, and a large table holds up nobody.  Behind each list stands one more entry, a row that
+// does not exist (it lives nowhere, like an id outside the table), whose start is where the table's last row ends.
 template <int ITEMS>
-__device__ uint32_t table_unique(TableShared& sh, const State& s, const Work& w, const uint2* buf, const uint2* spilled, const TableJob& job,
-                                 int count, unsigned long long* words, uint32_t tag, uint32_t* first, bool* ok) {
+__device__ uint32_t table_unique(TableShared& sh, const Work& w, const uint2* buf, const uint2* spilled, const TableJob& job, int count,
+                                 uint32_t* first) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
     constexpr int CHUNK = ITEMS * TBL_THREADS;
@@ -327,15 +328,12 @@ __device__ uint32_t table_unique(TableShared& sh, const State& s, const Work& w,
     const uint32_t U = __reduce_add_sync(0xffffffffU, in_block);
     const uint32_t before = __reduce_add_sync(0xffffffffU, lane < (int)job.rank ? in_block : 0u);
     if (job.rank == 0 && warp == 0) {
-        if (lane == 0) tile_publish(words, (uint32_t)job.t, U, tag);
-        bool poison;
-        const uint32_t b = tile_look_back(words, (uint32_t)job.t, U, tag, &poison);
-        if (lane < (int)job.blocks) {
-            if (job.blocks == 1) { sh.base[0] = b; sh.base[1] = poison; }
-            else peer_st2(sh.base, (uint32_t)lane, b, poison);
-        }
+        uint32_t b = 0;
+        if (lane == 0 && U) b = atomicAdd(&w.ctr->U, U + 1u);
+        b = __shfl_sync(0xffffffffU, b, 0);
+        if (lane < (int)job.blocks) { if (job.blocks == 1) sh.base = b; else peer_st(&sh.base, (uint32_t)lane, b); }
     }
-    // the samples in sorted order, while block 0 waits for the other tables
+    // the samples in sorted order, while block 0 takes the table's place
     for (int c0 = 0; c0 < count; c0 += CHUNK) {
         const int n = min(CHUNK, count - c0), items = (n + TBL_THREADS - 1) / TBL_THREADS;
         const uint32_t m = c0 == 0 ? edges1 : edges(c0, n, items);
@@ -345,10 +343,8 @@ __device__ uint32_t table_unique(TableShared& sh, const State& s, const Work& w,
         }
     }
     cluster_sync(job.blocks);
-    const uint32_t ubase = sh.base[0];
-    *ok = sh.base[1] == 0;
+    const uint32_t ubase = sh.base;
     *first = ubase;
-    if (!*ok) return U;
     uint32_t run = ubase + before;
     for (int c0 = 0; c0 < count; c0 += CHUNK) {
         const int n = min(CHUNK, count - c0), items = (n + TBL_THREADS - 1) / TBL_THREADS;
@@ -374,8 +370,8 @@ __device__ uint32_t table_unique(TableShared& sh, const State& s, const Work& w,
         }
     }
     if (job.rank == 0 && threadIdx.x == 0) {
-        w.ustart[job.t] = (int32_t)ubase;
-        if (job.t == s.T - 1) { w.ustart[s.T] = (int32_t)(ubase + U); w.seg[ubase + U] = job.start + job.n; w.ctr->U = ubase + U; }
+        w.ustart[job.t] = (int32_t)ubase; w.uend[job.t] = (int32_t)(ubase + U);
+        if (U) { w.uniq_row[ubase + U] = job.N; w.uniq_t[ubase + U] = job.t; w.seg[ubase + U] = job.start + job.n; }
     }
     return U;
 }
@@ -453,6 +449,7 @@ __device__ void table_state(TableShared& sh, int2* scratch, const State& s, cons
             }
         }
     }
+    if (threadIdx.x == 0 && U) { w.loc[ubase + U] = w.final_loc[ubase + U] = LOC_INVALID; w.cand_key[ubase + U] = CAND_NONE; }
     m_all = __reduce_add_sync(0xffffffffU, m_all); m_hit = __reduce_add_sync(0xffffffffU, m_hit);
     n_rows = __reduce_add_sync(0xffffffffU, n_rows); n_hit = __reduce_add_sync(0xffffffffU, n_hit);
     n_byp = __reduce_add_sync(0xffffffffU, n_byp);
@@ -489,8 +486,7 @@ __device__ void table_state(TableShared& sh, int2* scratch, const State& s, cons
 // clusters, most of it waiting, one set after the other).
 template <int ITEMS, bool STATE>
 __global__ void __launch_bounds__(TBL_THREADS, 1)
-k_table(State s, Work w, uint2* __restrict__ records, uint2* __restrict__ spill, unsigned long long* __restrict__ words, SortCtl* __restrict__ ctl,
-        uint32_t step, uint32_t epoch) {
+k_table(State s, Work w, uint2* __restrict__ records, uint2* __restrict__ spill, uint32_t step, uint32_t epoch) {
     extern __shared__ __align__(16) unsigned char table_smem[];
     uint2* buf = reinterpret_cast<uint2*>(table_smem);
     TableShared& sh = *reinterpret_cast<TableShared*>(table_smem + (size_t)ITEMS * TBL_THREADS * sizeof(uint2));
@@ -498,28 +494,10 @@ k_table(State s, Work w, uint2* __restrict__ records, uint2* __restrict__ spill,
     TableJob job;
     job.blocks = cluster_size(); job.rank = job.blocks == 1 ? 0u : cluster_rank();
     job.t = (int)(blockIdx.x / job.blocks);
-    if (threadIdx.x == 0) {
-        sh.n_heads = 0;
-        if (job.rank == 0) {
-            sh.base[0] = (ctl->seq + 1u) & SORT_TAG_MASK;                   // the pass number of this launch; moved on when every cluster is done
-            sh.base[1] = w.ctr->abort;                                      // an abandoned step: nothing to do, the same for the whole cluster
-            // a cluster waits for the tables before its own: drawn in the order in which clusters start, those are held by running ones
-            sh.table = atomicAdd(&ctl->ticket, 1u);
-        }
-    }
+    if (w.ctr->abort) return;                                  // an abandoned step: nothing to do, the same for every block
+    if (threadIdx.x == 0) sh.n_heads = 0;
     if (threadIdx.x < 8) sh.stats[threadIdx.x] = 0;
-    cluster_sync(job.blocks);
-    const uint32_t tag = job.blocks == 1 ? sh.base[0] : peer_ld(&sh.base[0], 0);
-    const bool off = (job.blocks == 1 ? sh.base[1] : peer_ld(&sh.base[1], 0)) != 0;
-    job.t = (int)(job.blocks == 1 ? sh.table : peer_ld(&sh.table, 0));
-    auto finished = [&]() {                                        // the cluster that finishes last ends the pass
-        if (job.rank == 0 && threadIdx.x == 0 && atomicAdd(&ctl->done, 1u) == (uint32_t)s.T - 1u) close_pass(ctl, tag);
-    };
-    if (off) {
-        cluster_sync(job.blocks);                                  // everybody has read block 0's words
-        finished();
-        return;
-    }
+    cluster_sync(job.blocks);                                  // the cluster's blocks have all begun: their shared memory can be written to
     job.start = w.table_start[job.t]; job.n = w.table_start[job.t + 1] - job.start;
     job.N = s.tables[job.t].N;
     job.q = max(32u, (((uint32_t)job.n + job.blocks - 1) / job.blocks + 31u) & ~31u);
@@ -534,17 +512,11 @@ k_table(State s, Work w, uint2* __restrict__ records, uint2* __restrict__ spill,
         spilled = records;
         table_sort_spilled<ITEMS>(sh, &spilled, spill, job, count, bits);
     }
-    bool ok;
     uint32_t ubase;
-    const uint32_t U = table_unique<ITEMS>(sh, s, w, buf, spilled, job, count, words, tag, &ubase, &ok);
-    if (!ok && threadIdx.x == 0) {                             // a look-back gave up: abandon the step
-        if (job.rank == 0) atomicAdd(&ctl->timeout, 1u);
-        w.ctr->abort = 1;
-    }
-    cluster_sync(job.blocks);                                  // the lists are complete
-    finished();
-    if (!ok) return;
-    if (STATE) table_state<2>(sh, reinterpret_cast<int2*>(buf), s, w, job, ubase, U, step, epoch);
+    const uint32_t U = table_unique<ITEMS>(sh, w, buf, spilled, job, count, &ubase);
+    if (!STATE) return;
+    __syncthreads();                                           // the lists are complete
+    table_state<2>(sh, reinterpret_cast<int2*>(buf), s, w, job, ubase, U, step, epoch);
 }
 
 }  // namespace mpe

@@ -152,3 +152,55 @@ def test_step_on_a_non_blocking_stream_straight_after_reserve(count):
     """The workspace grows between two steps of a stream that does not wait for the default one."""
     for seed in (6, 7):
         _ahead(_cfg([70001, 900], 64, seed=seed), [count // 3, count, count, 2 * count, 2 * count], torch.cuda.Stream(), 0)
+
+
+class _OneStepMore:
+    """A handle that has counted a step which the oracle never saw."""
+    def __init__(self, h):
+        self._h = h
+
+    def __getattr__(self, name):
+        return getattr(self._h, name)
+
+    def stats(self, t):
+        s = np.array(self._h.stats(t))
+        s[7] -= 1
+        return s
+
+
+def _abandon(cfg, counts, abandoned):
+    """Three steps; before the second one the look-backs of the next sort are made to give up."""
+    from paper_2010_11305_b200 import binding as mpe
+    from parity_util import compare_state, make_pair
+    h, o = make_pair(cfg)
+    rng = np.random.default_rng(cfg.seed)
+    every = range(cfg.num_tables)
+    for step in (1, 2, 3):
+        idx, off, grad = _batch(rng, [_skewed(rng, r, c) for r, c in zip(cfg.num_rows, counts)], cfg.batch, cfg.dim)
+        if step == 2:
+            h.selftest(mpe.SELFTEST_ABANDON_NEXT_SORT)
+        out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, device="cuda")
+        h.forward(torch.from_numpy(idx).cuda(), torch.from_numpy(off).cuda(), cfg.batch, out)
+        assert np.array_equal(out.cpu().numpy(), o.forward(idx, off, cfg.batch)), f"step {step}"
+        h.backward(torch.from_numpy(grad).cuda(), cfg.lr, step)
+        code, detail = h.last_error()
+        if step == 2 and abandoned:
+            assert code == mpe.ERR_TIMEOUT and detail > 0
+        else:
+            assert (code, detail) == (0, 0)
+            o.backward(grad, cfg.lr, step)
+        compare_state(_OneStepMore(h) if abandoned and step >= 2 else h, o, cfg, every, rng)
+    h.close()
+
+
+@pytest.mark.parametrize("policy,optimizer", [(wl.LFU, wl.ROWWISE_ADAGRAD), (wl.LRU, wl.SGD)])
+@pytest.mark.parametrize("counts", [(3000, 900, 0, 31), (8000, 7000), (20000, 90000)])
+def test_steps_sorted_inside_clusters_have_no_wait_that_could_abandon_them(counts, policy, optimizer):
+    """No table waits for another one, so a step cannot be left with some tables' priorities and caches changed and others' not."""
+    _abandon(_cfg([9000] * len(counts), 64, policy=policy, optimizer=optimizer), counts, abandoned=False)
+
+
+@pytest.mark.parametrize("policy,optimizer", [(wl.LFU, wl.ROWWISE_ADAGRAD), (wl.LRU, wl.SGD)])
+def test_a_step_whose_sort_is_abandoned_changes_nothing(policy, optimizer):
+    """Tables, caches, counters, accumulators and statistics stay as they were, and the next step goes on from there."""
+    _abandon(_cfg([90000, 900], 64, policy=policy, optimizer=optimizer), (302000, 500), abandoned=True)
