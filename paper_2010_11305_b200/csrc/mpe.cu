@@ -23,6 +23,9 @@ namespace {
 
 struct ProfRec { int name; cudaEvent_t a, b; };
 
+// How a batch's index work is done (table_plan)
+struct TablePlan { int blocks = 0; int items = 0; };
+
 }  // namespace
 
 struct mpe_handle {
@@ -59,6 +62,7 @@ struct mpe_handle {
         int64_t sort_n = 0;
         const uint32_t *skey = nullptr;
         std::vector<void*> allocs;
+        TablePlan plan;
         cudaEvent_t ev_free = nullptr, ev_keys = nullptr, ev_prep = nullptr;
         uint64_t bytes = 0;
     } alt;
@@ -90,6 +94,8 @@ struct mpe_handle {
     int32_t B = 0; int64_t L = 0;
     const uint32_t* skey = nullptr;         // the sorted keys of the current batch
     bool chain_done = false;                // the current batch has been sorted and its distinct rows are known
+    TablePlan plan;                         // ... by these kernels
+    volatile uint32_t* uneven_seen = nullptr;              // (pinned) what the kernels last found of how uneven the tables' segments are
     StepArgs args{};                        // the current call's arguments (passed by value when launching directly)
     Route* d_route = nullptr;               // destinations of the pooled vectors when the tables are spread over several GPUs
     bool graphs_enabled = true;             // accepted and remembered; see mpe_use_graphs
@@ -192,7 +198,7 @@ void swap_sets(mpe_handle* h) {
     std::swap(h->ghist, h->alt.ghist); std::swap(h->block_sums, h->alt.block_sums);
     std::swap(h->sort_status, h->alt.sort_status); std::swap(h->sort_ctl, h->alt.sort_ctl);
     std::swap(h->sort_n, h->alt.sort_n);
-    std::swap(h->skey, h->alt.skey);
+    std::swap(h->skey, h->alt.skey); std::swap(h->plan, h->alt.plan);
     std::swap(h->ws_allocs, h->alt.allocs);
     std::swap(h->ev_free, h->alt.ev_free); std::swap(h->ev_keys, h->alt.ev_keys); std::swap(h->ev_prep, h->alt.ev_prep);
     std::swap(h->ws_bytes, h->alt.bytes);
@@ -277,7 +283,7 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags, cudaStream_t first_use) {
     h->sort_n = (n + 3) & ~int64_t(3);
     A(h->sortA, 2 * h->sort_n); A(h->sortB, 2 * h->sort_n);
     A(h->block_sums, n / SCAN_TILE + 2);
-    A(w.table_start, T + 1); A(w.tile_base, T + 1); A(w.ustart, 2 * T + 1);
+    A(w.table_start, T + 1); A(w.tile_base, T + 1); A(w.ustart, 2 * T + 1);          // (both kinds of list ends, see Work)
     A(w.occ_b, n);
     A(w.uniq_row, nu); A(w.uniq_t, nu); A(w.seg, nu + 1); A(w.loc, nu); A(w.final_loc, nu);
     A(w.victim, nu); A(w.defer_k, nu); A(w.heads, nu);
@@ -292,13 +298,15 @@ int alloc_set(mpe_handle* h, int64_t L, int64_t bags, cudaStream_t first_use) {
     }
     uint8_t* base = nullptr;
     if ((rc = dmalloc(h, &base, total, tr)) != MPE_OK) return rc;
-    CK(h, cudaMemsetAsync(base, 0, (size_t)zeroed, first_use));
-    CK(h, cudaEventRecord(h->ev_prep, first_use));       // whoever prepares a batch here on another stream waits for this
+    uint8_t* const first = base;
     for (const Piece& x : pieces) {
         std::memcpy(x.p, &base, sizeof(base));
         base += (x.bytes + 255) / 256 * 256;
         h->ws_bytes += (uint64_t)x.bytes;
     }
+    CK(h, cudaMemsetAsync(first, 0, (size_t)zeroed, first_use));
+    CK(h, cudaMemcpyAsync(&w.ctr->uneven_seen, &h->uneven_seen, sizeof(h->uneven_seen), cudaMemcpyHostToDevice, first_use));
+    CK(h, cudaEventRecord(h->ev_prep, first_use));       // whoever prepares a batch here on another stream waits for this
     return MPE_OK;
 }
 
@@ -478,6 +486,8 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
     int rc = MPE_OK;
     auto fail = [&](int code) { mpe_destroy(h); return code; };
     if ((rc = dmalloc(h, &h->d_tables, num_tables, nullptr)) != MPE_OK) return fail(rc);
+    if (cudaHostAlloc((void**)&h->uneven_seen, sizeof(uint32_t), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) return fail(MPE_ERR_NOMEM);
+    *h->uneven_seen = 0;
     s.tables = h->d_tables;
     if (h->table_on_host) {
         // capacity tiering: the low-precision table stays in pinned host memory and is read and written in place over
@@ -559,21 +569,34 @@ int mpe_reserve(mpe_handle* h, int32_t max_batch, int64_t max_total_indices) {
 
 namespace {
 
-// How a step's index work is done.  Table by table, a cluster of `blocks` thread blocks each (mpe_table.cuh), if the tables'
-// segments are of a size for that; else (blocks == 0) by grid-wide kernels.
-// Only the average segment is known here.  A table with a larger one than its cluster's shared memory holds is sorted through
-// global memory by the same kernel: slower, not wrong.
-struct TablePlan { int blocks; int items; };
+// How a batch's index work is done.  Table by table, a cluster of `blocks` thread blocks each (mpe_table.cuh), if the tables'
+// segments are of a size for that; else (blocks == 0) by grid-wide kernels, whose time depends on the batch's size alone.
+// The host does not read a batch, so it goes by the average segment and by how much larger than the average the largest one was in
+// the batches before (tell_uneven; step_host_submit has this batch's offsets): a table that does not fit its cluster is sorted
+// through global memory by the cluster alone, which is right but slow.  Until a batch has been seen, and wherever the largest
+// table would need more than the clusters of all tables can be given at a time, the grid-wide kernels do it.
+// Step in us (1M rows of 32 INT8 values per table, LRU) going by the average alone / by this rule / with grid-wide kernels for
+// every batch (an earlier build): 26 tables, bags of 100 and 25 times 1, 16384 samples 1478 / 603 / 1078, 512 samples 725 / 182 / 202;
+// 26 tables, bags of 10, 5 and 24 times 1, 2048 samples 445 / 121 / 151; 64 tables, bags of 60 and 63 times 2, 1024 samples
+// 830 / 216 / 246; 8 tables, bags of 80 and 7 times 4, 4096 samples 311 / 270 / 353; even bags 56 / 56 / 111 (26 times 1, 2048 samples).
 constexpr int TBL_ITEMS_SMALL = 4, TBL_ITEMS_LARGE = 12;            // elements per thread: 4096 and 12288 per block
 constexpr int64_t TBL_MAX_SEGMENT = 150000;                         // average; sixteen blocks hold 196608
-TablePlan table_plan(const mpe_handle* h, int64_t L) {
+TablePlan table_plan(const mpe_handle* h, int64_t L, int64_t largest = -1) {
     const int64_t avg = (L + h->T - 1) / h->T;
-    if (avg > TBL_MAX_SEGMENT) return {0, 0};
+    if (largest < 0) {
+        const uint32_t seen = *h->uneven_seen;
+        if (seen == 0) return {};
+        largest = avg * seen / UNEVEN_ONE;
+    }
+    if (avg > TBL_MAX_SEGMENT || largest > TBL_MAX_SEGMENT) return {};
+    // batches vary a little: the average one by an eighth, a table that is larger than that by a sixteenth
+    const int64_t need = std::max(avg + avg / 8, largest + largest / 16);
     // about four elements per thread keep a block's phases short; more where the clusters would not fit the GPU side by side
     int blocks = 1;
-    while (blocks < TBL_MAX_CLUSTER && (int64_t)blocks * TBL_ITEMS_SMALL * TBL_THREADS < avg + avg / 8) blocks *= 2;
-    while (blocks > 1 && (int64_t)h->T * blocks > h->num_sms && (int64_t)(blocks / 2) * TBL_ITEMS_LARGE * TBL_THREADS >= avg + avg / 8) blocks /= 2;
-    const int items = (int64_t)blocks * TBL_ITEMS_SMALL * TBL_THREADS >= avg + avg / 8 ? TBL_ITEMS_SMALL : TBL_ITEMS_LARGE;
+    while (blocks < TBL_MAX_CLUSTER && (int64_t)blocks * TBL_ITEMS_SMALL * TBL_THREADS < need) blocks *= 2;
+    while (blocks > 1 && (int64_t)h->T * blocks > h->num_sms && (int64_t)(blocks / 2) * TBL_ITEMS_LARGE * TBL_THREADS >= need) blocks /= 2;
+    if (largest > 2 * avg && (int64_t)h->T * blocks > h->num_sms) return {};
+    const int items = (int64_t)blocks * TBL_ITEMS_SMALL * TBL_THREADS >= need ? TBL_ITEMS_SMALL : TBL_ITEMS_LARGE;
     return {blocks, items};
 }
 
@@ -600,7 +623,7 @@ int launch_table(mpe_handle* h, int blocks, const StepArgs& av) {
 }
 // the sort and the distinct rows; `state`: the priorities and the admission too (a cluster of one block)
 int enqueue_table(mpe_handle* h, const TablePlan& plan, const StepArgs& av, bool state) {
-    h->wk.uend = h->wk.ustart + h->T + 1;            // the tables' lists stand in any order
+    h->wk.end_at = h->T + 1;                         // the tables' lists stand in any order
     if (plan.items == TBL_ITEMS_LARGE) return launch_table<TBL_ITEMS_LARGE, false>(h, plan.blocks, av);
     return state ? launch_table<TBL_ITEMS_SMALL, true>(h, plan.blocks, av) : launch_table<TBL_ITEMS_SMALL, false>(h, plan.blocks, av);
 }
@@ -608,11 +631,11 @@ int enqueue_table(mpe_handle* h, const TablePlan& plan, const StepArgs& av, bool
 // What backward needs of the batch and the indices alone decide (no table, cache or policy state): the sorted batch and its
 // distinct rows.  The records to sort are in sort_input().  Launch sizes follow L, an upper bound of what the kernels read from
 // device memory.
-int enqueue_index_chain(mpe_handle* h, int64_t L) {
+int enqueue_index_chain(mpe_handle* h, int64_t L, const TablePlan& plan) {
     Work& w = h->wk;
-    const TablePlan plan = table_plan(h, L);
+    h->plan = plan;
     if (plan.blocks) return enqueue_table(h, plan, StepArgs{}, false);
-    w.uend = w.ustart + 1;                           // a table's distinct rows end where the next one's begin
+    w.end_at = 1;                                    // a table's distinct rows end where the next one's begin
     // sort the row indices of the mini-batch (Section 5.1), table by table
     seg_sort(h, sort_bufs(h), w.table_start, w.tile_base, bits_for((uint32_t)h->max_rows), L, reinterpret_cast<uint32_t*>(w.occ_b), &h->skey);
     // distinct rows
@@ -638,7 +661,7 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool chain) {
     const State& s = h->st;
     Work& w = h->wk;
     const StepArgs av = h->args;
-    const TablePlan plan = table_plan(h, L);
+    const TablePlan plan = chain ? table_plan(h, L) : h->plan;
     int rc = MPE_OK;
     // the hot rows' partial gradient sums: on a second stream, next to the kernels that leave most of the machine idle
     auto hot_partial = [&]() -> int {
@@ -666,7 +689,7 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool chain) {
         // (the cluster kernel leaves the hot rows to k_priority; the grid-wide kernels list them with the distinct rows, so that
         // their partial sums can start before it)
         const bool by_table = plan.blocks != 0;
-        if (chain) rc = enqueue_index_chain(h, L);
+        if (chain) rc = enqueue_index_chain(h, L, plan);
         if (rc == MPE_OK && !by_table) rc = hot_partial();
         LAUNCH_NEXT(h, "priority", k_priority, grid_for(h, L, PRI_CHUNK, 8), 256, 0, s, w, av, by_table ? 1 : 0);
         if (rc == MPE_OK && by_table) rc = hot_partial();
@@ -739,9 +762,9 @@ int forward_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
     return MPE_OK;
 }
 
-// see mpe_prepare in mpe.h
+// see mpe_prepare in mpe.h; `largest`: of the tables' segments, if the caller knows it
 int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offsets, int32_t batch, int64_t total_indices,
-                 cudaStream_t stream) {
+                 cudaStream_t stream, int64_t largest = -1) {
     const int64_t bags = (int64_t)h->T * batch;
     h->prepared = false;
     // only what fits the reserved workspace: otherwise the step simply does all of its work itself
@@ -766,7 +789,7 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
         LAUNCH(h, "prelude", k_prelude, 1, 32, 0, h->wk, h->T, av);
         LAUNCH(h, "make_keys", k_make_keys, grid_for(h, bags, 32, 8), 256, 0, h->st, h->wk, sort_input(sort_bufs(h)), av);
         e = cudaEventRecord(h->ev_keys, stream);
-        rc = enqueue_index_chain(h, total_indices);
+        rc = enqueue_index_chain(h, total_indices, table_plan(h, total_indices, largest));
         if (e == cudaSuccess) e = cudaEventRecord(h->ev_prep, stream);
     }
     if (rc == MPE_OK) rc = check_launch(h);
@@ -1063,7 +1086,9 @@ int mpe_step_host_submit(mpe_handle* h, const int32_t* h_indices, const int32_t*
     // the part of forward that needs the indices only starts as soon as they have arrived, beside whatever the previous
     // step still has to do
     CK(h, cudaStreamWaitEvent(h->prep, sl.ev_idx, 0));
-    int rc = prepare_impl(h, sl.idx, sl.off, batch, total_indices, h->prep);
+    int64_t largest = 0;                                                  // (inconsistent offsets are the kernels' business)
+    for (int t = 0; t < h->T; ++t) largest = std::max<int64_t>(largest, (int64_t)h_offsets[(int64_t)(t + 1) * batch] - h_offsets[(int64_t)t * batch]);
+    int rc = prepare_impl(h, sl.idx, sl.off, batch, total_indices, h->prep, largest);
     if (rc != MPE_OK) { cudaStreamSynchronize(h->copy_in); return rc; }
     CK(h, cudaStreamWaitEvent(st, sl.ev_idx, 0));
     if (sl.used) CK(h, cudaStreamWaitEvent(st, sl.ev_down, 0));           // the slot's previous output has left the device
@@ -1133,7 +1158,7 @@ int mpe_destroy(mpe_handle* h) {
     if (h->table_on_host) { cudaFreeHost(s.low.codes); cudaFreeHost(s.low.sb); cudaFree(s.home); }
     else if (h->row_records) cudaFree(h->row_records);
     else { cudaFree(s.low.codes); cudaFree(s.low.sb); cudaFree(s.home); }
-    cudaFree(h->d_route);
+    cudaFree(h->d_route); cudaFreeHost(const_cast<uint32_t*>(h->uneven_seen));
     cudaFree(h->d_tables); cudaFree(s.G); cudaFree(s.slab);
     cudaFree(s.tags); cudaFree(s.ts); cudaFree(s.hit_epoch); cudaFree(s.hit_k); cudaFree(s.floor); cudaFree(s.set_cnt); cudaFree(s.chain); cudaFree(s.bucket); cudaFree(s.stats);
     for (auto& r : h->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
@@ -1240,7 +1265,7 @@ int mpe_step_info(mpe_handle* h, int64_t* out6) {
     if (!h->wk.ctr) return MPE_OK;
     DeviceGuard guard(h->device);
     if (h->have_forward && !h->chain_done) {           // a forward alone does not sort its batch: the distinct rows are counted on demand
-        int rc = enqueue_index_chain(h, h->L);
+        int rc = enqueue_index_chain(h, h->L, table_plan(h, h->L));
         if (rc != MPE_OK) return rc;
         h->chain_done = true;
     }
@@ -1248,10 +1273,10 @@ int mpe_step_info(mpe_handle* h, int64_t* out6) {
     if (h->prep_running) CK(h, cudaEventSynchronize(h->ev_prep));
     Counters c;
     CK(h, cudaMemcpy(&c, h->wk.ctr, sizeof(c), cudaMemcpyDeviceToHost));
-    if (c.abort || !h->wk.uend) return MPE_OK;
+    if (c.abort || !h->wk.end_at) return MPE_OK;
     std::vector<int32_t> us(h->T), ue(h->T);
     CK(h, cudaMemcpy(us.data(), h->wk.ustart, sizeof(int32_t) * h->T, cudaMemcpyDeviceToHost));
-    CK(h, cudaMemcpy(ue.data(), h->wk.uend, sizeof(int32_t) * h->T, cudaMemcpyDeviceToHost));
+    CK(h, cudaMemcpy(ue.data(), h->wk.ustart + h->wk.end_at, sizeof(int32_t) * h->T, cudaMemcpyDeviceToHost));
     out4[0] = (int64_t)c.L - (int64_t)c.dropped;
     for (int t = 0; t < h->T; ++t) {
         out4[1] += ue[t] - us[t];

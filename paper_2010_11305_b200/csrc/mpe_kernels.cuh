@@ -50,6 +50,8 @@ struct Counters {
     unsigned long long dropped;      // out-of-range indices in this batch
     unsigned long long hot_occ;      // indices that belong to hot rows
     unsigned long long err[2];       // sticky: ERR_INDEX, ERR_OFFSETS
+    volatile uint32_t* uneven_seen;  // where tell_uneven tells the host (pinned host memory),
+    uint32_t uneven;       // and what it last did from this workspace
 };
 
 struct State {
@@ -96,7 +98,7 @@ struct StepArgs {
 struct Work {
     Counters* ctr;
     int32_t *table_start, *tile_base;            // [T+1]
-    int32_t *ustart, *uend;                      // [T] where each table's distinct rows are listed
+    int32_t* ustart;       // [T] where each table's distinct rows are listed from; ustart[end_at + t]: ... to
     int32_t* occ_b;        // [L] by sorted order: sample of the element; sign bit: last occurrence of its row
     int32_t *uniq_row, *uniq_t, *seg, *loc, *final_loc, *victim, *hot_base, *hot_left;   // per unique row
     int32_t* task_k;       // [hot tasks]
@@ -107,12 +109,25 @@ struct Work {
     int2* heads;           // [sets with candidates] {set of the concatenated cache, table}
     float* partial;        // [hot tasks][dim]
     int32_t sort_tile;     // keys per tile of the sorts of this workspace
+    int32_t end_at;        // see ustart
 };
 
 // the counters of a step, as its first kernel leaves them
 __device__ __forceinline__ void reset_step(Counters* c, uint32_t L, uint32_t abort, unsigned long long dropped) {
     c->L = L; c->U = 0; c->hot_rows = 0; c->hot_tasks = 0; c->mid_rows = 0; c->abort = abort; c->dropped = dropped; c->hot_occ = 0; c->deferred = 0;
     c->n_heads = 0; c->upd_next = 0;
+}
+
+// How much larger than the average the batch's largest segment is, in units of 1 / UNEVEN_ONE, for the host, which picks the kernels of
+// later index work by it (table_plan) and never reads the batch itself.  One lane; the store crosses the host link, so it is made only
+// when the figure rises or falls by a quarter.
+constexpr uint32_t UNEVEN_ONE = 64;
+__device__ __forceinline__ void tell_uneven(const Work& w, uint32_t largest, int T, uint32_t L) {
+    if (L == 0) return;
+    const uint32_t v = (uint32_t)ceilf((float)largest * (float)T * (float)UNEVEN_ONE / (float)L), told = w.ctr->uneven;
+    if (v <= told && 4 * v >= 3 * told) return;
+    w.ctr->uneven = v;
+    *w.ctr->uneven_seen = v;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -149,7 +164,8 @@ __global__ void k_prelude(Work w, int T, StepArgs a) {
         if (lane == 0) { c->abort = 1; atomicAdd(&c->err[ERR_OFFSETS], 1ULL); }
     }
     __syncwarp();
-    warp_tile_bases(w.table_start, T, w.tile_base, bad, w.sort_tile);     // the sort's tiles, table by table
+    const uint32_t largest = warp_tile_bases(w.table_start, T, w.tile_base, bad, w.sort_tile);     // the sort's tiles, table by table
+    if (lane == 0 && !bad) tell_uneven(w, largest, T, L);
 }
 
 // Records for the sort of a batch that is sorted ahead: the row id, or N_t for an id outside [0, N_t), and the sample;
@@ -366,7 +382,8 @@ __device__ __forceinline__ void forward_close(const State& s, const Work& w, con
             if (a.B == 0) for (int t = 0; t < s.T; ++t) w.table_start[t] = 0;
         }
         __syncwarp();
-        warp_tile_bases<true>(w.table_start, s.T, w.tile_base, nbad != 0, w.sort_tile);
+        const uint32_t largest = warp_tile_bases<true>(w.table_start, s.T, w.tile_base, nbad != 0, w.sort_tile);
+        if (threadIdx.x == 0 && !nbad) tell_uneven(w, largest, s.T, a.L);
     }
     if (nbad) {
         const int64_t row4 = (int64_t)s.T * s.dim / 4, total = (int64_t)a.B * row4;
@@ -380,7 +397,7 @@ __device__ __forceinline__ void forward_close(const State& s, const Work& w, con
             *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
-    if (threadIdx.x == 0) { c->fwd_bad = 0; c->fwd_done = 0; c->fwd_dropped = 0; }
+    if (threadIdx.x == 0) { c->fwd_bad = 0; c->fwd_done = 0; if (MODE == FWD_RECORD) c->fwd_dropped = 0; }
 }
 
 
@@ -917,7 +934,7 @@ k_policy(State s, Work w, StepArgs a) {
         const int2 head = w.heads[h];
         const int t = head.y;
         const TableDev tb = s.tables[t];
-        const int32_t ub = w.ustart[t], ue = w.uend[t];
+        const int32_t ub = w.ustart[t], ue = w.ustart[w.end_at + t];
         const PolicyCounts pc = policy_set<WAYS>(s, w, tb, head.x, ub, ue - ub, (uint32_t)a.step, a.epoch, gmask,
                                            gbase, way, scratch + grp * cap);
         if (way == 0) {

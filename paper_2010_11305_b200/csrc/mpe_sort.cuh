@@ -64,14 +64,16 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* t
 // tile_base[t] = number of tiles (of `tile` keys) of segments 0..t-1; tile_base[T] = total.  Called by one warp whose
 // lanes all take part; `off` (the step was abandoned) yields zero tiles, which turns the whole sort into a no-op.
 // FRESH: the starts were written by other blocks of the running kernel (read them from L2).
+// Returns the number of keys of the largest segment.
 template <bool FRESH = false>
-__device__ __forceinline__ void warp_tile_bases(const int32_t* seg_start, int T, int32_t* tile_base, bool off, int tile) {
+__device__ __forceinline__ uint32_t warp_tile_bases(const int32_t* seg_start, int T, int32_t* tile_base, bool off, int tile) {
     const int lane = threadIdx.x & 31;
-    int32_t run = 0;
+    int32_t run = 0, largest = 0;
     for (int t0 = 0; t0 < T; t0 += 32) {
         const int t = t0 + lane;
         int32_t len = 0;
         if (t < T && !off) len = FRESH ? __ldcg(seg_start + t + 1) - __ldcg(seg_start + t) : seg_start[t + 1] - seg_start[t];
+        largest = max(largest, len);
         const int32_t c = (len + tile - 1) / tile;
         int32_t inc = c;
 #pragma unroll
@@ -80,6 +82,7 @@ __device__ __forceinline__ void warp_tile_bases(const int32_t* seg_start, int T,
         run += __shfl_sync(0xffffffffU, inc, 31);
     }
     if (lane == 0) tile_base[T] = run;
+    return (uint32_t)__reduce_max_sync(0xffffffffU, largest);
 }
 
 __device__ __forceinline__ int find_segment(const int32_t* __restrict__ base, int T, int32_t v) {

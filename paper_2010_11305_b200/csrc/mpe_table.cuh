@@ -370,7 +370,7 @@ __device__ uint32_t table_unique(TableShared& sh, const Work& w, const uint2* bu
         }
     }
     if (job.rank == 0 && threadIdx.x == 0) {
-        w.ustart[job.t] = (int32_t)ubase; w.uend[job.t] = (int32_t)(ubase + U);
+        w.ustart[job.t] = (int32_t)ubase; w.ustart[w.end_at + job.t] = (int32_t)(ubase + U);
         if (U) { w.uniq_row[ubase + U] = job.N; w.uniq_t[ubase + U] = job.t; w.seg[ubase + U] = job.start + job.n; }
     }
     return U;

@@ -204,3 +204,61 @@ def test_steps_sorted_inside_clusters_have_no_wait_that_could_abandon_them(count
 def test_a_step_whose_sort_is_abandoned_changes_nothing(policy, optimizer):
     """Tables, caches, counters, accumulators and statistics stay as they were, and the next step goes on from there."""
     _abandon(_cfg([90000, 900], 64, policy=policy, optimizer=optimizer), (302000, 500), abandoned=True)
+
+
+def _planned(num_rows, seen, counts, busy, **kw):
+    """A step with `counts` indices per table after a step with `seen` (None: it is the handle's first).  `busy`: the GPU has other work
+    while the host chooses the kernels of the step, so that it knows of the earlier batches only.  Returns the kernels it chose."""
+    from parity_util import compare_state, make_pair
+    cfg = _cfg(num_rows, 16, **kw)
+    h, o = make_pair(cfg)
+    rng = np.random.default_rng(cfg.seed)
+    batches = [_batch(rng, [_skewed(rng, r, c) for r, c in zip(num_rows, cs)], cfg.batch, cfg.dim) for cs in (seen, counts) if cs]
+    dev = [tuple(torch.from_numpy(x).cuda() for x in b) for b in batches]
+    h.reserve(cfg.batch, max(b[0].size for b in batches))
+    for step, ((idx, off, grad), (d_idx, d_off, d_grad)) in enumerate(zip(batches, dev), start=1):
+        out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, device="cuda")
+        last = step == len(batches)
+        h.profile(last)
+        torch.cuda.synchronize()
+        if busy and last:
+            torch.cuda._sleep(40_000_000)
+        h.forward(d_idx, d_off, cfg.batch, out)
+        if not (busy and last):
+            torch.cuda.synchronize()
+        h.backward(d_grad, cfg.lr, step)
+        assert np.array_equal(out.cpu().numpy(), o.forward(idx, off, cfg.batch)), f"step {step}"
+        o.backward(grad, cfg.lr, step)
+    chosen = set(h.profile_read())
+    assert h.last_error() == (0, 0)
+    compare_state(h, o, cfg, range(cfg.num_tables), rng)
+    h.close()
+    return chosen
+
+
+@pytest.mark.parametrize("counts,kernel", [
+    ((3000,) * 5, "table"), ((3641, 3641, 10), "table"),            # one block per table
+    ((7000, 7000, 3000), "table_sort"),                             # several
+    ((20000, 10000) + (2000,) * 18, "table_sort"),                  # a larger one among small ones: all clusters grow with it
+    ((51200,) + (512,) * 25, "sort_scatter"),                       # one that would take more than the GPU has for each
+    ((512,) * 25 + (151000,), "sort_scatter"),                      # one that fits no cluster
+])
+def test_kernels_follow_the_largest_table_not_only_the_average(counts, kernel):
+    chosen = _planned([max(3, c // 3) for c in counts], counts, counts, busy=False)
+    assert kernel in chosen and len(chosen & {"table", "table_sort", "sort_scatter"}) == 1, chosen
+
+
+@pytest.mark.parametrize("counts", [(8000, 10, 0), (60000, 5, 5), (5000,) * 99 + (12289,), (199000, 900)])
+def test_a_table_larger_than_the_batches_before_let_expect(counts):
+    """Its cluster sorts it through global memory: one block, sixteen small ones, one large one, sixteen large ones."""
+    even = [max(1, sum(counts) // len(counts) - 100)] * len(counts)
+    num_rows = [max(3, c // 3) for c in counts]
+    num_rows[0] = 70001
+    assert _planned(num_rows, even, counts, busy=True) & {"table", "table_sort"}
+
+
+@pytest.mark.parametrize("counts", [(1,), (0, 0), (0, 1, 31, 33, 1023, 1025, 3000), (2048, 2049, 0), (4097,) * 30, (57000,)])
+def test_first_step_of_a_handle_has_no_earlier_batch_to_go_by(counts):
+    num_rows = [max(3, c // 3) for c in counts]
+    num_rows[0] = 70001
+    assert "sort_scatter" in _planned(num_rows, None, counts, busy=True)
