@@ -50,19 +50,29 @@ __device__ __forceinline__ uint32_t group_mask(int lanes_per_row) {
 
 // The four stored values of one lane (columns 4*sub .. 4*sub+3) are BITS*4 adjacent bits of the row: one byte (INT2),
 // one u16 (INT4), one u32 (INT8) or two u32 (FP16 table, BITS = 16); the lowest column sits in the lowest bits.
-// read-only loads of data that is used once (a low-precision row on its way to FP32): through the non-coherent path and
-// without taking a line of L1, which is better spent on the FP32 rows that many bags share
-__device__ __forceinline__ uint32_t ld_once_u8(const void* p) { uint32_t v; asm("ld.global.nc.L1::no_allocate.u8 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
-__device__ __forceinline__ uint32_t ld_once_u16(const void* p) { unsigned short v; asm("ld.global.nc.L1::no_allocate.u16 %0, [%1];" : "=h"(v) : "l"(p)); return v; }
-__device__ __forceinline__ uint32_t ld_once_u32(const void* p) { uint32_t v; asm("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
-__device__ __forceinline__ uint2 ld_once_u32x2(const void* p) { uint2 v; asm("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p)); return v; }
-__device__ __forceinline__ float2 ld_once_f32x2(const void* p) { float2 v; asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p)); return v; }
+// Loads of memory that the running kernel does not write, so that the compiler may move them past its stores.  Not through the
+// non-coherent path (ld.global.nc, __ldg): that one is for memory nobody writes while the kernel is resident, and a kernel launched by
+// LAUNCH_NEXT is resident while the one before it still writes.  ld_once_*: data that is used once (a low-precision row on its way
+// to FP32), without taking a line of L1, which is better spent on the FP32 rows that many bags share.
+__device__ __forceinline__ float4 ld_f32x4(const void* p) {
+    float4 v; asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p)); return v;
+}
+__device__ __forceinline__ int32_t ld_i32(const int32_t* p) { int32_t v; asm("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
+__device__ __forceinline__ uint32_t ld_once_u8(const void* p) { uint32_t v; asm("ld.global.L1::no_allocate.u8 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
+__device__ __forceinline__ uint32_t ld_once_u16(const void* p) { unsigned short v; asm("ld.global.L1::no_allocate.u16 %0, [%1];" : "=h"(v) : "l"(p)); return v; }
+__device__ __forceinline__ uint32_t ld_once_u32(const void* p) { uint32_t v; asm("ld.global.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
+__device__ __forceinline__ uint2 ld_once_u32x2(const void* p) { uint2 v; asm("ld.global.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p)); return v; }
+__device__ __forceinline__ float2 ld_once_f32x2(const void* p) { float2 v; asm("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p)); return v; }
 
 // First statement of every kernel that is launched by LAUNCH_NEXT: lets the kernel behind it in the stream be set up from now on,
-// and waits until the one before it has finished and its writes are visible.  Nothing of memory may be touched before.
-__device__ __forceinline__ void after_previous_kernel() {
+// and waits until the one before it has finished and its writes are visible.  Nothing of memory that another kernel writes may be
+// touched before.  Returns the thread's number, which the compiler takes for a result of the wait: addresses formed from it, and what
+// is loaded from there, cannot be moved in front of it, not even loads that may be moved past stores.
+__device__ __forceinline__ uint32_t after_previous_kernel() {
+    uint32_t thread = threadIdx.x;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" : "+r"(thread) :: "memory");
+    return thread;
 }
 
 // Where the low-precision rows are: codes and (scale, bias) of row r at codes + r * code_stride and sb + r * sb_stride.  On the GPU
@@ -127,7 +137,7 @@ __device__ __forceinline__ float4 decode4(uint2 qq, float2 p) {
     return fma4(p.x, x, make_float4(p.y, p.y, p.y, p.y));      // q * s + b
 }
 
-// RO = the table is not written by the running kernel, so the read-only data path may serve the loads
+// RO = the table is not written by the running kernel
 template <int BITS, bool RO>
 __device__ __forceinline__ float4 dequant4(const LowRows& low, int64_t grow, int sub) {
     float2 p = make_float2(1.0f, 0.0f);

@@ -344,7 +344,7 @@ template <int BITS, bool RO>
 __device__ __forceinline__ float4 fetch4(const State& s, const TableDev& tb, int32_t row, int loc, int sub) {
     if (loc >= 0) {
         const float4* src = reinterpret_cast<const float4*>(s.slab + (int64_t)loc * s.dim) + sub;
-        return RO ? __ldg(src) : *src;
+        return RO ? ld_f32x4(src) : *src;
     }
     return dequant4<BITS, RO>(s.low, tb.row_base + row, sub);
 }
@@ -408,21 +408,21 @@ __device__ __forceinline__ void forward_close(const State& s, const Work& w, con
 template <int BITS, int LANES, int MODE>
 __global__ void __launch_bounds__(256, 4)
 k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
-    after_previous_kernel();
-    const int32_t* __restrict__ indices = a.indices;
-    const int32_t* __restrict__ offsets = a.offsets;
-    float* __restrict__ out = a.out;
+    const uint32_t thread = after_previous_kernel();
+    const int32_t* indices = a.indices;
+    const int32_t* offsets = a.offsets;
+    float* out = a.out;
     const int B = a.B;
     const int32_t L = (int32_t)a.L;
     constexpr int NB = LANES < 4 ? LANES : 4;        // rows per batch; two batches are in flight
     constexpr int dim = 4 * LANES;
-    const int sub = threadIdx.x & (LANES - 1);
-    const int gbase = (threadIdx.x & 31) & ~(LANES - 1);
+    const int sub = thread & (LANES - 1);
+    const int gbase = (thread & 31) & ~(LANES - 1);
     const uint32_t gmask = group_mask(LANES);
     const int64_t nbags = (int64_t)s.T * B;
     const int64_t gpb = blockDim.x / LANES, ng = gpb * gridDim.x;
     const char* slab_col = reinterpret_cast<const char*>(s.slab) + 16 * sub;
-    const int64_t bag0 = blockIdx.x * gpb + threadIdx.x / LANES;
+    const int64_t bag0 = blockIdx.x * gpb + thread / LANES;
     int t = (int)(bag0 / B), b = (int)(bag0 - (int64_t)t * B);
     const int32_t* off = offsets + bag0;             // of the bag whose offsets are fetched next
     int32_t to_fetch = bag0 < nbags ? (int32_t)((nbags - bag0 + ng - 1) / ng) : 0, to_pool = to_fetch;
@@ -431,19 +431,19 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
     int32_t lo0, hi0, lo1, hi1;                      // this bag's range and the next one's
     auto next_range = [&](int32_t* lo, int32_t* hi) {
         *lo = *hi = 0;
-        if (to_fetch > 0) { *lo = off[0]; *hi = off[1]; off += ng; --to_fetch; }
+        if (to_fetch > 0) { *lo = ld_i32(off); *hi = ld_i32(off + 1); off += ng; --to_fetch; }
     };
     auto check_range = [&](int32_t* lo, int32_t* hi) {       // a bag whose offsets make no sense is not read
         if (*lo < 0 || *hi < *lo || *hi > L) { bad_offsets = true; *lo = *hi = 0; }
     };
     next_range(&lo0, &hi0);
     check_range(&lo0, &hi0);
-    int32_t row0 = lo0 + sub < hi0 ? indices[lo0 + sub] : 0;
+    int32_t row0 = lo0 + sub < hi0 ? ld_i32(indices + lo0 + sub) : 0;
     next_range(&lo1, &hi1);
     auto slot_at = [&](const TableDev& tb, int32_t row, bool live) {
         if (!live) return LOC_INVALID;
         if (row < 0 || row >= tb.N) { ++bad_rows; return LOC_INVALID; }
-        return __ldg(slot_of(s, tb.row_base + row));
+        return ld_i32(slot_of(s, tb.row_base + row));
     };
     auto record = [&](const TableDev& tb, int32_t p, int32_t row) {
         if (MODE == FWD_RECORD) __stcs(pairs + p, make_uint2(row < 0 || row >= tb.N ? (uint32_t)tb.N : (uint32_t)row, (uint32_t)b));
@@ -459,7 +459,7 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
         // the next bag's first row ids are on their way while this bag is pooled, and the offsets of the one after it
         check_range(&lo1, &hi1);
         lo0 = lo1; hi0 = hi1;
-        row0 = lo0 + sub < hi0 ? indices[lo0 + sub] : 0;
+        row0 = lo0 + sub < hi0 ? ld_i32(indices + lo0 + sub) : 0;
         next_range(&lo1, &hi1);
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         // one row: cache resident -> the FP32 row; uncached -> up-convert the codes; out of range -> +0 (never changes the sum)
@@ -467,7 +467,7 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
             const int lc = __shfl_sync(gmask, myloc, gbase + src_lane);
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
             if (lc >= 0) {
-                x = __ldg(reinterpret_cast<const float4*>(slab_col + (size_t)(uint32_t)lc * (size_t)(dim * 4)));
+                x = ld_f32x4(slab_col + (size_t)(uint32_t)lc * (size_t)(dim * 4));
             } else if (lc == LOC_MISS) {
                 const int32_t rw = __shfl_sync(gmask, myrow, gbase + src_lane);
                 x = dequant4<BITS, true>(s.low, row_base + rw, sub);
@@ -476,12 +476,12 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
         };
         auto fetch_hit = [&](int src_lane) {          // the row is known to be cache resident
             const uint32_t lc = (uint32_t)__shfl_sync(gmask, myloc, gbase + src_lane);
-            return __ldg(reinterpret_cast<const float4*>(slab_col + (size_t)lc * (size_t)(dim * 4)));
+            return ld_f32x4(slab_col + (size_t)lc * (size_t)(dim * 4));
         };
         for (int32_t p0 = clo; p0 < chi; p0 += LANES) {
             if (p0 > clo) {                           // later windows of a long bag
                 const bool live = p0 + sub < chi;
-                myrow = live ? indices[p0 + sub] : 0;
+                myrow = live ? ld_i32(indices + p0 + sub) : 0;
                 myloc = slot_at(tb, myrow, live);
                 if (live) record(tb, p0 + sub, myrow);
             }
@@ -525,7 +525,7 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
         }
         float* dst = out + ((int64_t)b * s.T + t) * dim;
         if (a.route) {                                // the owner of sample b gets the vector, straight into its buffer
-            const Route* __restrict__ r = a.route;
+            const Route* r = a.route;
             const int g = b / r->B_local;
             dst = r->out[g] + ((int64_t)(b - g * r->B_local) * r->T_global + r->t_base + t) * dim;
         }
@@ -534,7 +534,7 @@ k_pool(State s, Work w, uint2* __restrict__ pairs, StepArgs a) {
         while (nb >= B) { nb -= B; ++t; }
         b = (int)nb;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0 && (offsets[0] != 0 || offsets[nbags] != L)) bad_offsets = true;
+    if (blockIdx.x == 0 && thread == 0 && (ld_i32(offsets) != 0 || ld_i32(offsets + nbags) != L)) bad_offsets = true;
     forward_close<MODE>(s, w, a, bad_offsets, bad_rows);
 }
 
@@ -956,7 +956,7 @@ k_policy(State s, Work w, StepArgs a) {
 // gcol points at the group's lane-th float4 of column block t; stride_bytes is the size of one sample's row of grad_out.
 // FULL: the chunk has all 32 (most chunks of a hot row do): no bounds to check.
 template <int LANES, bool FULL>
-__device__ __forceinline__ float4 sum_chunk_of(const int32_t* __restrict__ occ_b, const char* __restrict__ gcol, uint32_t stride_bytes,
+__device__ __forceinline__ float4 sum_chunk_of(const int32_t* occ_b, const char* gcol, uint32_t stride_bytes,
                                                int32_t first, int len, uint32_t gmask, int gbase, int sub) {
     if (FULL) len = 32;
     constexpr int NW = LANES >= 4 ? 32 / LANES : 1;        // groups of one or two lanes read the ids one by one
@@ -970,7 +970,7 @@ __device__ __forceinline__ float4 sum_chunk_of(const int32_t* __restrict__ occ_b
         const uint32_t b = LANES >= 4 ? __shfl_sync(gmask, id[LANES >= 4 ? u / LANES : 0], gbase + (u & (LANES - 1)))
                                       : (uint32_t)occ_b[first + min(u, len - 1)] & 0x7fffffffu;
         float4 v = make_float4(NZ, NZ, NZ, NZ);
-        if (FULL || u < len) v = __ldg(reinterpret_cast<const float4*>(gcol + (size_t)b * stride_bytes));
+        if (FULL || u < len) v = ld_f32x4(gcol + (size_t)b * stride_bytes);
         return v;
     };
     float4 va[4], vb[4], acc;
@@ -1001,7 +1001,7 @@ __device__ __forceinline__ float4 sum_chunk_of(const int32_t* __restrict__ occ_b
 }
 
 template <int LANES>
-__device__ __forceinline__ float4 sum_chunk(const int32_t* __restrict__ occ_b, const char* __restrict__ gcol, uint32_t stride_bytes,
+__device__ __forceinline__ float4 sum_chunk(const int32_t* occ_b, const char* gcol, uint32_t stride_bytes,
                                             int32_t first, int len, uint32_t gmask, int gbase, int sub) {
     return len == 32 ? sum_chunk_of<LANES, true>(occ_b, gcol, stride_bytes, first, len, gmask, gbase, sub)
                      : sum_chunk_of<LANES, false>(occ_b, gcol, stride_bytes, first, len, gmask, gbase, sub);
@@ -1028,7 +1028,7 @@ __device__ __forceinline__ float4 tree_reduce(const Term& term, int64_t first, i
 // sum is left with group 0.
 constexpr int HOT_THREADS = 256;
 template <int LANES>
-__device__ __forceinline__ float4 hot_task_sum(const State& s, const Work& w, const float* __restrict__ grad, uint32_t task, int32_t k, float* chunk_sums /* [32][dim] */) {
+__device__ __forceinline__ float4 hot_task_sum(const State& s, const Work& w, const float* grad, uint32_t task, int32_t k, float* chunk_sums /* [32][dim] */) {
     constexpr int dim = 4 * LANES, ngrp = HOT_THREADS / LANES;
     const int sub = threadIdx.x & (LANES - 1), grp = threadIdx.x / LANES;
     const int gbase = (threadIdx.x & 31) & ~(LANES - 1);

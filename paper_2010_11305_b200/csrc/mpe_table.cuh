@@ -159,7 +159,7 @@ __device__ __forceinline__ void table_digit_starts(TableShared& sh, const TableJ
 // registers and puts it in order within the block; the blocks exchange their digit counts; then the piece goes out to wherever it
 // belongs in runs of equal digits (single keys scattered over sixteen blocks' memories took 3.7 us a pass, runs take 1).
 template <int ITEMS>
-__device__ void table_sort(TableShared& sh, uint2* buf, const uint2* __restrict__ records, const TableJob& job, int count, int bits) {
+__device__ void table_sort(TableShared& sh, uint2* buf, const uint2* records, const TableJob& job, int count, int bits) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int passes = (bits + TBL_RADIX_BITS - 1) / TBL_RADIX_BITS, width = max(1, (bits + passes - 1) / passes);
     const uint32_t mask = (1u << width) - 1u;
@@ -486,7 +486,7 @@ __device__ void table_state(TableShared& sh, int2* scratch, const State& s, cons
 // clusters, most of it waiting, one set after the other).
 template <int ITEMS, bool STATE>
 __global__ void __launch_bounds__(TBL_THREADS, 1)
-k_table(State s, Work w, uint2* __restrict__ records, uint2* __restrict__ spill, uint32_t step, uint32_t epoch) {
+k_table(State s, Work w, uint2* records, uint2* spill, uint32_t step, uint32_t epoch) {
     extern __shared__ __align__(16) unsigned char table_smem[];
     uint2* buf = reinterpret_cast<uint2*>(table_smem);
     TableShared& sh = *reinterpret_cast<TableShared*>(table_smem + (size_t)ITEMS * TBL_THREADS * sizeof(uint2));

@@ -84,3 +84,20 @@ def test_device_memory_is_cleared_in_front_of_its_first_use():
     bench = open(os.path.join(ROOT, "bench.py")).read()
     made, switched = bench.index("stream_gen.batch(s) for s in"), bench.index("torch.cuda.set_stream(")
     assert "torch.cuda.synchronize(" in bench[made:switched]           # the batches are made on the default stream
+
+
+def _source(name):
+    return open(os.path.join(ROOT, "paper_2010_11305_b200", "csrc", name)).read()
+
+
+def test_kernels_set_up_beside_their_predecessor_load_through_the_coherent_path():
+    """A kernel that begins with after_previous_kernel() is resident while the kernel before it still writes; ld.global.nc and __ldg
+    are for memory nobody writes meanwhile.  The one place left is k_update, which is launched when all before it has finished."""
+    text = {f: _source(f) for f in ("mpe_device.cuh", "mpe_sort.cuh", "mpe_kernels.cuh", "mpe_table.cuh")}
+    code = "".join(re.sub(r"//[^\n]*", "", t) for t in text.values())
+    assert "ld.global.nc" not in code and code.count("__ldg(") == 1
+    kernels = re.sub(r"//[^\n]*", "", text["mpe_kernels.cuh"])
+    at = kernels.index("__ldg(")
+    assert "k_update(State s" in kernels[kernels.rindex("__global__", 0, at):at]
+    launched = set(re.findall(r'LAUNCH_NEXT\(h, "[a-z]+", (\w+)', _source("mpe.cu")))
+    assert launched == {"kern", "k_priority"}                          # k_pool, k_update_small, k_priority (and k_table, by launch_table)

@@ -262,3 +262,73 @@ def test_first_step_of_a_handle_has_no_earlier_batch_to_go_by(counts):
     num_rows = [max(3, c // 3) for c in counts]
     num_rows[0] = 70001
     assert "sort_scatter" in _planned(num_rows, None, counts, busy=True)
+
+
+@pytest.mark.parametrize("count,rows,steps,ahead", [(700, 3000, 150, False), (30000, 40000, 60, True), (160000, 60000, 30, True)])
+def test_forward_behind_a_backward_reads_what_that_one_wrote(count, rows, steps, ahead):
+    """The forward's blocks may be on the GPU before the last kernel of the step before has finished.  A second forward of the same
+    batch, behind a wait, must give the same values to the bit."""
+    from paper_2010_11305_b200 import binding as mpe
+    T, dim, B = 3, 32, 64
+    rng = np.random.default_rng(count)
+    h = mpe.Mpe([rows] * T, dim, 4, 0.05, 4, mpe.LFU, seed=5)
+    batches = [tuple(torch.from_numpy(x).cuda() for x in _batch(rng, [_skewed(rng, rows, count) for _ in range(T)], B, dim)) for _ in range(4)]
+    h.reserve(B, T * count)
+    outs = torch.zeros(2, B, T * dim, device="cuda")
+    wrong = torch.zeros(1, dtype=torch.int64, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for step in range(1, steps + 1):
+        idx, off, grad = batches[step % 4]
+        h.forward(idx, off, B, outs[0])
+        if ahead:
+            side.wait_stream(torch.cuda.current_stream())
+            h.prepare(batches[(step + 1) % 4][0], batches[(step + 1) % 4][1], B, side.cuda_stream)
+        h.backward(grad, 0.5, step)
+        if step % 5 == 0:                             # the next batch once more: behind the backward, then behind a wait
+            nxt = batches[(step + 1) % 4]
+            h.forward(nxt[0], nxt[1], B, outs[0])
+            torch.cuda.synchronize()
+            h.forward(nxt[0], nxt[1], B, outs[1])
+            wrong += (outs[0] != outs[1]).sum()
+    assert int(wrong) == 0 and h.last_error() == (0, 0)
+    h.close()
+
+
+@pytest.mark.parametrize("what", ["event", "copy"])
+def test_forward_waits_for_what_the_caller_put_in_front_of_it(what):
+    """Between a backward, whose last kernel lets the next one be set up early, and the next forward the caller makes the stream wait
+    for another one that writes the batch, or copies the batch in."""
+    from parity_util import make_pair
+    cfg = _cfg([3000, 500], 64, dim=16)
+    h, o = make_pair(cfg)
+    rng = np.random.default_rng(1)
+    batches = [_batch(rng, [_skewed(rng, n, 400) for n in cfg.num_rows], cfg.batch, cfg.dim) for _ in range(12)]
+    pinned = [tuple(torch.from_numpy(x).pin_memory() for x in b) for b in batches]
+    dev = [tuple(torch.from_numpy(x).cuda() for x in b) for b in batches]
+    idx, off, grad = (torch.zeros_like(x) for x in dev[0])
+    big, big_host = torch.empty(1 << 23, device="cuda"), torch.empty(1 << 23).pin_memory()
+    outs = [torch.empty(cfg.batch, cfg.num_tables * cfg.dim, device="cuda") for _ in batches]
+    own, other = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(own):
+        for k in range(len(batches)):
+            if what == "event":
+                other.wait_stream(own)
+                with torch.cuda.stream(other):
+                    torch.cuda._sleep(500_000)
+                    for to, frm in zip((idx, off, grad), dev[k]):
+                        to.copy_(frm)
+                own.wait_stream(other)
+            else:
+                big.copy_(big_host, non_blocking=True)
+                for to, frm in zip((idx, off, grad), pinned[k]):
+                    to.copy_(frm, non_blocking=True)
+            h.forward(idx, off, cfg.batch, outs[k], own.cuda_stream)
+            h.backward(grad, cfg.lr, k + 1)
+    torch.cuda.synchronize()
+    assert h.last_error() == (0, 0)
+    for k, b in enumerate(batches):
+        assert np.array_equal(outs[k].cpu().numpy(), o.forward(b[0], b[1], cfg.batch)), f"step {k + 1}"
+        o.backward(b[2], cfg.lr, k + 1)
+    h.close()
