@@ -84,6 +84,7 @@ struct mpe_handle {
     uint64_t submitted = 0;
     // step state
     cudaStream_t stream = nullptr;
+    bool stream_waits = false;              // the handle's stream has been made to wait for an event since its last kernel
     cudaStream_t side = nullptr;            // runs the hot rows' partial sums next to the policy kernels
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStream_t copy_in = nullptr, copy_out = nullptr;   // mpe_step_host: host<->device copies next to the kernels
@@ -131,10 +132,15 @@ int prof_name(mpe_handle* h, const char* name) {
     return (int)h->prof_names.size() - 1;
 }
 
+// the handle's stream waits for an event
+cudaError_t wait_event(mpe_handle* h, cudaEvent_t e) { h->stream_waits = true; return cudaStreamWaitEvent(h->stream, e, 0); }
+
 struct LaunchScope {
     mpe_handle* h; cudaStream_t st; ProfRec rec{};
+    bool behind_kernel = true;              // what comes before it on its stream, as far as this handle knows, is a kernel
     LaunchScope(mpe_handle* h_, const char* name, cudaStream_t st_) : h(h_), st(st_) {
         ++h->launches;
+        if (st == h->stream) { behind_kernel = !h->stream_waits; h->stream_waits = false; }
         if (h->profiling) { rec.name = prof_name(h, name); rec.a = get_event(h); rec.b = get_event(h); cudaEventRecord(rec.a, st); }
     }
     ~LaunchScope() { if (h->profiling) { cudaEventRecord(rec.b, st); h->prof_recs.push_back(rec); } }
@@ -147,6 +153,8 @@ struct LaunchScope {
 // 37.5 -> 33.9 us, 26 tables of one id 51.1 -> 46.2 us, a small static forward 11.6 -> 9.6 us.
 // Not for the kernels that a step's other streams run beside (the policy, the row updates, the grid-wide sort): waiting blocks keep
 // the hot rows' sums and the next batch's sort off the SMs (configuration 4 5.2 -> 5.6 ms, 13 tables of FP16 rows 149 -> 151 us).
+// What such a kernel waits for by itself is the kernel before it, and with that all that kernel waited for.  So it is launched plainly
+// behind an event that this library makes the stream wait for (a batch prepared on another stream).
 template <class... K, class... A>
 void launch_next(mpe_handle* h, cudaStream_t st, const char* name, void (*kern)(K...), int grid, int block, size_t smem, A... args) {
     LaunchScope ls(h, name, st);
@@ -155,7 +163,7 @@ void launch_next(mpe_handle* h, cudaStream_t st, const char* name, void (*kern)(
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cfg.attrs = &attr; cfg.numAttrs = ls.behind_kernel ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);       // a failure is what check_launch finds
 }
 #define LAUNCH_NEXT(h, name, kern, grid, block, smem, ...) launch_next(h, (h)->stream, name, kern, grid, block, smem, __VA_ARGS__)
@@ -611,13 +619,14 @@ int launch_table(mpe_handle* h, int blocks, const StepArgs& av) {
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3((unsigned)(h->T * blocks)); cfg.blockDim = dim3(TBL_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = h->stream;
-    cfg.attrs = attr; cfg.numAttrs = 2;
+    cfg.attrs = attr;
     if (!h->table_ready.count(reinterpret_cast<const void*>(kern))) {
         CK(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         CK(h, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         h->table_ready.insert(reinterpret_cast<const void*>(kern));
     }
     LaunchScope ls(h, STATE ? "table" : "table_sort", h->stream);
+    cfg.numAttrs = ls.behind_kernel ? 2 : 1;
     CK(h, cudaLaunchKernelEx(&cfg, kern, h->st, h->wk, sort_input(sort_bufs(h)), reinterpret_cast<uint2*>(h->sortA), (uint32_t)av.step, av.epoch));
     return MPE_OK;
 }
@@ -707,7 +716,7 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool chain) {
         auto lst = k_update_list<BITS, LANES>;
         auto upd = k_update<BITS, LANES>;
         LAUNCH(h, "update", upd, gu, UPD_WARPS * 32, UPD_SMEM, s, w, av);
-        cudaStreamWaitEvent(h->stream, h->ev_join, 0);
+        wait_event(h, h->ev_join);
         LAUNCH(h, "update_hot", lst, gh, 256, 0, s, w, (const int32_t*)w.hot_k, (const uint32_t*)&w.ctr->hot_rows, 0, av);
         // a resident row that was touched in this step is never displaced under LRU, unless it is the set's only way
         if (h->max_sets > 0 && (h->policy == MPE_LFU || h->ways == 1))
@@ -720,7 +729,7 @@ int enqueue_backward(mpe_handle* h, int64_t L, bool chain) {
 int await_prepared(mpe_handle* h) {
     if (!h->prep_running) return MPE_OK;
     h->prep_running = false;
-    CK(h, cudaStreamWaitEvent(h->stream, h->ev_prep, 0));
+    CK(h, wait_event(h, h->ev_prep));
     return MPE_OK;
 }
 
@@ -746,7 +755,7 @@ int forward_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
         h->prepared = false;
         swap_sets(h);
         // pooling needs nothing of it, only the caller's indices must have been read; backward waits for the rest
-        CK(h, cudaStreamWaitEvent(h->stream, h->ev_keys, 0));
+        CK(h, wait_event(h, h->ev_keys));
         h->prep_running = true;
         enqueue_pool<FWD_PREPARED>(h, h->wk, nullptr, bags, h->args);
         h->chain_done = true;
@@ -781,10 +790,11 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
     StepArgs av{};
     av.indices = d_indices; av.offsets = d_offsets; av.B = batch; av.L = (uint32_t)total_indices;
     cudaStream_t user = h->stream;
+    const bool user_waits = h->stream_waits;
     swap_sets(h);
     h->stream = stream;
-    cudaError_t e = cudaStreamWaitEvent(stream, h->ev_free, 0);       // the step that used this workspace last has finished,
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, h->ev_prep, 0);   // and so has a batch that was prepared in it and discarded
+    cudaError_t e = wait_event(h, h->ev_free);                        // the step that used this workspace last has finished,
+    if (e == cudaSuccess) e = wait_event(h, h->ev_prep);              // and so has a batch that was prepared in it and discarded
     if (e == cudaSuccess) {
         LAUNCH(h, "prelude", k_prelude, 1, 32, 0, h->wk, h->T, av);
         LAUNCH(h, "make_keys", k_make_keys, grid_for(h, bags, 32, 8), 256, 0, h->st, h->wk, sort_input(sort_bufs(h)), av);
@@ -793,7 +803,7 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
         if (e == cudaSuccess) e = cudaEventRecord(h->ev_prep, stream);
     }
     if (rc == MPE_OK) rc = check_launch(h);
-    h->stream = user;
+    h->stream = user; h->stream_waits = user_waits;
     swap_sets(h);
     if (e != cudaSuccess) { h->last_cuda_error = (int)e; return MPE_ERR_CUDA; }
     if (rc != MPE_OK) return rc;
@@ -1090,15 +1100,15 @@ int mpe_step_host_submit(mpe_handle* h, const int32_t* h_indices, const int32_t*
     for (int t = 0; t < h->T; ++t) largest = std::max<int64_t>(largest, (int64_t)h_offsets[(int64_t)(t + 1) * batch] - h_offsets[(int64_t)t * batch]);
     int rc = prepare_impl(h, sl.idx, sl.off, batch, total_indices, h->prep, largest);
     if (rc != MPE_OK) { cudaStreamSynchronize(h->copy_in); return rc; }
-    CK(h, cudaStreamWaitEvent(st, sl.ev_idx, 0));
-    if (sl.used) CK(h, cudaStreamWaitEvent(st, sl.ev_down, 0));           // the slot's previous output has left the device
+    CK(h, wait_event(h, sl.ev_idx));
+    if (sl.used) CK(h, wait_event(h, sl.ev_down));                        // the slot's previous output has left the device
     rc = mpe_forward(h, sl.idx, sl.off, batch, total_indices, sl.out, (void*)st);
     if (rc != MPE_OK) { cudaStreamSynchronize(h->copy_in); return rc; }
     CK(h, cudaEventRecord(sl.ev_fwd, st));
     CK(h, cudaStreamWaitEvent(h->copy_out, sl.ev_fwd, 0));
     if (nout) CK(h, cudaMemcpyAsync(h_out, sl.out, sizeof(float) * nout, cudaMemcpyDeviceToHost, h->copy_out));
     CK(h, cudaEventRecord(sl.ev_down, h->copy_out));
-    CK(h, cudaStreamWaitEvent(st, sl.ev_grad, 0));
+    CK(h, wait_event(h, sl.ev_grad));
     rc = mpe_backward(h, sl.grad, lr, step);
     if (rc != MPE_OK) { cudaStreamSynchronize(h->copy_in); cudaStreamSynchronize(st); h->have_forward = false; return rc; }
     CK(h, cudaEventRecord(sl.ev_done, st));

@@ -101,3 +101,10 @@ def test_kernels_set_up_beside_their_predecessor_load_through_the_coherent_path(
     assert "k_update(State s" in kernels[kernels.rindex("__global__", 0, at):at]
     launched = set(re.findall(r'LAUNCH_NEXT\(h, "[a-z]+", (\w+)', _source("mpe.cu")))
     assert launched == {"kern", "k_priority"}                          # k_pool, k_update_small, k_priority (and k_table, by launch_table)
+
+
+def test_waits_of_the_step_stream_are_known_to_its_launches():
+    """A kernel behind an event the library makes the step's stream wait for is launched plainly: such waits go through one place."""
+    src = _source("mpe.cu")
+    assert src.count("cudaStreamWaitEvent(h->stream") == 1 and src.count("cudaStreamWaitEvent(st,") == 0
+    assert src.count("ls.behind_kernel ?") == 2
