@@ -269,7 +269,8 @@ int mpe_selftest(mpe_handle* h, int32_t which);
 /* Geometry of table `table`'s cache. */
 int mpe_cache_geometry(mpe_handle* h, int32_t table, int32_t* n_sets, int32_t* ways);
 /* Figures of the last step: out6 = {valid indices, distinct rows, dropped indices, rows whose gradient
- * is summed by the multi-block tree (more than 256 occurrences), indices that belong to such rows,
+ * is summed by the multi-block tree (more than 256 occurrences, more than 64 in steps of at most 2^20
+ * indices), indices that belong to such rows,
  * newcomers that had to wait for the write-back of a row updated in the same step (known after
  * mpe_backward)}. */
 int mpe_step_info(mpe_handle* h, int64_t* out6);

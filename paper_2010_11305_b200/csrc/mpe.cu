@@ -1288,12 +1288,25 @@ int mpe_step_info(mpe_handle* h, int64_t* out6) {
     CK(h, cudaMemcpy(us.data(), h->wk.ustart, sizeof(int32_t) * h->T, cudaMemcpyDeviceToHost));
     CK(h, cudaMemcpy(ue.data(), h->wk.ustart + h->wk.end_at, sizeof(int32_t) * h->T, cudaMemcpyDeviceToHost));
     out4[0] = (int64_t)c.L - (int64_t)c.dropped;
+    // the cluster kernel leaves it to backward to list the long rows: until then they are counted here
+    std::vector<int32_t> seg;
+    if (h->have_forward && h->plan.blocks && c.U) {
+        seg.resize(c.U);                         // (a table's last row ends where the entry behind it begins)
+        CK(h, cudaMemcpy(seg.data(), h->wk.seg, sizeof(int32_t) * c.U, cudaMemcpyDeviceToHost));
+        c.hot_rows = 0; c.hot_occ = 0;
+    }
     for (int t = 0; t < h->T; ++t) {
-        out4[1] += ue[t] - us[t];
-        if (c.dropped && ue[t] > us[t]) {        // the sort puts a table's out-of-range ids into one pseudo row behind the others; leave it out
+        int32_t rows = ue[t] - us[t];
+        if (c.dropped && rows > 0) {             // the sort puts a table's out-of-range ids into one pseudo row behind the others; leave it out
             int32_t last = 0;
             CK(h, cudaMemcpy(&last, h->wk.uniq_row + ue[t] - 1, sizeof(int32_t), cudaMemcpyDeviceToHost));
-            if (last >= h->tables[t].N) --out4[1];
+            if (last >= h->tables[t].N) --rows;
+        }
+        out4[1] += rows;
+        if (seg.empty()) continue;
+        for (int32_t k = us[t]; k < us[t] + rows; ++k) {
+            const uint32_t m = (uint32_t)(seg[k + 1] - seg[k]);
+            if (m > hot_threshold(c.L)) { ++c.hot_rows; c.hot_occ += m; }
         }
     }
     out4[2] = (int64_t)c.dropped;

@@ -332,3 +332,26 @@ def test_forward_waits_for_what_the_caller_put_in_front_of_it(what):
         assert np.array_equal(outs[k].cpu().numpy(), o.forward(b[0], b[1], cfg.batch)), f"step {k + 1}"
         o.backward(b[2], cfg.lr, k + 1)
     h.close()
+
+
+@pytest.mark.parametrize("counts", [(3000, 900), (8000, 7000), (160000, 150100)])
+def test_step_info_is_the_same_before_and_after_backward(counts):
+    from paper_2010_11305_b200 import binding as mpe
+    rng = np.random.default_rng(2)
+    ids = [np.concatenate([_skewed(rng, 5000, c - 700), np.full(400, 7), np.full(300, 9000 + t)]) for t, c in enumerate(counts)]
+    idx, off, grad = (torch.from_numpy(x).cuda() for x in _batch(rng, [rng.permutation(x) for x in ids], 16, 4))
+    h = mpe.Mpe([5000] * len(counts), 4, 8, 0.05, 8, mpe.LFU)
+    out = torch.empty(16, 4 * len(counts), device="cuda")
+    ref = np.array([0] * 6, np.int64)
+    threshold = 64 if sum(counts) <= 1 << 20 else 256
+    for x in ids:
+        n = np.bincount(x[x < 5000])
+        ref += [int(n.sum()), int((n > 0).sum()), 300, int((n > threshold).sum()), int(n[n > threshold].sum()), 0]
+    for step in (1, 2):
+        h.forward(idx, off, 16, out)
+        torch.cuda.synchronize()
+        before = np.array(h.step_info())
+        h.backward(grad, 0.1, step)
+        after = np.array(h.step_info())
+        assert np.array_equal(before[:5], ref[:5]) and np.array_equal(after[:5], ref[:5]) and ref[3] > 0, (before, after, ref)
+    h.close()
