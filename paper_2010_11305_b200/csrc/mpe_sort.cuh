@@ -324,11 +324,10 @@ k_sort_scatter(const uint2* __restrict__ pairs_in, uint2* __restrict__ pairs_out
             gb = (uint32_t)seg_start[t] + block_exclusive_scan<SORT_THREADS>(mine, &all, scan_tmp);
         } else {
             gb = sort_look_back(word, local, tag, &poison);
-            poison |= s_ticket[2] != 0;
         }
         st_relaxed_u64(word, sort_word(tag, SORT_PREFIX | (poison ? SORT_POISON : 0ULL), gb + tot));
         goff[threadIdx.x] = gb - ds;                                           // global position = goff + tile-local position
-        if (__syncthreads_or(poison)) {                                        // a look-back gave up: write nothing, abandon the step
+        if (__syncthreads_or(poison || (s_ticket[2] && local))) {              // a look-back gave up: write nothing, abandon the step
             if (threadIdx.x == 0) { atomicAdd(&ctl->timeout, 1u); *abort_flag = 1; }
             continue;
         }
