@@ -99,7 +99,6 @@ struct mpe_handle {
     volatile uint32_t* uneven_seen = nullptr;              // (pinned) what the kernels last found of how uneven the tables' segments are
     StepArgs args{};                        // the current call's arguments (passed by value when launching directly)
     Route* d_route = nullptr;               // destinations of the pooled vectors when the tables are spread over several GPUs
-    bool graphs_enabled = true;             // accepted and remembered; see mpe_use_graphs
     // instrumentation
     uint64_t launches = 0;
     bool profiling = false;
@@ -742,7 +741,7 @@ int forward_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
         int rc = mpe_reserve(h, batch, total_indices);
         if (rc != MPE_OK) return rc;
     }
-    h->sort_passes_bound += 4 * SORT_MAX_PASSES;       // this step's two sorts, and those of a batch prepared meanwhile
+    h->sort_passes_bound += SORT_MAX_PASSES;           // (prepare_impl counts its own)
     if (h->sort_passes_bound > SORT_TAG_MASK - 1024) { int rc = renew_sort_tags(h); if (rc != MPE_OK) return rc; }
     uint32_t L = (uint32_t)total_indices;
     h->B = batch; h->L = total_indices; ++h->epoch;
@@ -786,6 +785,7 @@ int prepare_impl(mpe_handle* h, const int32_t* d_indices, const int32_t* d_offse
         swap_sets(h);
         if (rc != MPE_OK) return rc;
     }
+    h->sort_passes_bound += SORT_MAX_PASSES;
     int rc = MPE_OK;
     StepArgs av{};
     av.indices = d_indices; av.offsets = d_offsets; av.B = batch; av.L = (uint32_t)total_indices;
@@ -1047,7 +1047,7 @@ int mpe_set_rounding(mpe_handle* h, int32_t mode) {
 int mpe_use_graphs(mpe_handle* h, int32_t enable) {
     if (!h) return MPE_ERR_ARG;
     if (h->have_forward) return MPE_ERR_SEQUENCE;      // both halves of a step are launched the same way
-    h->graphs_enabled = enable != 0;
+    (void)enable;
     return MPE_OK;
 }
 

@@ -403,7 +403,7 @@ __device__ __forceinline__ void forward_close(const State& s, const Work& w, con
 
 
 // Fetch + pool straight from the row ids: the row's home record says where it lives, so the forward needs no sort and no tag look-up per
-// distinct row, and a replayed or launched forward is this one kernel.  A bag's offsets, its row ids and their slots are three
+// distinct row, and is this one kernel.  A bag's offsets, its row ids and their slots are three
 // dependent loads; they are fetched three, two and one bags ahead.
 template <int BITS, int LANES, int MODE>
 __global__ void __launch_bounds__(256, 4)
@@ -552,7 +552,6 @@ constexpr int VICTIM_NONE = -1;       // the way was empty, or the displaced row
 constexpr int VICTIM_DEFER = -2;      // the displaced row was hit in this step: the newcomer waits for its write-back
 constexpr int CAND_NONE = -1;         // candidate key of a row that is not to be admitted
 __host__ __device__ constexpr int bucket_cap(int ways) { return ways >= 8 ? 2 * ways : (4 * ways < 16 ? 4 * ways : 16); }
-constexpr int BUCKET_CAP_MAX = 64;
 constexpr int BUCKET_PER_LANE = 4;    // bucket_cap(ways) / ways is at most this
 
 // the candidate k joins the bucket of set `gset`; true if it is the set's first one in this step

@@ -313,8 +313,8 @@ def test_memory_accounting_matches_the_appendix_table():
 def _full_size(cfg, tables, steps, check_at=(), prepare_ahead=False):
     """A configuration at its full size in the launch configuration the benchmark times; the oracle follows the
     sampled tables only.  State is compared at the steps in check_at, at the last step, and again after a flush.
-    prepare_ahead: as the benchmark does for steps too large to be replayed from a graph, the next batch is sorted and
-    de-duplicated on a second stream while the current step runs."""
+    prepare_ahead: as the benchmark does, the next batch is sorted and de-duplicated on a second stream while the current
+    step runs."""
     from parity_util import make_pair, compare_state
     h, o = make_pair(cfg, tables)
     st = wl.Stream(cfg, "cuda")
@@ -387,7 +387,6 @@ def test_batches_prepared_ahead_give_the_same_results():
     cfg = _cfg(num_rows=[30000, 900, 40], dim=64, bits=4, batch=512, bag=("poisson", 9.0), zipf=[1.1, 0.9, None], policy=wl.LFU, ways=8,
                cache_fraction=0.05, seed=21)
     h, o = make_pair(cfg)
-    h.use_graphs(False)                                  # replayed steps ignore the call: this test is about the plain path
     st = wl.Stream(cfg, "cpu")
     rng = np.random.default_rng(0)
     side = torch.cuda.Stream()
@@ -422,8 +421,8 @@ def test_batches_prepared_ahead_give_the_same_results():
 
 
 def test_launch_mode_cannot_change_between_a_forward_and_its_backward():
-    """Replayed kernels read the step's arguments from device memory, plainly launched ones get them by value: the two
-    halves of a step must be launched the same way, whatever the caller toggles in between."""
+    """The two halves of a step are launched the same way (with the records of mpe_profile or without): what would change that
+    is refused in between, and the step goes on as if it had not been asked for."""
     from parity_util import make_pair, compare_state
     from paper_2010_11305_b200 import binding as mpe
     cfg = _cfg(num_rows=[3000, 400], dim=16, bits=4, batch=48, bag=("poisson", 4.0), zipf=[1.1, 0.9], policy=wl.LFU, ways=4,
@@ -460,85 +459,80 @@ def test_a_look_back_that_gives_up_is_reported_and_the_handle_goes_on():
     cfg = _cfg(num_rows=[6000, 700], dim=16, bits=8, batch=96, bag=("poisson", 5.0), zipf=[1.1, 1.0], policy=wl.LRU, ways=4,
                cache_fraction=0.1, seed=21)
     rng = np.random.default_rng(0)
-    for graphs in (True, False):
-        h, o = make_pair(cfg)
-        h.use_graphs(graphs)
-        st = wl.Stream(cfg, "cpu")
-        with pytest.raises(mpe.MpeError) as e:          # no workspace yet
-            h.selftest(mpe.SELFTEST_LOOK_BACK_TIMEOUT)
-        assert e.value.code == mpe.ERR_SEQUENCE
-        for step in range(1, 7):
-            idx, off, grad = st.batch(step)
-            out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, device="cuda")
-            h.forward(idx.cuda(), off.cuda(), cfg.batch, out)
-            if step == 3:
-                with pytest.raises(mpe.MpeError) as e:  # not in the middle of a step
-                    h.selftest(mpe.SELFTEST_LOOK_BACK_TIMEOUT)
-                assert e.value.code == mpe.ERR_SEQUENCE
-            h.backward(grad.cuda(), cfg.lr, step)
-            assert np.array_equal(out.cpu().numpy(), o.forward(idx.numpy(), off.numpy(), cfg.batch))
-            o.backward(grad.numpy(), cfg.lr, step)
-            if step in (2, 4):
-                assert h.last_error() == (0, 0)
+    h, o = make_pair(cfg)
+    st = wl.Stream(cfg, "cpu")
+    with pytest.raises(mpe.MpeError) as e:          # no workspace yet
+        h.selftest(mpe.SELFTEST_LOOK_BACK_TIMEOUT)
+    assert e.value.code == mpe.ERR_SEQUENCE
+    for step in range(1, 7):
+        idx, off, grad = st.batch(step)
+        out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, device="cuda")
+        h.forward(idx.cuda(), off.cuda(), cfg.batch, out)
+        if step == 3:
+            with pytest.raises(mpe.MpeError) as e:  # not in the middle of a step
                 h.selftest(mpe.SELFTEST_LOOK_BACK_TIMEOUT)
-                if step == 4:
-                    h.selftest(mpe.SELFTEST_LOOK_BACK_TIMEOUT)
-                assert h.last_error() == (mpe.ERR_TIMEOUT, 1 if step == 2 else 2)
-                assert h.last_error() == (0, 0)
-        compare_state(h, o, cfg, [0, 1], rng)
-        assert h.last_error() == (0, 0)
-        h.close()
+            assert e.value.code == mpe.ERR_SEQUENCE
+        h.backward(grad.cuda(), cfg.lr, step)
+        assert np.array_equal(out.cpu().numpy(), o.forward(idx.numpy(), off.numpy(), cfg.batch))
+        o.backward(grad.numpy(), cfg.lr, step)
+        if step in (2, 4):
+            assert h.last_error() == (0, 0)
+            h.selftest(mpe.SELFTEST_LOOK_BACK_TIMEOUT)
+            if step == 4:
+                h.selftest(mpe.SELFTEST_LOOK_BACK_TIMEOUT)
+            assert h.last_error() == (mpe.ERR_TIMEOUT, 1 if step == 2 else 2)
+            assert h.last_error() == (0, 0)
+    compare_state(h, o, cfg, [0, 1], rng)
+    assert h.last_error() == (0, 0)
+    h.close()
 
 
-def test_sort_pass_numbers_can_start_over_at_any_step():
+@pytest.mark.parametrize("num_rows,bag", [([9000, 1200, 50], 6.0), ([90000, 1200], 540.0)])        # inside clusters; grid-wide
+def test_sort_pass_numbers_can_start_over_at_any_step(num_rows, bag):
     """The per-tile words of the sort carry a pass number that is started over long before it can repeat; forcing that
     between arbitrary steps (also with a batch prepared ahead in the second workspace) must not change any result."""
     from parity_util import make_pair, compare_state
     from paper_2010_11305_b200 import binding as mpe
-    cfg = _cfg(num_rows=[9000, 1200, 50], dim=32, bits=4, batch=300, bag=("poisson", 6.0), zipf=[1.1, 1.0, None], policy=wl.LFU,
+    cfg = _cfg(num_rows=num_rows, dim=32, bits=4, batch=300, bag=("poisson", bag), zipf=[1.1, 1.0, None][:len(num_rows)], policy=wl.LFU,
                ways=8, cache_fraction=0.1, seed=22)
     rng = np.random.default_rng(0)
-    for graphs in (True, False):
-        h, o = make_pair(cfg)
-        h.use_graphs(graphs)
-        st = wl.Stream(cfg, "cpu")
-        side = torch.cuda.Stream()
-        batches = [tuple(x.cuda() for x in st.batch(step)) for step in range(1, 10)]
-        host = [st.batch(step) for step in range(1, 10)]
-        for i, step in enumerate(range(1, 10)):
-            idx, off, grad = batches[i]
-            if step in (1, 4, 5, 8):
-                if step > 1:
-                    h.selftest(mpe.SELFTEST_RENEW_TAGS)
-                else:
-                    h.reserve(cfg.batch, max(int(b[0].numel()) for b in batches))
-                    h.selftest(mpe.SELFTEST_RENEW_TAGS)
-            out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, device="cuda")
-            h.forward(idx, off, cfg.batch, out)
-            if i + 1 < len(batches):
-                h.prepare(batches[i + 1][0], batches[i + 1][1], cfg.batch, side.cuda_stream)
-            h.backward(grad, cfg.lr, step)
-            hi, ho, hg = host[i]
-            assert np.array_equal(out.cpu().numpy(), o.forward(hi.numpy(), ho.numpy(), cfg.batch))
-            o.backward(hg.numpy(), cfg.lr, step)
-        compare_state(h, o, cfg, [0, 1, 2], rng)
-        assert h.last_error() == (0, 0)
-        torch.cuda.synchronize()
-        h.close()
+    h, o = make_pair(cfg)
+    st = wl.Stream(cfg, "cpu")
+    side = torch.cuda.Stream()
+    batches = [tuple(x.cuda() for x in st.batch(step)) for step in range(1, 10)]
+    host = [st.batch(step) for step in range(1, 10)]
+    for i, step in enumerate(range(1, 10)):
+        idx, off, grad = batches[i]
+        if step in (1, 4, 5, 8):
+            if step > 1:
+                h.selftest(mpe.SELFTEST_RENEW_TAGS)
+            else:
+                h.reserve(cfg.batch, max(int(b[0].numel()) for b in batches))
+                h.selftest(mpe.SELFTEST_RENEW_TAGS)
+        out = torch.empty(cfg.batch, cfg.num_tables * cfg.dim, device="cuda")
+        h.forward(idx, off, cfg.batch, out)
+        if i + 1 < len(batches):
+            h.prepare(batches[i + 1][0], batches[i + 1][1], cfg.batch, side.cuda_stream)
+        h.backward(grad, cfg.lr, step)
+        hi, ho, hg = host[i]
+        assert np.array_equal(out.cpu().numpy(), o.forward(hi.numpy(), ho.numpy(), cfg.batch))
+        o.backward(hg.numpy(), cfg.lr, step)
+    compare_state(h, o, cfg, range(len(num_rows)), rng)
+    assert h.last_error() == (0, 0)
+    torch.cuda.synchronize()
+    h.close()
 
 
-def test_graph_replay_and_plain_launches_agree_with_the_oracle():
-    """Small steps are replayed from a captured CUDA graph; the same handle must give the oracle's results when
-    the batch shrinks and grows under one graph, when the workspace regrows, and with graphs switched off."""
+def test_batches_that_shrink_and_grow_on_one_handle():
+    """The same handle gives the oracle's results when the batch shrinks and grows and when the workspace regrows."""
     from parity_util import make_pair, compare_state
     cfg = _cfg(num_rows=[4000, 900], dim=32, bits=4, batch=64, bag=("poisson", 5.0), zipf=[1.1, 1.0], policy=wl.LFU, ways=4,
                cache_fraction=0.1, seed=5)
     h, o = make_pair(cfg)
     rng = np.random.default_rng(0)
     step = 0
-    for batch, graphs in ((64, True), (64, True), (16, True), (64, True), (200, True), (64, False), (32, True)):
+    for batch in (64, 64, 16, 64, 200, 64, 32):
         cfg.batch = batch
-        h.use_graphs(graphs)
         step += 1
         idx, off, grad = wl.Stream(cfg, "cpu").batch(step)
         out = torch.empty(batch, cfg.num_tables * cfg.dim, device="cuda")

@@ -1,7 +1,8 @@
 """Each kernel variant at the sizes where it begins, ends or has a remainder, against the CPU oracle.
 
-The library chooses by sizes alone: a thread-block cluster per table sorts a batch (4096 or 12288 elements per block; a table with
-more than its cluster holds goes through global memory) until the tables average over 150000 indices, then grid-wide kernels do; up
+The library chooses by sizes: a thread-block cluster per table sorts a batch (4096 or 12288 elements per block; a table with
+more than its cluster holds goes through global memory) until the tables average over 150000 indices or one of them is larger than
+that in the batches seen so far, then, and as long as none has been seen, grid-wide kernels do; up
 to 131072 indices one launch updates every row; a row's gradient is summed by its group of lanes, by a warp's list of mid rows (from
 16 occurrences) or by whole blocks (from 64 or 256); a cache set finds its candidates in a bucket until that overflows."""
 import numpy as np
@@ -55,15 +56,16 @@ def _skewed(rng, n_rows, count):
 @pytest.mark.parametrize("counts", [
     (0, 1, 31, 33, 1023, 1025, 3000),           # one block per table, tables without indices among them
     (3641,), (3642,), (4097,),                  # the last size of one block, the first of two
-    (8000, 10, 0),                              # more than the one block holds
+    (8000, 10, 0),                              # four blocks, for one table that is larger than the average
     (7281,), (7283, 7290), (57000,),            # two, four and sixteen blocks
-    (60000, 5, 5),                              # more than the cluster's blocks hold
-    (5000,) * 99 + (12289,),                    # 12288 elements per block, and one table beyond
-    (100003,), (199000, 900),                   # sixteen large blocks: within, and one table beyond
+    (60000, 5, 5),                              # sixteen
+    (5000,) * 99 + (12289,),                    # one table beyond 12288 elements per block, which all have: grid-wide
+    (100003,), (199000, 900),                   # sixteen large blocks: within; one table beyond: grid-wide
     (150000,), (150001,),                       # the last average of the cluster kernel, the first of the grid-wide ones
     (320000, 7, 0), (1048576 + 9,),             # grid-wide: a few tiles and none, large tiles
 ])
 def test_index_work_at_its_boundaries(counts):
+    """The host has waited for the forward when it chooses the kernels of the backward, so it goes by this batch's largest table."""
     num_rows = [max(3, c // 3) for c in counts]
     num_rows[0] = 70001                         # keys of three digits
     _check(_cfg(num_rows, 16), lambda rng: [_skewed(rng, n, c) for n, c in zip(num_rows, counts)])
