@@ -125,7 +125,7 @@ class Mpe:
         self.ways = self.cache_geometry(0)[1]
 
     def close(self):
-        if getattr(self, "_h", None):
+        if getattr(self, "_h", None) and _lib is not None:          # (the module may be gone already when the interpreter ends)
             _lib.mpe_destroy(self._h)
             self._h = None
 

@@ -187,6 +187,41 @@ int resident_blocks(mpe_handle* h, K kernel, int threads, size_t smem) {
     return n;
 }
 
+// One word of pinned host memory per handle.  Page-locking memory costs about 2 ms however little it is, so the process's handles share a
+// page, which goes with the last of them; a handle that finds all of its words taken locks a page of its own.
+class HostWords {
+public:
+    volatile uint32_t* take() {
+        std::lock_guard<std::mutex> lock(lock_);
+        if (!page_ && !(page_ = lock_page())) return nullptr;
+        for (int i = 0; i < WORDS; ++i)
+            if (!taken_[i]) { taken_[i] = true; ++live_; page_[i] = 0; return page_ + i; }
+        uint32_t* own = lock_page();
+        if (own) *own = 0;
+        return own;
+    }
+    void give_back(volatile uint32_t* word) {
+        if (!word) return;
+        std::lock_guard<std::mutex> lock(lock_);
+        uint32_t* p = const_cast<uint32_t*>(word);
+        if (!page_ || p < page_ || p >= page_ + WORDS) { cudaFreeHost(p); return; }
+        taken_[p - page_] = false;
+        if (--live_ == 0) { cudaFreeHost(page_); page_ = nullptr; }
+    }
+private:
+    static constexpr int WORDS = 64;
+    static uint32_t* lock_page() {
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, WORDS * sizeof(uint32_t), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+        return static_cast<uint32_t*>(p);
+    }
+    std::mutex lock_;
+    uint32_t* page_ = nullptr;
+    bool taken_[WORDS] = {};
+    int live_ = 0;
+};
+HostWords g_host_words;
+
 int bits_for(uint32_t v) { int b = 1; while (b < 32 && (v >> b) != 0) ++b; return b; }
 
 template <class T>
@@ -493,8 +528,7 @@ int mpe_create_placed(mpe_handle** out, const mpe_table_spec* tables, int32_t nu
     int rc = MPE_OK;
     auto fail = [&](int code) { mpe_destroy(h); return code; };
     if ((rc = dmalloc(h, &h->d_tables, num_tables, nullptr)) != MPE_OK) return fail(rc);
-    if (cudaHostAlloc((void**)&h->uneven_seen, sizeof(uint32_t), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) return fail(MPE_ERR_NOMEM);
-    *h->uneven_seen = 0;
+    if (!(h->uneven_seen = g_host_words.take())) return fail(MPE_ERR_NOMEM);
     s.tables = h->d_tables;
     if (h->table_on_host) {
         // capacity tiering: the low-precision table stays in pinned host memory and is read and written in place over
@@ -1164,11 +1198,12 @@ int mpe_destroy(mpe_handle* h) {
         cudaFree(sl.idx); cudaFree(sl.off); cudaFree(sl.grad); cudaFree(sl.out);
     }
     free_workspace(h);
+    g_host_words.give_back(h->uneven_seen);
     State& s = h->st;
     if (h->table_on_host) { cudaFreeHost(s.low.codes); cudaFreeHost(s.low.sb); cudaFree(s.home); }
     else if (h->row_records) cudaFree(h->row_records);
     else { cudaFree(s.low.codes); cudaFree(s.low.sb); cudaFree(s.home); }
-    cudaFree(h->d_route); cudaFreeHost(const_cast<uint32_t*>(h->uneven_seen));
+    cudaFree(h->d_route);
     cudaFree(h->d_tables); cudaFree(s.G); cudaFree(s.slab);
     cudaFree(s.tags); cudaFree(s.ts); cudaFree(s.hit_epoch); cudaFree(s.hit_k); cudaFree(s.floor); cudaFree(s.set_cnt); cudaFree(s.chain); cudaFree(s.bucket); cudaFree(s.stats);
     for (auto& r : h->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }

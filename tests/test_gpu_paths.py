@@ -357,3 +357,38 @@ def test_step_info_is_the_same_before_and_after_backward(counts):
         after = np.array(h.step_info())
         assert np.array_equal(before[:5], ref[:5]) and np.array_equal(after[:5], ref[:5]) and ref[3] > 0, (before, after, ref)
     h.close()
+
+
+def test_many_handles_at_once():
+    """Handles share a page of host words: 70 are more than it holds, and a word is as good as new for its next handle."""
+    from paper_2010_11305_b200 import binding as mpe
+    idx, off, grad = (torch.from_numpy(x).cuda() for x in _batch(np.random.default_rng(3), [np.arange(300) % 90], 8, 4))
+    outs = []
+
+    def use(h):
+        out = torch.empty(8, 4, device="cuda")
+        for step in (1, 2):
+            h.forward(idx, off, 8, out)
+            torch.cuda.synchronize()
+            h.backward(grad, 0.1, step)
+        h.forward(idx, off, 8, out)
+        assert h.last_error() == (0, 0)
+        outs.append(out.cpu())
+
+    def make(n):
+        return [mpe.Mpe([100], 4, 8, 0.1, 2, mpe.LRU, seed=9) for _ in range(n)]
+
+    first = make(70)
+    for h in first[::7] + first[-2:]:
+        use(h)
+    for h in first[1::2]:
+        h.close()
+    second = make(40)
+    for h in second[::9]:
+        use(h)
+    for h in first[::2] + second:
+        h.close()
+    for h in make(2):
+        use(h)
+        h.close()
+    assert all(torch.equal(outs[0], o) for o in outs)
