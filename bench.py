@@ -35,28 +35,25 @@ NOMINAL_HBM_GBS = 8000.0
 # proportion to the indices processed): dram__bytes_read.sum + dram__bytes_write.sum per index of the batch, and the
 # limiter the counters point at.  The summaries under profiles/ give the commands and the counters.
 KERNEL_EVIDENCE = {
-    "update": {"dram_bytes_per_index": 103.6, "bound": "issue",
-               "evidence": "74 % of the issue slots used, 321 warp instructions per distinct row; DRAM 25 %, L2 30 % of peak",
+    "update": {"dram_bytes_per_index": 123.6, "bound": "issue",
+               "evidence": "71 % of the issue slots used, 310 warp instructions per distinct row; DRAM 30 %, L2 32 % of peak",
                "profile": "profiles/step_kernels_cfg4_8tables.md"},
-    "pool": {"dram_bytes_per_index": 67.6, "bound": "latency",
-             "evidence": "6.1 long-scoreboard stall cycles per issue at 49 % of the warp slots (64 registers); DRAM 18 %, L2 20 % of peak; 60 % of the sectors hit in L1",
+    "pool": {"dram_bytes_per_index": 80.8, "bound": "latency",
+             "evidence": "5.6 long-scoreboard stall cycles per issue at 49 % of the warp slots (64 registers); DRAM 22 %, L2 23 % of peak; 58 % of the sectors hit in L1",
              "profile": "profiles/step_kernels_cfg4_8tables.md"},
-    "hot_partial": {"dram_bytes_per_index": 22.8, "bound": "l2-latency",
-                    "evidence": "gradient rows come from L2 (82 % hits, 37 % of its throughput), 7.5 long-scoreboard stall cycles per issue at 24 % of the warp slots (kept small on purpose: it runs beside other kernels)",
+    "hot_partial": {"dram_bytes_per_index": 23.0, "bound": "l2-latency",
+                    "evidence": "gradient rows come from L2 (81 % hits, 39 % of its throughput), 7.2 long-scoreboard stall cycles per issue at 24 % of the warp slots (kept small on purpose: it runs beside other kernels)",
                     "profile": "profiles/step_kernels_cfg4_8tables.md"},
     # on the small case a pass of the sort is L2 resident, so its DRAM traffic does not scale to the full size: none given
     "sort_scatter": {"dram_bytes_per_index": None, "bound": "latency",
-                     "evidence": "short scoreboard 6.1 (ranking through shared-memory counters), long scoreboard 5.6 (tile load, look-back) and barrier 2.6 stall cycles per issue; 35 % of the issue slots; DRAM 14 %, L2 24 % of peak",
-                     "profile": "profiles/k_sort_scatter_cfg4_9tables.md"},
-    "broadcast": {"dram_bytes_per_index": 14.1, "bound": "l2",
-                  "evidence": "64 % of the L2 throughput (4-byte scatters and gathers inside a table's window), 80 long-scoreboard and 13.6 lg_throttle stall cycles per issue",
-                  "profile": "profiles/k_broadcast_cfg4_8tables.md"},
-    "priority": {"dram_bytes_per_index": 16.2, "bound": "dram-latency",
-                 "evidence": "one random read-modify-write of a counter per distinct row: 30 long-scoreboard stall cycles per issue, 13 % of the issue slots",
-                 "profile": "profiles/small_kernels_cfg4_8tables.md"},
-    "policy": {"dram_bytes_per_index": 6.3, "bound": "latency",
-               "evidence": "8.8 long-scoreboard stall cycles per issue, 47 % of the issue slots",
-               "profile": "profiles/small_kernels_cfg4_8tables.md"},
+                     "evidence": "short scoreboard 5.8 (ranking through shared-memory counters), long scoreboard 5.7 (tile load, look-back) and barrier 2.7 stall cycles per issue; 34 % of the issue slots; DRAM 14 %, L2 25 % of peak",
+                     "profile": "profiles/step_kernels_cfg4_8tables.md"},
+    "priority": {"dram_bytes_per_index": 19.2, "bound": "dram-latency",
+                 "evidence": "one random read-modify-write of a home record per distinct row: 42 long-scoreboard stall cycles per issue, 11 % of the issue slots",
+                 "profile": "profiles/step_kernels_cfg4_8tables.md"},
+    "policy": {"dram_bytes_per_index": 7.8, "bound": "latency",
+               "evidence": "4.8 long-scoreboard stall cycles per issue, 49 % of the issue slots",
+               "profile": "profiles/step_kernels_cfg4_8tables.md"},
 }
 
 
@@ -129,7 +126,7 @@ def describe(cfg):
             f"cache {cfg.cache_fraction:g} x rows, {cfg.ways or 32}-way {pol}, batch {cfg.batch}, bags {cfg.bag}, {opt}")
 
 
-def byte_model(cfg, L, U, U_hit, occ_hit, admissions, evictions, hot_occ, passes_main, passes_cand):
+def byte_model(cfg, L, U, U_hit, occ_hit, admissions, evictions, hot_occ, passes):
     """Algorithmic bytes of one step, counted both ways.
 
     per access  -- what the METHOD moves if every access goes to memory (the paper's effective-bandwidth numerator,
@@ -142,8 +139,8 @@ def byte_model(cfg, L, U, U_hit, occ_hit, admissions, evictions, hot_occ, passes
 
     Returns (per_access_step, compulsory_step, per_kernel) with per_kernel[name] = (per-access bytes, compulsory bytes,
     basis).  The per-kernel figures hold the method's bytes only (none of this implementation's bookkeeping arrays);
-    kernels that are bookkeeping of this implementation and nothing else (the sort passes, the scatter of the probe
-    results) are given the bytes their own algorithm has to move, and say so in `basis`.
+    kernels that are bookkeeping of this implementation and nothing else (the sort passes, the lists of distinct rows)
+    are given the bytes their own algorithm has to move, and say so in `basis`.
     """
     d, T, B = cfg.dim, cfg.num_tables, cfg.batch
     rb = d * cfg.bits // 8 + (0 if cfg.bits == 16 else 8)      # codes + FP32 scale + FP32 bias (none for an FP16 table)
@@ -164,16 +161,14 @@ def byte_model(cfg, L, U, U_hit, occ_hit, admissions, evictions, hot_occ, passes
     m["update"] = (cold_occ * fb + rows_rw + opt, min(cold_occ * fb, out_bytes) + rows_rw + opt, "method")
     m["hot_partial"] = (hot_occ * fb, min(hot_occ * fb, out_bytes), "method")
     m["priority"] = (pv, pv, "method")
-    m["probe"] = (4 * cfg.ways * U, 4 * cfg.ways * U, "method (tag reads)")
     m["policy"] = (U_miss * (4 if cfg.policy == wl.LFU else 0) + admissions * 8 * cfg.ways,) * 2 + ("method (priority values of candidates and sets)",)
-    sort_rw = passes_main * 16 * L + passes_cand * 16 * U
+    sort_rw = passes * 16 * L
     m["sort_scatter"] = (sort_rw, sort_rw, "radix-sort pass: key + payload read and written")
-    m["sort_digits"] = (4 * L + 8 * U,) * 2 + ("radix sort: the keys read once, ahead of the passes",)
+    m["sort_digits"] = (8 * L,) * 2 + ("radix sort: the keys read once, ahead of the passes",)
     m["make_keys"] = (4 * L + 4 * T * B, 4 * L + 4 * T * B, "indices and offsets read")
-    m["unique"] = (4 * L + 4 * U, 4 * L + 4 * U, "sorted keys read, distinct rows written")
+    m["table_sort"] = (8 * L + 4 * L + 12 * U,) * 2 + ("records read, samples in order and distinct rows written",)
     m["unique_count"] = (4 * L, 4 * L, "sorted keys read")
     m["unique_write"] = (4 * L + 4 * U, 4 * L + 4 * U, "sorted keys read, distinct rows written")
-    m["broadcast"] = (8 * L, 8 * L, "bookkeeping: per-index slot and sample id written")
     return per_access, compulsory, m
 
 
@@ -366,10 +361,8 @@ def run_ours(args, cfg, rank, world, local_rank):
     if rank != 0:
         return None
 
-    passes_main = (max(cfg.num_rows).bit_length() + 7) // 8
-    max_sets = max(h.cache_geometry(t)[0] for t in range(cfg.num_tables))
-    passes_cand = (max(max_sets, 1).bit_length() + 7) // 8 if max_sets else 0
-    per_access, compulsory, model = byte_model(cfg, L, U, U_hit, occ_hit, adm, evi, hot_occ, passes_main, passes_cand)
+    passes = (max(cfg.num_rows).bit_length() + 7) // 8
+    per_access, compulsory, model = byte_model(cfg, L, U, U_hit, occ_hit, adm, evi, hot_occ, passes)
     per_access, compulsory = float(per_access), float(compulsory)
     ms_step = ms / K
     ms_median = float(np.median(per_step_ms))
@@ -384,7 +377,7 @@ def run_ours(args, cfg, rank, world, local_rank):
         "warmup": args.warmup, "ms_per_step": ms_step, "ms_per_step_median": ms_median, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": describe(cfg), "l2": "inputs larger than L2; a new batch every step",
-                   "launch": "plain launches; per-kernel times from a second pass without the preparation",
+                   "launch": "kernel by kernel; per-kernel times from a second pass without the preparation",
                    "next_batch": "sorted ahead on a second stream (mpe_prepare) while the current step runs" if ahead else "not prepared ahead",
                    "sharding": "each rank trains its own tables (no data-path collective)" if world > 1 else "one GPU"},
         "clocks": clocks,

@@ -64,7 +64,7 @@ def test_bench_evidence_points_at_committed_summaries():
     import sys
     sys.path.insert(0, ROOT)
     import bench
-    assert {"update", "pool", "hot_partial", "sort_scatter", "broadcast"} <= set(bench.KERNEL_EVIDENCE)
+    assert {"update", "pool", "hot_partial", "sort_scatter", "priority", "policy"} == set(bench.KERNEL_EVIDENCE)
     for name, ev in bench.KERNEL_EVIDENCE.items():
         path = os.path.join(ROOT, ev["profile"])
         assert os.path.isfile(path) and path.endswith(".md"), f"{name}: {ev['profile']}"
